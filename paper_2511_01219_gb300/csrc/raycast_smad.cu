@@ -46,7 +46,23 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 
 __device__ __forceinline__ uint32_t isqrt_q16(int c2) {
-    // floor(sqrt(c2 * 2^32)): float estimate, one Newton correction, exact fix-up
+    // floor(sqrt(c2 * 2^32)).  Up to 2^20 (1024 cells: every range limit of 50 m at 5 cm) the float estimate is off
+    // by less than 8 (2 roundings of 2^-24 on a root below 2^26), so err = c2 2^32 - r^2 lies within 2 r 8 < 2^30 and
+    // 32-bit arithmetic holds it (the low word of c2 2^32 is 0); a few steps then make it exact.
+    if ((unsigned)c2 <= (1u << 20)) {
+        uint32_t r = (uint32_t)(sqrtf((float)c2) * 65536.0f);
+        int err = (int)(0u - r * r);
+        while (err < 0) {
+            --r;
+            err += (int)(2u * r + 1u);
+        }
+        while (err > (int)(2u * r)) {
+            err -= (int)(2u * r + 1u);
+            ++r;
+        }
+        return r;
+    }
+    // else float estimate, one Newton correction, exact fix-up
     const unsigned long long N = (unsigned long long)(unsigned)c2 << 32;
     unsigned long long r = (unsigned long long)(sqrtf((float)c2) * 65536.0f);
     long long err = (long long)(N - r * r);
@@ -182,99 +198,117 @@ __device__ __forceinline__ uint32_t cast_ray(const uint64_t *__restrict__ bits, 
 // and +y.  Each of the four frames is stored as a walk frame: cells outside
 // the map are set and a last column and row of full tiles follow the map, so
 // the first cell outside the map stops the ray like an occupied one and is
-// recognised after the loop, which needs no bounds test per tile.  In a tile
-// whose word is not zero, the word moved to the current cell
-// is ANDed with the table's bit board of the cells still ahead; on a
-// staircase that only moves +x and +y the cell order along the ray is the
-// row-major bit order, so the lowest common bit is the hit.  Otherwise the
-// ray leaves the tile at the cell of step min(selx[|dx| + nx], sely[|dy| +
-// ny]), nx and ny being the x- and y-steps to the tile's far edges.  An empty
-// tile is left as a whole box of empty tiles ahead (MapDev::reach) when that
-// box is larger: the run along the tile's row for a ray within about 14
-// degrees of the x axis, the run along its column within 14 degrees of the y
-// axis, the empty square otherwise; the same lookups then take the box's far
-// edges, since no cell inside it can stop the ray.  Same cells, same hit, same
-// range as cast_ray.
-__device__ __forceinline__ uint32_t walk_ray(const uint64_t *__restrict__ bits, const uint16_t *__restrict__ reach,
-                                             int W, int H, int TW, int TH, const RayTables &t, int ns, int j, int hx,
-                                             int hy, int2 d, int *hit, int *steps) {
-    const bool xneg = d.x <= 0, yneg = d.y <= 0;
-    const unsigned WB = (unsigned)TW + 1u;   // walk frame row, with the border column
-    const size_t frame = (size_t)((xneg ? 1 : 0) + (yneg ? 2 : 0)) * walk_frame_words(TW, TH);
-    const uint64_t *__restrict__ bq = bits + (size_t)TW * TH + frame;
-    const uint16_t *__restrict__ rq = reach + frame;
-    // which box of the packed reach the ray leaves: width (reach >> wsh) & 31, height (reach >> hsh) & 31, each
-    // at least 1 (bit 15 and up are 0, so a shift of 15 reads a side of 1 tile)
-    const long long adir = d.x < 0 ? -(long long)d.x : d.x, bdir = d.y < 0 ? -(long long)d.y : d.y;
-    const bool shallow = 4 * bdir <= adir, steep = 4 * adir <= bdir;
-    const unsigned wsh = shallow ? 5u : steep ? 15u : 0u;
-    const unsigned hsh = steep ? 10u : shallow ? 15u : 0u;
-    const int xlo = xneg ? 8 * TW - W : 0, ylo = yneg ? 8 * TH - H : 0;   // the map in the ray's frame
-    const int fx = xneg ? 8 * TW - 1 - hx : hx, fy = yneg ? 8 * TH - 1 - hy : hy;
-    const uint16_t *__restrict__ selx = t.selx + j;
-    const uint16_t *__restrict__ sely = t.sely + j;
-    const uint64_t *__restrict__ mk = t.mask + j;
-    const unsigned uns = (unsigned)ns;
+// recognised after the loop, which needs no bounds test per tile.
+//
+// The walk's state is the cell (cx, cy) alone: a cell k steps from the start
+// (fx, fy) has cx + cy = fx + fy + k, so a table's step index of a far edge
+// gives the other coordinate there with one subtraction, and the rows of the
+// tables are linear in cx, cy and cx + cy (the start is folded into the bases).
+// A tile is read through its boxes entry first (MapDev::reach: 0 exactly when
+// the tile is not empty).  A box of empty tiles is left at its far edges, the
+// run along the tile's row for a ray within about 14 degrees of the x axis, the
+// run along its column within 14 degrees of the y axis, the empty square
+// otherwise, at the cell of step min(selx[|dx| at the x edge], sely[|dy| at the
+// y edge]), since no cell inside it can stop the ray.  In a tile that is not
+// empty, the word moved to the current cell is ANDed with the table's bit board
+// of the cells still ahead; on a staircase that only moves +x and +y the cell
+// order along the ray is the row-major bit order, so the lowest common bit is
+// the hit; without one the ray leaves the tile as a box of one tile.  Only such
+// tiles load their word and board, together with the exit steps: two memory
+// round trips and at most five loads per move.  Same cells, same hit, same range
+// as cast_ray.
+//
+// Registers bound the kernel's warps: the tables share one allocation, and a
+// map's boxes lie behind its words in another, so a direction holds two 64-bit
+// bases and 32-bit indexes.
+struct RayDir {   // what the walks of one direction share
+    const uint64_t *__restrict__ bq;    // the direction's walk frame
+    const uint64_t *__restrict__ mk;    // the tables (RayTables)
+    unsigned rq;                        // the frame's boxes, 2-byte units from bq
+    unsigned selx, sely, jm;            // the direction's column: 2-byte units from mk, 8-byte units from mk
+    unsigned WB, ns;
+    unsigned wsh, hsh;                  // which sides of the packed boxes the ray leaves
+    int mx, my;                         // 8 TW - 1 (mirrored in x) or -1; 8 TH - 1 or -1
+
+    __device__ __forceinline__ void init(const uint64_t *bits, const uint16_t *reach, int TW, int TH,
+                                         const RayTables &t, int ns_, int j, int2 d) {
+        const bool xneg = d.x <= 0, yneg = d.y <= 0;
+        mx = xneg ? 8 * TW - 1 : -1;
+        my = yneg ? 8 * TH - 1 : -1;
+        WB = (unsigned)TW + 1u;   // walk frame row, with the border column
+        ns = (unsigned)ns_;
+        const size_t frame = (size_t)((xneg ? 1 : 0) + (yneg ? 2 : 0)) * walk_frame_words(TW, TH);
+        bq = bits + (size_t)TW * TH + frame;
+        rq = (unsigned)(reach + frame - reinterpret_cast<const uint16_t *>(bq));
+        mk = t.mask;
+        selx = t.selx + (unsigned)j;
+        sely = t.sely + (unsigned)j;
+        jm = (unsigned)j;
+        // box width (reach >> wsh) & 31, height (reach >> hsh) & 31, each at least 1 (bit 15 and up are 0, so a shift
+        // of 15 reads a side of 1 tile)
+        const long long adir = d.x < 0 ? -(long long)d.x : d.x, bdir = d.y < 0 ? -(long long)d.y : d.y;
+        const bool shallow = 4 * bdir <= adir, steep = 4 * adir <= bdir;
+        wsh = shallow ? 5u : steep ? 15u : 0u;
+        hsh = steep ? 10u : shallow ? 15u : 0u;
+    }
+    // between the map's x (y) and the frame's: the same involution both ways
+    __device__ __forceinline__ int flip_x(int x) const { return mx < 0 ? x : mx - x; }
+    __device__ __forceinline__ int flip_y(int y) const { return my < 0 ? y : my - y; }
+};
+
+__device__ __forceinline__ uint32_t walk_ray(const RayDir &r, int W, int H, unsigned kmax, int hx, int hy, int *hit,
+                                             int *steps) {
+    const int fx = r.flip_x(hx), fy = r.flip_y(hy);
+    const unsigned S = (unsigned)(fx + fy);
+    const uint16_t *__restrict__ sel = reinterpret_cast<const uint16_t *>(r.mk);
+    const uint16_t *__restrict__ rch = reinterpret_cast<const uint16_t *>(r.bq);
+    // unsigned 32-bit indexes: every table and map index fits, and the bases may wrap below zero before the row
+    // term brings the sum back
+    const unsigned bx = r.selx - (unsigned)fx * r.ns, by = r.sely - (unsigned)fy * r.ns, bm = r.jm - S * r.ns;
     // The loop only finds where the ray stops; the range is computed after it,
     // once for the whole warp, rather than in a divergent branch per lane.
-    // Cells outside the map are set in the walk frames, so leaving the map
-    // ends the loop as a hit and is told apart afterwards.  Indexes are
-    // unsigned 32-bit (every table and map index fits).
-    int adx = 0, ady = 0, cx = fx, cy = fy;
+    unsigned cx = (unsigned)fx, cy = (unsigned)fy;
     int stop;   // 1 hit (or left the map), 2 range limit
     for (;;) {
-        const int lx = cx & 7, ly = cy & 7;
-        // the tile's word, its boxes and the tile's exit steps are loaded together: one memory round trip
-        // per tile (a second one when the ray leaves a larger box)
-        const unsigned ti = (unsigned)(cy >> 3) * WB + (unsigned)(cx >> 3);
-        const uint64_t word = __ldg(bq + ti);
-        const unsigned rv = __ldg(rq + ti);
-        uint32_t kx = __ldg(selx + (unsigned)(adx + 8 - lx) * uns);
-        uint32_t ky = __ldg(sely + (unsigned)(ady + 8 - ly) * uns);
-        const unsigned bw = max(1u, (rv >> wsh) & 31u), bh = max(1u, (rv >> hsh) & 31u);   // the box, in tiles
-        const int ex = 8 * (int)bw - lx, ey = 8 * (int)bh - ly;   // x- and y-steps to its far edges
-        if ((bw | bh) > 1u) {
-            kx = __ldg(selx + (unsigned)(adx + ex) * uns);
-            ky = __ldg(sely + (unsigned)(ady + ey) * uns);
-        }
-        if (word) {
+        const unsigned tx = cx >> 3, ty = cy >> 3;
+        const unsigned ti = ty * r.WB + tx;
+        const unsigned rv = __ldg(rch + (r.rq + ti));
+        const unsigned ex = 8u * (tx + max(1u, (rv >> r.wsh) & 31u));   // the box's far edges
+        const unsigned ey = 8u * (ty + max(1u, (rv >> r.hsh) & 31u));
+        const unsigned kx = __ldg(sel + (ex * r.ns + bx));
+        const unsigned ky = __ldg(sel + (ey * r.ns + by));
+        if (rv == 0u) {
+            const uint64_t word = __ldg(r.bq + ti);
+            const uint64_t board = __ldg(r.mk + ((cx + cy) * r.ns + bm));
             // move the current cell to bit 0; bits that wrap into the row below
             // sit in columns the board's column mask removes
-            const uint64_t w = word >> (lx + 8 * ly);
+            const unsigned lx = cx & 7u, ly = cy & 7u;
             const uint32_t cm = 0x01010101u * (0xffu >> lx);   // board columns dx <= 7 - lx, every row
-            const uint64_t R = __ldg(mk + (unsigned)(adx + ady) * uns) & (((uint64_t)cm << 32) | cm);
-            const uint64_t hm = R & w;
+            const uint64_t hm = board & (((uint64_t)cm << 32) | cm) & (word >> (lx + 8u * ly));
             if (hm) {
-                const int b = __ffsll((long long)hm) - 1;
-                adx += b & 7;
-                ady += b >> 3;
+                const unsigned b = (unsigned)__ffsll((long long)hm) - 1u;
+                cx += b & 7u;
+                cy += b >> 3;
                 stop = 1;
                 break;
             }
         }
-        if (min(kx, ky) == kSelNone) {   // the next cell lies beyond the range limit
+        const unsigned k = min(kx, ky);
+        if (k == kSelNone) {   // the next cell lies beyond the range limit
             stop = 2;
             break;
         }
-        if (kx < ky) {
-            adx += ex;
-            ady = (int)kx - adx;
-        } else {
-            ady += ey;
-            adx = (int)ky - ady;
-        }
-        cx = fx + adx;
-        cy = fy + ady;
+        const unsigned sk = S + k;   // cx + cy at the exit
+        cx = kx < ky ? ex : sk - ey;
+        cy = sk - cx;
     }
-    if (stop == 1 && ((unsigned)(fx + adx - xlo) >= (unsigned)W || (unsigned)(fy + ady - ylo) >= (unsigned)H))
-        stop = 3;   // the first cell outside the map
-    const int sx = xneg ? -1 : 1, sy = yneg ? -1 : 1;
-    cx = hx + sx * adx;
-    cy = hy + sy * ady;
-    *hit = stop == 1 ? cy * W + cx : -1;
-    *steps = stop == 2 ? __ldg(t.kmax + j) + 1 : adx + ady;
-    const uint32_t r = isqrt_q16(stop == 1 ? adx * adx + ady * ady : 0);   // a hit lies within the range limit
-    return stop == 1 ? r : 0u;
+    const unsigned ax = (unsigned)r.flip_x((int)cx), ay = (unsigned)r.flip_y((int)cy);   // the map's cell
+    *steps = stop == 2 ? __ldg(reinterpret_cast<const int32_t *>(r.mk) + kmax) + 1 : (int)(cx + cy - S);
+    if (stop == 1 && (ax >= (unsigned)W || ay >= (unsigned)H)) stop = 3;   // the first cell outside the map
+    *hit = stop == 1 ? (int)ay * W + (int)ax : -1;
+    const int adx = (int)cx - fx, ady = (int)cy - fy;
+    const uint32_t q = isqrt_q16(stop == 1 ? adx * adx + ady * ady : 0);   // a hit lies within the range limit
+    return stop == 1 ? q : 0u;
 }
 
 // One thread per direction: the DDA of cast_ray from (0, 0), recorded.  The
@@ -410,14 +444,22 @@ __global__ void __launch_bounds__(kCastThreads, 5) k_cast(const ReqDesc *__restr
         const int j = (jc << 5) + lane;
         if (j < d.ns) {
             const int2 dir = d.D[j];
-            for (int h = h0; h < h1; ++h) {
-                const int2 hc = d.hyps[h];
-                int hit, steps = 0;
-                const uint32_t r = d.rt.mask ? walk_ray(d.bits, d.reach, d.W, d.H, d.TW, d.TH, d.rt, d.ns, j, hc.x, hc.y,
-                                                        dir, &hit, &steps)
-                                             : cast_ray(d.bits, d.W, d.H, d.TW, d.lim, hc.x, hc.y, dir, &hit, &steps);
-                d.scan_table[(size_t)h * d.ns + j] = r;
-                my_steps += (unsigned)steps;
+            uint32_t *out = d.scan_table + (size_t)h0 * d.ns + j;
+            int hit, steps = 0;
+            if (d.rt.mask) {
+                RayDir r;
+                r.init(d.bits, d.reach, d.TW, d.TH, d.rt, d.ns, j, dir);
+                for (int h = h0; h < h1; ++h, out += d.ns) {
+                    const int2 hc = d.hyps[h];
+                    *out = walk_ray(r, d.W, d.H, d.rt.kmax + (unsigned)j, hc.x, hc.y, &hit, &steps);
+                    my_steps += (unsigned)steps;
+                }
+            } else {
+                for (int h = h0; h < h1; ++h, out += d.ns) {
+                    const int2 hc = d.hyps[h];
+                    *out = cast_ray(d.bits, d.W, d.H, d.TW, d.lim, hc.x, hc.y, dir, &hit, &steps);
+                    my_steps += (unsigned)steps;
+                }
             }
         }
     }
@@ -730,18 +772,26 @@ __global__ void __launch_bounds__(256) k_win_read(const ReqDesc *__restrict__ re
     }
 }
 
+// One warp per (chunk of 32 directions, cell), cells fastest, as the ray cast
+// orders its work: the warps in flight then share a few directions' tables in
+// L1, and each stores whole 128-byte lines.
 __global__ void __launch_bounds__(256) k_synth(RayArgs a, uint32_t *__restrict__ ranges, int32_t *__restrict__ hits) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (warp >= a.n_hyp) return;
-    const int2 hc = a.hyps[warp];
-    for (int j = lane; j < a.ns; j += 32) {
-        int hit, steps;
-        uint32_t r = a.tab.mask ? walk_ray(a.bits, a.reach, a.W, a.H, a.TW, a.TH, a.tab, a.ns, j, hc.x, hc.y, a.D[j],
-                                           &hit, &steps)
-                                : cast_ray(a.bits, a.W, a.H, a.TW, a.lim, hc.x, hc.y, a.D[j], &hit, &steps);
-        ranges[(size_t)warp * a.ns + j] = r;
-        if (hits) hits[(size_t)warp * a.ns + j] = hit;
+    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    const int jc = (int)(warp / a.n_hyp), h = (int)(warp - (long long)jc * a.n_hyp), j = (jc << 5) + lane;
+    if (j >= a.ns) return;
+    const int2 hc = a.hyps[h];
+    int hit, steps;
+    uint32_t r;
+    if (a.tab.mask) {
+        RayDir dir;
+        dir.init(a.bits, a.reach, a.TW, a.TH, a.tab, a.ns, j, a.D[j]);
+        r = walk_ray(dir, a.W, a.H, a.tab.kmax + (unsigned)j, hc.x, hc.y, &hit, &steps);
+    } else {
+        r = cast_ray(a.bits, a.W, a.H, a.TW, a.lim, hc.x, hc.y, a.D[j], &hit, &steps);
     }
+    ranges[(size_t)h * a.ns + j] = r;
+    if (hits) hits[(size_t)h * a.ns + j] = hit;
 }
 
 }  // namespace
@@ -825,21 +875,23 @@ cudaError_t launch_win_read(const ReqDesc *reqs, int R, int total, cudaStream_t 
     return cudaGetLastError();
 }
 
-cudaError_t launch_ray_tables(const int2 *D, int ns, int lim, uint64_t *mask, uint16_t *selx, uint16_t *sely,
-                              int32_t *kmax, cudaStream_t s) {
-    const size_t rows_m = (size_t)ray_mask_rows(lim), rows_s = (size_t)ray_sel_rows(lim);
-    cudaError_t e = cudaMemsetAsync(mask, 0, sizeof(uint64_t) * rows_m * ns, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(selx, 0xff, sizeof(uint16_t) * rows_s * ns, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(sely, 0xff, sizeof(uint16_t) * rows_s * ns, s);
+cudaError_t launch_ray_tables(const int2 *D, int ns, int lim, void *tab, cudaStream_t s) {
+    const size_t mask_bytes = sizeof(uint64_t) * (size_t)ray_mask_rows(lim) * ns;
+    const RayTables t = ray_tables_at(tab, ns, lim);
+    uint64_t *mask = static_cast<uint64_t *>(tab);
+    uint16_t *sel = static_cast<uint16_t *>(tab);
+    cudaError_t e = cudaMemsetAsync(mask, 0, mask_bytes, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(sel + t.selx, 0xff, ray_tables_bytes(ns, lim) - mask_bytes, s);
     if (e != cudaSuccess) return e;
-    k_ray_tables<<<(ns + 127) / 128, 128, 0, s>>>(D, ns, lim, mask, selx, sely, kmax);
+    k_ray_tables<<<(ns + 127) / 128, 128, 0, s>>>(D, ns, lim, mask, sel + t.selx, sel + t.sely,
+                                                  static_cast<int32_t *>(tab) + t.kmax);
     return cudaGetLastError();
 }
 
 cudaError_t launch_synth(const RayArgs &a, uint32_t *ranges, int32_t *hit, cudaStream_t s) {
     if (a.n_hyp <= 0) return cudaSuccess;
-    int blocks = (a.n_hyp * 32 + 255) / 256;
-    k_synth<<<blocks, 256, 0, s>>>(a, ranges, hit);
+    const long long warps = (long long)a.n_hyp * (a.ns_pad >> 5);
+    k_synth<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(a, ranges, hit);
     return cudaGetLastError();
 }
 

@@ -63,10 +63,8 @@ struct ScanTable {
 // Per-direction traversal tables of one (N_s, range limit); see RayTables.
 struct RayTab {
     int ns = 0, lim = 0;
-    uint64_t *mask = nullptr;
-    uint16_t *selx = nullptr, *sely = nullptr;
-    int32_t *kmax = nullptr;
-    size_t bytes_mask = 0, bytes_sel = 0;
+    void *data = nullptr;             // one allocation (ray_tables_at)
+    size_t bytes = 0;
     cudaEvent_t built = nullptr;      // recorded after the build kernel
     unsigned long long last_use = 0;
     unsigned long long pin = 0;       // batch sequence number of the last batch that used it
@@ -616,10 +614,7 @@ ScanTable *new_table(relo_ctx *ctx, MapSlot &m, int ns, int lim) {
 // ---- per-direction traversal tables ---------------------------------------------------------------
 
 void free_raytab(relo_ctx *ctx, RayTab *t) {
-    dev_free(ctx, t->mask, t->bytes_mask);
-    dev_free(ctx, t->selx, t->bytes_sel);
-    dev_free(ctx, t->sely, t->bytes_sel);
-    dev_free(ctx, t->kmax, sizeof(int32_t) * (size_t)t->ns);
+    dev_free(ctx, t->data, t->bytes);
     if (t->built) cudaEventDestroy(t->built);
     delete t;
 }
@@ -635,9 +630,8 @@ RayTab *ray_tables_for(relo_ctx *ctx, const SensorPlan &P, int lim, cudaStream_t
             t->pin = ctx->batch_seq;
             return t;
         }
-    const size_t bm = sizeof(uint64_t) * (size_t)ray_mask_rows(lim) * P.ns;
-    const size_t bs = sizeof(uint16_t) * (size_t)ray_sel_rows(lim) * P.ns;
-    if (bm + 2 * bs > kMaxRayTabBytes) return nullptr;
+    const size_t bytes = ray_tables_bytes(P.ns, lim);
+    if (bytes > kMaxRayTabBytes) return nullptr;
     if ((int)ctx->raytabs.size() >= kMaxRayTabs) {
         auto it = ctx->raytabs.end();
         for (auto i = ctx->raytabs.begin(); i != ctx->raytabs.end(); ++i)
@@ -651,15 +645,11 @@ RayTab *ray_tables_for(relo_ctx *ctx, const SensorPlan &P, int lim, cudaStream_t
     if (!t) return nullptr;
     t->ns = P.ns;
     t->lim = lim;
-    t->bytes_mask = bm;   // free_raytab releases whatever was allocated
-    t->bytes_sel = bs;
+    t->bytes = bytes + sizeof(int32_t) * (size_t)P.ns;
     const std::string saved = ctx->err;
-    bool ok = dev_alloc(ctx, (void **)&t->mask, bm, "ray tables") == RELO_OK &&
-              dev_alloc(ctx, (void **)&t->selx, bs, "ray tables") == RELO_OK &&
-              dev_alloc(ctx, (void **)&t->sely, bs, "ray tables") == RELO_OK &&
-              dev_alloc(ctx, (void **)&t->kmax, sizeof(int32_t) * (size_t)P.ns, "ray tables") == RELO_OK &&
+    bool ok = dev_alloc(ctx, &t->data, t->bytes, "ray tables") == RELO_OK &&
               cudaEventCreateWithFlags(&t->built, cudaEventDisableTiming) == cudaSuccess &&
-              launch_ray_tables(P.D_dev, P.ns, lim, t->mask, t->selx, t->sely, t->kmax, st) == cudaSuccess &&
+              launch_ray_tables(P.D_dev, P.ns, lim, t->data, st) == cudaSuccess &&
               cudaEventRecord(t->built, st) == cudaSuccess;
     if (!ok) {
         ctx->err = saved;
@@ -674,14 +664,7 @@ RayTab *ray_tables_for(relo_ctx *ctx, const SensorPlan &P, int lim, cudaStream_t
 }
 
 RayTables ray_tables_view(const RayTab *t) {
-    RayTables v{nullptr, nullptr, nullptr, nullptr};
-    if (t) {
-        v.mask = t->mask;
-        v.selx = t->selx;
-        v.sely = t->sely;
-        v.kmax = t->kmax;
-    }
-    return v;
+    return t ? ray_tables_at(t->data, t->ns, t->lim) : RayTables{nullptr, 0, 0, 0};
 }
 
 // A new, unbuilt window table of scan table t for plan P, or nullptr when the
@@ -722,8 +705,8 @@ void free_map(relo_ctx *ctx, MapSlot &m) {
     dev_free(ctx, m.dev.summ, sizeof(int2) * (size_t)m.dev.W * edt_segments(m.dev.H));
     dev_free(ctx, m.dev.grid, (size_t)m.dev.W * m.dev.H);
     dev_free(ctx, m.dev.field, sizeof(uint16_t) * (size_t)m.dev.Wp * m.dev.Hp);
-    dev_free(ctx, m.dev.bits, sizeof(uint64_t) * occupancy_words(m.dev.TW, m.dev.TH));
-    dev_free(ctx, m.dev.reach, walk_reach_bytes(m.dev.TW, m.dev.TH));
+    dev_free(ctx, m.dev.bits, sizeof(uint64_t) * occupancy_words(m.dev.TW, m.dev.TH) +
+                                  walk_reach_bytes(m.dev.TW, m.dev.TH));   // reach lies behind bits
     dev_free(ctx, m.hyps, sizeof(int2) * (size_t)m.hyp_cap);
     dev_free(ctx, m.lut, sizeof(float2) * (kMaxClamp + 2));
     dev_free(ctx, m.sq_off, sizeof(int32_t) * (kMaxClamp + 2));
@@ -756,8 +739,8 @@ int load_map_impl(relo_ctx *ctx, const int8_t *grid, bool on_device, int32_t w, 
     const size_t fcells = (size_t)m.dev.Wp * m.dev.Hp;
     struct { void **p; size_t bytes; } allocs[] = {
         {(void **)&m.dev.d2, cells * 4}, {(void **)&m.dev.colsq, cells * 4}, {(void **)&m.dev.grid, cells},
-        {(void **)&m.dev.field, fcells * 2}, {(void **)&m.dev.bits, occupancy_words(m.dev.TW, m.dev.TH) * 8},
-        {(void **)&m.dev.reach, walk_reach_bytes(m.dev.TW, m.dev.TH)},
+        {(void **)&m.dev.field, fcells * 2},
+        {(void **)&m.dev.bits, occupancy_words(m.dev.TW, m.dev.TH) * 8 + walk_reach_bytes(m.dev.TW, m.dev.TH)},
         {(void **)&m.dev.summ, sizeof(int2) * (size_t)w * edt_segments(h)}};
     for (auto &a : allocs) {
         rc = dev_alloc(ctx, a.p, a.bytes, "map tables");
@@ -767,6 +750,7 @@ int load_map_impl(relo_ctx *ctx, const int8_t *grid, bool on_device, int32_t w, 
         }
         m.bytes += a.bytes;
     }
+    m.dev.reach = reinterpret_cast<uint16_t *>(m.dev.bits + occupancy_words(m.dev.TW, m.dev.TH));
     cudaError_t e = cudaEventCreateWithFlags(&m.tiles_ready, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m.field_ready, cudaEventDisableTiming);
     if (e == cudaSuccess)

@@ -45,8 +45,8 @@ struct MapDev {
     int P = 0, Wp = 0, Hp = 0;  // border width; padded width and height (W + 2P, H + 2P rounded up to 8)
     uint64_t *bits = nullptr;   // occupancy, bit (y&7)*8 + (x&7): [TH*TW] the map (cells outside free), then the
                                 // four walk frames (walk_frame_words each: native, mirrored in x, y and both)
-    uint16_t *reach = nullptr;  // per walk-frame tile, the empty boxes of tiles ahead, then scratch (walk_reach_bytes);
-                                // nullptr: no ray is cast on this map
+    uint16_t *reach = nullptr;  // per walk-frame tile, the empty boxes of tiles ahead, then scratch (walk_reach_bytes),
+                                // in one allocation after bits; nullptr: no ray is cast on this map
     int32_t *colsq = nullptr;   // [H*W] EDT column-pass scratch
     int2 *summ = nullptr;       // [S*W] EDT column-segment summaries (scratch)
     int8_t *grid = nullptr;     // [H*W] device copy of the grid
@@ -147,10 +147,12 @@ struct SelectState {
 //               and within the range limit, as an 8x8 bit board anchored at
 //               cell k: bit 8 |dy| + |dx| for the offsets (dx, dy).
 //   kmax[j]:   the last cell index within the range limit.
+// One allocation holds the four, so the walk keeps one 64-bit base and 32-bit
+// indexes: mask at its start, selx and sely at 2-byte units from there, kmax
+// at 4-byte units.
 struct RayTables {
     const uint64_t *mask;
-    const uint16_t *selx, *sely;
-    const int32_t *kmax;
+    unsigned selx, sely, kmax;
 };
 constexpr uint32_t kSelNone = 0xffffu;
 
@@ -167,6 +169,14 @@ __host__ __device__ inline int ray_sel_rows(int lim) {
     while ((long long)(r + 1) * (r + 1) <= (long long)lim) ++r;
     while ((long long)r * r > (long long)lim) --r;
     return r + 8 * kReachMax + 1;   // a cell in range has |dx| <= sqrt(lim); leaving a square adds at most 8 kReachMax
+}
+__host__ __device__ inline RayTables ray_tables_at(const void *base, int ns, int lim) {
+    const size_t m = (size_t)ray_mask_rows(lim) * ns, r = (size_t)ray_sel_rows(lim) * ns;
+    return RayTables{static_cast<const uint64_t *>(base), (unsigned)(4 * m), (unsigned)(4 * m + r),
+                     (unsigned)(2 * m + r)};
+}
+inline size_t ray_tables_bytes(int ns, int lim) {   // boards and step indexes, without kmax
+    return (sizeof(uint64_t) * (size_t)ray_mask_rows(lim) + 2 * sizeof(uint16_t) * (size_t)ray_sel_rows(lim)) * ns;
 }
 
 // single-request arguments of the synthesized-scan export (relo_synth_scans_dev)
@@ -333,9 +343,8 @@ cudaError_t launch_check_cells(const int2 *cells, int n, const MapDev &m, int *b
 cudaError_t launch_xy_cells(const double *xy, int n, double ox, double oy, double res, const MapDev &m, int2 *cells,
                             int *flags, cudaStream_t s);
 cudaError_t launch_synth(const RayArgs &a, uint32_t *ranges, int32_t *hit, cudaStream_t s);
-// fills the traversal tables of directions D[0, ns) for range limit lim (buffers sized by ray_*_rows)
-cudaError_t launch_ray_tables(const int2 *D, int ns, int lim, uint64_t *mask, uint16_t *selx, uint16_t *sely,
-                              int32_t *kmax, cudaStream_t s);
+// fills the traversal tables of directions D[0, ns) for range limit lim (ray_tables_bytes, then ns int32)
+cudaError_t launch_ray_tables(const int2 *D, int ns, int lim, void *tab, cudaStream_t s);
 
 // batched stages; R requests, descriptors in device memory
 // scan preparation alone, for a batch that casts no rays (launch_cast does it otherwise)
