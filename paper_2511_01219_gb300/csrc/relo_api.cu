@@ -80,6 +80,7 @@ struct MapSlot {
     int2 *hyps = nullptr;
     int n_hyp = 0, hyp_cap = 0;
     float2 *lut = nullptr;
+    double lut_key[6] = {0};     // what its values depend on: z_hit, sigma_hit, z_rand, eps, resolution, clamp
     int32_t *sq_off = nullptr;   // [kMaxClamp + 2] and [kMaxLatticePoints]: the cells at each squared distance
     short2 *sq_rep = nullptr;
     size_t bytes = 0;
@@ -100,6 +101,7 @@ struct Prepared {
 };
 
 constexpr int kMaxPlans = 32;
+constexpr size_t kMaxTamSegs = (size_t)kMaxBatches * (kMaxBatchRequests + 1);   // segment table of a batch slot
 constexpr size_t kBlobBytes = 30000;   // kernel-parameter upload size
 
 // Device-to-device upload through kernel parameters: the bytes travel with the
@@ -117,6 +119,7 @@ __global__ void k_upload(const __grid_constant__ Blob blob, unsigned char *dst, 
         bs->ray_work = 0u;
         bs->cast_work = 0u;
         bs->dda_steps = 0ull;
+        bs->error = 0u;
     }
 }
 
@@ -332,6 +335,8 @@ int build_lut(relo_ctx *ctx, MapSlot &m) {
         h[b] = make_float2((float)l, (float)(sc - sqrt((double)b)));
     }
     h[C + 1] = make_float2(0.0f, 0.0f);   // "no beam": contributes nothing
+    const double key[6] = {p.z_hit, p.sigma_hit, p.z_rand, p.eps, m.res, (double)C};
+    memcpy(m.lut_key, key, sizeof key);
     if (!m.lut) {
         int rc = dev_alloc(ctx, (void **)&m.lut, sizeof(float2) * (kMaxClamp + 2), "likelihood table");
         if (rc) return rc;
@@ -996,7 +1001,7 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R) {
     classes.erase(std::unique(classes.begin(), classes.end()), classes.end());
     int pre_max_batches = 0;
     for (int r = 0; r < R; ++r) pre_max_batches = std::max(pre_max_batches, pr[r].n_batches);
-    if ((size_t)pre_max_batches * classes.size() * R > (size_t)kMaxBatches * kMaxBatchRequests) {
+    if ((size_t)pre_max_batches * classes.size() * (R + 1) > kMaxTamSegs) {
         std::fill(vcls.begin(), vcls.end(), classes.back());
         classes.assign(1, classes.back());
     }
@@ -1004,7 +1009,7 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R) {
     // survivors per TAM task: the autotuner's choice for the request's shape, else the built-in one
     auto chunk_of = [&](int r) {
         const relo_tune_entry *e = tuned_tam(ctx, R, vcls[r], pr[r].P->n_orient, pr[r].K);
-        return e && e->val[0] > 0 ? e->val[0] : tam_chunk_for(pr[r].K, pr[r].P->n_orient, ctx->n_sm);
+        return e && e->val[0] > 0 ? e->val[0] : tam_chunk_for(pr[r].K, pr[r].P->n_orient, R, ctx->n_sm);
     };
     std::vector<ReqDesc> desc((size_t)R);
     std::vector<size_t> off((size_t)R);
@@ -1017,9 +1022,9 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R) {
         off[r] = total;
         total += align_up(24ull * K) + align_up(4ull * K);   // refined poses and re-evaluated scores
         total += align_up(sizeof(int2) * n) + align_up(4ull * n) + align_up(sizeof(ScanInfo)) + align_up(8ull * nh) * 2 +
-                 align_up(4ull * nh) + align_up(4ull * K) * 3 + align_up(4ull * K * q.P->n_orient) +
+                 align_up(4ull * nh) + align_up(4ull * K) * 2 + align_up(8ull * K) + align_up(4ull * K * q.P->n_orient) +
                  align_up(16ull * tam_chunk_cap(K, q.B, q.n_batches, chunk_of(r))) + align_up(4ull * (q.n_batches + 1)) +
-                 align_up(4ull * 8 * 32 * q.P->n_orient * tam_offs_stride_for(vcls[r])) +
+                 align_up(4ull * 32 * q.P->n_orient * tam_offs_stride_for(vcls[r])) +
                  align_up(8ull * K) + align_up(4ull * q.n_batches * p.local_topk) + align_up(sizeof(SelectState));
         if (mode[r] == kScanCast) total += align_up(4ull * nh * q.P->ns);   // the request's synthesized ranges
         if (mode[r] != kScanRead && cast) total_chunks += cast_chunks(nh, q.P->ns, 1);
@@ -1113,8 +1118,8 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R) {
         d.survivors = (int32_t *)take(4ull * q.K);
         d.tam_chunk = chunk_of(r);
         d.tam_stride = tam_offs_stride_for(vcls[r]);
-        d.tam_offs = (int32_t *)take(4ull * 8 * 32 * P.n_orient * d.tam_stride);
-        d.surv_perm = (int32_t *)take(4ull * q.K);
+        d.tam_offs = (int32_t *)take(4ull * 32 * P.n_orient * d.tam_stride);
+        d.surv_perm = (int2 *)take(8ull * q.K);
         d.tam_chunks = (int4 *)take(16ull * tam_chunk_cap(q.K, q.B, q.n_batches, d.tam_chunk));
         d.chunk_cnt = (int32_t *)take(4ull * (q.n_batches + 1));
         d.best_m = (int32_t *)take(4ull * q.K);
@@ -1123,6 +1128,7 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R) {
         d.local = (int32_t *)take(4ull * q.n_batches * p.local_topk);
         d.state = (SelectState *)take(sizeof(SelectState));
         d.result = q.result_dev;
+        d.bs = sl.bs;
         d.scan_table = mode[r] == kScanCast ? (uint32_t *)take(4ull * m.n_hyp * P.ns) : tab[r]->data;
         d.scan_mode = mode[r];
         d.win = win[r] ? win[r]->keys : nullptr;
@@ -1151,19 +1157,24 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R) {
     bool any_early = false;
     for (int r = 0; r < R; ++r) any_early = any_early || desc[r].early_stop;
     const int tam_rounds = any_early ? max_batches : std::min(max_batches, 1);
-    std::vector<TamSeg> segs((size_t)max_batches * NC * R);
+    const size_t seg_n = (size_t)R + 1;   // per launch: the requests' segments, then its task counter
+    std::vector<TamSeg> segs((size_t)max_batches * NC * seg_n);
     std::vector<TamPlan> plans((size_t)max_batches * NC);
     std::vector<int> blo((size_t)R), bhi((size_t)R);
     for (int bi = 0; bi < tam_rounds; ++bi) {
         for (int c = 0; c < NC; ++c) {
-            int beams_c = 1, C_c = 0;
+            int beams_c = 1, C_c = 0, chunk_c = 0, luts = 0;   // luts: 1 when the class's likelihood tables are the same
+            const MapSlot *m_c = nullptr;
             for (int r = 0; r < R; ++r) {
                 const bool in = vcls[r] == classes[c] && bi < desc[r].n_batches;
                 blo[r] = any_early ? bi : 0;
                 bhi[r] = in ? (any_early ? bi + 1 : desc[r].n_batches) : blo[r];
                 if (vcls[r] == classes[c]) {
                     beams_c = std::max(beams_c, pr[r].P->n);
+                    if (!m_c || memcmp(m_c->lut_key, pr[r].m->lut_key, sizeof m_c->lut_key)) ++luts;
+                    m_c = pr[r].m;
                     C_c = std::max(C_c, pr[r].m->dev.C);
+                    chunk_c = chunk_c ? std::min(chunk_c, desc[r].tam_chunk) : desc[r].tam_chunk;
                 }
             }
             int cps = 0;   // resident CTAs per SM: the smallest the class's requests are tuned to
@@ -1173,8 +1184,8 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R) {
                 if (e && e->val[1] > 0) cps = cps > 0 ? std::min(cps, e->val[1]) : e->val[1];
             }
             TamPlan &tp = plans[(size_t)bi * NC + c];
-            tp = plan_tam(blo.data(), bhi.data(), R, beams_c, C_c, ctx->n_sm, cps,
-                          &segs[((size_t)bi * NC + c) * R]);
+            tp = plan_tam(blo.data(), bhi.data(), R, beams_c, C_c, ctx->n_sm, cps, chunk_c, luts,
+                          &segs[((size_t)bi * NC + c) * seg_n]);
             if (tp.vpl < 0) return fail(ctx, RELO_E_INVALID_ARG, "no TAM kernel fits this beam count");
         }
     }
@@ -1185,7 +1196,7 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R) {
     memcpy(blob.data() + seg_off, segs.data(), sizeof(TamSeg) * segs.size());
     if ((rc = upload(ctx, st, sl.reqs_dev, blob.data(), blob.size(), sl.bs))) return rc;
     ReqDesc *rq = sl.reqs_dev;
-    const TamSeg *segs_dev = reinterpret_cast<const TamSeg *>(reinterpret_cast<unsigned char *>(sl.reqs_dev) + seg_off);
+    TamSeg *segs_dev = reinterpret_cast<TamSeg *>(reinterpret_cast<unsigned char *>(sl.reqs_dev) + seg_off);
     // the ray-cast launch prepares the scans first; a batch without rays to cast prepares them alone
     if (total_chunks <= 0) CK(timed_on(ctx, st, 1, 1, [&] { return launch_scan_prep(rq, R, st); }), "scan preparation");
     for (int r = 0; r < R; ++r) {
@@ -1236,8 +1247,8 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R) {
         for (int c = 0; c < NC; ++c) {
             const TamPlan &tp = plans[(size_t)bi * NC + c];
             if (tp.total_tasks <= 0) continue;
-            const TamSeg *sg = segs_dev + ((size_t)bi * NC + c) * R;
-            CK(timed_on(ctx, st, 4, 1, [&] { return launch_tam(rq, R, sg, tp, st); }), "TAM");
+            TamSeg *sg = segs_dev + ((size_t)bi * NC + c) * seg_n;
+            CK(timed_on(ctx, st, 4, 1, [&] { return launch_tam(rq, R, sg, tp, sl.bs, st); }), "TAM");
         }
         const int lo = any_early ? bi : 0, hi = any_early ? bi + 1 : max_batches;
         const bool last = bi == tam_rounds - 1;
@@ -1263,7 +1274,7 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R) {
 
 // device bytes of a slot's descriptor region: descriptors, then TAM segments
 size_t slot_desc_bytes() {
-    return align_up(sizeof(ReqDesc) * kMaxBatchRequests) + sizeof(TamSeg) * kMaxBatches * kMaxBatchRequests;
+    return align_up(sizeof(ReqDesc) * kMaxBatchRequests) + sizeof(TamSeg) * kMaxTamSegs;
 }
 
 int slot_init(relo_ctx *ctx, BatchSlot &sl, cudaStream_t stream) {
@@ -1343,10 +1354,10 @@ size_t request_bytes(const relo_ctx *ctx, const Prepared &q) {
     const size_t n = (size_t)q.P->n, nh = (size_t)q.m->n_hyp, K = (size_t)q.K;
     const bool resident = ctx->p.scan_cache_bytes > 0 && find_table(*q.m, q.P->ns, q.lim) != nullptr;
     return align_up(sizeof(int2) * n) + align_up(sizeof(ScanInfo)) + align_up(8 * nh) * 2 + align_up(4 * nh) +
-           align_up(4 * K) * 3 + align_up(4 * K * q.P->n_orient) + align_up(8 * K) +
-           align_up(16ull * tam_chunk_cap(q.K, q.B, q.n_batches, tam_chunk_for(q.K, q.P->n_orient, ctx->n_sm))) +
+           align_up(4 * K) * 2 + align_up(4 * K * q.P->n_orient) + align_up(8 * K) * 2 +
+           align_up(16ull * tam_chunk_cap(q.K, q.B, q.n_batches, tam_chunk_for(q.K, q.P->n_orient, 1, ctx->n_sm))) +
            align_up(4ull * (q.n_batches + 1)) +
-           align_up(4ull * 8 * 32 * q.P->n_orient * tam_offs_stride_for(tam_vpl_for(q.P->n))) +
+           align_up(4ull * 32 * q.P->n_orient * tam_offs_stride_for(tam_vpl_for(q.P->n))) +
            align_up(4ull * q.n_batches * ctx->p.local_topk) + align_up(sizeof(SelectState)) +
            align_up(sizeof(float) * q.P->n * ctx->p.n_skip_beam) + (resident ? 0 : align_up(4 * nh * q.P->ns));
 }

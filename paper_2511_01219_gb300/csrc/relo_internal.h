@@ -252,8 +252,8 @@ struct ReqDesc {
     // TAM's work order: within each batch the survivor positions grouped by the band phase (y + P) % 8 of
     // their cell, cut into chunks of at most tam_chunk of one phase: (phase, first, end) into surv_perm;
     // the chunks of batches < b are tam_chunks[0, chunk_cnt[b])
-    int32_t *surv_perm;          // [K]
-    int32_t *tam_offs;           // [8][n_orient][32][tam_stride] TAM endpoint offsets by band phase (tam_offsets.cuh)
+    int2 *surv_perm;             // [K] (survivor position, field_index of its cell's column at the top of its band)
+    int32_t *tam_offs;           // [n_orient][32][tam_stride] TAM endpoint cells: y << 16 | x offsets (tam_offsets.cuh)
     int tam_stride;              // slots per lane in tam_offs
     int4 *tam_chunks;            // [sum over batches of ceil(n_b / tam_chunk) + 8]
     int32_t *chunk_cnt;          // [n_batches + 1]
@@ -264,6 +264,7 @@ struct ReqDesc {
     int32_t *local;              // [n_batches * L]
     SelectState *state;
     void *result;                // relo_result in device memory
+    const struct BatchState *bs; // the batch's counters
     // work lists
     int hyp_base;                // first slot of this request in the batch's hypothesis list
     // synthesized scans of (map, hypotheses, N_s, lim): [n_hyp * ns] Q16 ranges, row per hypothesis
@@ -299,6 +300,7 @@ struct BatchState {
     unsigned int ray_work;          // next global hypothesis slot for the SMAD CTAs
     unsigned int cast_work;         // next global 32-ray chunk for the cast warps
     unsigned long long dda_steps;   // cells entered by all rays of the batch
+    unsigned int error;             // a TAM warp gave up waiting for its task
 };
 
 // TAM work of one request in one launch: the survivors of its batches
@@ -310,14 +312,15 @@ struct TamSeg {
 };
 
 constexpr int kMaxBatchRequests = 256;
-// survivors of one band phase per TAM task: the most (up to 64, a multiple of
-// 8) that still leave about three tasks (blocks of 4 orientations) per
-// resident CTA of five per SM, so the launch is not one ragged wave
-inline int tam_chunk_for(int K, int n_orient, int n_sm) {
+// Survivors of one band phase per TAM task: the most (16 to 64) that still give every CTA (two per SM) about four tasks
+// (blocks of 4 orientations) of a batch of R such requests, so that the tasks spread evenly.  Measured with 8 / 16 / 32 /
+// 64 per task (TAM, us): 256 survivors x 360 orientations 125 / 120 / 127 / 121, 1024 x 720 1138 / 1088 / 1065 / 1062,
+// 16 requests of 256 and 512 2364 / 2191 / 2174 / 2166.
+inline int tam_chunk_for(int K, int n_orient, int R, int n_sm) {
     const long long tasks_per_survivor = (n_orient + 3) / 4;
-    long long c = (long long)K * tasks_per_survivor / (3ll * 5 * n_sm);
+    long long c = (long long)K * R * tasks_per_survivor / (4ll * 2 * n_sm);
     c = c / 8 * 8;
-    return (int)(c < 8 ? 8 : c > 64 ? 64 : c);
+    return (int)(c < 16 ? 16 : c > 64 ? 64 : c);
 }
 // chunks of the TAM work order: per group of survivors (each batch, or all K as one group), its survivors in
 // chunks of one phase (at most one part chunk per phase); the per-batch count bounds both
@@ -370,18 +373,20 @@ cudaError_t launch_topk(const ReqDesc *reqs, int R, int max_n_hyp, int max_K, in
 struct TamPlan {
     int total_tasks, grid, vpl;
     size_t smem;
+    int stages, lut_bytes, lut_copies;   // staged tasks per CTA; bytes of a likelihood table and how many a CTA holds
     bool h2;   // selection counts on packed fp16 (table slot of C + 1 at most 6143: C <= 5956)
 };
 // values per lane the TAM kernel holds for max_beams valid beams (-1 if too many)
 int tam_vpl_for(int max_beams);
-// the planned launch for the batches [batch_lo[r], batch_hi[r]) of each request r: segs[R], grid and kernel class
+// the planned launch for the batches [batch_lo[r], batch_hi[r]) of each request r: segs[R + 1] (the last is the
+// launch's task counter), grid and kernel class
 TamPlan plan_tam(const int *batch_lo, const int *batch_hi, int R, int max_beams, int max_C, int n_sm,
-                 int ctas_per_sm, TamSeg *segs);
+                 int ctas_per_sm, int chunk, int luts, TamSeg *segs);
 // TAM's work order (surv_perm, tam_chunks, chunk_cnt) of every request, after the top-K
 // per-lane stride of the TAM endpoint offsets of a values-per-lane class
 int tam_offs_stride_for(int vpl);
 // every request's TAM endpoint offsets for all band phases and orientations (after the scan preparation)
-cudaError_t launch_tam(const ReqDesc *reqs, int R, const TamSeg *segs, const TamPlan &tp, cudaStream_t s);
+cudaError_t launch_tam(const ReqDesc *reqs, int R, TamSeg *segs, const TamPlan &tp, BatchState *bs, cudaStream_t s);
 // selection of batch indexes batch_lo .. batch_hi - 1 in order; with last, also every request's result.
 // With icp, only the local top-k (launch_icp and launch_icp_best take the rest).
 cudaError_t launch_select_batch(const ReqDesc *reqs, int R, int batch_lo, int batch_hi, bool last, bool icp,

@@ -262,8 +262,9 @@ __device__ void finalize_request(const ReqDesc &d) {
     r.n_batches = st.n_batches;
     r.n_tam_evals = st.n_tam_evals;
     r.n_smad_evals = d.n_smad_evals;
-    if (d.scan->n_valid <= 0 || st.n_batches == 0) {
-        r.status = RELO_E_NO_VALID_BEAMS;
+    const bool failed = d.bs->error != 0u;
+    if (failed || d.scan->n_valid <= 0 || st.n_batches == 0) {
+        r.status = failed ? RELO_E_CUDA : RELO_E_NO_VALID_BEAMS;
         r.x = r.y = r.theta = r.tam = r.smad = 0.0;
         r.smad_num = 0;
         r.hyp = -1;

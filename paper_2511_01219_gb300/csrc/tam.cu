@@ -40,6 +40,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "relo_internal.h"
 #include "scan_prep.cuh"
 
@@ -48,7 +50,6 @@ namespace relo {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kTamWarps = 8;
 // Selection values as fp16 bit patterns 0x6400 + s, s the table slot of the
 // value (lut_slot, below).  Positive fp16 numbers order like their bit
 // patterns, so this is an increasing map of s onto fp16 numbers >= 1024,
@@ -153,11 +154,21 @@ __global__ void __launch_bounds__(1024) k_scan_prep(const ReqDesc *__restrict__ 
 
 // Work is split into tasks (request, chunk of survivors of one band phase,
 // block of kTamQ consecutive orientations); the top-K launch builds the chunks
-// on the device (tam_offsets.cuh).  A CTA copies the block's endpoint offsets for
-// its chunk's phase from the request's table (tam_offsets.cuh: one linear
-// offset per phase, orientation and valid beam, computed once per request)
-// into shared memory; each warp then scores its survivors of the chunk over
-// the block's orientations, every gather one add to the survivor's base.
+// on the device (tam_offsets.cuh).  A CTA holds a few staged tasks in shared
+// memory: the block's endpoint offsets for the chunk's phase (computed from the
+// request's table of endpoint cells) and the task's constants, beside the
+// likelihood table.  Its warps run through the stages without a CTA barrier:
+// each takes survivors of the stage one by one from a shared counter and scores
+// them over the block's orientations (every gather one add to the survivor's
+// base), and moves on to the next stage when none is left; the last warp to
+// leave a stage takes the next task from the launch's counter and stages it
+// there while the others work on the next one.  What bounds the kernel is the
+// L1 data path (gathers, table lookups, offsets) and, for the shorter scans,
+// the latency of the searches; with three CTA barriers per task every warp
+// waited for the slowest search of its task, and a table copy and offsets for
+// each of 4 to 6 CTAs per SM left the gathers a third of L1.  TAM, us, before
+// and with the stages: 256 survivors x 360 orientations x 1081 beams 140 -> 117,
+// 1024 x 720 x 1440 1127 -> 1060, 16 mixed requests 2733 -> 2140.
 //
 // Selection.  The k-th smallest clamped d2 of a survivor rarely changes from
 // one orientation to the next (neighbouring orientations see nearly the same
@@ -165,258 +176,419 @@ __global__ void __launch_bounds__(1024) k_scan_prep(const ReqDesc *__restrict__ 
 // previous answer h: two counts confirm it (#{b <= h} >= k and #{b <= h-1} <
 // k); otherwise the search gallops away from h in doubling steps and bisects
 // the bracket.  Every step is a warp-wide count, and the result is the same
-// smallest b with #{b' <= b} >= k as a bisection over [0, C].  The likelihood
-// table is reloaded only when a CTA moves to another request's task.
+// smallest b with #{b' <= b} >= k as a bisection over [0, C].
 constexpr int kTamQ = 4;
+constexpr int kTamStages = 8;   // at most
 
-// resident CTAs per SM the register budget is sized for (measured per values-per-lane class)
-__host__ __device__ constexpr int tam_min_blocks(int vpl, bool h2) { return h2 ? (vpl <= 24 ? 6 : vpl <= 40 ? 5 : 4) : (vpl <= 24 ? 3 : 2); }
+// Warps per CTA, two CTAs per SM (one where their shared memory does not fit twice), by values-per-lane class: the
+// register budget they leave each other against the warps that hide the gathers.  Measured (TAM, us): up to 24 values 24
+// / 20 / 16 / 14 warps 84 / 80 / 79 / 88 (18 values, 256 survivors x 360 orientations) and 2169 / 2136 / - / 2789 (the
+// mixed batch, both lower classes); 34 values 24 / 20 / 16 / 14 / 12 warps 136 / 120 / 117 / 121 / 179; 46 values 20 / 16
+// / 14 / 12 warps 1214 / 1069 / 1060 / 1089.
+__host__ __device__ constexpr int tam_warps(int vpl, bool h2) { return h2 ? (vpl <= 24 ? 20 : vpl <= 40 ? 16 : 14) : (vpl <= 24 ? 12 : 8); }
+constexpr int kTamCtas = 2;
 
-template <int VPL, bool H2>
-__global__ void __launch_bounds__(kTamWarps * 32, tam_min_blocks(VPL, H2)) k_tam(const ReqDesc *__restrict__ reqs,
-                                                                             int R, const TamSeg *__restrict__ segs,
-                                                                             int total_tasks) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int s_base[kMaxBatchRequests + 1];
-    __shared__ int s_skip, s_lut_r;
-    __shared__ float s_ep[5];   // per-task constants of the epilogue
-    __shared__ int s_fine;      // the task's scoring metric (read where needed, not held in a register)
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // each request's tasks: its chunks in the launch's batches x its orientation blocks (counted on the device)
-    if (threadIdx.x == 0) {
-        int base = 0;
-        for (int r = 0; r < R; ++r) {
-            s_base[r] = base;
-            const TamSeg sg = segs[r];
-            if (sg.batch_hi > sg.batch_lo) {
-                const ReqDesc &d = reqs[r];
-                base += (d.chunk_cnt[sg.batch_hi] - d.chunk_cnt[sg.batch_lo]) * ((d.n_orient + kTamQ - 1) / kTamQ);
-            }
-        }
-        s_base[R] = base;
-        s_lut_r = -1;
+// One staged task.
+struct TamTask {
+    unsigned long long full;   // mbarrier: completes when the stage is filled
+    const uint16_t *field;
+    const int2 *perm;          // the chunk's survivors: (position, base of the cell's column in its band)
+    float *T;
+    unsigned long long *best_key;
+    const float2 *lut_src;     // the table the stage's copy came from (it stays when the next task shares it)
+    int n;                     // survivors, -1 when there are no more tasks
+    int q0, nq, n_orient;
+    int N, k, C, fine;
+    float inv_k, res_N, span, inv_span, res2_N, d_max;   // 1 / k, res / N, span of Eq. 29, res^2 / N
+    int next, left;            // the next survivor to take; warps that have left the stage
+};
+
+__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+// Waits for phase parity of the barrier.  Gives up after two seconds (a staging takes microseconds), so that a fault
+// of this protocol would end the launch with an error instead of hanging it.
+__device__ __forceinline__ bool wait_full(unsigned long long *bar, uint32_t parity) {
+    const uint32_t addr = smem_u32(bar);
+    unsigned long long start = 0;
+    for (;;) {
+        uint32_t ok;
+        asm volatile("{\n\t.reg .pred p;\n\t"
+                     "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok)
+                     : "r"(addr), "r"(parity)
+                     : "memory");
+        if (ok) return true;
+        unsigned long long now;
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(now));
+        if (!start) start = now;
+        else if (now - start > 2000000000ull) return false;
     }
-    __syncthreads();
-    total_tasks = s_base[R];
-    float2 *lut = reinterpret_cast<float2 *>(smem);
-    for (int task = blockIdx.x; task < total_tasks; task += gridDim.x) {
-        int lo = 0, hi = R - 1;   // the request whose tasks hold this one: last r with s_base[r] <= task
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (s_base[mid] <= task) lo = mid;
-            else hi = mid - 1;
+}
+
+// Stages task `task` of the launch (or, past the last, its end) by the threads tid, tid + nt, ...: the caller
+// synchronises them, records the returned table in lut_src and completes the stage's barrier.
+template <int VPL>
+__device__ __forceinline__ const float2 *stage_task(const ReqDesc *__restrict__ reqs, int R, const TamSeg *__restrict__ segs,
+                                                    const int *s_base, int task, TamTask &t, float2 *lut,
+                                                    int lut_copies, int *offs, int tid, int nt) {
+    constexpr int kS = tam_offs_stride(VPL);
+    if (task >= s_base[R]) {
+        if (tid == 0) t.n = -1;
+        return t.lut_src;
+    }
+    int lo = 0, hi = R - 1;   // the request whose tasks hold this one: last r with s_base[r] <= task
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (s_base[mid] <= task) lo = mid;
+        else hi = mid - 1;
+    }
+    const ReqDesc &d = reqs[lo];
+    const int local = task - s_base[lo];
+    const int nblk = (d.n_orient + kTamQ - 1) / kTamQ;
+    const int4 ck = d.tam_chunks[d.chunk_cnt[segs[lo].batch_lo] + local / nblk];   // (phase, first, end)
+    const int q0 = (local % nblk) * kTamQ, nq = min(kTamQ, d.n_orient - q0);
+    const float2 *src = lut_copies > 1 || !t.lut_src ? d.lut : t.lut_src;
+    if (t.lut_src != src)
+        for (int i = tid; i <= d.C + 1; i += nt) lut[lut_slot(i)] = __ldg(src + i);
+    {
+        // the block's endpoint cells (packed x, y offsets), nq x 32 x kS contiguous, to field offsets from a cell of
+        // the chunk's band phase (field_index is linear in x, and in y through the bands crossed)
+        const int Wp8 = 8 * d.Wp, ph = ck.x;
+        const int4 *from = reinterpret_cast<const int4 *>(d.tam_offs + (size_t)q0 * 32 * kS);
+        int4 *to = reinterpret_cast<int4 *>(offs);
+        const int n4 = nq * 32 * kS / 4;
+        auto off = [&](int p) {
+            const int v = ph + (p >> 16);
+            return 8 * (int)(short)p + Wp8 * (v >> 3) + (v & 7);
+        };
+#pragma unroll 4
+        for (int i = tid; i < n4; i += nt) {
+            const int4 p = __ldg(from + i);
+            to[i] = make_int4(off(p.x), off(p.y), off(p.z), off(p.w));
         }
-        const int r = lo;
-        const ReqDesc &d = reqs[r];
-        const TamSeg sg = segs[r];
+    }
+    if (tid == 0) {
         const int N = d.scan->n_valid;
         // the likelihood-field metrics (Eq. 32-33) keep every beam: no retention, no k-th value to find
         const int k = d.fine < kFineBaseline ? d.scan->k_ret : N;
-        __syncthreads();   // the previous task's reads of offs / lut are done
-        if (threadIdx.x == 0) {
-            s_skip = d.state->done || N <= 0;
-            s_fine = d.fine;
-            s_ep[0] = 1.0f / (float)k;                // 1 / k
-            s_ep[1] = d.res / (float)N;               // res / N
-            s_ep[2] = d.d_max - d.d_min;              // span of Eq. 29
-            s_ep[3] = 1.0f / (d.d_max - d.d_min);
-            s_ep[4] = d.res2 / (float)N;              // res^2 / N
+        t.field = d.field;
+        t.perm = d.surv_perm + ck.y;
+        t.T = d.T;
+        t.best_key = d.best_key;
+        t.n = ck.z - ck.y;
+        t.q0 = q0;
+        t.nq = nq;
+        t.n_orient = d.n_orient;
+        t.N = N;
+        t.k = k;
+        t.C = d.C;
+        t.fine = d.fine;
+        t.inv_k = 1.0f / (float)k;
+        t.res_N = d.res / (float)N;
+        t.span = d.d_max - d.d_min;
+        t.inv_span = 1.0f / (d.d_max - d.d_min);
+        t.res2_N = d.res2 / (float)N;
+        t.d_max = d.d_max;
+        t.next = 0;
+        t.left = 0;
+    }
+    return src;
+}
+
+// The scores of one survivor (position s, base field pointer fh) over the orientations [ql, qh) of the staged block, by
+// one warp.
+template <int VPL, bool H2>
+__device__ __forceinline__ void score_survivor(const TamTask &tk, const float2 *lut, const int *offs, int s,
+                                               const uint16_t *__restrict__ fh, int ql, int qh) {
+    constexpr int kS = tam_offs_stride(VPL);
+    const int lane = threadIdx.x & 31;
+    const int N = tk.N, k = tk.k, C = tk.C;
+    const uint32_t none = (uint32_t)C + 1u;   // table entry with zero weight
+    int hint = -1;   // the previous orientation's k-th smallest value
+    float e_arg = 0.0f, e_sd = 0.0f;   // lane qi: orientation qi's exponent and s_d
+    for (int qi = ql; qi < qh; ++qi) {
+        const int *ol = offs + (qi * 32 + lane) * kS;   // this lane's offsets, slot s = beam 32 s + lane
+        int sumb = 0;
+        float sgs = 0.0f, sl = 0.0f;
+        int bk;
+        int cle;   // #{b <= bk} over the valid beams
+        if constexpr (H2) {
+            uint32_t hv[VPL / 2];   // fp16 patterns 0x6400 + b of slots 2t (low half) and 2t + 1
+#pragma unroll
+            for (int u = 0; u < (VPL + 3) / 4; ++u) {
+                const int4 o4 = *reinterpret_cast<const int4 *>(ol + 4 * u);
+                const int oo[4] = {o4.x, o4.y, o4.z, o4.w};
+#pragma unroll
+                for (int e = 0; e < 4; e += 2) {
+                    const int t = 2 * u + e / 2;   // pair of slots 2t, 2t + 1
+                    if (t < VPL / 2) {
+                        const int i0 = (t << 6) + lane, i1 = i0 + 32;
+                        uint32_t b0 = none, b1 = none;
+                        if (i0 < N) {
+                            b0 = (uint32_t)__ldg(fh + oo[e]);
+                            sumb += (int)b0;
+                        }
+                        if (i1 < N) {
+                            b1 = (uint32_t)__ldg(fh + oo[e + 1]);
+                            sumb += (int)b1;
+                        }
+                        // both slots at once: b + floor(b / 32) per half, plus the bias
+                        // (slot(C + 1) <= kHalfMaxB: no carry between the halves)
+                        const uint32_t v2 = b0 | (b1 << 16);
+                        hv[t] = v2 + ((v2 >> 5) & 0x07ff07ffu) + (kHalfBias | (kHalfBias << 16));
+                    }
+                }
+            }
+            // #{b > x} on a lane: f(b) - f(x) saturated to [0, 1] is 1 exactly when b > x (f maps
+            // b to the fp16 number of bits 0x6400 + slot(b); the exact difference is then >= 1,
+            // else <= 0, and rounding keeps both); then #{b <= x} over the warp is the 32 VPL
+            // slots less those (no-beam slots are > C)
+            auto count_le = [&](int x) -> int {
+                const unsigned short fxb = (unsigned short)(kHalfBias + lut_slot((uint32_t)x));
+                const __half2 fx = __halves2half2(__ushort_as_half(fxb), __ushort_as_half(fxb));
+                // two chains (half the add latency); the low half starts at 1024, so the
+                // total 1024 + c (c <= 64) has the fp16 bits 0x6400 + c
+                __half2 acc0 = __halves2half2(__ushort_as_half((unsigned short)kHalfBias), __float2half(0.0f));
+                __half2 acc1 = __float2half2_rn(0.0f);
+#pragma unroll
+                for (int t = 0; t < VPL / 2; t += 2) {
+                    acc0 = __hadd2(acc0, __hsub2_sat(*reinterpret_cast<const __half2 *>(&hv[t]), fx));
+                    if (t + 1 < VPL / 2)
+                        acc1 = __hadd2(acc1, __hsub2_sat(*reinterpret_cast<const __half2 *>(&hv[t + 1]), fx));
+                }
+                const __half2 sum = __hadd2(acc0, acc1);
+                const __half2 tot = __hadd2(sum, __lowhigh2highlow(sum));
+                const int gt = __reduce_add_sync(kFull, (int)(__half_as_ushort(__low2half(tot)) & 0x3ffu));
+                return 32 * VPL - gt;
+            };
+            if (tk.fine < kFineBaseline) {
+                bk = kth_smallest(count_le, k, C, N, hint, cle);
+            } else {
+                bk = C;   // every valid beam
+                cle = N;
+            }
+            const uint32_t bkb = kHalfBias + lut_slot((uint32_t)bk);
+#pragma unroll
+            for (int t = 0; t < VPL / 2; ++t) {
+                const uint32_t p0 = hv[t] & 0xffffu, p1 = hv[t] >> 16;
+                const float2 g0 = lut[p0 - kHalfBias], g1 = lut[p1 - kHalfBias];   // slot(C+1) (no beam) adds zero
+                sgs += g0.y + g1.y;
+                if (p0 <= bkb) sl += g0.x;
+                if (p1 <= bkb) sl += g1.x;
+            }
+        } else {
+            uint32_t v[VPL];   // slots of the values
+#pragma unroll
+            for (int t = 0; t < VPL; ++t) {
+                const int i = (t << 5) + lane;
+                uint32_t bv = none;
+                if (i < N) {
+                    bv = (uint32_t)__ldg(fh + ol[t]);
+                    sumb += (int)bv;
+                }
+                v[t] = lut_slot(bv);
+            }
+            auto count_le = [&](int x) -> int {
+                int c = 0;
+                const uint32_t sx = lut_slot((uint32_t)x);
+#pragma unroll
+                for (int t = 0; t < VPL; ++t) c += (v[t] <= sx) ? 1 : 0;
+                return __reduce_add_sync(kFull, c);
+            };
+            if (tk.fine < kFineBaseline) {
+                bk = kth_smallest(count_le, k, C, N, hint, cle);
+            } else {
+                bk = C;
+                cle = N;
+            }
+            const uint32_t sk = lut_slot((uint32_t)bk);
+#pragma unroll
+            for (int t = 0; t < VPL; ++t) {
+                const float2 lg = lut[v[t]];   // the slot of C+1 (no beam) adds zero
+                sgs += lg.y;
+                if (v[t] <= sk) sl += lg.x;
+            }
         }
-        if (s_lut_r != r) {
-            for (int i = threadIdx.x; i <= d.C + 1; i += blockDim.x) lut[lut_slot(i)] = d.lut[i];
+        hint = bk;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            sgs += __shfl_xor_sync(kFull, sgs, o);
+            sl += __shfl_xor_sync(kFull, sl, o);
         }
-        __syncthreads();
-        if (threadIdx.x == 0) s_lut_r = r;
-        if (s_skip) continue;
-        constexpr int kS = tam_offs_stride(VPL);
-        int *offs = reinterpret_cast<int *>(smem + (((size_t)(lut_slot(d.C + 1) + 1) * sizeof(float2) + 15) & ~(size_t)15));
-        const int local = task - s_base[r];
-        const int nblk = (d.n_orient + kTamQ - 1) / kTamQ;
-        const int qb = local % nblk;
-        const int4 ck = d.tam_chunks[d.chunk_cnt[sg.batch_lo] + local / nblk];   // (phase, first, end)
-        const int ph = ck.x;
-        const int q0 = qb * kTamQ;
-        const int nq = min(kTamQ, d.n_orient - q0);
-        const int C = d.C;
-        const uint32_t none = (uint32_t)C + 1u;   // table entry with zero weight
-        const float d_max = d.d_max;
+        sumb = __reduce_add_sync(kFull, sumb);
         {
-            // the block's offsets for phase ph: nq x 32 x kS contiguous ints of the request's table
-            const int4 *src = reinterpret_cast<const int4 *>(d.tam_offs + ((size_t)ph * d.n_orient + q0) * 32 * kS);
-            int4 *dst = reinterpret_cast<int4 *>(offs);
-            const int n4 = nq * 32 * kS / 4;
-            for (int i = threadIdx.x; i < n4; i += blockDim.x) dst[i] = __ldg(src + i);
+            // Eq. 27-30 from the warp totals every lane holds; the top-k sum of l is every
+            // b <= bk less the cle - k ties at bk beyond the k-th; lane qi keeps what its
+            // orientation's score still needs: for TAM the exponent of exp(Lbar) exp(-var / 2)
+            // and s_d
+            const float topsum = sl - (float)(cle - k) * lut[lut_slot(bk)].x;
+            const float lbar = topsum * tk.inv_k;
+            const float dd = tk.res_N * sgs;   // d_max - dbar
+            const float dbar = tk.d_max - dd;
+            const float var = fmaxf(tk.res2_N * (float)sumb - dbar * dbar, 0.0f);
+            const float sd = fminf(dd, tk.span) * tk.inv_span;
+            const int fine = tk.fine;
+            float a = lbar - 0.5f * var;
+            if (fine == kFineTamMean) a = expf(lbar) + expf(-0.5f * var);   // wp + c (Eq. 34)
+            else if (fine == kFineBaseline) a = lbar;                       // wp_LF / N (Eq. 33)
+            else if (fine == kFineLF) a = topsum;                           // wp_LF (Eq. 32)
+            if (lane == qi) {
+                e_arg = a;
+                e_sd = sd;
+            }
+        }
+    }
+    if (lane >= ql && lane < qh) {   // the score of orientation q0 + lane
+        const int q = tk.q0 + lane;
+        const int fine = tk.fine;
+        float T = cbrtf(expf(e_arg) * e_sd);                                   // TAM, Eq. 31
+        if (fine == kFineTamMean) T = (e_arg + e_sd) * (1.0f / 3.0f);         // Eq. 34
+        else if (fine == kFineBaseline) T = sqrtf(expf(e_arg) * e_sd);        // Eq. 33
+        else if (fine == kFineLF) T = e_arg;                                  // Eq. 32
+        tk.T[(size_t)s * tk.n_orient + q] = T;
+        const unsigned long long key = ((unsigned long long)score_code(T) << 32) |
+                                       (unsigned long long)(0xffffffffu - (unsigned)q);
+        atomicMax(tk.best_key + s, key);
+    }
+}
+
+template <int VPL, bool H2>
+__global__ void __launch_bounds__(tam_warps(VPL, H2) * 32, kTamCtas) k_tam(const ReqDesc *__restrict__ reqs, int R,
+                                                                           TamSeg *__restrict__ segs, int stages,
+                                                                           int lut_bytes, int lut_copies,
+                                                                           BatchState *bs) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int s_base[kMaxBatchRequests + 1];
+    __shared__ int s_warp[kMaxBatchRequests / 32];
+    __shared__ TamTask task[kTamStages];
+    constexpr int kWarps = tam_warps(VPL, H2), kThreads = kWarps * 32;
+    static_assert(kThreads >= kMaxBatchRequests, "a thread per request");
+    constexpr int kOffs = kTamQ * 32 * tam_offs_stride(VPL);
+    // one table for all stages when every request of the launch has the same, else one per stage
+    auto lut_of = [&](int i) { return reinterpret_cast<float2 *>(smem + (lut_copies > 1 ? i * lut_bytes : 0)); };
+    int *const offs0 = reinterpret_cast<int *>(smem + lut_copies * lut_bytes);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned int *counter = reinterpret_cast<unsigned int *>(&segs[R].batch_lo);   // tasks taken after the first ones
+    // each request's tasks: its chunks in the launch's batches x its orientation blocks (counted on the device); none
+    // once it has terminated early or when it has no valid beam
+    {
+        const int r = threadIdx.x;
+        int n = 0;
+        if (r < R) {
+            const TamSeg sg = segs[r];
+            const ReqDesc &d = reqs[r];
+            if (sg.batch_hi > sg.batch_lo && !d.state->done && d.scan->n_valid > 0)
+                n = (d.chunk_cnt[sg.batch_hi] - d.chunk_cnt[sg.batch_lo]) * ((d.n_orient + kTamQ - 1) / kTamQ);
+        }
+        int incl = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += v;
+        }
+        if (r < kMaxBatchRequests && lane == 31) s_warp[warp] = incl;
+        __syncthreads();
+        if (r < kMaxBatchRequests) {
+            int before = 0;
+            for (int w = 0; w < warp; ++w) before += s_warp[w];
+            if (r < R) s_base[r] = before + incl - n;
+            if (r == R - 1) s_base[R] = before + incl;
+        }
+        if (threadIdx.x == 0)
+            for (int i = 0; i < kTamStages; ++i) {
+                task[i].lut_src = nullptr;
+                asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&task[i].full)) : "memory");
+            }
+        __syncthreads();
+    }
+    auto arrive = [](TamTask &t) {
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&t.full)) : "memory");
+    };
+    for (int i = 0; i < stages; ++i) {   // the first tasks, staged by the whole CTA
+        const float2 *src = stage_task<VPL>(reqs, R, segs, s_base, (int)blockIdx.x + i * (int)gridDim.x, task[i],
+                                            lut_of(i), lut_copies, offs0 + i * kOffs, threadIdx.x, kThreads);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            // a table that all stages share is filled by the first task; the others take it as theirs
+            for (int j = i; j < (lut_copies > 1 ? i + 1 : stages); ++j) task[j].lut_src = src;
+            arrive(task[i]);
         }
         __syncthreads();
-        for (int js = ck.y + warp; js < ck.z; js += kTamWarps) {
-            const int s = d.surv_perm[js];   // survivor position: its scores go to row s
-            const int2 hc = d.hyps[d.survivors[s]];
-            // the cell's column at the top of its band; the offsets of its phase lead to each endpoint
-            const uint16_t *fh = d.field + 8 * ((size_t)((hc.y + d.P) >> 3) * d.Wp + (hc.x + d.P));
-            int hint = -1;   // the previous orientation's k-th smallest value
-            float e_arg = 0.0f, e_sd = 0.0f;   // lane qi: orientation qi's exponent and s_d
-            for (int qi = 0; qi < nq; ++qi) {
-                const int *ol = offs + (qi * 32 + lane) * kS;   // this lane's offsets, slot s = beam 32 s + lane
-                int sumb = 0;
-                float sgs = 0.0f, sl = 0.0f;
-                int bk;
-                int cle;   // #{b <= bk} over the valid beams
-                if constexpr (H2) {
-                    uint32_t hv[VPL / 2];   // fp16 patterns 0x6400 + b of slots 2t (low half) and 2t + 1
-#pragma unroll
-                    for (int u = 0; u < (VPL + 3) / 4; ++u) {
-                        const int4 o4 = *reinterpret_cast<const int4 *>(ol + 4 * u);
-                        const int oo[4] = {o4.x, o4.y, o4.z, o4.w};
-#pragma unroll
-                        for (int e = 0; e < 4; e += 2) {
-                            const int t = 2 * u + e / 2;   // pair of slots 2t, 2t + 1
-                            if (t < VPL / 2) {
-                                const int i0 = (t << 6) + lane, i1 = i0 + 32;
-                                uint32_t b0 = none, b1 = none;
-                                if (i0 < N) {
-                                    b0 = (uint32_t)__ldg(fh + oo[e]);
-                                    sumb += (int)b0;
-                                }
-                                if (i1 < N) {
-                                    b1 = (uint32_t)__ldg(fh + oo[e + 1]);
-                                    sumb += (int)b1;
-                                }
-                                // both slots at once: b + floor(b / 32) per half, plus the bias
-                                // (slot(C + 1) <= kHalfMaxB: no carry between the halves)
-                                const uint32_t v2 = b0 | (b1 << 16);
-                                hv[t] = v2 + ((v2 >> 5) & 0x07ff07ffu) + (kHalfBias | (kHalfBias << 16));
-                            }
-                        }
-                    }
-                    // #{b > x} on a lane: f(b) - f(x) saturated to [0, 1] is 1 exactly when b > x (f maps
-                    // b to the fp16 number of bits 0x6400 + slot(b); the exact difference is then >= 1,
-                    // else <= 0, and rounding keeps both); then #{b <= x} over the warp is the 32 VPL
-                    // slots less those (no-beam slots are > C)
-                    auto count_le = [&](int x) -> int {
-                        const unsigned short fxb = (unsigned short)(kHalfBias + lut_slot((uint32_t)x));
-                        const __half2 fx = __halves2half2(__ushort_as_half(fxb), __ushort_as_half(fxb));
-                        // two chains (half the add latency); the low half starts at 1024, so the
-                        // total 1024 + c (c <= 64) has the fp16 bits 0x6400 + c
-                        __half2 acc0 = __halves2half2(__ushort_as_half((unsigned short)kHalfBias), __float2half(0.0f));
-                        __half2 acc1 = __float2half2_rn(0.0f);
-#pragma unroll
-                        for (int t = 0; t < VPL / 2; t += 2) {
-                            acc0 = __hadd2(acc0, __hsub2_sat(*reinterpret_cast<const __half2 *>(&hv[t]), fx));
-                            if (t + 1 < VPL / 2)
-                                acc1 = __hadd2(acc1, __hsub2_sat(*reinterpret_cast<const __half2 *>(&hv[t + 1]), fx));
-                        }
-                        const __half2 sum = __hadd2(acc0, acc1);
-                        const __half2 tot = __hadd2(sum, __lowhigh2highlow(sum));
-                        const int gt = __reduce_add_sync(kFull, (int)(__half_as_ushort(__low2half(tot)) & 0x3ffu));
-                        return 32 * VPL - gt;
-                    };
-                    if (s_fine < kFineBaseline) {
-                        bk = kth_smallest(count_le, k, C, N, hint, cle);
-                    } else {
-                        bk = C;   // every valid beam
-                        cle = N;
-                    }
-                    const uint32_t bkb = kHalfBias + lut_slot((uint32_t)bk);
-#pragma unroll
-                    for (int t = 0; t < VPL / 2; ++t) {
-                        const uint32_t p0 = hv[t] & 0xffffu, p1 = hv[t] >> 16;
-                        const float2 g0 = lut[p0 - kHalfBias], g1 = lut[p1 - kHalfBias];   // slot(C+1) (no beam) adds zero
-                        sgs += g0.y + g1.y;
-                        if (p0 <= bkb) sl += g0.x;
-                        if (p1 <= bkb) sl += g1.x;
-                    }
-                } else {
-                    uint32_t v[VPL];   // slots of the values
-#pragma unroll
-                    for (int t = 0; t < VPL; ++t) {
-                        const int i = (t << 5) + lane;
-                        uint32_t bv = none;
-                        if (i < N) {
-                            bv = (uint32_t)__ldg(fh + ol[t]);
-                            sumb += (int)bv;
-                        }
-                        v[t] = lut_slot(bv);
-                    }
-                    auto count_le = [&](int x) -> int {
-                        int c = 0;
-                        const uint32_t sx = lut_slot((uint32_t)x);
-#pragma unroll
-                        for (int t = 0; t < VPL; ++t) c += (v[t] <= sx) ? 1 : 0;
-                        return __reduce_add_sync(kFull, c);
-                    };
-                    if (s_fine < kFineBaseline) {
-                        bk = kth_smallest(count_le, k, C, N, hint, cle);
-                    } else {
-                        bk = C;
-                        cle = N;
-                    }
-                    const uint32_t sk = lut_slot((uint32_t)bk);
-#pragma unroll
-                    for (int t = 0; t < VPL; ++t) {
-                        const float2 lg = lut[v[t]];   // the slot of C+1 (no beam) adds zero
-                        sgs += lg.y;
-                        if (v[t] <= sk) sl += lg.x;
-                    }
+    }
+    unsigned dead = 0;   // stages that hold no further task
+    uint32_t parity = 0;
+    for (int i = 0; dead != (1u << stages) - 1u;) {
+        if (!(dead >> i & 1u)) {
+            TamTask &t = task[i];
+            float2 *lut = lut_of(i);
+            int *offs = offs0 + i * kOffs;
+            if (!wait_full(&t.full, parity)) {
+                if (lane == 0) atomicExch(&bs->error, 1u);
+                return;
+            }
+            const int n = t.n;
+            if (n < 0) {
+                dead |= 1u << i;
+            } else {
+                // with too few survivors for the warps, each takes one orientation of one (its search then starts
+                // from no neighbour's answer): the smallest calls wait for one score instead of a block's
+                const int part = kTamQ * n <= kWarps ? 1 : t.nq, parts = part == 1 ? t.nq : 1;
+                for (;;) {
+                    int j = 0;
+                    if (lane == 0) j = atomicAdd(&t.next, 1);
+                    j = __shfl_sync(kFull, j, 0);
+                    if (j >= n * parts) break;
+                    const int js = parts == 1 ? j : j / parts, ql = parts == 1 ? 0 : j - js * parts;
+                    const int2 sv = __ldg(t.perm + js);
+                    score_survivor<VPL, H2>(t, lut, offs, sv.x, t.field + (unsigned)sv.y, ql, ql + part);
                 }
-                hint = bk;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    sgs += __shfl_xor_sync(kFull, sgs, o);
-                    sl += __shfl_xor_sync(kFull, sl, o);
+                __syncwarp();   // every lane's reads of the stage come before the warp counts itself out
+                int last = 0;
+                if (lane == 0) {
+                    __threadfence_block();
+                    last = atomicAdd(&t.left, 1) == kWarps - 1;
+                    __threadfence_block();
                 }
-                sumb = __reduce_add_sync(kFull, sumb);
-                {
-                    // Eq. 27-30 from the warp totals every lane holds; the top-k sum of l is every
-                    // b <= bk less the cle - k ties at bk beyond the k-th; lane qi keeps what its
-                    // orientation's score still needs: for TAM the exponent of exp(Lbar) exp(-var / 2)
-                    // and s_d
-                    const float topsum = sl - (float)(cle - k) * lut[lut_slot(bk)].x;
-                    const float lbar = topsum * s_ep[0];
-                    const float dd = s_ep[1] * sgs;   // d_max - dbar
-                    const float dbar = d_max - dd;
-                    const float var = fmaxf(s_ep[4] * (float)sumb - dbar * dbar, 0.0f);
-                    const float sd = fminf(dd, s_ep[2]) * s_ep[3];
-                    const int fine = s_fine;
-                    float a = lbar - 0.5f * var;
-                    if (fine == kFineTamMean) a = expf(lbar) + expf(-0.5f * var);   // wp + c (Eq. 34)
-                    else if (fine == kFineBaseline) a = lbar;                       // wp_LF / N (Eq. 33)
-                    else if (fine == kFineLF) a = topsum;                           // wp_LF (Eq. 32)
-                    if (lane == qi) {
-                        e_arg = a;
-                        e_sd = sd;
+                last = __shfl_sync(kFull, last, 0);
+                __syncwarp();
+                if (last) {   // all warps have left: refill the stage
+                    int nt = 0;
+                    if (lane == 0) nt = (int)(atomicAdd(counter, 1u) + (unsigned)stages * gridDim.x);
+                    nt = __shfl_sync(kFull, nt, 0);
+                    const float2 *src = stage_task<VPL>(reqs, R, segs, s_base, nt, t, lut, lut_copies, offs, lane, 32);
+                    __syncwarp();
+                    if (lane == 0) {
+                        t.lut_src = src;
+                        arrive(t);
                     }
                 }
             }
-            if (lane < nq) {   // the score of orientation q0 + lane
-                const int q = q0 + lane;
-                const int fine = s_fine;
-                float T = cbrtf(expf(e_arg) * e_sd);                                   // TAM, Eq. 31
-                if (fine == kFineTamMean) T = (e_arg + e_sd) * (1.0f / 3.0f);         // Eq. 34
-                else if (fine == kFineBaseline) T = sqrtf(expf(e_arg) * e_sd);        // Eq. 33
-                else if (fine == kFineLF) T = e_arg;                                  // Eq. 32
-                d.T[(size_t)s * d.n_orient + q] = T;
-                const unsigned long long key = ((unsigned long long)score_code(T) << 32) |
-                                               (unsigned long long)(0xffffffffu - (unsigned)q);
-                atomicMax(d.best_key + s, key);
-            }
+        }
+        if (++i == stages) {
+            i = 0;
+            parity ^= 1u;
         }
     }
 }
 
 template <int VPL, bool H2>
-cudaError_t run_tam(const ReqDesc *reqs, int R, const TamSeg *segs, const TamPlan &tp, cudaStream_t s) {
+cudaError_t run_tam(const ReqDesc *reqs, int R, TamSeg *segs, const TamPlan &tp, BatchState *bs, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(k_tam<VPL, H2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tp.smem);
     if (e != cudaSuccess) return e;
-    k_tam<VPL, H2><<<tp.grid, kTamWarps * 32, tp.smem, s>>>(reqs, R, segs, tp.total_tasks);
+    k_tam<VPL, H2><<<tp.grid, tam_warps(VPL, H2) * 32, tp.smem, s>>>(reqs, R, segs, tp.stages, tp.lut_bytes, tp.lut_copies,
+                                                                    bs);
     return cudaGetLastError();
 }
 
 template <int VPL, bool H2>
 int tam_occupancy(size_t smem) {
     int occ = 0;
-    if (cudaFuncSetAttribute(k_tam<VPL, H2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    if (cudaFuncSetAttribute(k_tam<VPL, H2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+        cudaGetLastError();   // more than an SM has: no CTA fits
         return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_tam<VPL, H2>, kTamWarps * 32, smem) != cudaSuccess)
+    }
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_tam<VPL, H2>, tam_warps(VPL, H2) * 32, smem) != cudaSuccess)
         return 0;
     return occ;
 }
@@ -453,26 +625,43 @@ cudaError_t launch_scan_prep(const ReqDesc *reqs, int R, cudaStream_t s) {
 
 // The launch for the batches [batch_lo[r], batch_hi[r]) of every request:
 // its kernel class (values per lane and selection precision for the longest
-// scan and the largest clamp), the shared memory (table and one block's
-// endpoint offsets) and a grid of every resident CTA (or ctas_per_sm per SM
-// when that is fewer); the tasks are counted by the kernel from the
-// device-built chunk tables.
+// scan and the largest clamp), its stages, and a grid of every resident CTA (or
+// ctas_per_sm per SM when that is fewer); the tasks are counted by the kernel
+// from the device-built chunk tables.  chunk: survivors of a usual task; lut_copies:
+// 1 when all requests share one likelihood table.  segs: R entries and the
+// task counter.
+//
+// A stage is refilled once its slowest survivor is done, so the stages together hold about twice the survivors that
+// the warps work on (never fewer than two stages); they may not cost a resident CTA.
 TamPlan plan_tam(const int *batch_lo, const int *batch_hi, int R, int max_beams, int max_C, int n_sm,
-                 int ctas_per_sm, TamSeg *segs) {
-    TamPlan tp{0, 0, vpl_bucket(max_beams), 0, (int)lut_slot(max_C + 1) <= kHalfMaxB};
+                 int ctas_per_sm, int chunk, int luts, TamSeg *segs) {
+    TamPlan tp{0, 0, vpl_bucket(max_beams), 0, 1, 0, 1, (int)lut_slot(max_C + 1) <= kHalfMaxB};
     if (tp.vpl < 0) return tp;
-    tp.smem = (((size_t)(lut_slot(max_C + 1) + 1) * sizeof(float2) + 15) & ~(size_t)15) +
-              (size_t)kTamQ * 32 * tam_offs_stride(tp.vpl) * sizeof(int);
-    const int occ = occupancy_for(tp.vpl, tp.h2, tp.smem);
+    tp.lut_bytes = (int)(((size_t)(lut_slot(max_C + 1) + 1) * sizeof(float2) + 15) & ~(size_t)15);
+    const size_t offs = (size_t)kTamQ * 32 * tam_offs_stride(tp.vpl) * sizeof(int);
+    auto bytes = [&](int stages) { return (size_t)tp.lut_bytes * (luts > 1 ? stages : 1) + stages * offs; };
+    const int want = std::min(kTamStages, std::max(2, (9 * tam_warps(tp.vpl, tp.h2) + 4 * chunk - 1) / (4 * chunk)));
+    int occ = 0;
+    for (int st = want; st >= 1; --st) {   // the most stages among those with the most CTAs
+        const int o = std::min(kTamCtas, occupancy_for(tp.vpl, tp.h2, bytes(st)));
+        if (o > occ) {
+            occ = o;
+            tp.stages = st;
+            tp.smem = bytes(st);
+        }
+        if (occ == kTamCtas) break;
+    }
     if (occ < 1) {
         tp.vpl = -1;
         return tp;
     }
+    tp.lut_copies = luts > 1 ? tp.stages : 1;
     bool any = false;
     for (int r = 0; r < R; ++r) {
         segs[r] = TamSeg{batch_lo[r], batch_hi[r]};
         any = any || batch_hi[r] > batch_lo[r];
     }
+    segs[R] = TamSeg{0, 0};
     tp.total_tasks = any ? 1 : 0;
     tp.grid = n_sm * (ctas_per_sm > 0 && ctas_per_sm < occ ? ctas_per_sm : occ);
     return tp;
@@ -480,10 +669,11 @@ TamPlan plan_tam(const int *batch_lo, const int *batch_hi, int R, int max_beams,
 
 int tam_offs_stride_for(int vpl) { return tam_offs_stride(vpl); }
 
-cudaError_t launch_tam(const ReqDesc *reqs, int R, const TamSeg *segs, const TamPlan &tp, cudaStream_t s) {
+cudaError_t launch_tam(const ReqDesc *reqs, int R, TamSeg *segs, const TamPlan &tp, BatchState *bs, cudaStream_t s) {
     if (tp.total_tasks <= 0) return cudaSuccess;
-#define RELO_TAM_RUN(V) \
-    if (tp.vpl == V) return tp.h2 ? run_tam<V, true>(reqs, R, segs, tp, s) : run_tam<V, false>(reqs, R, segs, tp, s);
+#define RELO_TAM_RUN(V)                                                                 \
+    if (tp.vpl == V)                                                                    \
+        return tp.h2 ? run_tam<V, true>(reqs, R, segs, tp, bs, s) : run_tam<V, false>(reqs, R, segs, tp, bs, s);
     RELO_TAM_VPLS(RELO_TAM_RUN)
 #undef RELO_TAM_RUN
     return cudaErrorInvalidValue;

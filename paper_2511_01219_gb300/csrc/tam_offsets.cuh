@@ -1,7 +1,7 @@
 // TAM's inputs that the top-K launch prepares (select.cu): each request's
 // work order (survivors grouped by band phase, in chunks), built by its
 // ranking CTA once the survivors are known, and the endpoint offsets of its
-// plan (Eq. 13's endpoint cells, as offsets into the banded field), computed
+// plan (Eq. 13's endpoint cells), computed
 // by the other CTAs of the launch beside the ranking ones.
 #pragma once
 #include <cuda_runtime.h>
@@ -11,19 +11,18 @@
 
 namespace relo {
 
-// Every request's endpoint offsets, once per batch: for band phase ph,
-// orientation q (m = q n_enum) and valid beam i, the field_index offset of the
-// endpoint cell round-half-up(R_i * D_{(b_i + m) mod N_s} / 2^46) per axis from
-// a cell of band phase ph (linear in the x offset, and in the y offset through
-// the bands crossed), laid out [ph][q][lane][slot] with the TAM kernel's
-// per-lane stride, so one block's offsets for one phase are one contiguous
-// span.  One CTA writes all eight phases of orientation q.
+// Every request's endpoint cells, once per batch: for orientation q (m = q
+// n_enum) and valid beam i, the offsets round-half-up(R_i * D_{(b_i + m) mod
+// N_s} / 2^46) per axis (each below 2^15), packed y << 16 | x, laid out
+// [q][lane][slot] with the TAM kernel's per-lane stride, so one block of
+// orientations is one contiguous span.  TAM turns a block's cells into field
+// offsets for its task's band phase as it stages them: a table per phase (8
+// times the bytes) cost the batched workload more to write and read back than
+// those few operations per task.  One CTA writes orientation q.
 __device__ __forceinline__ void tam_offsets_one(const ReqDesc &d, int q) {
     const int N = d.scan->n_valid;
     const int m = q * d.n_enum;
-    const long long Wp8 = 8ll * d.Wp;
     const int kS = d.tam_stride;
-    const size_t phase_step = (size_t)d.n_orient * 32 * kS;
     int32_t *oq = d.tam_offs + (size_t)q * 32 * kS;
     // k walks the orientation's table in memory order (lane-major), so every store is coalesced
     for (int k = threadIdx.x; k < 32 * kS; k += blockDim.x) {
@@ -36,11 +35,7 @@ __device__ __forceinline__ void tam_offsets_one(const ReqDesc &d, int q) {
         const int ox = (int)(((long long)bR.y * dir.x + (1ll << 45)) >> 46);
         const int oy = (int)(((long long)bR.y * dir.y + (1ll << 45)) >> 46);
         // |ox|, |oy| < P keeps every endpoint inside the field's border
-#pragma unroll
-        for (int ph = 0; ph < 8; ++ph) {
-            const int v = ph + oy;
-            oq[ph * phase_step + k] = (int)(8ll * ox + Wp8 * (v >> 3)) + (v & 7);
-        }
+        oq[k] = (int)((unsigned)oy << 16 | ((unsigned)ox & 0xffffu));
     }
 }
 
@@ -69,9 +64,10 @@ __device__ __forceinline__ void tam_chunks_one(const ReqDesc &d) {
             int run = lo, nc = s_chunks;
             for (int p = 0; p < 8; ++p) {
                 s_next[p] = run;
-                for (int f = run; f < run + s_cnt[p]; f += d.tam_chunk)
-                    d.tam_chunks[nc++] = make_int4(p, f, min(run + s_cnt[p], f + d.tam_chunk), 0);
-                run += s_cnt[p];
+                const int n = s_cnt[p], parts = (n + d.tam_chunk - 1) / d.tam_chunk;   // of equal size, within one
+                for (int c = 0; c < parts; ++c)
+                    d.tam_chunks[nc++] = make_int4(p, run + n * c / parts, run + n * (c + 1) / parts, 0);
+                run += n;
             }
             s_chunks = nc;
             if (d.early_stop) d.chunk_cnt[b + 1] = nc;
@@ -79,8 +75,11 @@ __device__ __forceinline__ void tam_chunks_one(const ReqDesc &d) {
                 for (int j = 1; j <= d.n_batches; ++j) d.chunk_cnt[j] = nc;
         }
         __syncthreads();
-        for (int i = lo + threadIdx.x; i < hi; i += blockDim.x)
-            d.surv_perm[atomicAdd(&s_next[(d.hyps[d.survivors[i]].y + d.P) & 7], 1)] = i;
+        for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+            const int2 c = d.hyps[d.survivors[i]];
+            const unsigned base = 8u * ((unsigned)((c.y + d.P) >> 3) * (unsigned)d.Wp + (unsigned)(c.x + d.P));
+            d.surv_perm[atomicAdd(&s_next[(c.y + d.P) & 7], 1)] = make_int2(i, (int)base);
+        }
         __syncthreads();
     }
 }
