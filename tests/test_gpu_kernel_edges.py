@@ -1,0 +1,93 @@
+"""Kernels at the sizes where their tiling changes: remainders of tiles and
+stages, the smallest and the largest of a range, both sides of a dispatch."""
+import numpy as np
+import pytest
+
+import oracle
+import workloads
+from test_gpu_parity import full_case, relo, small_case   # noqa: F401  (relo: the module fixture)
+
+pytestmark = pytest.mark.gpu
+RES = 0.05
+
+
+@pytest.mark.parametrize("early", [False, True])
+@pytest.mark.parametrize("n_orient", [6, 120])
+@pytest.mark.parametrize("K", [1, 5, 17, 30])
+def test_tam_tasks_of_few_survivors(relo, K, n_orient, early):
+    """TAM tasks that split by orientation and tasks that do not, blocks of 4 and a remainder of 2 orientations: scores,
+    argmax and survivors against the oracle (full_case's bounds)."""
+    wl = small_case(n_orient=n_orient)
+    full_case(relo, wl, K, early_stop=early, batch=7, local_topk=2, tau=2.0)[0].close()
+
+
+@pytest.mark.parametrize("d_max_cells", [40, 80, 90])
+def test_tam_tables_of_different_resolutions_in_one_batch(relo, d_max_cells):
+    """Maps of different resolution have different likelihood tables: one launch scores both (a table per stage, and at
+    the largest clamp a single stage), every result and the first request's scores as alone, bit for bit."""
+    import torch
+    wl = small_case()
+    ctx = relo.Relo(n_orient=40, topk=30, batch=11, local_topk=3, early_stop=0, d_max=0.05 * d_max_cells)
+    reqs = []
+    for res in (0.05, 0.1, 0.05):
+        mid = ctx.load_map(wl.grid, res)
+        ctx.set_hypotheses(mid, workloads.cell_centres(wl.hyps, res))
+        reqs.append((mid, wl.ranges * (res / 0.05), wl.angles, wl.max_range * (res / 0.05)))
+
+    def scores(rows):
+        return ctx.stage(relo.STAGE_TAM, torch.empty((rows, 40), device="cuda")).cpu().numpy()
+    alone = []
+    for q in reqs:
+        alone.append((ctx.relocalize(*q).as_dict(), scores(30)))
+    for first in range(3):
+        order = [reqs[(first + i) % 3] for i in range(3)]
+        got = ctx.relocalize_batch(order)
+        assert [g.as_dict() for g in got] == [alone[(first + i) % 3][0] for i in range(3)]
+        assert np.array_equal(scores(30).view(np.uint32), alone[first][1].view(np.uint32))
+    ctx.close()
+
+
+@pytest.mark.parametrize("cells,ns", [(1, 360), (33, 90), (7, 361)])
+def test_synth_scans_beyond_the_32_bit_root(relo, cells, ns):
+    """Hits on both sides of 1024 cells (where the range's square root changes form), against cell-by-cell stepping and
+    the oracle."""
+    import torch
+    g = np.zeros((40, 1500), np.int8)
+    g[0] = g[-1] = 100
+    g[:, 0] = g[:, -1] = 100
+    g[10:14, 1100] = 100
+    xy = np.array([[3 + 2 * i, 20] for i in range(cells)], np.int32)
+    ang = workloads.beam_angles(ns, ns)
+    out = []
+    for tables in (1, 0):
+        ctx = relo.Relo(n_orient=0, ray_tables=tables)
+        mid = ctx.load_map(g, RES)
+        r, h = ctx.synth_scans(mid, torch.from_numpy(xy).cuda(), ang, 80.0, ns)
+        out.append((r.cpu().numpy(), h.cpu().numpy()))
+        ctx.close()
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+    pl = oracle.plan(np.full(ns, 1.0, np.float32), ang, 80.0, RES, oracle.Params(n_orient=0))
+    for k in range(cells):
+        want, hx, hy = oracle.synth_scan(g, int(xy[k, 0]), int(xy[k, 1]), pl)
+        assert np.array_equal(out[0][0][k].astype(np.int64), want)
+    assert (out[0][0] >= 1024 << 16).any() and (out[0][0] < 1024 << 16).any()
+
+
+@pytest.mark.parametrize("rho,points", [(0.25, 164), (0.2, 256), (0.1998, 257), (0.14, 523)])
+def test_rrt_sub_batches(relo, rho, points):
+    """A round shorter than a sub-batch, exactly one, one point more, and two with a remainder: the serial tree, bit for
+    bit, over several rounds."""
+    import math
+
+    import torch
+    from rrt_f32 import serial_rrt
+    g = workloads.make_room(1000)
+    assert math.ceil(g.size * RES * RES / (rho * rho)) == points
+    clr = workloads.clearance_table(g, RES)
+    p0 = workloads.free_start(g, RES, 0.21, 7, clr)
+    want, rounds, nodes = serial_rrt(clr, RES, p0, rho, 0.6, 0.21, 0, 5, max_rounds=6)
+    ctx = relo.Relo()
+    got, r, n = ctx.rrt_hypotheses(torch.tensor(clr, device="cuda"), RES, p0, rho, 0.6, 0.21, 0, seed=5, max_rounds=6)
+    ctx.close()
+    assert (r, n) == (rounds, nodes)
+    assert np.array_equal(got.cpu().numpy(), want)
