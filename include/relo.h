@@ -416,7 +416,7 @@ int relo_rrt_sample(relo_ctx *ctx, const int8_t *grid, int32_t w, int32_t h, dou
  * has no occupied cell), asynchronously on stream (a cudaStream_t; NULL = the
  * default stream), with no context and no allocation: the caller owns the
  * input and the output, and the scratch is a file-scope device array of
- * fixed size (4.5 MiB per device, held until the process exits).
+ * fixed size (0.7 MiB per device, held until the process exits).
  * Returns RELO_E_INVALID_ARG for null pointers or w, h outside [1, 1024],
  * RELO_E_CUDA if a CUDA call or a launch fails, or if a CUDA error from
  * earlier work is already pending in the calling thread (nothing is then

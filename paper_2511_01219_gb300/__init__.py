@@ -266,11 +266,11 @@ class Relo:
         import torch
         H, W = shape
         d2 = torch.empty((H, W), dtype=torch.int32, device="cuda")
-        fld = torch.empty((H, W), dtype=torch.int16, device="cuda")
+        fld = torch.empty((H, W), dtype=torch.uint16, device="cuda")
         occ = torch.empty((H, W), dtype=torch.uint8, device="cuda")
         self._check(self._L.relo_map_tables_dev(self._h, map_id, _t_ptr(d2), _t_ptr(fld), _t_ptr(occ)),
                     "map_tables")
-        return d2, fld.to(torch.int32) & 0xFFFF, occ
+        return d2, fld.to(torch.int32), occ
 
     def walk_boxes(self, map_id: int, shape):
         """The ray walk's empty boxes of tiles (relo_map_walk_boxes_dev) as an int32 numpy array

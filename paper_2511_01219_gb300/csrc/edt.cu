@@ -8,157 +8,43 @@
 // of P cells holding C on every side, P at least the longest beam in cells, so
 // every beam endpoint of TAM falls inside the array and needs no bounds test.
 //
-// d2(x, y) = min over occupied (x', y') of (x - x')^2 + (y - y')^2 separates
-// into a column term g2(x', y) = min over occupied y' in column x' of
-// (y - y')^2 and a row minimisation d2(x, y) = min over x' of (x - x')^2 +
-// g2(x', y).  The column term comes from two sweeps per column (coalesced
-// across columns); the row minimisation stages one row in shared memory and
-// each thread scans outward from its cell, stopping once (x - x')^2 alone
-// reaches the best value found, which no further column can beat.
+// The distance passes themselves are in edt_band.cuh; the tile pass here also
+// lays out the walk frames and, where the caller's grid allows it, writes the
+// map's own copy of the grid.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "edt_band.cuh"
 #include "relo_internal.h"
 
 namespace relo {
 
 namespace {
 
-constexpr int kInf = 0x7fffffff;
-
-// Column term, step 1: for every (column, segment of L rows) the first and the
-// last occupied row inside the segment (-1 if none).  The same pass builds the
-// occupancy bitmaps: a warp covers 32 consecutive columns (four 8x8 tiles) and
-// L is a multiple of 8, so the ballot of each row gives four tile rows, which
-// lanes 0-3 collect into their tile's word (cells outside the map are free).
-// The word is stored as is, and, with the cells outside the map set, into the
-// four walk frames: as is, and mirrored in x (x' = 8 TW - 1 - x: tile TW - 1 -
-// tx, bits reversed within each row), in y (rows reversed) and in both (all 64
-// bits reversed), which the ray cast uses so that every ray travels towards +x
-// and +y.
-__global__ void k_edt_col_summary(const int8_t *__restrict__ grid, int W, int H, int L, int TW, int TH,
-                                  int2 *__restrict__ summ, uint64_t *__restrict__ bits) {
-    const int lane = threadIdx.x & 31;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int x0 = x - lane;
-    const int sgm = blockIdx.y;
-    if (x0 >= W) return;   // the whole warp lies right of the map
-    const int y0 = sgm * L;
-    int first = -1, last = -1;
-    // a tile row (8 grid rows; L and y0 are multiples of 8) at a time, its 8 loads issued together
-    for (int yb = y0; yb < y0 + L; yb += 8) {
-        bool occ8[8], in8[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            in8[u] = x < W && yb + u < H;
-            occ8[u] = in8[u] && grid[(size_t)(yb + u) * W + x] >= 65;
-        }
-        uint64_t word = 0ull, wword = 0ull;   // the map's word; the walk frames' word (outside cells set)
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            if (occ8[u]) {
-                if (first < 0) first = yb + u;
-                last = yb + u;
-            }
-            const unsigned b = __ballot_sync(0xffffffffu, occ8[u]);
-            const unsigned bw = __ballot_sync(0xffffffffu, occ8[u] || !in8[u]);
-            word |= (uint64_t)((b >> (8 * (lane & 3))) & 0xffu) << (8 * u);
-            wword |= (uint64_t)((bw >> (8 * (lane & 3))) & 0xffu) << (8 * u);
-        }
-        const int tx = (x0 >> 3) + lane, ty = yb >> 3;
-        if (lane < 4 && tx < TW && ty < TH) {
-            const size_t WB = (size_t)TW + 1, n = walk_frame_words(TW, TH);
-            uint64_t *wf = bits + (size_t)TW * TH;
-            const uint64_t rev = __brevll(wword);   // both mirrors
-            const uint64_t ymir = ((uint64_t)__byte_perm((uint32_t)wword, 0u, 0x0123u) << 32) |
-                                  (uint64_t)__byte_perm((uint32_t)(wword >> 32), 0u, 0x0123u);
-            const uint64_t xmir = ((uint64_t)__byte_perm((uint32_t)rev, 0u, 0x0123u) << 32) |
-                                  (uint64_t)__byte_perm((uint32_t)(rev >> 32), 0u, 0x0123u);
-            bits[(size_t)ty * TW + tx] = word;
-            wf[(size_t)ty * WB + tx] = wword;
-            wf[n + (size_t)ty * WB + (TW - 1 - tx)] = xmir;
-            wf[2 * n + (size_t)(TH - 1 - ty) * WB + tx] = ymir;
-            wf[3 * n + (size_t)(TH - 1 - ty) * WB + (TW - 1 - tx)] = rev;
-        }
-    }
-    if (x < W) summ[(size_t)sgm * W + x] = make_int2(first, last);
+// Occupancy tiles, column summaries and walk frames: the map's word as is, and, with the cells outside the map set, the
+// four walk frames: as is, and mirrored in x (x' = 8 TW - 1 - x: tile TW - 1 - tx, bits reversed within each row), in y
+// (rows reversed) and in both (all 64 bits reversed), which the ray cast uses so that every ray travels towards +x and
+// +y.  A thread reads a tile's 8 rows of 8 bytes with 8 loads in flight (32 bytes a row of the warp are 8 tiles wide); a
+// ballot per row of 32 columns with a byte load per cell took 26 us on the 4096 x 4096 warehouse, this takes 9 us
+// (with the copy of the grid, which was another 9 us).
+__global__ void __launch_bounds__(256) k_edt_tiles(const int8_t *__restrict__ grid, EdtTiles t, bool vec, int8_t *copy,
+                                                   uint64_t *wf) {
+    edt_tiles(grid, t, vec, copy, [&](uint64_t w, int tx, int ty) {
+        const size_t WB = (size_t)t.TW + 1, n = walk_frame_words(t.TW, t.TH);
+        const uint64_t rev = __brevll(w);   // both mirrors
+        const uint64_t ymir = ((uint64_t)__byte_perm((uint32_t)w, 0u, 0x0123u) << 32) |
+                              (uint64_t)__byte_perm((uint32_t)(w >> 32), 0u, 0x0123u);
+        const uint64_t xmir = ((uint64_t)__byte_perm((uint32_t)rev, 0u, 0x0123u) << 32) |
+                              (uint64_t)__byte_perm((uint32_t)(rev >> 32), 0u, 0x0123u);
+        const int mx = t.TW - 1 - tx, my = t.TH - 1 - ty;
+        wf[(size_t)ty * WB + tx] = w;
+        wf[n + (size_t)ty * WB + mx] = xmir;
+        wf[2 * n + (size_t)my * WB + tx] = ymir;
+        wf[3 * n + (size_t)my * WB + mx] = rev;
+    });
 }
 
-// Column term, step 2: the nearest occupied rows above and below the segment
-// come from the other segments' summaries; one downward and one upward sweep
-// inside the segment then give g(x, y) = distance to the nearest occupied
-// cell of the column, stored squared (kInf when the column has none).
-__global__ void k_edt_col_final(const int8_t *__restrict__ grid, int W, int H, int L, int S,
-                                const int2 *__restrict__ summ, int32_t *__restrict__ colsq) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int sgm = blockIdx.y;
-    if (x >= W) return;
-    int last = -1;    // nearest occupied row above the segment
-    for (int t = 0; t < sgm; ++t) {
-        const int v = summ[(size_t)t * W + x].y;
-        if (v >= 0) last = v;
-    }
-    int next = -1;    // nearest occupied row below the segment
-    for (int t = S - 1; t > sgm; --t) {
-        const int v = summ[(size_t)t * W + x].x;
-        if (v >= 0) next = v;
-    }
-    const int y0 = sgm * L, y1 = min(H, y0 + L);
-    for (int y = y0; y < y1; ++y) {
-        const size_t i = (size_t)y * W + x;
-        if (grid[i] >= 65) last = y;
-        colsq[i] = last < 0 ? kInf : y - last;
-    }
-    for (int y = y1 - 1; y >= y0; --y) {
-        const size_t i = (size_t)y * W + x;
-        if (grid[i] >= 65) next = y;
-        const int up = colsq[i];
-        const int dn = next < 0 ? kInf : next - y;
-        const int g = up < dn ? up : dn;
-        colsq[i] = g == kInf ? kInf : g * g;
-    }
-}
-
-// The row is staged with W + 4 cells of sentinel on each side and "no
-// obstacle in this column" as the same sentinel, a value larger than any
-// squared distance that still leaves room for dx^2, so the outward scan needs
-// no bounds or sentinel tests: a sentinel never improves the minimum.  The
-// scan takes four distances per step (their loads independent of each other),
-// so a cell waits on a shared-memory round trip once per four columns; the up
-// to three columns it looks at beyond the stopping distance are ordinary
-// candidates and leave the minimum exact.
-constexpr int kRowSentinel = 0x3fffffff;
-constexpr int kRowPad = 4;   // the scan's step, and the extra sentinels it may read past the row's reach
-
-__global__ void k_edt_rows(const int32_t *__restrict__ colsq, int W, int C, int P, int Wp, int32_t *__restrict__ d2,
-                           uint16_t *__restrict__ field) {
-    extern __shared__ int32_t rowbuf[];   // [3W + 2 kRowPad]: sentinels, the row, sentinels
-    int32_t *row = rowbuf + W + kRowPad;
-    const int y = blockIdx.x;
-    const int32_t *src = colsq + (size_t)y * W;
-    for (int x = threadIdx.x; x < W + kRowPad; x += blockDim.x) {
-        rowbuf[x] = kRowSentinel;
-        row[W + x] = kRowSentinel;
-    }
-    for (int x = threadIdx.x; x < W; x += blockDim.x) {
-        const int v = src[x];
-        row[x] = v == kInf ? kRowSentinel : v;
-    }
-    __syncthreads();
-    for (int x = threadIdx.x; x < W; x += blockDim.x) {
-        int best = row[x];
-        const int reach = x > W - 1 - x ? x : W - 1 - x;   // past this both sides are sentinels
-        for (int dx = 1; dx <= reach && dx * dx < best; dx += kRowPad) {
-            const int a = min(row[x - dx], row[x + dx]) + dx * dx;
-            const int b = min(row[x - dx - 1], row[x + dx + 1]) + (dx + 1) * (dx + 1);
-            const int c = min(row[x - dx - 2], row[x + dx + 2]) + (dx + 2) * (dx + 2);
-            const int e4 = min(row[x - dx - 3], row[x + dx + 3]) + (dx + 3) * (dx + 3);
-            best = min(best, min(min(a, b), min(c, e4)));
-        }
-        d2[(size_t)y * W + x] = best >= kRowSentinel ? kD2None : best;
-        field[field_index(x + P, y + P, Wp)] = (uint16_t)(best > C ? C : best);
-    }
-}
+EdtTiles tiles_of(const MapDev &m) { return EdtTiles{m.bits, m.summ, edt_span_of(m), m.far, m.W, m.H, m.TW, m.TH}; }
 
 // the border of the padded field: every cell outside the map reads C (d = d_max)
 __global__ void k_field_border(uint16_t *__restrict__ fieldp, int W, int H, int P, int Wp, int Hp, int C) {
@@ -229,16 +115,45 @@ __global__ void k_walk_border(uint64_t *__restrict__ wf, int TW, int TH) {
     for (int i = threadIdx.x; i < TW; i += blockDim.x) f[(size_t)TH * WB + i] = ~0ull;
 }
 
-__global__ void k_map_tables(const int32_t *__restrict__ d2s, const uint16_t *__restrict__ fs,
-                             const uint64_t *__restrict__ bs, int W, int H, int TW, int P, int Wp, int32_t *d2,
-                             uint16_t *field,
-                             uint8_t *occ) {
-    size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (size_t)W * H) return;
-    int x = (int)(i % W), y = (int)(i / W);
-    if (d2) d2[i] = d2s[i];
-    if (field) field[i] = fs[field_index(x + P, y + P, Wp)];
-    if (occ) occ[i] = (uint8_t)((bs[(size_t)(y >> 3) * TW + (x >> 3)] >> (((y & 7) << 3) | (x & 7))) & 1ull);
+// The tables row-major: a thread takes kCols columns (4 where rows and buffers are aligned for vector stores, else 1) of
+// one field band (8 rows, each column 16 contiguous bytes of the field), so every field load is 16 bytes and the lanes
+// of a warp store neighbouring columns; one cell per thread read 2 of every 16 field bytes and divided for its
+// coordinates (87 us on 4001 x 3500, now 38).
+template <int kCols>
+__global__ void __launch_bounds__(128) k_map_tables(const int32_t *__restrict__ d2s, const uint16_t *__restrict__ fs,
+                                                    const uint64_t *__restrict__ bs, int W, int H, int TW, int P, int Wp,
+                                                    int32_t *__restrict__ d2, uint16_t *__restrict__ field,
+                                                    uint8_t *__restrict__ occ) {
+    const int B = (P >> 3) + (int)blockIdx.y, y0 = 8 * B - P, x0 = kCols * ((int)blockIdx.x * 128 + (int)threadIdx.x);
+    if (x0 >= W) return;   // kCols divides W
+    uint4 f[kCols] = {};
+    if (field)
+#pragma unroll
+        for (int i = 0; i < kCols; ++i) f[i] = *reinterpret_cast<const uint4 *>(fs + 8 * ((size_t)B * Wp + (x0 + i + P)));
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const int y = y0 + u;
+        if (y < 0 || y >= H) continue;
+        const size_t at = (size_t)y * W + x0;
+        uint32_t h[kCols];
+#pragma unroll
+        for (int i = 0; i < kCols; ++i) {
+            const uint32_t w = u < 2 ? f[i].x : u < 4 ? f[i].y : u < 6 ? f[i].z : f[i].w;
+            h[i] = w >> (16 * (u & 1)) & 0xffffu;
+        }
+        uint32_t o = 0u;   // the cells' occupancy bits (of one tile row)
+        if (occ) o = (uint32_t)(bs[(size_t)(y >> 3) * TW + (x0 >> 3)] >> (((y & 7) << 3) | (x0 & 7)));
+        if constexpr (kCols == 4) {
+            if (d2) *reinterpret_cast<int4 *>(d2 + at) = *reinterpret_cast<const int4 *>(d2s + at);
+            if (field) *reinterpret_cast<uint2 *>(field + at) = make_uint2(h[0] | h[1] << 16, h[2] | h[3] << 16);
+            if (occ)
+                *reinterpret_cast<uint32_t *>(occ + at) = (o & 1u) | (o & 2u) << 7 | (o & 4u) << 14 | (o & 8u) << 21;
+        } else {
+            if (d2) d2[at] = d2s[at];
+            if (field) field[at] = (uint16_t)h[0];
+            if (occ) occ[at] = (uint8_t)(o & 1u);
+        }
+    }
 }
 
 __global__ void k_check_cells(const int2 *__restrict__ cells, int n, const uint64_t *__restrict__ bits, int W,
@@ -283,10 +198,17 @@ cudaError_t launch_xy_cells(const double *xy, int n, double ox, double oy, doubl
     return cudaGetLastError();
 }
 
-cudaError_t launch_edt_tiles(const MapDev &m, cudaStream_t s) {
-    const int L = edt_segment_rows(m.H), S = (m.H + L - 1) / L;
-    const dim3 cgrid((m.W + 127) / 128, S);
-    k_edt_col_summary<<<cgrid, 128, 0, s>>>(m.grid, m.W, m.H, L, m.TW, m.TH, m.summ, m.bits);
+cudaError_t launch_edt_tiles(const MapDev &m, const int8_t *grid, cudaStream_t s) {
+    const EdtTiles t = tiles_of(m);
+    const bool vec = (m.W & 7) == 0 && (reinterpret_cast<uintptr_t>(grid) & 7) == 0;
+    int8_t *copy = grid != m.grid ? m.grid : nullptr;
+    if (copy && !vec) {
+        const cudaError_t e = cudaMemcpyAsync(m.grid, grid, (size_t)m.W * m.H, cudaMemcpyDeviceToDevice, s);
+        if (e != cudaSuccess) return e;
+        return launch_edt_tiles(m, m.grid, s);
+    }
+    k_edt_tiles<<<dim3((m.TW + 31) / 32, edt_summary_rows(m.H)), dim3(32, 8), 0, s>>>(grid, t, vec, copy,
+                                                                                      m.bits + (size_t)m.TW * m.TH);
     if (m.reach) {
         // the walk frames' empty boxes (their border tiles, full, were written when the map was loaded)
         const unsigned WB = (unsigned)m.TW + 1u, SW = walk_empty_row_words(m.TW), rows = 4u * ((unsigned)m.TH + 1u);
@@ -297,24 +219,13 @@ cudaError_t launch_edt_tiles(const MapDev &m, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_edt_field(const MapDev &m, cudaStream_t s) {
-    const int L = edt_segment_rows(m.H), S = (m.H + L - 1) / L;
-    const dim3 cgrid((m.W + 127) / 128, S);
-    k_edt_col_final<<<cgrid, 128, 0, s>>>(m.grid, m.W, m.H, L, S, m.summ, m.colsq);
-    size_t smem = ((size_t)3 * m.W + 2 * kRowPad) * sizeof(int32_t);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_edt_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    // 512 threads: shared memory admits 4 rows of 49 KB per SM at W = 4096, and 16 warps each fill all 64 warp
-    // slots (256 threads left half of them empty: 171 -> 148 us per warehouse launch)
-    k_edt_rows<<<m.H, 512, smem, s>>>(m.colsq, m.W, m.C, m.P, m.Wp, m.d2, m.field);
-    return cudaGetLastError();
+cudaError_t launch_edt_field(const MapDev &m, int n_sm, cudaStream_t s) {
+    return launch_edt_bands(tiles_of(m), EdtOut{m.d2, m.field, m.C, m.P, m.Wp}, n_sm, s);
 }
 
-cudaError_t launch_edt(const MapDev &m, cudaStream_t s) {
-    cudaError_t e = launch_edt_tiles(m, s);
-    return e == cudaSuccess ? launch_edt_field(m, s) : e;
+cudaError_t launch_edt(const MapDev &m, int n_sm, cudaStream_t s) {
+    cudaError_t e = launch_edt_tiles(m, m.grid, s);
+    return e == cudaSuccess ? launch_edt_field(m, n_sm, s) : e;
 }
 
 cudaError_t launch_field_border(const MapDev &m, cudaStream_t s) {
@@ -324,9 +235,15 @@ cudaError_t launch_field_border(const MapDev &m, cudaStream_t s) {
 }
 
 cudaError_t launch_map_tables(const MapDev &m, int32_t *d2, uint16_t *field, uint8_t *occ, cudaStream_t s) {
-    size_t n = (size_t)m.W * m.H;
-    k_map_tables<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(m.d2, m.field, m.bits, m.W, m.H, m.TW, m.P, m.Wp, d2, field,
-                                                             occ);
+    const bool vec = (m.W & 3) == 0 && (reinterpret_cast<uintptr_t>(d2) & 15) == 0 &&
+                     (reinterpret_cast<uintptr_t>(field) & 7) == 0 && (reinterpret_cast<uintptr_t>(occ) & 3) == 0;
+    const int bands = edt_bands(m.H, m.P);
+    if (vec)
+        k_map_tables<4><<<dim3((m.W + 511) / 512, bands), 128, 0, s>>>(m.d2, m.field, m.bits, m.W, m.H, m.TW, m.P, m.Wp,
+                                                                       d2, field, occ);
+    else
+        k_map_tables<1><<<dim3((m.W + 127) / 128, bands), 128, 0, s>>>(m.d2, m.field, m.bits, m.W, m.H, m.TW, m.P, m.Wp,
+                                                                       d2, field, occ);
     return cudaGetLastError();
 }
 

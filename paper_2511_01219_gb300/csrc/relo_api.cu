@@ -497,19 +497,15 @@ int plan_for(relo_ctx *ctx, const float *angles_raw, int n_raw, SensorPlan **out
     return RELO_OK;
 }
 
-int edt_segments(int H) {
-    const int L = edt_segment_rows(H);
-    return (H + L - 1) / L;
-}
-
-// The EDT of a map whose grid the context stream is about to hold: the occupancy tiles on the context stream, then
-// the field and d2 on the side stream (after the tiles, whose summaries they read).  Every later reader of the field
-// or d2 waits on field_ready; the next EDT of the map waits on it before its grid is overwritten.
-cudaError_t map_edt(relo_ctx *ctx, MapSlot &m) {
-    cudaError_t e = timed(ctx, 0, m.dev.reach ? 3 : 1, [&] { return launch_edt_tiles(m.dev, ctx->stream); });
+// The EDT of a map from a device grid that the context stream is about to hold (the map's own, or the caller's, which
+// the tile pass then copies): the occupancy tiles on the context stream, then the field and d2 on the side stream (from
+// the tiles and their summaries).  Every later reader of the field or d2 waits on field_ready; the next EDT of the map
+// waits on it before its tiles are overwritten.
+cudaError_t map_edt(relo_ctx *ctx, MapSlot &m, const int8_t *grid) {
+    cudaError_t e = timed(ctx, 0, m.dev.reach ? 3 : 1, [&] { return launch_edt_tiles(m.dev, grid, ctx->stream); });
     if (e == cudaSuccess) e = cudaEventRecord(m.tiles_ready, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->side, m.tiles_ready, 0);
-    if (e == cudaSuccess) e = timed_on(ctx, ctx->side, 7, 2, [&] { return launch_edt_field(m.dev, ctx->side); });
+    if (e == cudaSuccess) e = timed_on(ctx, ctx->side, 7, 3, [&] { return launch_edt_field(m.dev, ctx->n_sm, ctx->side); });
     if (e == cudaSuccess) e = cudaEventRecord(m.field_ready, ctx->side);
     return e;
 }
@@ -706,8 +702,7 @@ void free_map(relo_ctx *ctx, MapSlot &m) {
     if (m.field_ready) cudaEventDestroy(m.field_ready);
     drop_tables(ctx, m);
     dev_free(ctx, m.dev.d2, sizeof(int32_t) * (size_t)m.dev.W * m.dev.H);
-    dev_free(ctx, m.dev.colsq, sizeof(int32_t) * (size_t)m.dev.W * m.dev.H);
-    dev_free(ctx, m.dev.summ, sizeof(int2) * (size_t)m.dev.W * edt_segments(m.dev.H));
+    dev_free(ctx, m.dev.summ, edt_scratch_bytes(m.dev.W, m.dev.H));
     dev_free(ctx, m.dev.grid, (size_t)m.dev.W * m.dev.H);
     dev_free(ctx, m.dev.field, sizeof(uint16_t) * (size_t)m.dev.Wp * m.dev.Hp);
     dev_free(ctx, m.dev.bits, sizeof(uint64_t) * occupancy_words(m.dev.TW, m.dev.TH) +
@@ -743,10 +738,10 @@ int load_map_impl(relo_ctx *ctx, const int8_t *grid, bool on_device, int32_t w, 
     const size_t cells = (size_t)w * h;
     const size_t fcells = (size_t)m.dev.Wp * m.dev.Hp;
     struct { void **p; size_t bytes; } allocs[] = {
-        {(void **)&m.dev.d2, cells * 4}, {(void **)&m.dev.colsq, cells * 4}, {(void **)&m.dev.grid, cells},
+        {(void **)&m.dev.d2, cells * 4}, {(void **)&m.dev.grid, cells},
         {(void **)&m.dev.field, fcells * 2},
         {(void **)&m.dev.bits, occupancy_words(m.dev.TW, m.dev.TH) * 8 + walk_reach_bytes(m.dev.TW, m.dev.TH)},
-        {(void **)&m.dev.summ, sizeof(int2) * (size_t)w * edt_segments(h)}};
+        {(void **)&m.dev.summ, edt_scratch_bytes(w, h)}};
     for (auto &a : allocs) {
         rc = dev_alloc(ctx, a.p, a.bytes, "map tables");
         if (rc) {
@@ -756,6 +751,7 @@ int load_map_impl(relo_ctx *ctx, const int8_t *grid, bool on_device, int32_t w, 
         m.bytes += a.bytes;
     }
     m.dev.reach = reinterpret_cast<uint16_t *>(m.dev.bits + occupancy_words(m.dev.TW, m.dev.TH));
+    m.dev.far = edt_far_of(m.dev.summ, w, h);
     cudaError_t e = cudaEventCreateWithFlags(&m.tiles_ready, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m.field_ready, cudaEventDisableTiming);
     if (e == cudaSuccess)
@@ -763,7 +759,7 @@ int load_map_impl(relo_ctx *ctx, const int8_t *grid, bool on_device, int32_t w, 
                             ctx->stream);
     if (e == cudaSuccess) e = launch_field_border(m.dev, ctx->stream);
     if (e == cudaSuccess) ctx->kernels += 2;
-    if (e == cudaSuccess) e = map_edt(ctx, m);
+    if (e == cudaSuccess) e = map_edt(ctx, m, m.dev.grid);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->stream, m.field_ready, 0);
     if (e != cudaSuccess) {
         free_map(ctx, m);
@@ -1682,7 +1678,7 @@ int relo_set_params(relo_ctx *ctx, const relo_params *p) {
             m.dev.C = C;
             CK(cudaStreamWaitEvent(ctx->stream, m.field_ready, 0), "map rebuild");
             CK(launch_field_border(m.dev, ctx->stream), "map rebuild");
-            CK(map_edt(ctx, m), "map rebuild");
+            CK(map_edt(ctx, m, m.dev.grid), "map rebuild");
             CK(cudaStreamWaitEvent(ctx->stream, m.field_ready, 0), "map rebuild");
             if ((rc = build_lut(ctx, m))) return rc;
         }
@@ -1706,10 +1702,8 @@ int relo_update_map_dev(relo_ctx *ctx, int32_t map_id, const int8_t *grid_dev) {
     MapSlot *m = get_map(ctx, map_id);
     if (!m) return fail(ctx, RELO_E_NOT_FOUND, "unknown map id");
     drop_tables(ctx, *m);
-    CK(cudaStreamWaitEvent(ctx->stream, m->field_ready, 0), "map update");   // the last EDT still reads the grid
-    CK(cudaMemcpyAsync(m->dev.grid, grid_dev, (size_t)m->dev.W * m->dev.H, cudaMemcpyDeviceToDevice, ctx->stream),
-       "map update");
-    CK(map_edt(ctx, *m), "map update");
+    CK(cudaStreamWaitEvent(ctx->stream, m->field_ready, 0), "map update");   // the last EDT still reads the tiles
+    CK(map_edt(ctx, *m, grid_dev), "map update");
     return RELO_OK;
 }
 
@@ -1718,10 +1712,10 @@ int relo_update_map(relo_ctx *ctx, int32_t map_id, const int8_t *grid) {
     MapSlot *m = get_map(ctx, map_id);
     if (!m) return fail(ctx, RELO_E_NOT_FOUND, "unknown map id");
     drop_tables(ctx, *m);
-    CK(cudaStreamWaitEvent(ctx->stream, m->field_ready, 0), "map update");   // the last EDT still reads the grid
+    CK(cudaStreamWaitEvent(ctx->stream, m->field_ready, 0), "map update");   // the last EDT still reads the tiles
     CK(cudaMemcpyAsync(m->dev.grid, grid, (size_t)m->dev.W * m->dev.H, cudaMemcpyHostToDevice, ctx->stream),
        "map update");
-    CK(map_edt(ctx, *m), "map update");
+    CK(map_edt(ctx, *m, m->dev.grid), "map update");
     return RELO_OK;
 }
 
@@ -2046,15 +2040,14 @@ int relo_rrt_sample(relo_ctx *ctx, const int8_t *grid, int32_t w, int32_t h, dou
     t.C = 65535;
     t.P = 0;
     t.Wp = (t.W + 7) & ~7;
-    t.Hp = (t.H + 7) & ~7;
-    const size_t pc = (size_t)t.W * t.H, fc = (size_t)t.Wp * t.Hp;
+    t.Hp = (t.H + 7) & ~7;   // no field: only the distances are wanted
+    const size_t pc = (size_t)t.W * t.H;
     int8_t *raw = nullptr;
     float *clr = nullptr;
     float2 *xy = nullptr;
     struct { void **p; size_t bytes; } allocs[] = {
-        {(void **)&raw, cells}, {(void **)&t.grid, pc}, {(void **)&t.d2, pc * 4}, {(void **)&t.colsq, pc * 4},
-        {(void **)&t.summ, sizeof(int2) * (size_t)t.W * edt_segments(t.H)}, {(void **)&t.field, fc * 2},
-        {(void **)&t.bits, occupancy_words(t.TW, t.TH) * 8}, {(void **)&clr, cells * 4},
+        {(void **)&raw, cells}, {(void **)&t.grid, pc}, {(void **)&t.d2, pc * 4},
+        {(void **)&t.summ, edt_scratch_bytes(t.W, t.H)}, {(void **)&t.bits, occupancy_words(t.TW, t.TH) * 8}, {(void **)&clr, cells * 4},
         {(void **)&xy, sizeof(float2) * (size_t)(cap > 0 ? cap : 1)}};
     int rc = RELO_OK;
     for (auto &a : allocs)
@@ -2063,7 +2056,8 @@ int relo_rrt_sample(relo_ctx *ctx, const int8_t *grid, int32_t w, int32_t h, dou
     if (rc == RELO_OK) {
         e = cudaMemcpyAsync(raw, grid, cells, cudaMemcpyHostToDevice, st);
         if (e == cudaSuccess) e = launch_rrt_blocked(raw, w, h, t.grid, st);
-        if (e == cudaSuccess) e = launch_edt(t, st);
+        t.far = edt_far_of(t.summ, t.W, t.H);
+        if (e == cudaSuccess) e = launch_edt(t, ctx->n_sm, st);
         if (e == cudaSuccess) e = launch_rrt_clearance(t.d2, w, h, res, clr, st);
         if (e == cudaSuccess) ctx->kernels += 5;
         if (e != cudaSuccess) rc = cuda_fail(ctx, e, "RRT clearance table");

@@ -47,8 +47,8 @@ struct MapDev {
                                 // four walk frames (walk_frame_words each: native, mirrored in x, y and both)
     uint16_t *reach = nullptr;  // per walk-frame tile, the empty boxes of tiles ahead, then scratch (walk_reach_bytes),
                                 // in one allocation after bits; nullptr: no ray is cast on this map
-    int32_t *colsq = nullptr;   // [H*W] EDT column-pass scratch
-    int2 *summ = nullptr;       // [S*W] EDT column-segment summaries (scratch)
+    short2 *summ = nullptr;     // EDT column-segment summaries (edt_band.cuh), [edt_summary_rows(H)][W] (scratch)
+    int *far = nullptr;         // [TH + 1] bands the EDT's 32-bit pass has work in, after summ (scratch)
     int8_t *grid = nullptr;     // [H*W] device copy of the grid
 };
 
@@ -63,12 +63,16 @@ __host__ __device__ inline size_t field_index(int x, int y, int Wp) {
     return (((size_t)(y >> 3) * (unsigned)Wp + (unsigned)x) << 3) + (unsigned)(y & 7);
 }
 
-// rows per column segment of the EDT column pass: at least 16, at most 64
-// segments, a multiple of 8 (the segment pass also builds the 8x8 tiles)
-__host__ __device__ inline int edt_segment_rows(int H) {
-    int L = (H + 63) / 64;
-    L = L < 16 ? 16 : L;
-    return (L + 7) & ~7;
+// The EDT's scratch (edt_band.cuh) in one allocation at MapDev::summ: the column summaries of 64-row segments, the spans
+// of every tile row, the bands' flags (MapDev::far).
+inline size_t edt_summary_cells(int W, int H) { return (size_t)W * (((H + 7) / 8 + 7) / 8); }
+inline size_t edt_span_cells(int W, int H) { return (size_t)W * ((H + 7) / 8); }
+inline size_t edt_scratch_bytes(int W, int H) {
+    return (edt_summary_cells(W, H) + edt_span_cells(W, H)) * sizeof(short2) + (size_t)((H + 7) / 8 + 1) * sizeof(int);
+}
+inline short2 *edt_span_of(const MapDev &m) { return m.summ + edt_summary_cells(m.W, m.H); }
+inline int *edt_far_of(short2 *summ, int W, int H) {
+    return reinterpret_cast<int *>(summ + edt_summary_cells(W, H) + edt_span_cells(W, H));
 }
 
 // A walk frame holds TW+1 x TH+1 tiles: the map's tiles with every cell
@@ -334,11 +338,11 @@ inline int tam_chunk_cap(int K, int B, int n_batches, int chunk) {
 }
 constexpr int kMaxBatches = 64;      // ceil(K / batch) limit, bounds the TamSeg table
 
-cudaError_t launch_edt(const MapDev &m, cudaStream_t s);          // interior of the field, d2, bitmap
-// the same in two parts: the occupancy tiles and column summaries (all the ray cast needs), then, reading the
-// summaries and the grid, the column terms, d2 and the interior of the field (TAM and ICP)
-cudaError_t launch_edt_tiles(const MapDev &m, cudaStream_t s);
-cudaError_t launch_edt_field(const MapDev &m, cudaStream_t s);
+cudaError_t launch_edt(const MapDev &m, int n_sm, cudaStream_t s);   // interior of the field, d2, bitmap
+// the same in two parts: the occupancy tiles and column summaries (all the ray cast needs) from a device grid (m.grid,
+// or another buffer, which is then copied there), then, from those, d2 and the interior of the field (TAM and ICP)
+cudaError_t launch_edt_tiles(const MapDev &m, const int8_t *grid, cudaStream_t s);
+cudaError_t launch_edt_field(const MapDev &m, int n_sm, cudaStream_t s);
 cudaError_t launch_field_border(const MapDev &m, cudaStream_t s); // the constant borders of the field and walk frames (once per map)
 cudaError_t launch_map_tables(const MapDev &m, int32_t *d2, uint16_t *field, uint8_t *occ, cudaStream_t s);
 cudaError_t launch_check_cells(const int2 *cells, int n, const MapDev &m, int *bad, cudaStream_t s);

@@ -91,3 +91,46 @@ def test_rrt_sub_batches(relo, rho, points):
     ctx.close()
     assert (r, n) == (rounds, nodes)
     assert np.array_equal(got.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("max_range", [30.0, 29.95, 30.3])   # border widths 601, 600 and 607: band phases 1, 0 and 7
+@pytest.mark.parametrize("shape,density", [
+    ((1, 1), 0.0), ((1, 1), 1.0), ((7, 300), 0.02), ((9, 1025), 0.001), ((65, 8), 0.05), ((64, 257), 0.01),
+    ((129, 1024), 0.3), ((73, 1030), 0.0001),
+    ((400, 700), -1.0),    # one occupied cell: distances beyond 16 bits, in both directions
+    ((330, 515), -2.0),    # an occupied column at each end: far cells in the middle only
+    ((40, 620), 0.0),      # none
+])
+def test_edt_bands(relo, shape, density, max_range):
+    """Squared distances, likelihood field and occupancy from packed 16-bit bands and from the 32-bit pass, with sides and
+    bands that do not divide, against the oracle; the allocation-free entry point where it applies."""
+    import torch
+    rng = np.random.default_rng(3)
+    H, W = shape
+    g = np.zeros(shape, np.int8)
+    if density == -1.0:
+        g[H // 3, W // 4] = 100
+    elif density == -2.0:
+        g[:, 0] = g[:, -1] = 65
+    else:
+        g[rng.random(shape) < density] = 100
+        g[rng.random(shape) < 0.1] -= 1   # unknown cells, and occupied ones of other values
+    want = oracle.edt(g)
+    occ = g >= 65
+    ctx = relo.Relo(max_range=max_range)
+    gt = torch.from_numpy(g).cuda()
+    for mid in (ctx.load_map(np.zeros_like(g), RES), ctx.load_map_dev(gt, RES)):
+        ctx.update_map_dev(mid, gt)
+        d2, field, o = (t.cpu().numpy() for t in ctx.map_tables(mid, g.shape))
+        assert np.array_equal(d2, want)
+        assert np.array_equal(field, np.where((want < 0) | (want > 1600), 1600, want))
+        assert np.array_equal(o, occ)
+    ctx.close()
+    if max(shape) <= 1024:
+        out = torch.full(shape, 7, dtype=torch.int32, device="cuda")
+        odd = torch.empty(H * W + 1, dtype=torch.int8, device="cuda")   # a grid at an odd address
+        odd[1:] = gt.reshape(-1)
+        for ptr in (gt.data_ptr(), odd.data_ptr() + 1):
+            out.fill_(7)
+            assert relo.lib().relo_edt_noalloc(ptr, W, H, out.data_ptr(), torch.cuda.current_stream().cuda_stream) == 0
+            assert np.array_equal(out.cpu().numpy(), want)
