@@ -1217,6 +1217,8 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R) {
         CK(timed_on(ctx, st, 6, 1,
                     [&] {
                         if (!cast) return launch_rank_by_index(rq, R, total_smad, ctx->n_sm, st);
+                        if (p.coarse_metric == RELO_COARSE_CAER)
+                            return launch_caer(rq, R, total_smad, max_ns_pad, sl.bs, ctx->n_sm, st);
                         return p.coarse_metric == RELO_COARSE_SMAD_DIRECT
                                    ? launch_smad_direct(rq, R, total_smad, max_ns_pad, sl.bs, ctx->n_sm, st)
                                    : launch_smad(rq, R, total_smad, max_ns_pad, sl.bs, ctx->n_sm, st);

@@ -362,6 +362,9 @@ cudaError_t launch_cast(const ReqDesc *reqs, int R, int total_chunks, int cast_h
 // SMAD of every hypothesis of the batch from the requests' scan tables
 cudaError_t launch_smad(const ReqDesc *reqs, int R, int total_hyp, int max_ns_pad, BatchState *bs, int n_sm,
                         cudaStream_t s);
+// CAER of every hypothesis of the batch (caer.cu)
+cudaError_t launch_caer(const ReqDesc *reqs, int R, int total_hyp, int max_ns_pad, BatchState *bs, int n_sm,
+                        cudaStream_t s);
 // the same SMAD by direct window sums, without the prefix sums of Eq. 17 (the Table II ablation)
 cudaError_t launch_smad_direct(const ReqDesc *reqs, int R, int total_hyp, int max_ns_pad, BatchState *bs, int n_sm,
                                cudaStream_t s);

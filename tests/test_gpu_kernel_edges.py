@@ -134,3 +134,41 @@ def test_edt_bands(relo, shape, density, max_range):
             out.fill_(7)
             assert relo.lib().relo_edt_noalloc(ptr, W, H, out.data_ptr(), torch.cuda.current_stream().cuda_stream) == 0
             assert np.array_equal(out.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("n_beams,ns,n_orient,gap", [
+    (90, 120, 120, 0),     # every direction an orientation
+    (90, 120, 40, 7),      # two intervals, three residue classes
+    (100, 120, 2, 0),      # fewer orientations than a lane holds: lanes split the beams
+    (300, 500, 500, 11),   # more orientations than one pass of a warp
+    (31, 32, 16, 0),       # one beam short of the circle
+])
+def test_caer_orientation_groups(relo, n_beams, ns, n_orient, gap):
+    """CAER numerators, shifts and survivors equal the oracle's across group, class and interval remainders."""
+    wl = small_case(n_beams=n_beams, ns=ns, n_orient=n_orient)
+    keep = np.ones(n_beams, bool)
+    keep[n_beams // 3:n_beams // 3 + gap] = False
+    wl.ranges, wl.angles = wl.ranges[keep].copy(), wl.angles[keep]
+    wl.ranges[::9] = 100.0   # invalid beams
+    full_case(relo, wl, 12, batch=5, local_topk=2, coarse=1)[0].close()
+
+
+def test_caer_ranges_beyond_a_block_of_32_bits(relo):
+    """A coarse map resolution makes the range limit 8000 cells: sums of differences leave 32 bits within a block."""
+    g = np.zeros((30, 9000), np.int8)
+    g[0] = g[-1] = 100
+    g[:, 0] = g[:, -1] = 100
+    hyps = np.array([[x, 15] for x in range(500, 1000, 100)], np.int32)
+    ang = workloads.beam_angles(40, 60)
+    z = np.random.default_rng(1).uniform(1.0, 399.0, 40).astype(np.float32)   # far from every synthesized range
+    prm = dict(n_orient=60, topk=3, coarse=1)
+    ctx = relo.Relo(n_orient=60, topk=3, coarse_metric=1, max_range=400.0, ray_tables=0)
+    mid = ctx.load_map(g, RES)
+    ctx.set_hypotheses(mid, workloads.cell_centres(hyps, RES))
+    ctx.relocalize(mid, z, ang, 400.0)
+    import torch
+    got = ctx.stage(relo.STAGE_SMAD_NUM, torch.empty(len(hyps), dtype=torch.int64, device="cuda")).cpu().numpy()
+    ctx.close()
+    pl = oracle.plan(z, ang, 400.0, RES, oracle.Params(**prm))
+    want, _ = oracle.coarse(g, hyps, pl, oracle.Params(**prm))
+    assert np.array_equal(got, want) and want.max() > 1 << 32
