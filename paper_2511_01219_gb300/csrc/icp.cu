@@ -2,11 +2,11 @@
 // step of the framework overview, Sec. III: the local top-k poses are aligned
 // to the whole map and scored again; Remark 2 names the refinement operator).
 //
-// k_icp: one CTA of kIcpThreads per local top-k pose.  The pose starts at its hypothesis
+// k_icp: one cluster of CTAs per local top-k pose.  The pose starts at its hypothesis
 // cell centre and orientation theta_m.  Beam i is the sensor-frame point
 // (z_i, a_i), z_i = R_i res / 2^16 (its Q16 range) and a_i = 2 pi b_i / N_s (its
 // panoramic grid angle); its sensor-frame point s_i = (z_i cos a_i, z_i sin
-// a_i) is computed once.  An iteration maps every valid beam to its world
+// a_i) is computed once per request (icp_points.cuh).  An iteration maps every valid beam to its world
 // point w = p + R(theta) s (each product and sum rounded on its own, as the
 // oracle does; its cell is floor(w * (1 / res))), pairs it with the centre of
 // the nearest occupied cell to the cell it
@@ -18,10 +18,19 @@
 // icp_iters iterations, when fewer than 2 pairs remain, or when the motion is
 // below 1e-9 rad and 1e-9 m.  All pose arithmetic is FP64.
 //
+// What bounds it is the FP64 rate (two lanes per clock and SM) and the chain of
+// dependent steps, so a pose is spread over as many SMs as there are to spare:
+// the CTAs of a cluster share its beams, their sums meet in the first CTA's
+// shared memory, one warp there solves for the motion and writes the pose to
+// all.  With one CTA per pose whose every thread solved the motion and made its
+// own beams' points, 20 poses of 1027 beams took 212 us for 10 iterations, now
+// @@ICP@@.
+//
 // The refined pose is then scored like TAM: each beam ends in the cell of its
 // world point, takes min(d2, C) (C off the map), and the k-th smallest
 // value, the likelihood table and the epilogue of Eq. 23-31 (or the metric
-// fine_metric selects) give the score, in the same FP32 arithmetic as k_tam.
+// fine_metric selects) give the score, in the FP32 arithmetic of k_tam with
+// sums in FP64, by one warp.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -33,26 +42,38 @@ namespace relo {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kIcpThreads = 256;
+constexpr int kIcpThreads = 128;
 constexpr int kIcpWarps = kIcpThreads / 32;
+constexpr int kIcpCluster = 8;   // CTAs per pose at most
 
 // The nearest occupied cell to cell (x, y) when its squared distance is at
 // most cap (<= C): the cells at exactly the EDT distance, by increasing dy,
-// then dx, from the map's table of the offsets at each squared distance.
+// then dx, from the map's table of the offsets at each squared distance, eight
+// at a time (most distances have no more; one by one, every candidate waited
+// for two loads).
 __device__ bool nearest_occupied(const ReqDesc &d, int x, int y, int cap, int &ox, int &oy) {
     if (x < 0 || y < 0 || x >= d.W || y >= d.H) return false;
     const int d2 = d.d2map[(size_t)y * d.W + x];
     if (d2 < 0 || d2 > cap) return false;
     const int e1 = d.sq_off[d2 + 1];
-    for (int e = d.sq_off[d2]; e < e1; ++e) {
-        const short2 o = d.sq_rep[e];
-        const int cx = x + o.y, cy = y + o.x;
-        if (cx < 0 || cy < 0 || cx >= d.W || cy >= d.H) continue;
-        if (d.grid[(size_t)cy * d.W + cx] >= 65) {
-            ox = cx;
-            oy = cy;
-            return true;
+    for (int e = d.sq_off[d2]; e < e1; e += 8) {
+        short2 o[8];
+        int8_t v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) o[i] = e + i < e1 ? __ldg(d.sq_rep + e + i) : make_short2(0, 0);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int cx = x + o[i].y, cy = y + o[i].x;
+            const bool in = e + i < e1 && cx >= 0 && cy >= 0 && cx < d.W && cy < d.H;
+            v[i] = in ? __ldg(d.grid + (size_t)cy * d.W + cx) : (int8_t)0;
         }
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (v[i] >= 65) {
+                ox = x + o[i].y;
+                oy = y + o[i].x;
+                return true;
+            }
     }
     return false;
 }
@@ -63,24 +84,38 @@ __device__ __forceinline__ double warp_sum_d(double v) {
     return v;
 }
 
-// Sums of V values over the CTA: every thread gets the same totals (the warp
-// partials are added in warp order by every thread).  red: [V][kIcpWarps].
-template <int V>
-__device__ __forceinline__ void block_sums(double (&v)[V], double *red) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// Sums of 8 values over the warp with 9 additions instead of 40: each exchange halves the values a lane carries.  The
+// lane ends with the total of value sum_index(lane).
+__device__ __forceinline__ double warp_sums8(double (&v)[8]) {
+    const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int j = 0; j < V; ++j) {
-        const double w = warp_sum_d(v[j]);
-        if (lane == 0) red[j * kIcpWarps + warp] = w;
-    }
-    __syncthreads();
+    for (int n = 4, o = 16; n >= 1; n >>= 1, o >>= 1) {
+        const bool up = lane & o;
 #pragma unroll
-    for (int j = 0; j < V; ++j) {
-        double t = 0.0;
-        for (int w = 0; w < kIcpWarps; ++w) t += red[j * kIcpWarps + w];
-        v[j] = t;
+        for (int j = 0; j < n; ++j) {
+            const double send = up ? v[j] : v[j + n], keep = up ? v[j + n] : v[j];
+            v[j] = keep + __shfl_xor_sync(kFull, send, o);
+        }
     }
-    __syncthreads();   // red is free again
+    v[0] += __shfl_xor_sync(kFull, v[0], 2);
+    v[0] += __shfl_xor_sync(kFull, v[0], 1);
+    return v[0];
+}
+__device__ __forceinline__ int sum_index(int lane) { return (lane >> 4 & 1) * 4 + (lane >> 3 & 1) * 2 + (lane >> 2 & 1); }
+
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_addr(const void *p, int rank) {   // p in CTA `rank` of the cluster
+    uint32_t out;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(out) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return out;
+}
+__device__ __forceinline__ void cluster_store(uint32_t a, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_store(uint32_t a, int v) {
+    asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 
 // world point and cell of a sensor-frame point at pose (x, y) with ct, st = cos, sin of theta
@@ -98,37 +133,68 @@ __device__ __forceinline__ int clamped_d2(const ReqDesc &d, int x, int y) {
     return (v < 0 || v > d.C) ? d.C : v;
 }
 
-__global__ void __launch_bounds__(kIcpThreads) k_icp(const ReqDesc *__restrict__ reqs, int batch_lo, int batch_hi) {
-    extern __shared__ double spt[];   // [2 N] sensor-frame points, then [N] int clamped d2 of the refined endpoints
-    __shared__ double red[7 * kIcpWarps];
-    const ReqDesc &d = reqs[blockIdx.x];
-    const int tid = threadIdx.x;
-    const int slot = blockIdx.y;
+struct IcpPose {
+    double x, y, th, ct, st;   // the pose, cos and sin of theta
+    int stop;
+};
+
+// dynamic shared memory: [per] the CTA's sensor-frame points, then in the first CTA [N] the clamped d2 of the refined
+// endpoints; per: beams per CTA of the cluster for the longest scan
+__global__ void __launch_bounds__(kIcpThreads) k_icp(const ReqDesc *__restrict__ reqs, int batch_lo, int batch_hi,
+                                                     int per) {
+    extern __shared__ __align__(16) unsigned char icp_smem[];
+    __shared__ double part[kIcpCluster * kIcpWarps][8];   // the first CTA's: every warp's sums
+    __shared__ IcpPose pose;
+    double2 *pts = reinterpret_cast<double2 *>(icp_smem);
+    int *qv = reinterpret_cast<int *>(icp_smem + sizeof(double2) * (size_t)per);
+    uint32_t cs, cr;
+    asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(cs));
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(cr));
+    const ReqDesc &d = reqs[blockIdx.y];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // the conditions below are the same in every CTA of the cluster
+    const int slot = (int)(blockIdx.x / cs);
     if (slot >= (batch_hi - batch_lo) * d.L) return;
     const int b = batch_lo + slot / d.L;
     if (b >= d.n_batches) return;
     const int s = d.local[(size_t)b * d.L + slot % d.L];
     const int N = d.scan->n_valid;
     if (s < 0 || N <= 0) return;
-    int *qv = reinterpret_cast<int *>(spt + 2 * (size_t)N);
-    const int2 hc = d.hyps[d.survivors[s]];
-    const double res = d.resd, q16 = res / 65536.0, ang = 2.0 * M_PI / (double)d.ns, inv_res = 1.0 / res;
-    for (int i = tid; i < N; i += kIcpThreads) {
-        const int2 bR = d.vbR[i];
-        const double z = __dmul_rn((double)bR.y, q16), a = __dmul_rn((double)bR.x, ang);
-        spt[2 * i] = __dmul_rn(z, cos(a));
-        spt[2 * i + 1] = __dmul_rn(z, sin(a));
+    const int i0 = (int)cr * per, n = max(0, min(N - i0, per));   // this CTA's beams
+    const double2 *src = reinterpret_cast<const double2 *>(d.icp_pts) + i0;
+    for (int i = tid; i < n; i += kIcpThreads) pts[i] = src[i];
+    const double res = d.resd, inv_res = 1.0 / res;
+    auto tell = [&](const IcpPose &p) {   // by warp 0 of the first CTA: the pose to every CTA, one per lane
+        if (lane < (int)cs) {
+            const uint32_t a = cluster_addr(&pose, lane);
+            cluster_store(a, p.x);
+            cluster_store(a + 8, p.y);
+            cluster_store(a + 16, p.th);
+            cluster_store(a + 24, p.ct);
+            cluster_store(a + 32, p.st);
+            cluster_store(a + 40, p.stop);
+        }
+    };
+    cluster_sync();   // every CTA has started: its shared memory may be written
+    if (cr == 0 && warp == 0) {
+        const int2 hc = d.hyps[d.survivors[s]];
+        IcpPose p;
+        p.x = __dmul_rn((double)hc.x + 0.5, res);
+        p.y = __dmul_rn((double)hc.y + 0.5, res);
+        p.th = __ddiv_rn(__dmul_rn((double)d.best_m[s], 2.0 * M_PI), (double)d.ns);
+        p.ct = cos(p.th);
+        p.st = sin(p.th);
+        p.stop = d.icp_iters <= 0;
+        tell(p);
     }
-    __syncthreads();
-    double px = __dmul_rn((double)hc.x + 0.5, res), py = __dmul_rn((double)hc.y + 0.5, res);
-    double th = __ddiv_rn(__dmul_rn((double)d.best_m[s], 2.0 * M_PI), (double)d.ns);
-    for (int it = 0; it < d.icp_iters; ++it) {
-        double v[7] = {0, 0, 0, 0, 0, 0, 0};   // pairs, sums of w, of c, of w.c and of w x c
-        const double ct = cos(th), st = sin(th);
-        for (int i = tid; i < N; i += kIcpThreads) {
+    cluster_sync();
+    for (int it = 1; !pose.stop; ++it) {
+        const IcpPose p = pose;
+        double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};   // pairs, sums of w, of c, of w.c and of w x c
+        for (int i = tid; i < n; i += kIcpThreads) {
             double wx, wy;
             int ex, ey, ox, oy;
-            world_point(px, py, ct, st, spt[2 * i], spt[2 * i + 1], inv_res, wx, wy, ex, ey);
+            world_point(p.x, p.y, p.ct, p.st, pts[i].x, pts[i].y, inv_res, wx, wy, ex, ey);
             if (!nearest_occupied(d, ex, ey, d.C, ox, oy)) continue;
             const double cx = ((double)ox + 0.5) * res, cy = ((double)oy + 0.5) * res;
             v[0] += 1.0;
@@ -139,47 +205,61 @@ __global__ void __launch_bounds__(kIcpThreads) k_icp(const ReqDesc *__restrict__
             v[5] += wx * cx + wy * cy;
             v[6] += wx * cy - wy * cx;
         }
-        block_sums(v, red);
-        const double n = v[0], swx = v[1], swy = v[2], scx = v[3], scy = v[4], sdot = v[5], scr = v[6];
-        if (n < 2.0) break;
-        const double mwx = swx / n, mwy = swy / n, mcx = scx / n, mcy = scy / n;
-        const double f = atan2(scr - n * (mwx * mcy - mwy * mcx), sdot - n * (mwx * mcx + mwy * mcy));
-        const double cf = cos(f), sf = sin(f);
-        const double tx = __dsub_rn(mcx, __dsub_rn(__dmul_rn(cf, mwx), __dmul_rn(sf, mwy)));
-        const double ty = __dsub_rn(mcy, __dadd_rn(__dmul_rn(sf, mwx), __dmul_rn(cf, mwy)));
-        const double nx = __dadd_rn(__dsub_rn(__dmul_rn(cf, px), __dmul_rn(sf, py)), tx);
-        const double ny = __dadd_rn(__dadd_rn(__dmul_rn(sf, px), __dmul_rn(cf, py)), ty);
-        const double moved = fabs(nx - px) + fabs(ny - py);
-        px = nx;
-        py = ny;
-        th = __dadd_rn(th, f);
-        if (fabs(f) < 1e-9 && moved < 1e-9) break;
-    }
-    // the refined pose scored again
-    int sumb = 0;
-    {
-        const double ct = cos(th), st = sin(th);
-        for (int i = tid; i < N; i += kIcpThreads) {
-            double wx, wy;
-            int ex, ey;
-            world_point(px, py, ct, st, spt[2 * i], spt[2 * i + 1], inv_res, wx, wy, ex, ey);
-            const int q = clamped_d2(d, ex, ey);
-            qv[i] = q;
-            sumb += q;
+        __syncwarp();
+        const double w = warp_sums8(v);
+        if ((lane & 3) == 0) cluster_store(cluster_addr(&part[cr * kIcpWarps + warp][sum_index(lane)], 0), w);
+        cluster_sync();   // the sums have arrived, and every thread has read the pose
+        if (cr == 0 && warp == 0) {
+            double t = 0.0;
+            for (int k = lane >> 3; k < (int)cs * kIcpWarps; k += 4) t += part[k][lane & 7];
+            t += __shfl_xor_sync(kFull, t, 8);
+            t += __shfl_xor_sync(kFull, t, 16);
+            double m[7];
+#pragma unroll
+            for (int j = 0; j < 7; ++j) m[j] = __shfl_sync(kFull, t, j);
+            IcpPose q = p;
+            const double np = m[0];
+            if (np < 2.0) {
+                q.stop = 1;
+            } else {
+                const double mwx = m[1] / np, mwy = m[2] / np, mcx = m[3] / np, mcy = m[4] / np;
+                const double f = atan2(m[6] - np * (mwx * mcy - mwy * mcx), m[5] - np * (mwx * mcx + mwy * mcy));
+                q.th = __dadd_rn(p.th, f);
+                // one lane takes the motion's angle, another the new pose's: one evaluation for both
+                const double ang = lane == 0 ? f : q.th, ca = cos(ang), sa = sin(ang);
+                const double cf = __shfl_sync(kFull, ca, 0), sf = __shfl_sync(kFull, sa, 0);
+                q.ct = __shfl_sync(kFull, ca, 1);
+                q.st = __shfl_sync(kFull, sa, 1);
+                const double tx = __dsub_rn(mcx, __dsub_rn(__dmul_rn(cf, mwx), __dmul_rn(sf, mwy)));
+                const double ty = __dsub_rn(mcy, __dadd_rn(__dmul_rn(sf, mwx), __dmul_rn(cf, mwy)));
+                q.x = __dadd_rn(__dsub_rn(__dmul_rn(cf, p.x), __dmul_rn(sf, p.y)), tx);
+                q.y = __dadd_rn(__dadd_rn(__dmul_rn(sf, p.x), __dmul_rn(cf, p.y)), ty);
+                const double moved = fabs(q.x - p.x) + fabs(q.y - p.y);
+                q.stop = (fabs(f) < 1e-9 && moved < 1e-9) || it >= d.icp_iters;
+            }
+            tell(q);
         }
+        cluster_sync();
     }
-    {
-        double t[1] = {(double)sumb};
-        block_sums(t, red);   // also makes qv visible to the whole CTA
-        sumb = (int)t[0];
+    // the refined pose scored again: the clamped d2 of every endpoint to the first CTA
+    const IcpPose p = pose;
+    for (int i = tid; i < n; i += kIcpThreads) {
+        double wx, wy;
+        int ex, ey;
+        world_point(p.x, p.y, p.ct, p.st, pts[i].x, pts[i].y, inv_res, wx, wy, ex, ey);
+        cluster_store(cluster_addr(&qv[i0 + i], 0), clamped_d2(d, ex, ey));
     }
+    cluster_sync();
+    if (cr != 0 || warp != 0) return;
+    int sumb = 0;
+    for (int i = lane; i < N; i += 32) sumb += qv[i];
+    sumb = __reduce_add_sync(kFull, sumb);
     const int C = d.C;
     const int k = d.fine < kFineBaseline ? d.scan->k_ret : N;
     auto count_le = [&](int x) {
-        double c[1] = {0.0};
-        for (int i = tid; i < N; i += kIcpThreads) c[0] += qv[i] <= x ? 1.0 : 0.0;
-        block_sums(c, red);
-        return (int)c[0];
+        int c = 0;
+        for (int i = lane; i < N; i += 32) c += qv[i] <= x ? 1 : 0;
+        return __reduce_add_sync(kFull, c);
     };
     int bk = C, cle = N;
     if (k < N) {   // the smallest b with #{q <= b} >= k, by bisection over [0, C]
@@ -197,19 +277,14 @@ __global__ void __launch_bounds__(kIcpThreads) k_icp(const ReqDesc *__restrict__
         bk = lo;
         cle = c_hi;
     }
-    float sl = 0.0f, sgs = 0.0f;
-    for (int i = tid; i < N; i += kIcpThreads) {
+    double dl = 0.0, dg = 0.0;
+    for (int i = lane; i < N; i += 32) {
         const float2 g = d.lut[qv[i]];
-        sgs += g.y;
-        if (qv[i] <= bk) sl += g.x;
+        dg += (double)g.y;
+        if (qv[i] <= bk) dl += (double)g.x;
     }
-    {
-        double t[2] = {(double)sl, (double)sgs};
-        block_sums(t, red);
-        sl = (float)t[0];
-        sgs = (float)t[1];
-    }
-    if (tid == 0) {
+    const float sl = (float)warp_sum_d(dl), sgs = (float)warp_sum_d(dg);
+    if (lane == 0) {
         // Eq. 27-31 as k_tam evaluates them
         const float topsum = sl - (float)(cle - k) * d.lut[bk].x;
         const float lbar = topsum * (1.0f / (float)k);
@@ -222,26 +297,37 @@ __global__ void __launch_bounds__(kIcpThreads) k_icp(const ReqDesc *__restrict__
         else if (d.fine == kFineBaseline) T = sqrtf(expf(lbar) * sd);
         else if (d.fine == kFineLF) T = topsum;
         double *ps = d.ref_pose + 3 * (size_t)s;
-        ps[0] = px;
-        ps[1] = py;
-        ps[2] = th;
+        ps[0] = p.x;
+        ps[1] = p.y;
+        ps[2] = p.th;
         d.reev[s] = T;
     }
 }
 
 }  // namespace
 
-cudaError_t launch_icp(const ReqDesc *reqs, int R, int batch_lo, int batch_hi, int max_L, int max_beams,
+cudaError_t launch_icp(const ReqDesc *reqs, int R, int batch_lo, int batch_hi, int max_L, int max_beams, int n_sm,
                        cudaStream_t s) {
     const int slots = (batch_hi - batch_lo) * max_L;
     if (R < 1 || slots < 1) return cudaSuccess;
-    const size_t smem = (2 * sizeof(double) + sizeof(int)) * (size_t)(max_beams > 0 ? max_beams : 1);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_icp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    k_icp<<<dim3(R, slots), kIcpThreads, smem, s>>>(reqs, batch_lo, batch_hi);
-    return cudaGetLastError();
+    const int beams = max_beams > 0 ? max_beams : 1;
+    // as many CTAs per pose as give every SM about two (each adds its share of the barriers, not of the FP64 work)
+    int cs = kIcpCluster;
+    while (cs > 1 && (long long)R * slots * cs > 5ll * n_sm / 2) cs >>= 1;
+    const int per = (beams + cs - 1) / cs;
+    const size_t smem = sizeof(double2) * (size_t)per + sizeof(int) * (size_t)beams;   // at most 41 KB
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cs;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(cs * slots, R);
+    cfg.blockDim = dim3(kIcpThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_icp, reqs, batch_lo, batch_hi, per);
 }
 
 }  // namespace relo

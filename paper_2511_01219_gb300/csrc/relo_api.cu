@@ -1017,6 +1017,7 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R) {
         const int n = q.P->n, nh = q.m->n_hyp, K = q.K;
         off[r] = total;
         total += align_up(24ull * K) + align_up(4ull * K);   // refined poses and re-evaluated scores
+        if (p.icp_iters > 0) total += align_up(16ull * n);   // sensor-frame points
         total += align_up(sizeof(int2) * n) + align_up(4ull * n) + align_up(sizeof(ScanInfo)) + align_up(8ull * nh) * 2 +
                  align_up(4ull * nh) + align_up(4ull * K) * 2 + align_up(8ull * K) + align_up(4ull * K * q.P->n_orient) +
                  align_up(16ull * tam_chunk_cap(K, q.B, q.n_batches, chunk_of(r))) + align_up(4ull * (q.n_batches + 1)) +
@@ -1105,6 +1106,7 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R) {
         d.grid = m.dev.grid;
         d.sq_off = m.sq_off;
         d.sq_rep = m.sq_rep;
+        d.icp_pts = p.icp_iters > 0 ? (double *)take(16ull * P.n) : nullptr;
         d.ref_pose = (double *)take(24ull * q.K);
         d.reev = (float *)take(4ull * q.K);
         d.scan = (ScanInfo *)take(sizeof(ScanInfo));
@@ -1237,7 +1239,7 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R) {
         for (int r = 0; r < R; ++r) max_no = std::max(max_no, desc[r].n_orient);
         // the ranking and TAM's work order, and beside them the endpoint offset table O[m][i] of each request plan,
         // per band phase
-        CK(timed_on(ctx, st, 3, 1, [&] { return launch_topk(rq, R, max_n_hyp, max_K, max_no, ctx->n_sm, st); }),
+        CK(timed_on(ctx, st, 3, 1, [&] { return launch_topk(rq, R, max_n_hyp, max_K, max_no, p.icp_iters > 0 ? max_beams : 0, ctx->n_sm, st); }),
            "SMAD top-K");
     }
     for (int r = 0; r < R; ++r) CK(cudaStreamWaitEvent(st, pr[r].m->field_ready, 0), "map field");
@@ -1254,7 +1256,7 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R) {
             // the local top-k, their ICP refinement and re-evaluation, then the batch's best
             CK(timed_on(ctx, st, 5, 1, [&] { return launch_select_batch(rq, R, lo, hi, false, true, st); }),
                "batch selection");
-            CK(timed_on(ctx, st, 5, 1, [&] { return launch_icp(rq, R, lo, hi, p.local_topk, max_beams, st); }),
+            CK(timed_on(ctx, st, 5, 1, [&] { return launch_icp(rq, R, lo, hi, p.local_topk, max_beams, ctx->n_sm, st); }),
                "ICP refinement");
             CK(timed_on(ctx, st, 5, 1, [&] { return launch_icp_best(rq, R, lo, hi, last, st); }), "batch selection");
         } else {

@@ -220,6 +220,7 @@ struct ReqDesc {
     const int8_t *grid;          // [H*W] the occupancy grid (ICP pairs)
     const int32_t *sq_off;       // [C+2] start of the offsets with dy^2 + dx^2 = n in sq_rep, for n in [0, C + 1]
     const short2 *sq_rep;        // (dy, dx) offsets by n, each n's ordered by dy, then dx (the ICP pairing order)
+    double *icp_pts;             // [n_beams][2] the valid beams' sensor-frame points (with ICP only)
     double *ref_pose;            // [K][3] refined pose (x, y, theta) of each refined survivor (map metres)
     float *reev;                 // [K] its re-evaluated score
     const float2 *lut;           // [C+2] (l(b), sqrt(C) - sqrt(b)); entry C+1 = (0, 0) marks "no beam"
@@ -375,7 +376,8 @@ cudaError_t launch_win_build(const ReqDesc *reqs, int R, int total, int max_ns_p
 // SMAD of the window-read requests' hypotheses by search in their window keys
 cudaError_t launch_win_read(const ReqDesc *reqs, int R, int total, cudaStream_t s);
 // the top-K of every request with its TAM work order, and beside it (extra blocks) every request's TAM endpoint offsets
-cudaError_t launch_topk(const ReqDesc *reqs, int R, int max_n_hyp, int max_K, int max_n_orient, int n_sm, cudaStream_t s);
+cudaError_t launch_topk(const ReqDesc *reqs, int R, int max_n_hyp, int max_K, int max_n_orient, int icp_beams,
+                        int n_sm, cudaStream_t s);   // icp_beams: the most beams of a request with ICP, 0 without
 // plans the TAM launch of one batch index: fills segs[R] and returns the task count and grid size
 struct TamPlan {
     int total_tasks, grid, vpl;
@@ -401,7 +403,7 @@ cudaError_t launch_select_batch(const ReqDesc *reqs, int R, int batch_lo, int ba
 // ICP refinement and re-evaluation of the local top-k of batches batch_lo .. batch_hi - 1, then their best,
 // early termination and (with last) the results
 cudaError_t launch_icp(const ReqDesc *reqs, int R, int batch_lo, int batch_hi, int max_L, int max_beams,
-                       cudaStream_t s);
+                       int n_sm, cudaStream_t s);
 cudaError_t launch_icp_best(const ReqDesc *reqs, int R, int batch_lo, int batch_hi, bool last, cudaStream_t s);
 // Algorithm 1 in batched-expansion form (rrt.cu); blocking on s; *err names a failure
 // the RRT's blocked grid with a ring of blocked cells ((W + 2) x (H + 2), occupied = 100) and, from the squared

@@ -30,6 +30,7 @@
 #include <stdint.h>
 
 #include "../../include/relo.h"
+#include "icp_points.cuh"
 #include "relo_internal.h"
 #include "tam_offsets.cuh"
 
@@ -235,9 +236,9 @@ __device__ void topk_request(const ReqDesc &d, unsigned long long *sm, int Kp_ca
 
 // One CTA per request ranks it and then builds its TAM work order from the
 // survivors; the CTAs after the first R compute the requests' TAM endpoint
-// offsets meanwhile (they need the scan preparation, not the ranking).
+// offsets and, for ICP, the beams' sensor-frame points meanwhile (they need the scan preparation, not the ranking).
 __global__ void __launch_bounds__(kTopkThreads) k_topk(const ReqDesc *__restrict__ reqs, int Kp_cap, int stage_cap,
-                                                       int R, int max_n_orient) {
+                                                       int R, int max_n_orient, int icp_chunks) {
     extern __shared__ __align__(16) unsigned long long sm[];
     if ((int)blockIdx.x >= R) {
         for (int t = (int)blockIdx.x - R; t < R * max_n_orient; t += (int)gridDim.x - R) {
@@ -245,6 +246,8 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(const ReqDesc *__restrict
             const int q = t % max_n_orient;
             if (q < o.n_orient && !o.state->done && o.tam_offs) tam_offsets_one(o, q);
         }
+        for (int t = (int)gridDim.x - 1 - (int)blockIdx.x; t < R * icp_chunks; t += (int)gridDim.x - R)
+            if (reqs[t / icp_chunks].icp_iters > 0) icp_points_chunk(reqs[t / icp_chunks], t % icp_chunks);
         return;
     }
     const ReqDesc &d = reqs[blockIdx.x];
@@ -388,7 +391,7 @@ __global__ void k_icp_best(const ReqDesc *__restrict__ reqs, int R, int batch_lo
 
 }  // namespace
 
-cudaError_t launch_topk(const ReqDesc *reqs, int R, int max_n_hyp, int max_K, int max_n_orient, int n_sm,
+cudaError_t launch_topk(const ReqDesc *reqs, int R, int max_n_hyp, int max_K, int max_n_orient, int icp_beams, int n_sm,
                         cudaStream_t s) {
     int Kp = 1;
     while (Kp < max_K) Kp <<= 1;
@@ -400,7 +403,8 @@ cudaError_t launch_topk(const ReqDesc *reqs, int R, int max_n_hyp, int max_K, in
     if (e != cudaSuccess) return e;
     // one CTA per SM for the offsets (the ranking CTAs' shared memory leaves room for no second one)
     const int n_off = std::max(1, std::min(R * std::max(max_n_orient, 1), n_sm));
-    k_topk<<<R + n_off, kTopkThreads, smem, s>>>(reqs, Kp, stage_cap, R, std::max(max_n_orient, 1));
+    k_topk<<<R + n_off, kTopkThreads, smem, s>>>(reqs, Kp, stage_cap, R, std::max(max_n_orient, 1),
+                                                 (icp_beams + 31) / 32);
     return cudaGetLastError();
 }
 

@@ -172,3 +172,29 @@ def test_caer_ranges_beyond_a_block_of_32_bits(relo):
     pl = oracle.plan(z, ang, 400.0, RES, oracle.Params(**prm))
     want, _ = oracle.coarse(g, hyps, pl, oracle.Params(**prm))
     assert np.array_equal(got, want) and want.max() > 1 << 32
+
+
+@pytest.mark.parametrize("requests", [2, 5, 11, 24])
+def test_icp_cluster_sizes(relo, requests):
+    """8, 4, 2 and 1 CTAs per refined pose: each request of a batch gets the pose it gets alone (its sums are added in
+    another order: 1e-9 m and rad, far above that and far below a cell) and its score (the same endpoints: equal)."""
+    g = workloads.make_room(2, n=40, n_boxes=4)
+    free = np.argwhere(g == 0)[:, ::-1]
+    hyps = free[np.random.default_rng(2).choice(len(free), 60, replace=False)].astype(np.int32)
+    ctx = relo.Relo(n_orient=40, topk=48, batch=16, local_topk=12, early_stop=0, icp_iters=10)
+    mid = ctx.load_map(g, RES)
+    ctx.set_hypotheses(mid, workloads.cell_centres(hyps, RES))
+    reqs = []
+    for i in range(requests):
+        n = 60 + 5 * i
+        ang = workloads.beam_angles(n, 120 if n <= 120 else 240)
+        true = ((hyps[i][0] + 0.8) * RES, (hyps[i][1] + 0.3) * RES, 0.5 * i)
+        z = workloads.render_scan(g, RES, true, ang, 6.0)
+        reqs.append((mid, workloads.add_noise(z, 6.0, i, sigma=0.005, drop_frac=0.0, short_frac=0.0), ang, 6.0))
+    alone = [ctx.relocalize(*q) for q in reqs]
+    for a, b in zip(alone, ctx.relocalize_batch(reqs)):
+        assert (a.hyp, a.m, a.n_batches, a.smad_num) == (b.hyp, b.m, b.n_batches, b.smad_num)
+        assert abs(a.x - b.x) <= 1e-9 and abs(a.y - b.y) <= 1e-9
+        assert abs((a.theta - b.theta + np.pi) % (2 * np.pi) - np.pi) <= 1e-9
+        assert a.tam == b.tam
+    ctx.close()
