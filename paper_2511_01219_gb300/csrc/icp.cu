@@ -14,7 +14,8 @@
 // dy, then the smaller dx; pairs farther than the TAM clamp C = (d_max /
 // res)^2 are dropped), and applies the rigid motion that minimises the
 // squared pair distances: with the centroids mw, mc and the centred cross and
-// dot sums, phi = atan2(cross, dot) and t = mc - R(phi) mw.  It stops after
+// dot sums, phi = atan2(cross, dot) (whose cosine and sine are the two sums over
+// their length) and t = mc - R(phi) mw.  It stops after
 // icp_iters iterations, when fewer than 2 pairs remain, or when the motion is
 // below 1e-9 rad and 1e-9 m.  All pose arithmetic is FP64.
 //
@@ -23,8 +24,8 @@
 // the CTAs of a cluster share its beams, their sums meet in the first CTA's
 // shared memory, one warp there solves for the motion and writes the pose to
 // all.  With one CTA per pose whose every thread solved the motion and made its
-// own beams' points, 20 poses of 1027 beams took 212 us for 10 iterations, now
-// @@ICP@@.
+// own beams' points, 20 poses of 1027 beams took 420 us for 10 iterations; this
+// takes 130 (with the angle evaluated in every iteration 172).
 //
 // The refined pose is then scored like TAM: each beam ends in the cell of its
 // world point, takes min(d2, C) (C off the map), and the k-th smallest
@@ -51,16 +52,22 @@ constexpr int kIcpCluster = 8;   // CTAs per pose at most
 // then dx, from the map's table of the offsets at each squared distance, eight
 // at a time (most distances have no more; one by one, every candidate waited
 // for two loads).
-__device__ bool nearest_occupied(const ReqDesc &d, int x, int y, int cap, int &ox, int &oy) {
+__device__ bool nearest_occupied(const ReqDesc &d, const int32_t *sq_off, const short2 *sq_rep, int x, int y, int cap,
+                                 int &ox, int &oy) {
     if (x < 0 || y < 0 || x >= d.W || y >= d.H) return false;
     const int d2 = d.d2map[(size_t)y * d.W + x];
     if (d2 < 0 || d2 > cap) return false;
-    const int e1 = d.sq_off[d2 + 1];
-    for (int e = d.sq_off[d2]; e < e1; e += 8) {
+    if (d2 == 0) {
+        ox = x;
+        oy = y;
+        return true;
+    }
+    const int e1 = sq_off[d2 + 1];
+    for (int e = sq_off[d2]; e < e1; e += 8) {
         short2 o[8];
         int8_t v[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) o[i] = e + i < e1 ? __ldg(d.sq_rep + e + i) : make_short2(0, 0);
+        for (int i = 0; i < 8; ++i) o[i] = e + i < e1 ? sq_rep[e + i] : make_short2(0, 0);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int cx = x + o[i].y, cy = y + o[i].x;
@@ -84,12 +91,12 @@ __device__ __forceinline__ double warp_sum_d(double v) {
     return v;
 }
 
-// Sums of 8 values over the warp with 9 additions instead of 40: each exchange halves the values a lane carries.  The
+// Sums of 4 values over the warp with 6 additions instead of 20: each exchange halves the values a lane carries.  The
 // lane ends with the total of value sum_index(lane).
-__device__ __forceinline__ double warp_sums8(double (&v)[8]) {
+__device__ __forceinline__ double warp_sums4(double (&v)[4]) {
     const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int n = 4, o = 16; n >= 1; n >>= 1, o >>= 1) {
+    for (int n = 2, o = 16; n >= 1; n >>= 1, o >>= 1) {
         const bool up = lane & o;
 #pragma unroll
         for (int j = 0; j < n; ++j) {
@@ -97,11 +104,11 @@ __device__ __forceinline__ double warp_sums8(double (&v)[8]) {
             v[j] = keep + __shfl_xor_sync(kFull, send, o);
         }
     }
-    v[0] += __shfl_xor_sync(kFull, v[0], 2);
-    v[0] += __shfl_xor_sync(kFull, v[0], 1);
+#pragma unroll
+    for (int o = 4; o >= 1; o >>= 1) v[0] += __shfl_xor_sync(kFull, v[0], o);
     return v[0];
 }
-__device__ __forceinline__ int sum_index(int lane) { return (lane >> 4 & 1) * 4 + (lane >> 3 & 1) * 2 + (lane >> 2 & 1); }
+__device__ __forceinline__ int sum_index(int lane) { return (lane >> 4 & 1) * 2 + (lane >> 3 & 1); }
 
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -123,8 +130,8 @@ __device__ __forceinline__ void world_point(double x, double y, double ct, doubl
                                             double inv_res, double &wx, double &wy, int &cx, int &cy) {
     wx = __dadd_rn(x, __dsub_rn(__dmul_rn(ct, sx), __dmul_rn(st, sy)));
     wy = __dadd_rn(y, __dadd_rn(__dmul_rn(st, sx), __dmul_rn(ct, sy)));
-    cx = (int)floor(__dmul_rn(wx, inv_res));
-    cy = (int)floor(__dmul_rn(wy, inv_res));
+    cx = __double2int_rd(__dmul_rn(wx, inv_res));
+    cy = __double2int_rd(__dmul_rn(wy, inv_res));
 }
 
 __device__ __forceinline__ int clamped_d2(const ReqDesc &d, int x, int y) {
@@ -133,17 +140,30 @@ __device__ __forceinline__ int clamped_d2(const ReqDesc &d, int x, int y) {
     return (v < 0 || v > d.C) ? d.C : v;
 }
 
+// The pose: position, cos and sin of theta.  The rotation applied so far is carried as its cosine and sine (c, s),
+// renormalised after every step, and theta is read off it once at the end: an FP64 atan2, sine and cosine in every
+// iteration were half of the iteration's time.
 struct IcpPose {
-    double x, y, th, ct, st;   // the pose, cos and sin of theta
+    double x, y, ct, st, c, s;
     int stop;
 };
 
-// dynamic shared memory: [per] the CTA's sensor-frame points, then in the first CTA [N] the clamped d2 of the refined
-// endpoints; per: beams per CTA of the cluster for the longest scan
+// (c, s) scaled to unit length (its length is 1 within rounding: one Newton step of the reciprocal square root)
+__device__ __forceinline__ void unit_rotation(double &c, double &s) {
+    const double r = 1.5 - 0.5 * (c * c + s * s);
+    c *= r;
+    s *= r;
+}
+
+constexpr int kIcpTableBytes = 28 * 1024;   // the pairing table is staged up to this size (C = 1600: 26 KB)
+
+// dynamic shared memory: [per] the CTA's sensor-frame points, then in the first CTA [max_beams] the clamped d2 of the
+// refined endpoints, then with staged the map's pairing table; per: beams per CTA of the cluster for the longest scan
 __global__ void __launch_bounds__(kIcpThreads) k_icp(const ReqDesc *__restrict__ reqs, int batch_lo, int batch_hi,
-                                                     int per) {
+                                                     int per, int max_beams, bool staged) {
     extern __shared__ __align__(16) unsigned char icp_smem[];
-    __shared__ double part[kIcpCluster * kIcpWarps][8];   // the first CTA's: every warp's sums
+    __shared__ double part[kIcpCluster * kIcpWarps][4];   // the first CTA's: every warp's sums
+    __shared__ int parti[kIcpCluster * kIcpWarps][4];
     __shared__ IcpPose pose;
     double2 *pts = reinterpret_cast<double2 *>(icp_smem);
     int *qv = reinterpret_cast<int *>(icp_smem + sizeof(double2) * (size_t)per);
@@ -163,79 +183,117 @@ __global__ void __launch_bounds__(kIcpThreads) k_icp(const ReqDesc *__restrict__
     const int i0 = (int)cr * per, n = max(0, min(N - i0, per));   // this CTA's beams
     const double2 *src = reinterpret_cast<const double2 *>(d.icp_pts) + i0;
     for (int i = tid; i < n; i += kIcpThreads) pts[i] = src[i];
-    const double res = d.resd, inv_res = 1.0 / res;
+    // the pairing table next to the beams: two of the four loads that a pairing waits for in turn
+    const int32_t *sq_off = d.sq_off;
+    const short2 *sq_rep = d.sq_rep;
+    if (staged) {   // 16 bytes at a time: the tables end in padding
+        const int reps = __ldg(sq_off + d.C + 1), o4 = (d.C + 2 + 3) / 4, r4 = (reps + 3) / 4;
+        int4 *off = reinterpret_cast<int4 *>(qv + ((max_beams + 3) & ~3)), *rep = off + o4;
+#pragma unroll 4
+        for (int i = tid; i < o4; i += kIcpThreads) off[i] = __ldg(reinterpret_cast<const int4 *>(sq_off) + i);
+#pragma unroll 4
+        for (int i = tid; i < r4; i += kIcpThreads) rep[i] = __ldg(reinterpret_cast<const int4 *>(sq_rep) + i);
+        sq_off = reinterpret_cast<const int32_t *>(off);
+        sq_rep = reinterpret_cast<const short2 *>(rep);
+    }
+    const double res = d.resd, inv_res = 1.0 / res, half = 0.5 * res;
     auto tell = [&](const IcpPose &p) {   // by warp 0 of the first CTA: the pose to every CTA, one per lane
         if (lane < (int)cs) {
             const uint32_t a = cluster_addr(&pose, lane);
             cluster_store(a, p.x);
             cluster_store(a + 8, p.y);
-            cluster_store(a + 16, p.th);
-            cluster_store(a + 24, p.ct);
-            cluster_store(a + 32, p.st);
-            cluster_store(a + 40, p.stop);
+            cluster_store(a + 16, p.ct);
+            cluster_store(a + 24, p.st);
+            cluster_store(a + 32, p.c);
+            cluster_store(a + 40, p.s);
+            cluster_store(a + 48, p.stop);
         }
     };
+    const double th0 = __ddiv_rn(__dmul_rn((double)d.best_m[s], 2.0 * M_PI), (double)d.ns);
     cluster_sync();   // every CTA has started: its shared memory may be written
     if (cr == 0 && warp == 0) {
         const int2 hc = d.hyps[d.survivors[s]];
         IcpPose p;
         p.x = __dmul_rn((double)hc.x + 0.5, res);
         p.y = __dmul_rn((double)hc.y + 0.5, res);
-        p.th = __ddiv_rn(__dmul_rn((double)d.best_m[s], 2.0 * M_PI), (double)d.ns);
-        p.ct = cos(p.th);
-        p.st = sin(p.th);
+        p.ct = cos(th0);
+        p.st = sin(th0);
+        p.c = 1.0;
+        p.s = 0.0;
         p.stop = d.icp_iters <= 0;
         tell(p);
     }
     cluster_sync();
     for (int it = 1; !pose.stop; ++it) {
         const IcpPose p = pose;
-        double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};   // pairs, sums of w, of c, of w.c and of w x c
+        double v[4] = {0, 0, 0, 0};   // sums of w, of w.c and of w x c
+        int np = 0, sox = 0, soy = 0;   // pairs and sums of their cells, exact
         for (int i = tid; i < n; i += kIcpThreads) {
             double wx, wy;
             int ex, ey, ox, oy;
             world_point(p.x, p.y, p.ct, p.st, pts[i].x, pts[i].y, inv_res, wx, wy, ex, ey);
-            if (!nearest_occupied(d, ex, ey, d.C, ox, oy)) continue;
-            const double cx = ((double)ox + 0.5) * res, cy = ((double)oy + 0.5) * res;
-            v[0] += 1.0;
-            v[1] += wx;
-            v[2] += wy;
-            v[3] += cx;
-            v[4] += cy;
-            v[5] += wx * cx + wy * cy;
-            v[6] += wx * cy - wy * cx;
+            if (!nearest_occupied(d, sq_off, sq_rep, ex, ey, d.C, ox, oy)) continue;
+            const double cx = fma((double)ox, res, half), cy = fma((double)oy, res, half);
+            ++np;
+            sox += ox;
+            soy += oy;
+            v[0] += wx;
+            v[1] += wy;
+            v[2] = fma(wx, cx, fma(wy, cy, v[2]));
+            v[3] = fma(wx, cy, fma(-wy, cx, v[3]));
         }
         __syncwarp();
-        const double w = warp_sums8(v);
-        if ((lane & 3) == 0) cluster_store(cluster_addr(&part[cr * kIcpWarps + warp][sum_index(lane)], 0), w);
+        const double w = warp_sums4(v);
+        const int k0 = cr * kIcpWarps + warp;
+        np = __reduce_add_sync(kFull, np);
+        sox = __reduce_add_sync(kFull, sox);
+        soy = __reduce_add_sync(kFull, soy);
+        if ((lane & 7) == 0) cluster_store(cluster_addr(&part[k0][sum_index(lane)], 0), w);
+        if (lane < 3) cluster_store(cluster_addr(&parti[k0][lane], 0), lane == 0 ? np : lane == 1 ? sox : soy);
         cluster_sync();   // the sums have arrived, and every thread has read the pose
         if (cr == 0 && warp == 0) {
+            const int parts = (int)cs * kIcpWarps;
             double t = 0.0;
-            for (int k = lane >> 3; k < (int)cs * kIcpWarps; k += 4) t += part[k][lane & 7];
-            t += __shfl_xor_sync(kFull, t, 8);
-            t += __shfl_xor_sync(kFull, t, 16);
-            double m[7];
+            for (int k = lane >> 2; k < parts; k += 8) t += part[k][lane & 3];
 #pragma unroll
-            for (int j = 0; j < 7; ++j) m[j] = __shfl_sync(kFull, t, j);
+            for (int o = 4; o <= 16; o <<= 1) t += __shfl_xor_sync(kFull, t, o);
+            const double swx = __shfl_sync(kFull, t, 0), swy = __shfl_sync(kFull, t, 1), sdot = __shfl_sync(kFull, t, 2),
+                         scr = __shfl_sync(kFull, t, 3);
+            const int pairs = __reduce_add_sync(kFull, lane < parts ? parti[lane][0] : 0);
+            const int nox = __reduce_add_sync(kFull, lane < parts ? parti[lane][1] : 0);
+            const int noy = __reduce_add_sync(kFull, lane < parts ? parti[lane][2] : 0);
+            const double np = (double)pairs;
             IcpPose q = p;
-            const double np = m[0];
             if (np < 2.0) {
                 q.stop = 1;
             } else {
-                const double mwx = m[1] / np, mwy = m[2] / np, mcx = m[3] / np, mcy = m[4] / np;
-                const double f = atan2(m[6] - np * (mwx * mcy - mwy * mcx), m[5] - np * (mwx * mcx + mwy * mcy));
-                q.th = __dadd_rn(p.th, f);
-                // one lane takes the motion's angle, another the new pose's: one evaluation for both
-                const double ang = lane == 0 ? f : q.th, ca = cos(ang), sa = sin(ang);
-                const double cf = __shfl_sync(kFull, ca, 0), sf = __shfl_sync(kFull, sa, 0);
-                q.ct = __shfl_sync(kFull, ca, 1);
-                q.st = __shfl_sync(kFull, sa, 1);
+                // the four means by four lanes, so one division's latency; then the cross sum (even lanes) and the
+                // dot sum (odd lanes)
+                const int which = lane & 3;
+                const double mean = (which == 0 ? swx : which == 1 ? swy : which == 2 ? ((double)nox + 0.5 * np) * res
+                                                                                     : ((double)noy + 0.5 * np) * res) / np;
+                const double mwx = __shfl_sync(kFull, mean, 0), mwy = __shfl_sync(kFull, mean, 1);
+                const double mcx = __shfl_sync(kFull, mean, 2), mcy = __shfl_sync(kFull, mean, 3);
+                const bool odd = lane & 1;
+                const double a1 = odd ? mcx : mcy, a2 = odd ? mcy : mcx;
+                const double cd = (odd ? sdot : scr) - np * (odd ? mwx * a1 + mwy * a2 : mwx * a1 - mwy * a2);
+                const double cross = __shfl_sync(kFull, cd, 0), dot = __shfl_sync(kFull, cd, 1);
+                // the motion's rotation: cos and sin of atan2(cross, dot) (the identity for two zero sums)
+                const double len2 = cross * cross + dot * dot, inv = len2 > 0.0 ? rsqrt(len2) : 0.0;
+                double cf = len2 > 0.0 ? dot * inv : 1.0, sf = cross * inv;
+                unit_rotation(cf, sf);
+                q.ct = p.ct * cf - p.st * sf;
+                q.st = p.st * cf + p.ct * sf;
+                unit_rotation(q.ct, q.st);
+                q.c = p.c * cf - p.s * sf;
+                q.s = p.s * cf + p.c * sf;
+                unit_rotation(q.c, q.s);
                 const double tx = __dsub_rn(mcx, __dsub_rn(__dmul_rn(cf, mwx), __dmul_rn(sf, mwy)));
                 const double ty = __dsub_rn(mcy, __dadd_rn(__dmul_rn(sf, mwx), __dmul_rn(cf, mwy)));
                 q.x = __dadd_rn(__dsub_rn(__dmul_rn(cf, p.x), __dmul_rn(sf, p.y)), tx);
                 q.y = __dadd_rn(__dadd_rn(__dmul_rn(sf, p.x), __dmul_rn(cf, p.y)), ty);
                 const double moved = fabs(q.x - p.x) + fabs(q.y - p.y);
-                q.stop = (fabs(f) < 1e-9 && moved < 1e-9) || it >= d.icp_iters;
+                q.stop = (fabs(sf) < 1e-9 && cf > 0.0 && moved < 1e-9) || it >= d.icp_iters;
             }
             tell(q);
         }
@@ -299,15 +357,15 @@ __global__ void __launch_bounds__(kIcpThreads) k_icp(const ReqDesc *__restrict__
         double *ps = d.ref_pose + 3 * (size_t)s;
         ps[0] = p.x;
         ps[1] = p.y;
-        ps[2] = p.th;
+        ps[2] = th0 + atan2(p.s, p.c);
         d.reev[s] = T;
     }
 }
 
 }  // namespace
 
-cudaError_t launch_icp(const ReqDesc *reqs, int R, int batch_lo, int batch_hi, int max_L, int max_beams, int n_sm,
-                       cudaStream_t s) {
+cudaError_t launch_icp(const ReqDesc *reqs, int R, int batch_lo, int batch_hi, int max_L, int max_beams, int max_C,
+                       int max_reps, int n_sm, cudaStream_t s) {
     const int slots = (batch_hi - batch_lo) * max_L;
     if (R < 1 || slots < 1) return cudaSuccess;
     const int beams = max_beams > 0 ? max_beams : 1;
@@ -315,7 +373,13 @@ cudaError_t launch_icp(const ReqDesc *reqs, int R, int batch_lo, int batch_hi, i
     int cs = kIcpCluster;
     while (cs > 1 && (long long)R * slots * cs > 5ll * n_sm / 2) cs >>= 1;
     const int per = (beams + cs - 1) / cs;
-    const size_t smem = sizeof(double2) * (size_t)per + sizeof(int) * (size_t)beams;   // at most 41 KB
+    const size_t table = 16 * ((size_t)(max_C + 2 + 3) / 4 + (size_t)(max_reps + 3) / 4);
+    const bool staged = table <= (size_t)kIcpTableBytes;
+    const size_t smem = sizeof(double2) * (size_t)per + sizeof(int) * (size_t)((beams + 3) & ~3) + (staged ? table : 0);
+    if (smem > 46 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(k_icp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -327,7 +391,7 @@ cudaError_t launch_icp(const ReqDesc *reqs, int R, int batch_lo, int batch_hi, i
     cfg.stream = s;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_icp, reqs, batch_lo, batch_hi, per);
+    return cudaLaunchKernelEx(&cfg, k_icp, reqs, batch_lo, batch_hi, per, beams, staged);
 }
 
 }  // namespace relo

@@ -83,6 +83,7 @@ struct MapSlot {
     double lut_key[6] = {0};     // what its values depend on: z_hit, sigma_hit, z_rand, eps, resolution, clamp
     int32_t *sq_off = nullptr;   // [kMaxClamp + 2] and [kMaxLatticePoints]: the cells at each squared distance
     short2 *sq_rep = nullptr;
+    int n_reps = 0;              // entries of sq_rep
     size_t bytes = 0;
     std::vector<ScanTable *> tables;
     // the map's EDT runs in two parts: the occupancy tiles on the context stream (tiles_ready), then the field and
@@ -362,6 +363,7 @@ int build_lut(relo_ctx *ctx, MapSlot &m) {
         }
     }
     off[C + 1] = (int32_t)rep.size();
+    m.n_reps = (int)rep.size();
     if (!m.sq_off) {
         int rc = dev_alloc(ctx, (void **)&m.sq_off, sizeof(int32_t) * (kMaxClamp + 2), "pairing table");
         if (!rc) rc = dev_alloc(ctx, (void **)&m.sq_rep, sizeof(short2) * kMaxLatticePoints, "pairing table");
@@ -1010,7 +1012,7 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R) {
     std::vector<ReqDesc> desc((size_t)R);
     std::vector<size_t> off((size_t)R);
     size_t total = 0;
-    int total_hyp = 0, max_ns_pad = 32, max_n_hyp = 1, max_K = 1, max_beams = 1, max_C = 0, max_batches = 0;
+    int total_hyp = 0, max_ns_pad = 32, max_n_hyp = 1, max_K = 1, max_beams = 1, max_C = 0, max_reps = 0, max_batches = 0;
     long long total_chunks = 0;
     for (int r = 0; r < R; ++r) {
         const Prepared &q = pr[r];
@@ -1033,6 +1035,7 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R) {
         max_K = std::max(max_K, K);
         max_beams = std::max(max_beams, n);
         max_C = std::max(max_C, q.m->dev.C);
+        max_reps = std::max(max_reps, q.m->n_reps);
         max_batches = std::max(max_batches, q.n_batches);
     }
     // hypotheses per cast work item: group while every resident warp (5 CTAs of 8 warps per SM) keeps 16 or more items
@@ -1256,7 +1259,7 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R) {
             // the local top-k, their ICP refinement and re-evaluation, then the batch's best
             CK(timed_on(ctx, st, 5, 1, [&] { return launch_select_batch(rq, R, lo, hi, false, true, st); }),
                "batch selection");
-            CK(timed_on(ctx, st, 5, 1, [&] { return launch_icp(rq, R, lo, hi, p.local_topk, max_beams, ctx->n_sm, st); }),
+            CK(timed_on(ctx, st, 5, 1, [&] { return launch_icp(rq, R, lo, hi, p.local_topk, max_beams, max_C, max_reps, ctx->n_sm, st); }),
                "ICP refinement");
             CK(timed_on(ctx, st, 5, 1, [&] { return launch_icp_best(rq, R, lo, hi, last, st); }), "batch selection");
         } else {

@@ -403,7 +403,7 @@ cudaError_t launch_select_batch(const ReqDesc *reqs, int R, int batch_lo, int ba
 // ICP refinement and re-evaluation of the local top-k of batches batch_lo .. batch_hi - 1, then their best,
 // early termination and (with last) the results
 cudaError_t launch_icp(const ReqDesc *reqs, int R, int batch_lo, int batch_hi, int max_L, int max_beams,
-                       int n_sm, cudaStream_t s);
+                       int max_C, int max_reps, int n_sm, cudaStream_t s);   // max_reps: pairing offsets of max_C
 cudaError_t launch_icp_best(const ReqDesc *reqs, int R, int batch_lo, int batch_hi, bool last, cudaStream_t s);
 // Algorithm 1 in batched-expansion form (rrt.cu); blocking on s; *err names a failure
 // the RRT's blocked grid with a ring of blocked cells ((W + 2) x (H + 2), occupied = 100) and, from the squared

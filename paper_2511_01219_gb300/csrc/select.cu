@@ -359,34 +359,44 @@ __global__ void __launch_bounds__(1024) k_select_batch(const ReqDesc *__restrict
     }
 }
 
-// One thread per request, after k_icp: for batches batch_lo .. batch_hi - 1
+// One warp per request, after k_icp: for batches batch_lo .. batch_hi - 1
 // in order (each skipped when the request has fewer or already terminated),
 // the best re-evaluated local top-k pose (ties to the earlier survivor) joins
 // the running best, and early termination follows its score (the overview of
 // Sec. III: the test is made on the re-evaluated score).  With last, the
 // result.
-__global__ void k_icp_best(const ReqDesc *__restrict__ reqs, int R, int batch_lo, int batch_hi, int last) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= R) return;
-    const ReqDesc &d = reqs[r];
+__global__ void __launch_bounds__(32) k_icp_best(const ReqDesc *__restrict__ reqs, int batch_lo, int batch_hi, int last) {
+    const ReqDesc &d = reqs[blockIdx.x];
+    const int lane = threadIdx.x;
     SelectState *st = d.state;
     if (d.scan->n_valid > 0) {
-        for (int b = batch_lo; b < batch_hi && b < d.n_batches; ++b) {
-            if (st->done) break;
+        bool done = st->done;
+        unsigned long long best = st->best;
+        for (int b = batch_lo; b < batch_hi && b < d.n_batches && !done; ++b) {
             unsigned long long top = 0ull;
-            for (int i = 0; i < d.L; ++i) {
+            for (int i = lane; i < d.L; i += 32) {
                 const int s = d.local[(size_t)b * d.L + i];
                 if (s < 0) continue;
                 const unsigned long long key = ((unsigned long long)score_code(d.reev[s]) << 32) |
                                                (0xffffffffu - (unsigned)s);
                 top = key > top ? key : top;
             }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const unsigned long long t = __shfl_xor_sync(0xffffffffu, top, o);
+                top = t > top ? t : top;
+            }
             if (top == 0ull) continue;
-            if (top > st->best) st->best = top;
-            if (d.early_stop && (double)score_of((unsigned)(top >> 32)) >= d.tau) st->done = 1;
+            if (top > best) best = top;
+            if (d.early_stop && (double)score_of((unsigned)(top >> 32)) >= d.tau) done = true;
+        }
+        __syncwarp();   // every lane has read the state
+        if (lane == 0) {
+            st->best = best;
+            st->done = done ? 1 : 0;
         }
     }
-    if (last) finalize_request(d);
+    if (last && lane == 0) finalize_request(d);
 }
 
 }  // namespace
@@ -415,7 +425,7 @@ cudaError_t launch_select_batch(const ReqDesc *reqs, int R, int batch_lo, int ba
 }
 
 cudaError_t launch_icp_best(const ReqDesc *reqs, int R, int batch_lo, int batch_hi, bool last, cudaStream_t s) {
-    k_icp_best<<<(R + 63) / 64, 64, 0, s>>>(reqs, R, batch_lo, batch_hi, last ? 1 : 0);
+    k_icp_best<<<R, 32, 0, s>>>(reqs, batch_lo, batch_hi, last ? 1 : 0);
     return cudaGetLastError();
 }
 
