@@ -44,7 +44,8 @@ __global__ void __launch_bounds__(256) k_edt_tiles(const int8_t *__restrict__ gr
     });
 }
 
-EdtTiles tiles_of(const MapDev &m) { return EdtTiles{m.bits, m.summ, edt_span_of(m), m.far, m.W, m.H, m.TW, m.TH}; }
+EdtTiles tiles_of(const MapDev &m) { return EdtTiles{m.bits, m.summ, edt_span_of(m), m.far,
+                                                    m.reach ? walk_empty_bits(m.reach, m.TW, m.TH) : nullptr, m.W, m.H, m.TW, m.TH}; }
 
 // the border of the padded field: every cell outside the map reads C (d = d_max)
 __global__ void k_field_border(uint16_t *__restrict__ fieldp, int W, int H, int P, int Wp, int Hp, int C) {
@@ -56,42 +57,84 @@ __global__ void k_field_border(uint16_t *__restrict__ fieldp, int W, int H, int 
     }
 }
 
-// Which walk-frame tiles are empty, one bit per tile: word [row][k] of a
-// frame row holds tiles 32 k .. 32 k + 31 (tiles past the row count as not
-// empty, and one more word of zeros ends every row).
-__global__ void k_walk_empty(const uint64_t *__restrict__ wf, int TW, uint32_t *__restrict__ emp) {
-    const unsigned WB = (unsigned)TW + 1u, SW = walk_empty_row_words(TW);
-    const unsigned x = blockIdx.x * blockDim.x + threadIdx.x;
-    const size_t row = blockIdx.y;   // frame * (TH + 1) + ty
-    const unsigned bal = __ballot_sync(0xffffffffu, x < WB && wf[row * WB + x] == 0ull);
-    if ((threadIdx.x & 31) == 0 && (x >> 5) < SW) emp[row * SW + (x >> 5)] = bal;
+// The rows of emptiness that a warp's 32 tiles of a frame row see ahead: lanes k < kReachMax hold the emptiness bits of
+// row ty + k covering the tiles, lanes kReachMax + k the next 32.  For each of the kReachMax rows from theirs, a lane
+// shifts the 64 bits of that pair down by its own position (row_ahead), so bit i says whether the tile i to its right is
+// empty (i + 31 < 64: a window of kReachMax + 1 bits always fits).  The map's emptiness is stored once; a frame mirrored
+// in x reads the window from the other end, reversed, and tiles outside the map count as not empty.
+__device__ __forceinline__ uint32_t rows_ahead(const uint32_t *__restrict__ emp, int TW, int TH, unsigned strip) {
+    static_assert(2 * kReachMax <= 32, "one emptiness word per lane");
+    const int lane = threadIdx.x & 31, HB = TH + 1, words = walk_empty_row_words(TW);
+    const int frame = (int)blockIdx.y / HB, y = (int)blockIdx.y % HB + lane % kReachMax, s = (int)strip + lane / kReachMax;
+    if (y >= TH) return 0u;
+    const uint32_t *row = emp + (size_t)(frame & 2 ? TH - 1 - y : y) * words;
+    if (!(frame & 1)) return s < words ? row[s] : 0u;
+    const int p = TW - 32 * (s + 1), q = p >> 5;   // the map's tiles p .. p + 31
+    const uint32_t lo = q >= 0 ? row[q] : 0u, hi = q + 1 >= 0 && q + 1 < words ? row[q + 1] : 0u;
+    return __brev(__funnelshift_r(lo, hi, (unsigned)(p & 31)));
+}
+__device__ __forceinline__ uint32_t row_ahead(uint32_t words, int r) {
+    return __funnelshift_r(__shfl_sync(0xffffffffu, words, r), __shfl_sync(0xffffffffu, words, r + kReachMax),
+                           threadIdx.x & 31);
 }
 
-// The empty boxes ahead of every walk-frame tile (MapDev::reach).  A warp
-// takes 32 tiles of a row: lanes k < kReachMax load the emptiness word of row
-// ty + k covering its tiles and lanes kReachMax + k the next word.  For each
-// of the kReachMax rows from theirs, a lane shifts the 64 bits of that pair
-// down by its own position, so bit i says whether the tile i to its right is
-// empty (i + 31 < 64: a window of kReachMax + 1 bits always fits).  Its row
-// run is the block of set bits from bit 0 of the first row, its column run
-// the rows that keep bit 0, and its square the largest s whose s rows' AND
-// keeps bits 0 .. s - 1.
-__global__ void k_walk_reach(const uint32_t *__restrict__ emp, int TW, int TH, uint16_t *__restrict__ reach) {
-    static_assert(2 * kReachMax <= 32, "one emptiness word per lane");
+// The empty boxes ahead of every walk-frame tile, per slope class (MapDev::reach).  A warp takes 32 tiles of a row.  With
+// h rows' windows ANDed, the run of set bits from bit 0 is the widest box of height h; a class keeps the (w, h) whose far
+// edges a ray from the tile's middle at its angle reaches last, min((w - 1/2) / cos, (h - 1/2) / sin).  That value in
+// 1/128 tiles above the box's code is one integer, so a candidate is a product, a minimum, an OR and a maximum; a class
+// looks no further down than the height that no width up to kReachMax can use (2, 4 and 9 rows for the shallow ones).
+// Bound by those; with float values and a box beside each 39 us on the 4096 x 4096 warehouse (1.05 M tiles, 7 classes).
+__global__ void __launch_bounds__(256) k_walk_reach(const uint32_t *__restrict__ emp, int TW, int TH,
+                                                    uint16_t *__restrict__ reach) {
+    // 64 / cos and 64 / sin of the classes' middles: 3, 11, 26, 45, 64, 79 and 87 degrees
+    constexpr uint32_t kInvC[kReachClasses] = {64, 65, 71, 91, 146, 335, 1223};
+    constexpr uint32_t kInvS[kReachClasses] = {1223, 335, 146, 91, 71, 65, 64};
     const int lane = threadIdx.x & 31;
-    const unsigned WB = (unsigned)TW + 1u, HB = (unsigned)TH + 1u, SW = walk_empty_row_words(TW);
+    const unsigned WB = (unsigned)TW + 1u, HB = (unsigned)TH + 1u;
     const unsigned strip = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (strip * 32u >= WB) return;   // the whole warp lies past the row
-    const unsigned fy = blockIdx.y, ty = fy % HB;   // frame * HB + ty
-    const unsigned k = (unsigned)lane % kReachMax, y = ty + k;
-    const uint32_t wv = y < HB ? emp[(size_t)(fy + k) * SW + strip + lane / kReachMax] : 0u;
+    const uint32_t words = rows_ahead(emp, TW, TH, strip);
+    uint32_t a = ~0u, best[kReachClasses];
+#pragma unroll
+    for (int c = 0; c < kReachClasses; ++c) best[c] = 8u | 8u << 8 | 1u;   // not empty: the tile alone
+#pragma unroll
+    for (int r = 0; r < kReachMax; ++r) {
+        a &= row_ahead(words, r);
+        const uint32_t w = (uint32_t)__ffs((int)(~a | (1u << kReachMax))) - 1u;   // the sentinel bit caps the run
+        if (!__any_sync(0xffffffffu, w > 0u)) break;
+        if (w > 0u) {
+            const uint32_t w2 = 2u * w - 1u, e = 8u * w | 8u * (uint32_t)(r + 1) << 8;
+#pragma unroll
+            for (int c = 0; c < kReachClasses; ++c) {
+                // rows that r - 1 already offered at any width add nothing
+                if (r > 0 && (2u * r - 1u) * kInvS[c] >= (2u * kReachMax - 1u) * kInvC[c]) continue;
+                best[c] = max(best[c], min(w2 * (kInvC[c] << 16), ((2u * r + 1u) * kInvS[c]) << 16) | e);
+            }
+        }
+    }
+    const unsigned xa = strip * 32u + lane, frame = blockIdx.y / HB, ty = blockIdx.y % HB;
+    const size_t n = walk_frame_words(TW, TH);
+    if (xa < WB) {
+        uint16_t *out = reach + (size_t)frame * kReachClasses * n + (size_t)ty * WB + xa;
+#pragma unroll
+        for (int c = 0; c < kReachClasses; ++c) out[c * n] = (uint16_t)best[c];
+    }
+}
+
+// The exported boxes (relo_map_walk_boxes_dev): the row run is the block of set bits from bit 0 of the first row, the
+// column run the rows that keep bit 0, the square the largest s whose s rows' AND keeps bits 0 .. s - 1.
+__global__ void k_walk_export(const uint32_t *__restrict__ emp, int TW, int TH, uint16_t *__restrict__ boxes) {
+    const int lane = threadIdx.x & 31;
+    const unsigned WB = (unsigned)TW + 1u;
+    const unsigned strip = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (strip * 32u >= WB) return;
+    const uint32_t words = rows_ahead(emp, TW, TH, strip);
     uint32_t e0 = 0u, a = ~0u;
     int s = 0, yr = 0;
     bool sq = true, col = true;
 #pragma unroll
     for (int r = 0; r < kReachMax; ++r) {
-        const uint32_t e = __funnelshift_r(__shfl_sync(0xffffffffu, wv, r),
-                                           __shfl_sync(0xffffffffu, wv, r + kReachMax), (unsigned)lane);
+        const uint32_t e = row_ahead(words, r);
         if (r == 0) e0 = e;
         col = col && (e & 1u);
         if (col) yr = r + 1;
@@ -99,12 +142,10 @@ __global__ void k_walk_reach(const uint32_t *__restrict__ emp, int TW, int TH, u
         const uint32_t mr = (2u << r) - 1u;   // bits 0 .. r
         sq = sq && (a & mr) == mr;
         if (sq) s = r + 1;
-        if (!__any_sync(0xffffffffu, sq || col)) break;   // no lane's boxes grow further
     }
-    // the sentinel bit caps the row run at kReachMax
     const int xr = __ffs((int)(~e0 | (1u << kReachMax))) - 1;
     const unsigned xa = strip * 32u + lane;
-    if (xa < WB) reach[(size_t)fy * WB + xa] = (uint16_t)(s | (xr << 5) | (yr << 10));
+    if (xa < WB) boxes[(size_t)blockIdx.y * WB + xa] = (uint16_t)(s | (xr << 5) | (yr << 10));
 }
 
 // the last column and row of tiles of each walk frame: every bit set
@@ -209,12 +250,15 @@ cudaError_t launch_edt_tiles(const MapDev &m, const int8_t *grid, cudaStream_t s
     }
     k_edt_tiles<<<dim3((m.TW + 31) / 32, edt_summary_rows(m.H)), dim3(32, 8), 0, s>>>(grid, t, vec, copy,
                                                                                       m.bits + (size_t)m.TW * m.TH);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_walk_reach(const MapDev &m, cudaStream_t s) {
     if (m.reach) {
         // the walk frames' empty boxes (their border tiles, full, were written when the map was loaded)
-        const unsigned WB = (unsigned)m.TW + 1u, SW = walk_empty_row_words(m.TW), rows = 4u * ((unsigned)m.TH + 1u);
-        uint32_t *emp = walk_empty_bits(m.reach, m.TW, m.TH);
-        k_walk_empty<<<dim3((32u * SW + 255u) / 256u, rows), 256, 0, s>>>(m.bits + (size_t)m.TW * m.TH, m.TW, emp);
-        k_walk_reach<<<dim3((WB + 255u) / 256u, rows), 256, 0, s>>>(emp, m.TW, m.TH, m.reach);
+        const unsigned WB = (unsigned)m.TW + 1u, rows = 4u * ((unsigned)m.TH + 1u);
+        k_walk_reach<<<dim3((WB + 255u) / 256u, rows), 256, 0, s>>>(walk_empty_bits(m.reach, m.TW, m.TH), m.TW, m.TH,
+                                                                    m.reach);
     }
     return cudaGetLastError();
 }
@@ -226,6 +270,12 @@ cudaError_t launch_edt_field(const MapDev &m, int n_sm, cudaStream_t s) {
 cudaError_t launch_edt(const MapDev &m, int n_sm, cudaStream_t s) {
     cudaError_t e = launch_edt_tiles(m, m.grid, s);
     return e == cudaSuccess ? launch_edt_field(m, n_sm, s) : e;
+}
+
+cudaError_t launch_walk_boxes(const MapDev &m, uint16_t *boxes, cudaStream_t s) {
+    const unsigned WB = (unsigned)m.TW + 1u, rows = 4u * ((unsigned)m.TH + 1u);
+    k_walk_export<<<dim3((WB + 255u) / 256u, rows), 256, 0, s>>>(walk_empty_bits(m.reach, m.TW, m.TH), m.TW, m.TH, boxes);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_field_border(const MapDev &m, cudaStream_t s) {

@@ -33,12 +33,14 @@ constexpr int kFarMark = -2;          // d2 of a cell left to k_edt_far
 
 // Occupancy words, bit 8 (y & 7) + (x & 7), of tiles [TH][TW]; the segments' first and last occupied rows (-1: none),
 // [ceil(TH / kSegTiles)][W]; per tile row and column, the nearest occupied rows above and below the tile row (-1: none),
-// [TH][W]; per band, whether k_edt_far has work (TH + 1 bands at most).
+// [TH][W]; per band, whether k_edt_far has work (TH + 1 bands at most); which tiles have no occupied cell and lie inside
+// the map (nullptr: not wanted), a bit per tile, [TH][ceil(TW / 32)].
 struct EdtTiles {
     uint64_t *words;
     short2 *summ;
     short2 *span;
     int *far;
+    uint32_t *empty;
     int W, H, TW, TH;
 };
 
@@ -82,6 +84,7 @@ __device__ __forceinline__ void edt_tiles(const int8_t *__restrict__ grid, const
     const int tx = blockIdx.x * 32 + threadIdx.x, ty = blockIdx.y * 8 + threadIdx.y;
     const size_t cells = (size_t)t.W * t.H;
     uint64_t word = 0ull;
+    bool free = false;
     if (tx < t.TW && ty < t.TH) {
         uint2 v[8];
 #pragma unroll
@@ -101,8 +104,13 @@ __device__ __forceinline__ void edt_tiles(const int8_t *__restrict__ grid, const
         word &= inside;
         t.words[(size_t)ty * t.TW + tx] = word;
         frames(word | ~inside, tx, ty);
+        free = (word | ~inside) == 0ull;
         if (tx == 0) t.far[ty] = 0;
         if (tx == 0 && ty == 0) t.far[t.TH] = 0;
+    }
+    if (t.empty) {   // a warp is 32 tiles of a row
+        const unsigned bal = __ballot_sync(0xffffffffu, free);
+        if (threadIdx.x == 0 && ty < t.TH) t.empty[(size_t)ty * gridDim.x + blockIdx.x] = bal;
     }
     s_word[threadIdx.y][threadIdx.x] = word;
     __syncthreads();

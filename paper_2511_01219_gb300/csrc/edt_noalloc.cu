@@ -94,7 +94,7 @@ extern "C" int relo_edt_noalloc(const int8_t *grid_dev, int32_t w, int32_t h, in
     // an error left by the caller's own earlier work: report it, launch nothing, leave it pending
     if (cudaPeekAtLastError() != cudaSuccess) return RELO_E_CUDA;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const EdtTiles t{sc->words, sc->summ, sc->span, sc->far, w, h, (w + 7) / 8, (h + 7) / 8};
+    const EdtTiles t{sc->words, sc->summ, sc->span, sc->far, nullptr, w, h, (w + 7) / 8, (h + 7) / 8};
     const bool vec = (w & 7) == 0 && (reinterpret_cast<uintptr_t>(grid_dev) & 7) == 0;
     k_na_tiles<<<dim3((t.TW + 31) / 32, edt_summary_rows(h)), dim3(32, 8), 0, s>>>(grid_dev, t, vec);
     if (cudaGetLastError() != cudaSuccess) return RELO_E_CUDA;

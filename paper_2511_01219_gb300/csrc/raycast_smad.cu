@@ -204,19 +204,13 @@ __device__ __forceinline__ uint32_t cast_ray(const uint64_t *__restrict__ bits, 
 // (fx, fy) has cx + cy = fx + fy + k, so a table's step index of a far edge
 // gives the other coordinate there with one subtraction, and the rows of the
 // tables are linear in cx, cy and cx + cy (the start is folded into the bases).
-// A tile is read through its boxes entry first (MapDev::reach: 0 exactly when
-// the tile is not empty).  A box of empty tiles is left at its far edges, the
-// run along the tile's row for a ray within about 14 degrees of the x axis, the
-// run along its column within 14 degrees of the y axis, the empty square
-// otherwise, at the cell of step min(selx[|dx| at the x edge], sely[|dy| at the
-// y edge]), since no cell inside it can stop the ray.  In a tile that is not
-// empty, the word moved to the current cell is ANDed with the table's bit board
-// of the cells still ahead; on a staircase that only moves +x and +y the cell
-// order along the ray is the row-major bit order, so the lowest common bit is
-// the hit; without one the ray leaves the tile as a box of one tile.  Only such
-// tiles load their word and board, together with the exit steps: two memory
-// round trips and at most five loads per move.  Same cells, same hit, same range
-// as cast_ray.
+// A tile is read through its box entry first (MapDev::reach, of the ray's slope class).  A box of empty tiles is left at
+// its far edges, at the cell of step min(selx[|dx| at the x edge], sely[|dy| at the y edge]), since no cell inside it can
+// stop the ray.  In a tile that is not empty (bit 0 of its entry), the word moved to the current cell is ANDed with the
+// table's bit board of the cells still ahead; on a staircase that only moves +x and +y the cell order along the ray is
+// the row-major bit order, so the lowest common bit is the hit; without one the ray leaves the tile as a box of one tile.
+// Only such tiles load their word and board, together with the exit steps: two memory round trips and at most five loads
+// per move.  Same cells, same hit, same range as cast_ray.
 //
 // Registers bound the kernel's warps: the tables share one allocation, and a
 // map's boxes lie behind its words in another, so a direction holds two 64-bit
@@ -227,7 +221,6 @@ struct RayDir {   // what the walks of one direction share
     unsigned rq;                        // the frame's boxes, 2-byte units from bq
     unsigned selx, sely, jm;            // the direction's column: 2-byte units from mk, 8-byte units from mk
     unsigned WB, ns;
-    unsigned wsh, hsh;                  // which sides of the packed boxes the ray leaves
     int mx, my;                         // 8 TW - 1 (mirrored in x) or -1; 8 TH - 1 or -1
 
     __device__ __forceinline__ void init(const uint64_t *bits, const uint16_t *reach, int TW, int TH,
@@ -239,17 +232,15 @@ struct RayDir {   // what the walks of one direction share
         ns = (unsigned)ns_;
         const size_t frame = (size_t)((xneg ? 1 : 0) + (yneg ? 2 : 0)) * walk_frame_words(TW, TH);
         bq = bits + (size_t)TW * TH + frame;
-        rq = (unsigned)(reach + frame - reinterpret_cast<const uint16_t *>(bq));
+        // the class of the slope: any class's boxes are empty, so the split need not be exact
+        const float ax = fabsf((float)d.x), ay = fabsf((float)d.y), lo = fminf(ax, ay), hi = fmaxf(ax, ay);
+        const int c = lo < 0.1051f * hi ? 0 : lo < 0.3249f * hi ? 1 : lo < 0.7265f * hi ? 2 : 3;
+        const size_t box = frame * kReachClasses + (size_t)(ay > ax ? kReachClasses - 1 - c : c) * walk_frame_words(TW, TH);
+        rq = (unsigned)(reach + box - reinterpret_cast<const uint16_t *>(bq));
         mk = t.mask;
         selx = t.selx + (unsigned)j;
         sely = t.sely + (unsigned)j;
         jm = (unsigned)j;
-        // box width (reach >> wsh) & 31, height (reach >> hsh) & 31, each at least 1 (bit 15 and up are 0, so a shift
-        // of 15 reads a side of 1 tile)
-        const long long adir = d.x < 0 ? -(long long)d.x : d.x, bdir = d.y < 0 ? -(long long)d.y : d.y;
-        const bool shallow = 4 * bdir <= adir, steep = 4 * adir <= bdir;
-        wsh = shallow ? 5u : steep ? 15u : 0u;
-        hsh = steep ? 10u : shallow ? 15u : 0u;
     }
     // between the map's x (y) and the frame's: the same involution both ways
     __device__ __forceinline__ int flip_x(int x) const { return mx < 0 ? x : mx - x; }
@@ -270,14 +261,12 @@ __device__ __forceinline__ uint32_t walk_ray(const RayDir &r, int W, int H, unsi
     unsigned cx = (unsigned)fx, cy = (unsigned)fy;
     int stop;   // 1 hit (or left the map), 2 range limit
     for (;;) {
-        const unsigned tx = cx >> 3, ty = cy >> 3;
-        const unsigned ti = ty * r.WB + tx;
-        const unsigned rv = __ldg(rch + (r.rq + ti));
-        const unsigned ex = 8u * (tx + max(1u, (rv >> r.wsh) & 31u));   // the box's far edges
-        const unsigned ey = 8u * (ty + max(1u, (rv >> r.hsh) & 31u));
+        const unsigned ti = (cy >> 3) * r.WB + (cx >> 3);
+        const unsigned box = __ldg(rch + (r.rq + ti));
+        const unsigned ex = (cx & ~7u) + (box & 0xf8u), ey = (cy & ~7u) + (box >> 8);   // the box's far edges
         const unsigned kx = __ldg(sel + (ex * r.ns + bx));
         const unsigned ky = __ldg(sel + (ey * r.ns + by));
-        if (rv == 0u) {
+        if (box & 1u) {   // not empty
             const uint64_t word = __ldg(r.bq + ti);
             const uint64_t board = __ldg(r.mk + ((cx + cy) * r.ns + bm));
             // move the current cell to bit 0; bits that wrap into the row below

@@ -88,7 +88,8 @@ struct MapSlot {
     std::vector<ScanTable *> tables;
     // the map's EDT runs in two parts: the occupancy tiles on the context stream (tiles_ready), then the field and
     // d2 on the context's side stream (field_ready), overlapping the next request's ray cast
-    cudaEvent_t tiles_ready = nullptr, field_ready = nullptr;
+    // (words_ready: the tiles and summaries alone, all that the field pass reads)
+    cudaEvent_t words_ready = nullptr, tiles_ready = nullptr, field_ready = nullptr;
 };
 
 // One request prepared for a batch.
@@ -504,9 +505,13 @@ int plan_for(relo_ctx *ctx, const float *angles_raw, int n_raw, SensorPlan **out
 // the tiles and their summaries).  Every later reader of the field or d2 waits on field_ready; the next EDT of the map
 // waits on it before its tiles are overwritten.
 cudaError_t map_edt(relo_ctx *ctx, MapSlot &m, const int8_t *grid) {
-    cudaError_t e = timed(ctx, 0, m.dev.reach ? 3 : 1, [&] { return launch_edt_tiles(m.dev, grid, ctx->stream); });
+    cudaError_t e = timed(ctx, 0, 2, [&] {
+        cudaError_t t = launch_edt_tiles(m.dev, grid, ctx->stream);
+        if (t == cudaSuccess) t = cudaEventRecord(m.words_ready, ctx->stream);
+        return t == cudaSuccess ? launch_walk_reach(m.dev, ctx->stream) : t;
+    });
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->side, m.words_ready, 0);
     if (e == cudaSuccess) e = cudaEventRecord(m.tiles_ready, ctx->stream);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->side, m.tiles_ready, 0);
     if (e == cudaSuccess) e = timed_on(ctx, ctx->side, 7, 3, [&] { return launch_edt_field(m.dev, ctx->n_sm, ctx->side); });
     if (e == cudaSuccess) e = cudaEventRecord(m.field_ready, ctx->side);
     return e;
@@ -700,6 +705,7 @@ WinTable *new_win(relo_ctx *ctx, ScanTable *t, const SensorPlan &P, int n_hyp) {
 
 void free_map(relo_ctx *ctx, MapSlot &m) {
     if (ctx->side) cudaStreamSynchronize(ctx->side);
+    if (m.words_ready) cudaEventDestroy(m.words_ready);
     if (m.tiles_ready) cudaEventDestroy(m.tiles_ready);
     if (m.field_ready) cudaEventDestroy(m.field_ready);
     drop_tables(ctx, m);
@@ -754,7 +760,8 @@ int load_map_impl(relo_ctx *ctx, const int8_t *grid, bool on_device, int32_t w, 
     }
     m.dev.reach = reinterpret_cast<uint16_t *>(m.dev.bits + occupancy_words(m.dev.TW, m.dev.TH));
     m.dev.far = edt_far_of(m.dev.summ, w, h);
-    cudaError_t e = cudaEventCreateWithFlags(&m.tiles_ready, cudaEventDisableTiming);
+    cudaError_t e = cudaEventCreateWithFlags(&m.words_ready, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m.tiles_ready, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m.field_ready, cudaEventDisableTiming);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(m.dev.grid, grid, cells, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
@@ -1752,9 +1759,8 @@ int relo_map_walk_boxes_dev(relo_ctx *ctx, int32_t map_id, uint16_t *boxes_dev, 
     const int64_t n = (int64_t)(4 * walk_frame_words(m->dev.TW, m->dev.TH));
     if (n_out) *n_out = n;
     if (!boxes_dev || capacity < n) return fail(ctx, RELO_E_INVALID_ARG, "the buffer holds fewer than 4 (TW+1)(TH+1)");
-    // the boxes are written on the context stream with the occupancy tiles
-    CK(cudaMemcpyAsync(boxes_dev, m->dev.reach, sizeof(uint16_t) * (size_t)n, cudaMemcpyDeviceToDevice, ctx->stream),
-       "walk boxes");
+    // from the tiles' emptiness, which the context stream wrote with them
+    CK(launch_walk_boxes(m->dev, boxes_dev, ctx->stream), "walk boxes");
     CK(cudaStreamSynchronize(ctx->stream), "walk boxes");
     return RELO_OK;
 }

@@ -84,15 +84,15 @@ __host__ __device__ inline size_t occupancy_words(int TW, int TH) {
     return (size_t)TW * TH + 4 * walk_frame_words(TW, TH);
 }
 
-// Empty boxes ahead.  For every tile (tx, ty) of a walk frame, reach packs
-// three boxes of empty tiles that start at it, each side at most kReachMax
-// (all 0 when the tile itself is not empty): bits 0-4 the side s of the
-// largest square [tx, tx + s) x [ty, ty + s), bits 5-9 the run [tx, tx + r) x
-// {ty} along the tile's row, bits 10-14 the run {tx} x [ty, ty + r) along its
-// column.  A ray in that tile moves towards +x and +y, so every cell it enters
-// before it leaves a box lies inside it: the walk may leave the whole box in
-// one move.  The walk frames' last column and row are full, so a box never
-// leaves the map.
+// Empty boxes ahead.  A ray in an empty walk-frame tile (tx, ty) moves towards +x and +y, so every cell it enters before
+// it leaves a box of empty tiles [tx, tx + w) x [ty, ty + h) lies inside it: the walk leaves the whole box in one move.
+// MapDev::reach holds a box per tile for each of kReachClasses classes of ray slope, the one (sides at most kReachMax)
+// that a ray of the class's middle slope stays in longest: 8 w in bits 0-7 and 8 h in bits 8-15, and for a tile that is
+// not empty the tile itself with bit 0 set.  The walk frames' last column and row are full, so a box never leaves the
+// map.  Moves of a warp's longest ray, counted on the CPU (office 1024^2 / warehouse 2048^2): square, row run or column
+// run by slope 4.48 / 4.64, the best box of 3 classes 4.04 / 3.01, of 5 3.94 / 2.93, of 7 3.81 / 2.84, of 11 3.77 /
+// 2.90, of every ray's own slope 3.59 / 2.70.
+constexpr int kReachClasses = 7;   // by angle to the x axis: up to 6, 18, 36, 54, 72, 84 and 90 degrees
 constexpr int kReachMax = 16;
 // Hypotheses one ray-cast work item takes, for one chunk of 32 directions
 // (the directions' setup is then done once for all of them): at most
@@ -102,17 +102,17 @@ constexpr int kCastHypsMax = 4;
 __host__ __device__ inline long long cast_chunks(int n_hyp, int ns, int per_item) {
     return (long long)((n_hyp + per_item - 1) / per_item) * (((ns + 31) & ~31) >> 5);
 }
-// words per frame row of the tiles' emptiness bits (one more than the row needs: the 64-tile window of a row's last
-// 32 tiles reads it)
-__host__ __device__ inline unsigned walk_empty_row_words(int TW) { return ((unsigned)TW + 1u + 31u) / 32u + 1u; }
-// MapDev::reach: the packed boxes [4][TH + 1][TW + 1], then the emptiness bits [4 (TH + 1)][walk_empty_row_words]
+// words per tile row of the tiles' emptiness bits
+__host__ __device__ inline int walk_empty_row_words(int TW) { return (TW + 31) / 32; }
+// MapDev::reach: the boxes [4][kReachClasses][TH + 1][TW + 1], then the map's emptiness bits [TH][walk_empty_row_words]
+__host__ __device__ inline size_t walk_boxes_bytes(int TW, int TH) {
+    return (4 * kReachClasses * walk_frame_words(TW, TH) * sizeof(uint16_t) + 15) & ~(size_t)15;
+}
 __host__ __device__ inline size_t walk_reach_bytes(int TW, int TH) {
-    const size_t boxes = (4 * walk_frame_words(TW, TH) * sizeof(uint16_t) + 15) & ~(size_t)15;
-    return boxes + (size_t)4 * ((size_t)TH + 1) * walk_empty_row_words(TW) * sizeof(uint32_t);
+    return walk_boxes_bytes(TW, TH) + (size_t)TH * walk_empty_row_words(TW) * sizeof(uint32_t);
 }
 __host__ __device__ inline uint32_t *walk_empty_bits(uint16_t *reach, int TW, int TH) {
-    return reinterpret_cast<uint32_t *>(reinterpret_cast<unsigned char *>(reach) +
-                                        ((4 * walk_frame_words(TW, TH) * sizeof(uint16_t) + 15) & ~(size_t)15));
+    return reinterpret_cast<uint32_t *>(reinterpret_cast<unsigned char *>(reach) + walk_boxes_bytes(TW, TH));
 }
 
 __host__ __device__ inline size_t tile_index(int x, int y, int TW) {
@@ -343,9 +343,12 @@ cudaError_t launch_edt(const MapDev &m, int n_sm, cudaStream_t s);   // interior
 // the same in two parts: the occupancy tiles and column summaries (all the ray cast needs) from a device grid (m.grid,
 // or another buffer, which is then copied there), then, from those, d2 and the interior of the field (TAM and ICP)
 cudaError_t launch_edt_tiles(const MapDev &m, const int8_t *grid, cudaStream_t s);
+cudaError_t launch_walk_reach(const MapDev &m, cudaStream_t s);   // the walk frames' empty boxes, from the tiles
 cudaError_t launch_edt_field(const MapDev &m, int n_sm, cudaStream_t s);
 cudaError_t launch_field_border(const MapDev &m, cudaStream_t s); // the constant borders of the field and walk frames (once per map)
 cudaError_t launch_map_tables(const MapDev &m, int32_t *d2, uint16_t *field, uint8_t *occ, cudaStream_t s);
+// the exported boxes of relo_map_walk_boxes_dev: the largest empty square, row run and column run of every frame tile
+cudaError_t launch_walk_boxes(const MapDev &m, uint16_t *boxes, cudaStream_t s);
 cudaError_t launch_check_cells(const int2 *cells, int n, const MapDev &m, int *bad, cudaStream_t s);
 // metre coordinates (n (x, y) FP64 pairs on the device) to cells; flags[0] off the map, flags[1] on occupied cells
 cudaError_t launch_xy_cells(const double *xy, int n, double ox, double oy, double res, const MapDev &m, int2 *cells,

@@ -198,3 +198,34 @@ def test_icp_cluster_sizes(relo, requests):
         assert abs((a.theta - b.theta + np.pi) % (2 * np.pi) - np.pi) <= 1e-9
         assert a.tam == b.tam
     ctx.close()
+
+
+@pytest.mark.parametrize("shape,kind", [((700, 700), "free"), ((333, 1017), "sparse"), ((1017, 333), "sparse"),
+                                        ((264, 2050), "corridor"), ((2050, 264), "corridor")])
+def test_walk_boxes_of_every_slope(relo, shape, kind):
+    """Rays of every slope class across boxes of up to 16 x 16 tiles, long and flat, tall and narrow, in maps whose sides
+    are not multiples of 8: ranges and hit cells as cell-by-cell stepping gives them."""
+    import torch
+    rng = np.random.default_rng(11)
+    H, W = shape
+    g = np.zeros(shape, np.int8)
+    if kind == "sparse":
+        g[rng.random(shape) < 0.0002] = 100
+    elif kind == "corridor":
+        g[::89] = 100
+        g[:, ::97] = 100
+        g[rng.integers(0, H, 400), rng.integers(0, W, 400)] = 0
+        for _ in range(40):
+            y, x = int(rng.integers(0, H - 20)), int(rng.integers(0, W - 20))
+            g[y:y + 20, x:x + 20] = 0
+    free = np.argwhere(g == 0)[:, ::-1]
+    cells = free[rng.choice(len(free), 60, replace=False)].astype(np.int32)
+    ang = workloads.beam_angles(720, 720)
+    out = []
+    for tables in (1, 0):
+        ctx = relo.Relo(n_orient=0, ray_tables=tables)
+        mid = ctx.load_map(g, RES)
+        r, h = ctx.synth_scans(mid, torch.from_numpy(cells).cuda(), ang, 60.0, 720)
+        out.append((r.cpu().numpy(), h.cpu().numpy()))
+        ctx.close()
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
