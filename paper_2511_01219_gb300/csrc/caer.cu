@@ -188,10 +188,8 @@ cudaError_t launch_caer(const ReqDesc *reqs, int R, int total_hyp, int max_ns_pa
     if (R < 1 || R > kMaxBatchRequests || max_ns_pad < 1) return cudaErrorInvalidValue;
     const int warp_words = max_ns_pad;
     const size_t smem = (size_t)kCaerWarps * warp_words * 4;   // at most 128 KB
-    cudaError_t e = cudaFuncSetAttribute(k_caer, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_caer, kCaerWarps * 32, smem);
+    const cudaError_t e = resident_ctas((const void *)k_caer, kCaerWarps * 32, smem, &occ);
     if (e != cudaSuccess) return e;
     if (occ < 1) return cudaErrorInvalidConfiguration;
     const long long need = ((long long)total_hyp + kCaerWarps - 1) / kCaerWarps;

@@ -377,7 +377,7 @@ cudaError_t launch_icp(const ReqDesc *reqs, int R, int batch_lo, int batch_hi, i
     const bool staged = table <= (size_t)kIcpTableBytes;
     const size_t smem = sizeof(double2) * (size_t)per + sizeof(int) * (size_t)((beams + 3) & ~3) + (staged ? table : 0);
     if (smem > 46 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_icp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_smem((const void *)k_icp, smem);
         if (e != cudaSuccess) return e;
     }
     cudaLaunchConfig_t cfg = {};

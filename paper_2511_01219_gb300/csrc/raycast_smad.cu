@@ -751,7 +751,7 @@ cudaError_t launch_cast(const ReqDesc *reqs, int R, int total_chunks, int cast_h
         cast_hyps == 4 ? k_cast<4> : cast_hyps == 2 ? k_cast<2> : cast_hyps == 1 ? k_cast<1> : nullptr;
     if (!kern) return cudaErrorInvalidValue;
     int occ = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kCastThreads, 0);
+    cudaError_t e = resident_ctas((const void *)kern, kCastThreads, 0, &occ);
     if (e != cudaSuccess) return e;
     if (occ < 1) return cudaErrorInvalidConfiguration;
     if (ctas_per_sm > 0 && ctas_per_sm < occ) occ = ctas_per_sm;   // a tuned launch shape
@@ -770,14 +770,11 @@ cudaError_t launch_smad(const ReqDesc *reqs, int R, int total_hyp, int max_ns_pa
     // warps per CTA: the most resident warps per SM that shared memory allows
     // (a long row's scratch fills an SM before its thread limit; smaller CTAs
     // waste less of it), the larger CTA on ties
-    cudaError_t e = cudaFuncSetAttribute(k_smad, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)std::min((size_t)8 * wb, (size_t)200 * 1024));
-    if (e != cudaSuccess) return e;
     int wpc = 0, occ = 0;
     for (int w = 8; w >= 1; --w) {
         if ((size_t)w * wb > (size_t)200 * 1024) continue;
         int o = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_smad, w * 32, (size_t)w * wb);
+        const cudaError_t e = resident_ctas((const void *)k_smad, w * 32, (size_t)w * wb, &o);
         if (e != cudaSuccess) return e;
         if (o * w > occ * wpc) {
             wpc = w;
@@ -801,10 +798,8 @@ cudaError_t launch_win_build(const ReqDesc *reqs, int R, int total, int max_ns_p
     while (nm_pad < max_nm) nm_pad <<= 1;
     const size_t smem = (size_t)nm_pad * 8 + (((size_t)(max_ns_pad + 32) * 4 + 7) & ~(size_t)7) +
                         (size_t)(max_ns_pad / 32 + 1) * 8;
-    cudaError_t e = cudaFuncSetAttribute(k_win_build, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     int occ = 0, dev = 0, n_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_win_build, 256, smem);
+    cudaError_t e = resident_ctas((const void *)k_win_build, 256, smem, &occ);
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;

@@ -106,17 +106,22 @@ constexpr int kMaxPlans = 32;
 constexpr size_t kMaxTamSegs = (size_t)kMaxBatches * (kMaxBatchRequests + 1);   // segment table of a batch slot
 constexpr size_t kBlobBytes = 30000;   // kernel-parameter upload size
 
-// Device-to-device upload through kernel parameters: the bytes travel with the
-// launch, so no host buffer has to outlive the call and nothing is pinned.
+// Upload through kernel parameters: the bytes travel with the launch, so no host buffer has to outlive the call and
+// nothing is pinned.  The first n bytes go to dst, the n2 after them (from the next 16) to dst2.
 struct Blob {
-    unsigned int n;
-    unsigned char bytes[kBlobBytes];
+    unsigned int n, n2;
+    alignas(16) unsigned char bytes[kBlobBytes];
 };
 
 // copies the blob; with bs, also zeroes the batch's work counters
-__global__ void k_upload(const __grid_constant__ Blob blob, unsigned char *dst, BatchState *bs) {
-    for (unsigned int i = blockIdx.x * blockDim.x + threadIdx.x; i < blob.n; i += gridDim.x * blockDim.x)
-        dst[i] = blob.bytes[i];
+__global__ void __launch_bounds__(256) k_upload(const __grid_constant__ Blob blob, unsigned char *dst, unsigned char *dst2,
+                                                BatchState *bs) {
+    const uint4 *v = reinterpret_cast<const uint4 *>(blob.bytes);
+    const unsigned w = (blob.n + 15u) / 16u, w2 = (blob.n2 + 15u) / 16u;   // the destinations are padded to 16 bytes
+    for (unsigned int i = blockIdx.x * blockDim.x + threadIdx.x; i < w + w2; i += gridDim.x * blockDim.x) {
+        if (i < w) reinterpret_cast<uint4 *>(dst)[i] = v[i];
+        else reinterpret_cast<uint4 *>(dst2)[i - w] = v[i];
+    }
     if (bs && blockIdx.x == 0 && threadIdx.x == 0) {
         bs->ray_work = 0u;
         bs->cast_work = 0u;
@@ -845,14 +850,23 @@ int set_hyps_impl(relo_ctx *ctx, MapSlot &m, const int2 *cells, bool on_device, 
 
 // ---- batches ------------------------------------------------------------------------------------
 
-int upload(relo_ctx *ctx, cudaStream_t st, void *dst, const void *src, size_t bytes, BatchState *bs) {
+// bytes from src to dst, and with the last of them bytes2 from src2 to dst2 if they still fit that launch (*sent2 tells).
+// dst and dst2 hold their sizes rounded up to 16.
+int upload(relo_ctx *ctx, cudaStream_t st, void *dst, const void *src, size_t bytes, BatchState *bs, void *dst2 = nullptr,
+           const void *src2 = nullptr, size_t bytes2 = 0, bool *sent2 = nullptr) {
     const unsigned char *p = static_cast<const unsigned char *>(src);
     unsigned char *d = static_cast<unsigned char *>(dst);
     while (bytes > 0) {
-        const size_t n = bytes < kBlobBytes ? bytes : kBlobBytes;
+        const size_t n = bytes < kBlobBytes ? bytes : kBlobBytes, at = (n + 15) & ~(size_t)15;
         ctx->blob->n = (unsigned int)n;
         memcpy(ctx->blob->bytes, p, n);
-        k_upload<<<(unsigned)((n + 255) / 256 < 16 ? (n + 255) / 256 : 16), 256, 0, st>>>(*ctx->blob, d, bs);
+        const bool with2 = bytes2 > 0 && n == bytes && at + bytes2 <= kBlobBytes;
+        ctx->blob->n2 = with2 ? (unsigned int)bytes2 : 0u;
+        if (with2) memcpy(ctx->blob->bytes + at, src2, bytes2);
+        if (with2 && sent2) *sent2 = true;
+        const size_t units = (at + bytes2) / 16 + 1;
+        k_upload<<<(unsigned)std::min<size_t>((units + 255) / 256, 16), 256, 0, st>>>(
+            *ctx->blob, d, static_cast<unsigned char *>(dst2), bs);
         bs = nullptr;
         CK(cudaGetLastError(), "descriptor upload");
         ctx->kernels += 1;
@@ -901,8 +915,14 @@ int prepare(relo_ctx *ctx, int32_t map_id, const float *ranges_dev, const float 
     return RELO_OK;
 }
 
-// Lays out the batch's scratch, uploads its descriptors and launches every stage once.
-int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R) {
+// Scans in host memory that the batch's requests read at sl.ranges_dev.
+struct HostScans {
+    const float *ranges;
+    size_t n;
+};
+
+// Lays out the batch's scratch, uploads its descriptors (and scans) and launches every stage once.
+int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R, HostScans scans = {nullptr, 0}) {
     if (R < 1 || R > kMaxBatchRequests) return fail(ctx, RELO_E_INVALID_ARG, "1 to 256 requests per batch");
     const relo_params &p = ctx->p;
     ++ctx->batch_seq;
@@ -1202,7 +1222,13 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R) {
     std::vector<unsigned char> blob(seg_off + sizeof(TamSeg) * segs.size(), 0);
     memcpy(blob.data(), desc.data(), sizeof(ReqDesc) * R);
     memcpy(blob.data() + seg_off, segs.data(), sizeof(TamSeg) * segs.size());
-    if ((rc = upload(ctx, st, sl.reqs_dev, blob.data(), blob.size(), sl.bs))) return rc;
+    // scans that fit beside the descriptors travel in the same launch; more take one copy (the caller's one vector)
+    bool scans_sent = false;
+    if ((rc = upload(ctx, st, sl.reqs_dev, blob.data(), blob.size(), sl.bs, sl.ranges_dev, scans.ranges,
+                     sizeof(float) * scans.n, &scans_sent)))
+        return rc;
+    if (scans.n && !scans_sent)
+        CK(cudaMemcpyAsync(sl.ranges_dev, scans.ranges, sizeof(float) * scans.n, cudaMemcpyHostToDevice, st), "scan upload");
     ReqDesc *rq = sl.reqs_dev;
     TamSeg *segs_dev = reinterpret_cast<TamSeg *>(reinterpret_cast<unsigned char *>(sl.reqs_dev) + seg_off);
     // the ray-cast launch prepares the scans first; a batch without rays to cast prepares them alone
@@ -1394,16 +1420,13 @@ void launch_batch(relo_ctx *ctx, InFlight &f, std::vector<Ticket *> &batch, std:
         memcpy(host.data() + pos, batch[i]->ranges.data(), sizeof(float) * batch[i]->ranges.size());
         pos += batch[i]->ranges.size();
     }
-    int rc = ensure(ctx, &sl.ranges_dev, &sl.ranges_cap, total, "scan upload");
-    if (rc == RELO_OK && cudaMemcpyAsync(sl.ranges_dev, host.data(), sizeof(float) * total, cudaMemcpyHostToDevice,
-                                         sl.stream) != cudaSuccess)
-        rc = RELO_E_CUDA;
+    int rc = ensure(ctx, &sl.ranges_dev, &sl.ranges_cap, (total + 3) & ~(size_t)3, "scan upload");
     if (rc == RELO_OK) {
         for (size_t i = 0; i < batch.size(); ++i) {
             pr[i].ranges_dev = sl.ranges_dev + off[i];
             pr[i].result_dev = sl.results_dev + i;
         }
-        rc = run_batch(ctx, sl, pr.data(), (int)batch.size());
+        rc = run_batch(ctx, sl, pr.data(), (int)batch.size(), HostScans{host.data(), total});
     }
     if (rc == RELO_OK && cudaEventRecord(sl.done, sl.stream) != cudaSuccess) rc = RELO_E_CUDA;
     if (rc != RELO_OK) {
@@ -1834,18 +1857,19 @@ int relo_relocalize_batch(relo_ctx *ctx, const relo_request *reqs, int32_t n, re
         total += (size_t)reqs[i].n_beams;
     }
     BatchSlot &sl = ctx->main;
-    int rc = ensure(ctx, &sl.ranges_dev, &sl.ranges_cap, total, "scan upload");
+    int rc = ensure(ctx, &sl.ranges_dev, &sl.ranges_cap, (total + 3) & ~(size_t)3, "scan upload");
     if (rc) return rc;
-    std::vector<relo_request> dreq(reqs, reqs + n);
+    std::vector<float> all;   // several scans go up together
+    if (n > 1) all.reserve(total);
+    std::vector<Prepared> pr((size_t)n);
     size_t pos = 0;
-    for (int i = 0; i < n; ++i) {
-        CK(cudaMemcpyAsync(sl.ranges_dev + pos, reqs[i].ranges, sizeof(float) * reqs[i].n_beams,
-                           cudaMemcpyHostToDevice, ctx->stream),
-           "scan upload");
-        dreq[i].ranges = sl.ranges_dev + pos;
+    for (int i = 0; i < n && !rc; ++i) {
+        rc = prepare(ctx, reqs[i].map_id, sl.ranges_dev + pos, reqs[i].angles, reqs[i].n_beams, reqs[i].max_range,
+                     sl.results_dev + i, &pr[i], reqs[i].topk);
+        if (n > 1) all.insert(all.end(), reqs[i].ranges, reqs[i].ranges + reqs[i].n_beams);
         pos += (size_t)reqs[i].n_beams;
     }
-    rc = relo_relocalize_batch_dev(ctx, dreq.data(), n, sl.results_dev);
+    if (!rc) rc = run_batch(ctx, sl, pr.data(), n, HostScans{n > 1 ? all.data() : reqs[0].ranges, total});
     if (rc) {
         cudaStreamSynchronize(ctx->stream);
         return rc;

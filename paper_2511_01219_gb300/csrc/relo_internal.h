@@ -339,6 +339,10 @@ inline int tam_chunk_cap(int K, int B, int n_batches, int chunk) {
 }
 constexpr int kMaxBatches = 64;      // ceil(K / batch) limit, bounds the TamSeg table
 
+// (fit.cu) lets a kernel use that much dynamic shared memory; and that with the CTAs of the shape an SM holds
+cudaError_t allow_smem(const void *kernel, size_t smem);
+cudaError_t resident_ctas(const void *kernel, int threads, size_t smem, int *ctas);
+
 cudaError_t launch_edt(const MapDev &m, int n_sm, cudaStream_t s);   // interior of the field, d2, bitmap
 // the same in two parts: the occupancy tiles and column summaries (all the ray cast needs) from a device grid (m.grid,
 // or another buffer, which is then copied there), then, from those, d2 and the interior of the field (TAM and ICP)

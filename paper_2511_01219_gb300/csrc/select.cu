@@ -409,7 +409,7 @@ cudaError_t launch_topk(const ReqDesc *reqs, int R, int max_n_hyp, int max_K, in
     const size_t smem_max = 227 * 1024;
     const int stage_cap = (max_n_hyp <= kStageMax && fixed + (size_t)max_n_hyp * 8 <= smem_max) ? max_n_hyp : 0;
     const size_t smem = fixed + (size_t)stage_cap * 8;
-    cudaError_t e = cudaFuncSetAttribute(k_topk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem((const void *)k_topk, smem);
     if (e != cudaSuccess) return e;
     // one CTA per SM for the offsets (the ranking CTAs' shared memory leaves room for no second one)
     const int n_off = std::max(1, std::min(R * std::max(max_n_orient, 1), n_sm));

@@ -123,10 +123,8 @@ cudaError_t launch_smad_direct(const ReqDesc *reqs, int R, int total_hyp, int ma
     const int warp_words = (max_ns_pad + 3) & ~3;   // 16-byte aligned slices
     const size_t smem = (size_t)kDirectWarps * warp_words * 4;
     if (smem > (size_t)200 * 1024) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k_smad_direct, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_smad_direct, kDirectWarps * 32, smem);
+    const cudaError_t e = resident_ctas((const void *)k_smad_direct, kDirectWarps * 32, smem, &occ);
     if (e != cudaSuccess) return e;
     if (occ < 1) return cudaErrorInvalidConfiguration;
     long long grid = (long long)n_sm * occ;

@@ -574,8 +574,7 @@ __global__ void __launch_bounds__(tam_warps(VPL, H2) * 32, kTamCtas) k_tam(const
 
 template <int VPL, bool H2>
 cudaError_t run_tam(const ReqDesc *reqs, int R, TamSeg *segs, const TamPlan &tp, BatchState *bs, cudaStream_t s) {
-    cudaError_t e = cudaFuncSetAttribute(k_tam<VPL, H2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tp.smem);
-    if (e != cudaSuccess) return e;
+    // plan_tam has asked for this shape's residency, which also lets the kernel use its shared memory
     k_tam<VPL, H2><<<tp.grid, tam_warps(VPL, H2) * 32, tp.smem, s>>>(reqs, R, segs, tp.stages, tp.lut_bytes, tp.lut_copies,
                                                                     bs);
     return cudaGetLastError();
@@ -584,12 +583,10 @@ cudaError_t run_tam(const ReqDesc *reqs, int R, TamSeg *segs, const TamPlan &tp,
 template <int VPL, bool H2>
 int tam_occupancy(size_t smem) {
     int occ = 0;
-    if (cudaFuncSetAttribute(k_tam<VPL, H2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    if (resident_ctas((const void *)k_tam<VPL, H2>, tam_warps(VPL, H2) * 32, smem, &occ) != cudaSuccess) {
         cudaGetLastError();   // more than an SM has: no CTA fits
         return 0;
     }
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_tam<VPL, H2>, tam_warps(VPL, H2) * 32, smem) != cudaSuccess)
-        return 0;
     return occ;
 }
 
