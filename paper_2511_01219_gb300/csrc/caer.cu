@@ -22,6 +22,7 @@
 
 #include <algorithm>
 
+#include "chain.cuh"
 #include "relo_internal.h"
 
 namespace relo {
@@ -83,6 +84,8 @@ __global__ void __launch_bounds__(kCaerWarps * 32) k_caer(const ReqDesc *__restr
                                                           BatchState *bs, int warp_words) {
     extern __shared__ __align__(16) uint32_t s_rows[];
     __shared__ int s_base[kMaxBatchRequests + 1];
+    chain_wait();
+    chain_go();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int r = threadIdx.x; r < R; r += blockDim.x) s_base[r] = reqs[r].hyp_base;
     if (threadIdx.x == 0) s_base[R] = total_hyp;
@@ -194,8 +197,7 @@ cudaError_t launch_caer(const ReqDesc *reqs, int R, int total_hyp, int max_ns_pa
     if (occ < 1) return cudaErrorInvalidConfiguration;
     const long long need = ((long long)total_hyp + kCaerWarps - 1) / kCaerWarps;
     const long long grid = std::max(1ll, std::min((long long)n_sm * occ, need));
-    k_caer<<<(int)grid, kCaerWarps * 32, smem, s>>>(reqs, R, total_hyp, bs, warp_words);
-    return cudaGetLastError();
+    return launch_chained(k_caer, dim3((unsigned)grid), kCaerWarps * 32, smem, s, reqs, R, total_hyp, bs, warp_words);
 }
 
 }  // namespace relo

@@ -36,6 +36,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "chain.cuh"
 #include "relo_internal.h"
 
 namespace relo {
@@ -167,6 +168,8 @@ __global__ void __launch_bounds__(kIcpThreads) k_icp(const ReqDesc *__restrict__
     __shared__ IcpPose pose;
     double2 *pts = reinterpret_cast<double2 *>(icp_smem);
     int *qv = reinterpret_cast<int *>(icp_smem + sizeof(double2) * (size_t)per);
+    chain_wait();
+    chain_go();
     uint32_t cs, cr;
     asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(cs));
     asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(cr));
@@ -381,16 +384,18 @@ cudaError_t launch_icp(const ReqDesc *reqs, int R, int batch_lo, int batch_hi, i
         if (e != cudaSuccess) return e;
     }
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = cs;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // as launch_chained
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = dim3(cs * slots, R);
     cfg.blockDim = dim3(kIcpThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, k_icp, reqs, batch_lo, batch_hi, per, beams, staged);
 }
 

@@ -36,6 +36,7 @@
 #include <algorithm>
 #include <stdint.h>
 
+#include "chain.cuh"
 #include "relo_internal.h"
 #include "scan_prep.cuh"
 
@@ -366,6 +367,8 @@ template <int G>
 __global__ void __launch_bounds__(kCastThreads, 5) k_cast(const ReqDesc *__restrict__ reqs, int R, int total_chunks,
                                                        BatchState *bs) {
     __shared__ int s_base[kMaxBatchRequests + 1];
+    chain_wait();
+    chain_go();
     const int lane = threadIdx.x & 31;
     // first the scan preparation, which the later stages need and the cast does
     // not: every CTA fills its share of the TAM scores, CTA r prepares request r
@@ -433,6 +436,8 @@ __global__ void __launch_bounds__(256) k_smad(const ReqDesc *__restrict__ reqs, 
                                               BatchState *bs, int warp_bytes) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_base[kMaxBatchRequests + 1];
+    chain_wait();
+    chain_go();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int r = threadIdx.x; r < R; r += blockDim.x) s_base[r] = reqs[r].hyp_base;
     if (threadIdx.x == 0) s_base[R] = total_hyp;
@@ -558,6 +563,8 @@ __global__ void __launch_bounds__(256) k_win_build(const ReqDesc *__restrict__ r
     __shared__ int s_base[kMaxBatchRequests + 1];
     __shared__ unsigned long long s_best[8];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    chain_wait();
+    chain_go();
     const int nwarps = blockDim.x >> 5;
     for (int r = threadIdx.x; r < R; r += blockDim.x) s_base[r] = reqs[r].wbuild_base;
     if (threadIdx.x == 0) s_base[R] = total;
@@ -683,6 +690,8 @@ __device__ __forceinline__ int lower_bound_u64(const unsigned long long *__restr
 
 __global__ void __launch_bounds__(256) k_win_read(const ReqDesc *__restrict__ reqs, int R, int total) {
     __shared__ int s_base[kMaxBatchRequests + 1];
+    chain_wait();
+    chain_go();
     for (int r = threadIdx.x; r < R; r += blockDim.x) s_base[r] = reqs[r].wread_base;
     if (threadIdx.x == 0) s_base[R] = total;
     __syncthreads();
@@ -759,8 +768,7 @@ cudaError_t launch_cast(const ReqDesc *reqs, int R, int total_chunks, int cast_h
     long long grid = (long long)n_sm * occ;
     if (grid * (kCastThreads / 32) > warps) grid = (warps + kCastThreads / 32 - 1) / (kCastThreads / 32);
     if (grid < R) grid = R;   // one CTA per request for the scan preparation
-    kern<<<(int)grid, kCastThreads, 0, s>>>(reqs, R, total_chunks, bs);
-    return cudaGetLastError();
+    return launch_chained(kern, dim3((unsigned)grid), kCastThreads, 0, s, reqs, R, total_chunks, bs);
 }
 
 cudaError_t launch_smad(const ReqDesc *reqs, int R, int total_hyp, int max_ns_pad, BatchState *bs, int n_sm,
@@ -787,8 +795,7 @@ cudaError_t launch_smad(const ReqDesc *reqs, int R, int total_hyp, int max_ns_pa
     const long long need = ((long long)total_hyp + wpc - 1) / wpc;
     if (grid > need) grid = need;
     if (grid < 1) grid = 1;
-    k_smad<<<(int)grid, wpc * 32, smem, s>>>(reqs, R, total_hyp, bs, (int)wb);
-    return cudaGetLastError();
+    return launch_chained(k_smad, dim3((unsigned)grid), wpc * 32, smem, s, reqs, R, total_hyp, bs, (int)wb);
 }
 
 cudaError_t launch_win_build(const ReqDesc *reqs, int R, int total, int max_ns_pad, int max_nm, cudaStream_t s) {
@@ -805,15 +812,13 @@ cudaError_t launch_win_build(const ReqDesc *reqs, int R, int total, int max_ns_p
     if (e != cudaSuccess) return e;
     if (occ < 1) return cudaErrorInvalidConfiguration;
     const int grid = total < n_sm * occ ? total : n_sm * occ;
-    k_win_build<<<grid, 256, smem, s>>>(reqs, R, total, nm_pad);
-    return cudaGetLastError();
+    return launch_chained(k_win_build, dim3((unsigned)grid), 256, smem, s, reqs, R, total, nm_pad);
 }
 
 cudaError_t launch_win_read(const ReqDesc *reqs, int R, int total, cudaStream_t s) {
     if (R < 1 || R > kMaxBatchRequests) return cudaErrorInvalidValue;
     if (total <= 0) return cudaSuccess;
-    k_win_read<<<(total + 255) / 256, 256, 0, s>>>(reqs, R, total);
-    return cudaGetLastError();
+    return launch_chained(k_win_read, dim3((unsigned)((total + 255) / 256)), 256, 0, s, reqs, R, total);
 }
 
 cudaError_t launch_ray_tables(const int2 *D, int ns, int lim, void *tab, cudaStream_t s) {

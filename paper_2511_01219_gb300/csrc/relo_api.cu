@@ -1278,7 +1278,11 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R, HostScans
         CK(timed_on(ctx, st, 3, 1, [&] { return launch_topk(rq, R, max_n_hyp, max_K, max_no, p.icp_iters > 0 ? max_beams : 0, ctx->n_sm, st); }),
            "SMAD top-K");
     }
-    for (int r = 0; r < R; ++r) CK(cudaStreamWaitEvent(st, pr[r].m->field_ready, 0), "map field");
+    for (int r = 0; r < R; ++r)   // a field that is ready already (the map was not just updated) needs no wait
+        if (cudaEventQuery(pr[r].m->field_ready) != cudaSuccess) {
+            (void)cudaGetLastError();
+            CK(cudaStreamWaitEvent(st, pr[r].m->field_ready, 0), "map field");
+        }
     for (int bi = 0; bi < tam_rounds; ++bi) {
         for (int c = 0; c < NC; ++c) {
             const TamPlan &tp = plans[(size_t)bi * NC + c];

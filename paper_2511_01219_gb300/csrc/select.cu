@@ -30,6 +30,7 @@
 #include <stdint.h>
 
 #include "../../include/relo.h"
+#include "chain.cuh"
 #include "icp_points.cuh"
 #include "relo_internal.h"
 #include "tam_offsets.cuh"
@@ -240,6 +241,8 @@ __device__ void topk_request(const ReqDesc &d, unsigned long long *sm, int Kp_ca
 __global__ void __launch_bounds__(kTopkThreads) k_topk(const ReqDesc *__restrict__ reqs, int Kp_cap, int stage_cap,
                                                        int R, int max_n_orient, int icp_chunks) {
     extern __shared__ __align__(16) unsigned long long sm[];
+    chain_wait();
+    chain_go();
     if ((int)blockIdx.x >= R) {
         for (int t = (int)blockIdx.x - R; t < R * max_n_orient; t += (int)gridDim.x - R) {
             const ReqDesc &o = reqs[t / max_n_orient];
@@ -311,6 +314,8 @@ __global__ void __launch_bounds__(1024) k_select_batch(const ReqDesc *__restrict
                                                        int last, int icp) {
     __shared__ unsigned long long v[kMaxBatch];
     __shared__ int s_skip;
+    chain_wait();
+    chain_go();
     const ReqDesc &d = reqs[blockIdx.x];
     const int n_batches = d.n_batches;
     const bool none_valid = d.scan->n_valid <= 0, early = d.early_stop;
@@ -366,6 +371,8 @@ __global__ void __launch_bounds__(1024) k_select_batch(const ReqDesc *__restrict
 // Sec. III: the test is made on the re-evaluated score).  With last, the
 // result.
 __global__ void __launch_bounds__(32) k_icp_best(const ReqDesc *__restrict__ reqs, int batch_lo, int batch_hi, int last) {
+    chain_wait();
+    chain_go();
     const ReqDesc &d = reqs[blockIdx.x];
     const int lane = threadIdx.x;
     SelectState *st = d.state;
@@ -413,20 +420,18 @@ cudaError_t launch_topk(const ReqDesc *reqs, int R, int max_n_hyp, int max_K, in
     if (e != cudaSuccess) return e;
     // one CTA per SM for the offsets (the ranking CTAs' shared memory leaves room for no second one)
     const int n_off = std::max(1, std::min(R * std::max(max_n_orient, 1), n_sm));
-    k_topk<<<R + n_off, kTopkThreads, smem, s>>>(reqs, Kp, stage_cap, R, std::max(max_n_orient, 1),
-                                                 (icp_beams + 31) / 32);
-    return cudaGetLastError();
+    return launch_chained(k_topk, dim3((unsigned)(R + n_off)), kTopkThreads, smem, s, reqs, Kp, stage_cap, R,
+                          std::max(max_n_orient, 1), (icp_beams + 31) / 32);
 }
 
 cudaError_t launch_select_batch(const ReqDesc *reqs, int R, int batch_lo, int batch_hi, bool last, bool icp,
                                 cudaStream_t s) {
-    k_select_batch<<<R, 1024, 0, s>>>(reqs, batch_lo, batch_hi, last ? 1 : 0, icp ? 1 : 0);
-    return cudaGetLastError();
+    return launch_chained(k_select_batch, dim3((unsigned)R), 1024, 0, s, reqs, batch_lo, batch_hi, last ? 1 : 0,
+                          icp ? 1 : 0);
 }
 
 cudaError_t launch_icp_best(const ReqDesc *reqs, int R, int batch_lo, int batch_hi, bool last, cudaStream_t s) {
-    k_icp_best<<<R, 32, 0, s>>>(reqs, batch_lo, batch_hi, last ? 1 : 0);
-    return cudaGetLastError();
+    return launch_chained(k_icp_best, dim3((unsigned)R), 32, 0, s, reqs, batch_lo, batch_hi, last ? 1 : 0);
 }
 
 }  // namespace relo

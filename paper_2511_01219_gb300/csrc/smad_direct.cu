@@ -17,6 +17,7 @@
 #include <algorithm>
 
 #include "../../include/relo.h"
+#include "chain.cuh"
 #include "relo_internal.h"
 
 namespace relo {
@@ -30,6 +31,8 @@ __global__ void __launch_bounds__(kDirectWarps * 32) k_smad_direct(const ReqDesc
                                                                    int total_hyp, BatchState *bs, int warp_words) {
     extern __shared__ __align__(16) uint32_t s_rows[];
     __shared__ int s_base[kMaxBatchRequests + 1];
+    chain_wait();
+    chain_go();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int r = threadIdx.x; r < R; r += blockDim.x) s_base[r] = reqs[r].hyp_base;
     if (threadIdx.x == 0) s_base[R] = total_hyp;
@@ -88,6 +91,8 @@ __global__ void __launch_bounds__(kDirectWarps * 32) k_smad_direct(const ReqDesc
 // they were set.  One thread per hypothesis slot of the batch.
 __global__ void __launch_bounds__(256) k_rank_by_index(const ReqDesc *__restrict__ reqs, int R, int total_hyp) {
     __shared__ int s_base[kMaxBatchRequests + 1];
+    chain_wait();
+    chain_go();
     for (int r = threadIdx.x; r < R; r += blockDim.x) s_base[r] = reqs[r].hyp_base;
     if (threadIdx.x == 0) s_base[R] = total_hyp;
     __syncthreads();
@@ -113,8 +118,7 @@ cudaError_t launch_rank_by_index(const ReqDesc *reqs, int R, int total_hyp, int 
     long long grid = ((long long)total_hyp + 255) / 256;
     if (grid > 4ll * n_sm) grid = 4ll * n_sm;
     if (grid < 1) grid = 1;
-    k_rank_by_index<<<(int)grid, 256, 0, s>>>(reqs, R, total_hyp);
-    return cudaGetLastError();
+    return launch_chained(k_rank_by_index, dim3((unsigned)grid), 256, 0, s, reqs, R, total_hyp);
 }
 
 cudaError_t launch_smad_direct(const ReqDesc *reqs, int R, int total_hyp, int max_ns_pad, BatchState *bs, int n_sm,
@@ -131,8 +135,8 @@ cudaError_t launch_smad_direct(const ReqDesc *reqs, int R, int total_hyp, int ma
     const long long need = ((long long)total_hyp + kDirectWarps - 1) / kDirectWarps;
     if (grid > need) grid = need;
     if (grid < 1) grid = 1;
-    k_smad_direct<<<(int)grid, kDirectWarps * 32, smem, s>>>(reqs, R, total_hyp, bs, warp_words);
-    return cudaGetLastError();
+    return launch_chained(k_smad_direct, dim3((unsigned)grid), kDirectWarps * 32, smem, s, reqs, R, total_hyp, bs,
+                          warp_words);
 }
 
 }  // namespace relo

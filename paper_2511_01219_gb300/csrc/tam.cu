@@ -42,6 +42,7 @@
 
 #include <algorithm>
 
+#include "chain.cuh"
 #include "relo_internal.h"
 #include "scan_prep.cuh"
 
@@ -146,6 +147,8 @@ __host__ __device__ constexpr int tam_offs_stride(int vpl) {
 // batches whose requests all read resident synthesized scans (otherwise the
 // ray-cast launch does the same work first).
 __global__ void __launch_bounds__(1024) k_scan_prep(const ReqDesc *__restrict__ reqs) {
+    chain_wait();
+    chain_go();
     const ReqDesc &d = reqs[blockIdx.x];
     scan_prep_fill(d, blockIdx.y, gridDim.y);
     if (blockIdx.y == 0) scan_prep_request(d);
@@ -469,6 +472,8 @@ __global__ void __launch_bounds__(tam_warps(VPL, H2) * 32, kTamCtas) k_tam(const
     auto lut_of = [&](int i) { return reinterpret_cast<float2 *>(smem + (lut_copies > 1 ? i * lut_bytes : 0)); };
     int *const offs0 = reinterpret_cast<int *>(smem + lut_copies * lut_bytes);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    chain_wait();
+    chain_go();
     unsigned int *counter = reinterpret_cast<unsigned int *>(&segs[R].batch_lo);   // tasks taken after the first ones
     // each request's tasks: its chunks in the launch's batches x its orientation blocks (counted on the device); none
     // once it has terminated early or when it has no valid beam
@@ -575,9 +580,8 @@ __global__ void __launch_bounds__(tam_warps(VPL, H2) * 32, kTamCtas) k_tam(const
 template <int VPL, bool H2>
 cudaError_t run_tam(const ReqDesc *reqs, int R, TamSeg *segs, const TamPlan &tp, BatchState *bs, cudaStream_t s) {
     // plan_tam has asked for this shape's residency, which also lets the kernel use its shared memory
-    k_tam<VPL, H2><<<tp.grid, tam_warps(VPL, H2) * 32, tp.smem, s>>>(reqs, R, segs, tp.stages, tp.lut_bytes, tp.lut_copies,
-                                                                    bs);
-    return cudaGetLastError();
+    return launch_chained(k_tam<VPL, H2>, dim3((unsigned)tp.grid), tam_warps(VPL, H2) * 32, tp.smem, s, reqs, R, segs,
+                          tp.stages, tp.lut_bytes, tp.lut_copies, bs);
 }
 
 template <int VPL, bool H2>
@@ -616,8 +620,7 @@ int occupancy_for(int vpl, bool h2, size_t smem) {
 int tam_vpl_for(int max_beams) { return vpl_bucket(max_beams); }
 
 cudaError_t launch_scan_prep(const ReqDesc *reqs, int R, cudaStream_t s) {
-    k_scan_prep<<<dim3(R, 8), 1024, 0, s>>>(reqs);
-    return cudaGetLastError();
+    return launch_chained(k_scan_prep, dim3((unsigned)R, 8), 1024, 0, s, reqs);
 }
 
 // The launch for the batches [batch_lo[r], batch_hi[r]) of every request:
