@@ -367,7 +367,8 @@ cudaError_t launch_scan_prep(const ReqDesc *reqs, int R, cudaStream_t s);
 // casts the total_chunks 32-ray chunks of the batch into the requests' scan tables
 cudaError_t launch_cast(const ReqDesc *reqs, int R, int total_chunks, int cast_hyps, BatchState *bs, int n_sm, int ctas_per_sm,
                         cudaStream_t s);
-// SMAD of every hypothesis of the batch from the requests' scan tables
+// SMAD of every hypothesis of the batch from the requests' scan tables; max_ns_pad: the longest padded row of the
+// requests with more than one orientation, 0 when there is none
 cudaError_t launch_smad(const ReqDesc *reqs, int R, int total_hyp, int max_ns_pad, BatchState *bs, int n_sm,
                         cudaStream_t s);
 // CAER of every hypothesis of the batch (caer.cu)

@@ -229,3 +229,29 @@ def test_walk_boxes_of_every_slope(relo, shape, kind):
         out.append((r.cpu().numpy(), h.cpu().numpy()))
         ctx.close()
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("n_beams,ns,n_orient", [
+    (20, 32, 8), (70, 128, 16), (71, 132, 33), (100, 160, 40), (500, 768, 96), (520, 772, 193), (90, 130, 65), (61, 97, 97),
+])
+def test_smad_row_blocks(relo, n_beams, ns, n_orient):
+    """SMAD rows of less than a block, whole blocks and remainders, rows that are not 16-byte aligned, and gapped scans:
+    numerators, shifts and survivors equal the oracle's."""
+    wl = small_case(n_beams=n_beams, ns=ns, n_orient=n_orient)
+    full_case(relo, wl, 12, batch=5, local_topk=2)[0].close()
+    keep = np.ones(n_beams, bool)
+    keep[n_beams // 2:n_beams // 2 + 5] = False
+    wl.ranges, wl.angles = wl.ranges[keep].copy(), wl.angles[keep]
+    full_case(relo, wl, 12, batch=5, local_topk=2)[0].close()
+
+
+@pytest.mark.parametrize("ns,gap", [(64, 3), (130, 0), (131, 7), (720, 30), (721, 0)])
+def test_smad_single_orientation_rows(relo, ns, gap):
+    """Scans of 0.9 of the circle and more (m = 0 only): the row sums over aligned and unaligned intervals that may wrap."""
+    wl = small_case(n_beams=ns, ns=ns, n_orient=1 if ns in (131, 721) else 2)
+    for first in (0, ns // 3):   # the gap inside the scan, or the scan starting after it
+        keep = np.ones(ns, bool)
+        keep[first:first + gap] = False
+        z, a = wl.ranges.copy(), wl.angles
+        w = workloads.Workload("row", wl.grid, wl.res, wl.hyps, z[keep], a[keep], wl.max_range, wl.n_orient, 8, ns, (0, 0, 0))
+        full_case(relo, w, 12, batch=5, local_topk=2)[0].close()
