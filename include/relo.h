@@ -358,8 +358,8 @@ int relo_rrt_hypotheses_dev(relo_ctx *ctx, const float *clearance_dev, int32_t w
  *   RELO_TUNE_TAM   key = {values-per-lane class of the request's TAM kernel
  *                   (relo_tam_class), n_orient, K}; val = {survivors per TAM
  *                   task (a multiple of 8 in [8, 128]; 0 keeps the built-in
- *                   choice), resident CTAs per SM of the TAM launch (0: all
- *                   that fit; a launch takes the smallest of its requests')}.
+ *                   choice), CTAs per SM of the TAM launch (accepted, and
+ *                   without effect: the launch runs one CTA per SM)}.
  *   RELO_TUNE_TAM_ONE  as RELO_TUNE_TAM, for a launch that serves a single
  *                   request (its TAM tasks alone fill the GPU, so the best
  *                   shape differs from a mixed batch's); such a launch falls

@@ -1,12 +1,12 @@
 """Autotuner of the batched stages' launch shapes (relo_set_tuning).
 
 The library picks the launch shapes of its stage kernels by rule: TAM takes
-survivors in tasks of one band phase (a chunk of up to 64), the ray cast and
-TAM fill every resident CTA slot.  Which shape is fastest depends on the
+survivors in tasks of one band phase (a chunk of up to 64), the ray cast
+fills every resident CTA slot.  Which shape is fastest depends on the
 request shapes (beam count, orientations, K) and on the GPU, so this module
 measures: for the ray cast it tries CTAs per SM, and for every TAM shape
 bucket (values-per-lane class, n_orient, K) present in a workload it tries
-chunk sizes and CTAs per SM, one bucket at a time (the others at their best
+chunk sizes, one bucket at a time (the others at their best
 so far), timing the stage with the library's own CUDA events over a few
 repetitions of the workload.  Shapes never change results, only time.
 
@@ -28,7 +28,6 @@ from . import TUNE_CAST, TUNE_TAM, TUNE_TAM_ONE, tam_class
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CHUNKS = (8, 16, 24, 32, 48, 64)
-TAM_CTAS = (0, 4, 3)          # resident CTAs per SM (0: all that fit)
 CAST_CTAS = (0, 5, 4, 3)
 
 
@@ -103,16 +102,15 @@ def tune(ctx, run, shapes, reps: int = 3, log=None, single: bool = False) -> dic
     best_tam_ms = base_tam
     for b in buckets(shapes):
         for chunk in CHUNKS:
-            for cps in TAM_CTAS:
-                cand = dict(chosen)
-                cand[b] = (chunk, cps)
-                e = [(tam_kind, k, v) for k, v in cand.items()]
-                ctx.set_tuning(e)
-                ms = stage_ms(ctx, run, "tam", reps)
-                trials.append({"entries": e, "tam_ms": ms})
-                if ms < best_tam_ms:
-                    best_tam_ms = ms
-                    chosen = cand
+            cand = dict(chosen)
+            cand[b] = (chunk, 0)   # the TAM launch runs one CTA per SM
+            e = [(tam_kind, k, v) for k, v in cand.items()]
+            ctx.set_tuning(e)
+            ms = stage_ms(ctx, run, "tam", reps)
+            trials.append({"entries": e, "tam_ms": ms})
+            if ms < best_tam_ms:
+                best_tam_ms = ms
+                chosen = cand
         if log:
             log(f"bucket {b}: {chosen.get(b)} tam {best_tam_ms:.4f} ms ({time.time() - t0:.0f} s)")
     entries = [(tam_kind, k, v) for k, v in chosen.items()] + ([best_cast] if best_cast else [])

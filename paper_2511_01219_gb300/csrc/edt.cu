@@ -47,13 +47,13 @@ __global__ void __launch_bounds__(256) k_edt_tiles(const int8_t *__restrict__ gr
 EdtTiles tiles_of(const MapDev &m) { return EdtTiles{m.bits, m.summ, edt_span_of(m), m.far,
                                                     m.reach ? walk_empty_bits(m.reach, m.TW, m.TH) : nullptr, m.W, m.H, m.TW, m.TH}; }
 
-// the border of the padded field: every cell outside the map reads C (d = d_max)
-__global__ void k_field_border(uint16_t *__restrict__ fieldp, int W, int H, int P, int Wp, int Hp, int C) {
+// the border of the padded field: every cell outside the map reads the code of C (d = d_max), the last rank
+__global__ void k_field_border(uint16_t *__restrict__ fieldp, int W, int H, int P, int Wp, int Hp, uint32_t code) {
     const size_t n = (size_t)Hp * Wp;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const size_t c = i >> 3;   // column of a band, then the row inside the band (field_index)
         const int y = (int)(c / Wp) * 8 + (int)(i & 7) - P, x = (int)(c % Wp) - P;
-        if (x < 0 || y < 0 || x >= W || y >= H) fieldp[i] = (uint16_t)C;
+        if (x < 0 || y < 0 || x >= W || y >= H) fieldp[i] = (uint16_t)code;
     }
 }
 
@@ -164,7 +164,12 @@ template <int kCols>
 __global__ void __launch_bounds__(128) k_map_tables(const int32_t *__restrict__ d2s, const uint16_t *__restrict__ fs,
                                                     const uint64_t *__restrict__ bs, int W, int H, int TW, int P, int Wp,
                                                     int32_t *__restrict__ d2, uint16_t *__restrict__ field,
-                                                    uint8_t *__restrict__ occ) {
+                                                    uint8_t *__restrict__ occ, const uint16_t *__restrict__ value,
+                                                    int n_rank) {
+    extern __shared__ uint16_t s_value[];   // the value of every rank
+    if (field)
+        for (int i = threadIdx.x; i < n_rank; i += 128) s_value[i] = __ldg(value + i);
+    __syncthreads();
     const int B = (P >> 3) + (int)blockIdx.y, y0 = 8 * B - P, x0 = kCols * ((int)blockIdx.x * 128 + (int)threadIdx.x);
     if (x0 >= W) return;   // kCols divides W
     uint4 f[kCols] = {};
@@ -180,7 +185,7 @@ __global__ void __launch_bounds__(128) k_map_tables(const int32_t *__restrict__ 
 #pragma unroll
         for (int i = 0; i < kCols; ++i) {
             const uint32_t w = u < 2 ? f[i].x : u < 4 ? f[i].y : u < 6 ? f[i].z : f[i].w;
-            h[i] = w >> (16 * (u & 1)) & 0xffffu;
+            h[i] = field ? s_value[(w >> (16 * (u & 1)) & 0xffffu) - kFieldBias] : 0u;
         }
         uint32_t o = 0u;   // the cells' occupancy bits (of one tile row)
         if (occ) o = (uint32_t)(bs[(size_t)(y >> 3) * TW + (x0 >> 3)] >> (((y & 7) << 3) | (x0 & 7)));
@@ -264,7 +269,7 @@ cudaError_t launch_walk_reach(const MapDev &m, cudaStream_t s) {
 }
 
 cudaError_t launch_edt_field(const MapDev &m, int n_sm, cudaStream_t s) {
-    return launch_edt_bands(tiles_of(m), EdtOut{m.d2, m.field, m.C, m.P, m.Wp}, n_sm, s);
+    return launch_edt_bands(tiles_of(m), EdtOut{m.d2, m.field, m.code, m.C, m.P, m.Wp}, n_sm, s);
 }
 
 cudaError_t launch_edt(const MapDev &m, int n_sm, cudaStream_t s) {
@@ -279,7 +284,7 @@ cudaError_t launch_walk_boxes(const MapDev &m, uint16_t *boxes, cudaStream_t s) 
 }
 
 cudaError_t launch_field_border(const MapDev &m, cudaStream_t s) {
-    k_field_border<<<1024, 256, 0, s>>>(m.field, m.W, m.H, m.P, m.Wp, m.Hp, m.C);
+    k_field_border<<<1024, 256, 0, s>>>(m.field, m.W, m.H, m.P, m.Wp, m.Hp, kFieldBias + (uint32_t)m.n_rank - 1u);
     k_walk_border<<<4, 256, 0, s>>>(m.bits + (size_t)m.TW * m.TH, m.TW, m.TH);
     return cudaGetLastError();
 }
@@ -288,12 +293,13 @@ cudaError_t launch_map_tables(const MapDev &m, int32_t *d2, uint16_t *field, uin
     const bool vec = (m.W & 3) == 0 && (reinterpret_cast<uintptr_t>(d2) & 15) == 0 &&
                      (reinterpret_cast<uintptr_t>(field) & 7) == 0 && (reinterpret_cast<uintptr_t>(occ) & 3) == 0;
     const int bands = edt_bands(m.H, m.P);
+    const size_t smem = field ? (size_t)m.n_rank * sizeof(uint16_t) : 0;
     if (vec)
-        k_map_tables<4><<<dim3((m.W + 511) / 512, bands), 128, 0, s>>>(m.d2, m.field, m.bits, m.W, m.H, m.TW, m.P, m.Wp,
-                                                                       d2, field, occ);
+        k_map_tables<4><<<dim3((m.W + 511) / 512, bands), 128, smem, s>>>(m.d2, m.field, m.bits, m.W, m.H, m.TW, m.P, m.Wp,
+                                                                          d2, field, occ, m.value, m.n_rank);
     else
-        k_map_tables<1><<<dim3((m.W + 127) / 128, bands), 128, 0, s>>>(m.d2, m.field, m.bits, m.W, m.H, m.TW, m.P, m.Wp,
-                                                                       d2, field, occ);
+        k_map_tables<1><<<dim3((m.W + 127) / 128, bands), 128, smem, s>>>(m.d2, m.field, m.bits, m.W, m.H, m.TW, m.P, m.Wp,
+                                                                          d2, field, occ, m.value, m.n_rank);
     return cudaGetLastError();
 }
 

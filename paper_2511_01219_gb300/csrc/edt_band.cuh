@@ -199,11 +199,12 @@ __device__ __forceinline__ void column_distances(const EdtTiles &t, int x, int y
     }
 }
 
-// Where the results go: d2 row-major [H][W] (-1 when the map has no occupied cell), and, if field is not null,
-// min(d2, C) in 8-row bands with a border of P cells (relo_internal.h, field_index).
+// Where the results go: d2 row-major [H][W] (-1 when the map has no occupied cell), and, if field is not null, the code
+// of min(d2, C), code[0 .. C], in 8-row bands with a border of P cells (relo_internal.h, field_index).
 struct EdtOut {
     int32_t *d2;
     uint16_t *field;
+    const uint16_t *code;
     int C, P, Wp;
 };
 
@@ -220,6 +221,9 @@ template <int kCols, int kSplit>
 __global__ void __launch_bounds__(kCols / 4 * kSplit) k_edt_band(EdtTiles t, EdtOut o) {
     constexpr int kRow = kCols + 2 * kHalo, kGroups = kCols / 4, T = kGroups * kSplit, kPairs = 4 / kSplit;
     __shared__ __align__(16) uint32_t sq[4][kRow];
+    extern __shared__ uint16_t s_code[];   // [C + 1], with a field
+    if (o.field)
+        for (int i = threadIdx.x; i <= o.C; i += T) s_code[i] = __ldg(o.code + i);
     const int B = (o.P >> 3) + (int)blockIdx.y, y0 = 8 * B - o.P, X0 = (int)blockIdx.x * kCols;
 #pragma unroll 2
     for (int i = threadIdx.x; i < kRow; i += T) {
@@ -305,8 +309,8 @@ __global__ void __launch_bounds__(kCols / 4 * kSplit) k_edt_band(EdtTiles t, Edt
     }
     if (far) t.far[blockIdx.y] = 1;   // every writer writes 1
     if (!o.field) return;
-    // min(d2, C), C for the rows off the map (the border's value); what is left to k_edt_far is above kNear2
-    const uint32_t C = (uint32_t)min(o.C, 0xffff), C2 = C | C << 16;
+    // the code of min(d2, C), C's for the rows off the map (the border's value); what is left to k_edt_far is above kNear2
+    const uint32_t C = (uint32_t)o.C, C2 = C | C << 16;
     uint32_t off[kPairs];   // halves to replace by C
 #pragma unroll
     for (int p = 0; p < kPairs; ++p) {
@@ -318,7 +322,10 @@ __global__ void __launch_bounds__(kCols / 4 * kSplit) k_edt_band(EdtTiles t, Edt
         if (x0 + i >= t.W) continue;
         uint32_t f[kPairs];
 #pragma unroll
-        for (int p = 0; p < kPairs; ++p) f[p] = (__vminu2(best[p][i], C2) & ~off[p]) | (C2 & off[p]);
+        for (int p = 0; p < kPairs; ++p) {
+            const uint32_t b = (__vminu2(best[p][i], C2) & ~off[p]) | (C2 & off[p]);
+            f[p] = (uint32_t)s_code[b & 0xffffu] | (uint32_t)s_code[b >> 16] << 16;
+        }
         uint16_t *to = o.field + 8 * ((size_t)B * o.Wp + (x0 + i + o.P)) + 2 * p0;
         if constexpr (kPairs == 4) *reinterpret_cast<uint4 *>(to) = make_uint4(f[0], f[1], f[2], f[3]);
         else *reinterpret_cast<uint2 *>(to) = make_uint2(f[0], f[1]);
@@ -399,7 +406,7 @@ __global__ void __launch_bounds__(kFarThreads) k_edt_far(EdtTiles t, EdtOut o, i
                             *out = best[i] >= kFarNone * kFarNone ? -1 : best[i];
                             if (o.field)
                                 o.field[8 * ((size_t)B * o.Wp + (lx + i + o.P)) + u0 + lu] =
-                                    (uint16_t)(best[i] > o.C ? o.C : best[i]);
+                                    __ldg(o.code + (best[i] > o.C ? o.C : best[i]));
                         }
                     }
                     __syncthreads();
@@ -419,12 +426,13 @@ inline cudaError_t launch_edt_bands(const EdtTiles &t, const EdtOut &o, int n_sm
     const int bands = edt_bands(t.H, o.P);
     k_edt_spans<<<dim3((t.W + 127) / 128, edt_summary_rows(t.H)), 128, 0, s>>>(t);
     auto strips = [&](int cols) { return (t.W + cols - 1) / cols; };
+    const size_t code = o.field ? ((size_t)o.C + 1) * sizeof(uint16_t) : 0;   // at most 16 KB
     if ((long long)strips(1024) * bands >= 4ll * n_sm)
-        k_edt_band<1024, 1><<<dim3(strips(1024), bands), 256, 0, s>>>(t, o);
+        k_edt_band<1024, 1><<<dim3(strips(1024), bands), 256, code, s>>>(t, o);
     else if ((long long)strips(512) * bands >= 2ll * n_sm)
-        k_edt_band<512, 2><<<dim3(strips(512), bands), 256, 0, s>>>(t, o);
+        k_edt_band<512, 2><<<dim3(strips(512), bands), 256, code, s>>>(t, o);
     else
-        k_edt_band<256, 2><<<dim3(strips(256), bands), 128, 0, s>>>(t, o);
+        k_edt_band<256, 2><<<dim3(strips(256), bands), 128, code, s>>>(t, o);
     const size_t smem = (size_t)far_rows(t.W) * far_width(t.W) * sizeof(uint16_t);
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(k_edt_far, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -98,6 +98,6 @@ extern "C" int relo_edt_noalloc(const int8_t *grid_dev, int32_t w, int32_t h, in
     const bool vec = (w & 7) == 0 && (reinterpret_cast<uintptr_t>(grid_dev) & 7) == 0;
     k_na_tiles<<<dim3((t.TW + 31) / 32, edt_summary_rows(h)), dim3(32, 8), 0, s>>>(grid_dev, t, vec);
     if (cudaGetLastError() != cudaSuccess) return RELO_E_CUDA;
-    if (launch_edt_bands(t, EdtOut{d2_dev, nullptr, 0, 0, 0}, n_sm, s) != cudaSuccess) return RELO_E_CUDA;
+    if (launch_edt_bands(t, EdtOut{d2_dev, nullptr, nullptr, 0, 0, 0}, n_sm, s) != cudaSuccess) return RELO_E_CUDA;
     return RELO_OK;
 }

@@ -79,7 +79,7 @@ struct MapSlot {
     double res = 0, ox = 0, oy = 0;
     int2 *hyps = nullptr;
     int n_hyp = 0, hyp_cap = 0;
-    float2 *lut = nullptr;
+    float2 *lut = nullptr;       // [kMaxClamp + 2] by value, [kMaxClamp + 2] by rank, then the field codes and their values
     double lut_key[6] = {0};     // what its values depend on: z_hit, sigma_hit, z_rand, eps, resolution, clamp
     int32_t *sq_off = nullptr;   // [kMaxClamp + 2] and [kMaxLatticePoints]: the cells at each squared distance
     short2 *sq_rep = nullptr;
@@ -330,26 +330,49 @@ int clamp_for(relo_ctx *ctx, double d_max, double res, int *C) {
     return RELO_OK;
 }
 
-// likelihood table of Eq. 23 and sqrt(C) - sqrt(b), for b in [0, C]
-int build_lut(relo_ctx *ctx, MapSlot &m) {
+constexpr size_t kMapTableBytes = (2 * sizeof(float2) + 2 * sizeof(uint16_t)) * (kMaxClamp + 2);
+
+// The map's tables for its clamp C, in one allocation and one upload: the likelihood table of Eq. 23 and
+// sqrt(C) - sqrt(b), by value and by rank, and the field codes (relo_internal.h) of the values a clamped squared distance
+// can take (sums of two squares, and C) with their inverse.  Before the EDT, which writes the codes.  No entry is made
+// for a value that no cell can have.
+int build_tables(relo_ctx *ctx, MapSlot &m) {
     const relo_params &p = ctx->p;
     const int C = m.dev.C;
-    std::vector<float2> h(C + 2);
+    std::vector<char> can((size_t)C + 1, 0);
+    for (int y = 0; y * y <= C; ++y)
+        for (int x = 0; x <= y && y * y + x * x <= C; ++x) can[y * y + x * x] = 1;
+    can[C] = 1;
+    std::vector<char> h(kMapTableBytes, 0);
+    float2 *lut = reinterpret_cast<float2 *>(h.data()), *lut_rank = lut + (kMaxClamp + 2);
+    uint16_t *code = reinterpret_cast<uint16_t *>(lut_rank + (kMaxClamp + 2)), *value = code + (kMaxClamp + 2);
     const double sc = sqrt((double)C);
+    int n = 0;
     for (int b = 0; b <= C; ++b) {
-        double d = m.res * sqrt((double)b);
-        double l = log(p.z_hit * exp(-(d * d) / (2.0 * p.sigma_hit * p.sigma_hit)) + p.z_rand + p.eps);
-        h[b] = make_float2((float)l, (float)(sc - sqrt((double)b)));
-    }
-    h[C + 1] = make_float2(0.0f, 0.0f);   // "no beam": contributes nothing
+        if (!can[b]) continue;
+        const double d = m.res * sqrt((double)b);
+        const double l = log(p.z_hit * exp(-(d * d) / (2.0 * p.sigma_hit * p.sigma_hit)) + p.z_rand + p.eps);
+        lut[b] = lut_rank[n] = make_float2((float)l, (float)(sc - sqrt((double)b)));
+        value[n] = (uint16_t)b;
+        code[b] = (uint16_t)(kFieldBias + (uint32_t)n++);
+    }   // lut[C + 1] and lut_rank[n] stay (0, 0): "no beam", contributes nothing
     const double key[6] = {p.z_hit, p.sigma_hit, p.z_rand, p.eps, m.res, (double)C};
     memcpy(m.lut_key, key, sizeof key);
     if (!m.lut) {
-        int rc = dev_alloc(ctx, (void **)&m.lut, sizeof(float2) * (kMaxClamp + 2), "likelihood table");
+        int rc = dev_alloc(ctx, (void **)&m.lut, kMapTableBytes, "likelihood table");
         if (rc) return rc;
-        m.bytes += sizeof(float2) * (kMaxClamp + 2);
+        m.bytes += kMapTableBytes;
     }
-    CK(cudaMemcpyAsync(m.lut, h.data(), sizeof(float2) * (C + 2), cudaMemcpyHostToDevice, ctx->stream), "lut upload");
+    m.dev.code = reinterpret_cast<uint16_t *>(m.lut + 2 * (kMaxClamp + 2));
+    m.dev.value = m.dev.code + (kMaxClamp + 2);
+    m.dev.n_rank = n;
+    CK(cudaMemcpyAsync(m.lut, h.data(), kMapTableBytes, cudaMemcpyHostToDevice, ctx->stream), "lut upload");
+    return RELO_OK;
+}
+
+// ICP's pairing table for the map's clamp (no kernel of the map's precompute reads it)
+int build_pairing(relo_ctx *ctx, MapSlot &m) {
+    const int C = m.dev.C;
     // every (dy, dx) with dy^2 + dx^2 = n <= C, grouped by n and ordered by dy, then dx: the candidates ICP
     // tries, nearest first, when it pairs a beam with an occupied cell
     std::vector<int32_t> off(C + 2, 0);
@@ -721,7 +744,7 @@ void free_map(relo_ctx *ctx, MapSlot &m) {
     dev_free(ctx, m.dev.bits, sizeof(uint64_t) * occupancy_words(m.dev.TW, m.dev.TH) +
                                   walk_reach_bytes(m.dev.TW, m.dev.TH));   // reach lies behind bits
     dev_free(ctx, m.hyps, sizeof(int2) * (size_t)m.hyp_cap);
-    dev_free(ctx, m.lut, sizeof(float2) * (kMaxClamp + 2));
+    dev_free(ctx, m.lut, kMapTableBytes);
     dev_free(ctx, m.sq_off, sizeof(int32_t) * (kMaxClamp + 2));
     dev_free(ctx, m.sq_rep, sizeof(short2) * kMaxLatticePoints);
     m = MapSlot();
@@ -771,6 +794,10 @@ int load_map_impl(relo_ctx *ctx, const int8_t *grid, bool on_device, int32_t w, 
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(m.dev.grid, grid, cells, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                             ctx->stream);
+    if (e == cudaSuccess && (rc = build_tables(ctx, m))) {
+        free_map(ctx, m);
+        return rc;
+    }
     if (e == cudaSuccess) e = launch_field_border(m.dev, ctx->stream);
     if (e == cudaSuccess) ctx->kernels += 2;
     if (e == cudaSuccess) e = map_edt(ctx, m, m.dev.grid);
@@ -779,7 +806,7 @@ int load_map_impl(relo_ctx *ctx, const int8_t *grid, bool on_device, int32_t w, 
         free_map(ctx, m);
         return cuda_fail(ctx, e, "map precompute");
     }
-    rc = build_lut(ctx, m);
+    rc = build_pairing(ctx, m);
     if (rc) {
         free_map(ctx, m);
         return rc;
@@ -1083,6 +1110,8 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R, HostScans
         d.Wp = m.dev.Wp;
         d.P = m.dev.P;
         d.lut = m.lut;
+        d.lut_rank = m.lut + (kMaxClamp + 2);
+        d.n_rank = m.dev.n_rank;
         d.W = m.dev.W;
         d.H = m.dev.H;
         d.TW = m.dev.TW;
@@ -1192,7 +1221,8 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R, HostScans
     std::vector<int> blo((size_t)R), bhi((size_t)R);
     for (int bi = 0; bi < tam_rounds; ++bi) {
         for (int c = 0; c < NC; ++c) {
-            int beams_c = 1, C_c = 0, chunk_c = 0, luts = 0;   // luts: 1 when the class's likelihood tables are the same
+            int beams_c = 1, rank_c = 0, chunk_c = 0, luts = 0;   // luts: 1 when the class's likelihood tables are the same
+            long long poses_c = 0;
             const MapSlot *m_c = nullptr;
             for (int r = 0; r < R; ++r) {
                 const bool in = vcls[r] == classes[c] && bi < desc[r].n_batches;
@@ -1202,18 +1232,13 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R, HostScans
                     beams_c = std::max(beams_c, pr[r].P->n);
                     if (!m_c || memcmp(m_c->lut_key, pr[r].m->lut_key, sizeof m_c->lut_key)) ++luts;
                     m_c = pr[r].m;
-                    C_c = std::max(C_c, pr[r].m->dev.C);
+                    rank_c = std::max(rank_c, pr[r].m->dev.n_rank);
                     chunk_c = chunk_c ? std::min(chunk_c, desc[r].tam_chunk) : desc[r].tam_chunk;
+                    poses_c += (long long)(any_early ? desc[r].B : desc[r].K) * desc[r].n_orient;
                 }
             }
-            int cps = 0;   // resident CTAs per SM: the smallest the class's requests are tuned to
-            for (int r = 0; r < R; ++r) {
-                if (vcls[r] != classes[c]) continue;
-                const relo_tune_entry *e = tuned_tam(ctx, R, vcls[r], desc[r].n_orient, desc[r].K);
-                if (e && e->val[1] > 0) cps = cps > 0 ? std::min(cps, e->val[1]) : e->val[1];
-            }
             TamPlan &tp = plans[(size_t)bi * NC + c];
-            tp = plan_tam(blo.data(), bhi.data(), R, beams_c, C_c, ctx->n_sm, cps, chunk_c, luts,
+            tp = plan_tam(blo.data(), bhi.data(), R, beams_c, rank_c, ctx->n_sm, chunk_c, luts, poses_c,
                           &segs[((size_t)bi * NC + c) * seg_n]);
             if (tp.vpl < 0) return fail(ctx, RELO_E_INVALID_ARG, "no TAM kernel fits this beam count");
         }
@@ -1719,10 +1744,11 @@ int relo_set_params(relo_ctx *ctx, const relo_params *p) {
             if ((rc = clamp_for(ctx, p->d_max, m.res, &C))) return rc;
             m.dev.C = C;
             CK(cudaStreamWaitEvent(ctx->stream, m.field_ready, 0), "map rebuild");
+            if ((rc = build_tables(ctx, m))) return rc;
             CK(launch_field_border(m.dev, ctx->stream), "map rebuild");
             CK(map_edt(ctx, m, m.dev.grid), "map rebuild");
             CK(cudaStreamWaitEvent(ctx->stream, m.field_ready, 0), "map rebuild");
-            if ((rc = build_lut(ctx, m))) return rc;
+            if ((rc = build_pairing(ctx, m))) return rc;
         }
         CK(cudaStreamSynchronize(ctx->stream), "map rebuild");
     }

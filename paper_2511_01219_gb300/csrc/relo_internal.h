@@ -41,7 +41,10 @@ struct MapDev {
     int W = 0, H = 0, TW = 0, TH = 0;
     int C = 0;                  // clamp (d_max / res)^2 used by the TAM field
     int32_t *d2 = nullptr;      // [H*W] exact squared EDT, -1 = no obstacle
-    uint16_t *field = nullptr;  // [Hp * Wp] min(d2, C) with a border of P cells holding C, in 8-row bands
+    uint16_t *field = nullptr;  // [Hp * Wp] codes of min(d2, C) with a border of P cells holding C's, in 8-row bands
+    uint16_t *code = nullptr;   // [C + 1] the code of every value (field_code); that of a value no cell can have is unused
+    uint16_t *value = nullptr;  // [n_rank] the value of every rank
+    int n_rank = 0;             // values that a clamped squared distance can take
     int P = 0, Wp = 0, Hp = 0;  // border width; padded width and height (W + 2P, H + 2P rounded up to 8)
     uint64_t *bits = nullptr;   // occupancy, bit (y&7)*8 + (x&7): [TH*TW] the map (cells outside free), then the
                                 // four walk frames (walk_frame_words each: native, mirrored in x, y and both)
@@ -51,6 +54,11 @@ struct MapDev {
     int *far = nullptr;         // [TH + 1] bands the EDT's 32-bit pass has work in, after summ (scratch)
     int8_t *grid = nullptr;     // [H*W] device copy of the grid
 };
+
+// The field's code of a clamped squared distance is its rank among the sums of two squares up to C (and C itself), plus
+// kFieldBias: a positive finite fp16 bit pattern of a number >= 1024, consecutive codes at least 1 apart (TAM counts codes
+// as fp16 numbers).  There are at most 2258 ranks (C = 8100), so no pattern reaches infinity (0x7c00).
+constexpr uint32_t kFieldBias = 0x6400u;
 
 // The clamped field is stored in bands of 8 rows, each band column by
 // column: cell (x, y) of the padded grid (the map cell (x - P, y - P)) sits at
@@ -223,7 +231,9 @@ struct ReqDesc {
     double *icp_pts;             // [n_beams][2] the valid beams' sensor-frame points (with ICP only)
     double *ref_pose;            // [K][3] refined pose (x, y, theta) of each refined survivor (map metres)
     float *reev;                 // [K] its re-evaluated score
-    const float2 *lut;           // [C+2] (l(b), sqrt(C) - sqrt(b)); entry C+1 = (0, 0) marks "no beam"
+    const float2 *lut;           // [C+2] (l(b), sqrt(C) - sqrt(b)) by value (ICP's score)
+    const float2 *lut_rank;      // [n_rank + 1] the same by rank (TAM); the last entry = (0, 0) marks "no beam"
+    int n_rank;
     int W, H, TW, TH, C, Wp, P;
     float res, res2, d_max, d_min;
     double resd, ox, oy;
@@ -317,15 +327,15 @@ struct TamSeg {
 };
 
 constexpr int kMaxBatchRequests = 256;
-// Survivors of one band phase per TAM task: the most (16 to 64) that still give every CTA (two per SM) about four tasks
-// (blocks of 4 orientations) of a batch of R such requests, so that the tasks spread evenly.  Measured with 8 / 16 / 32 /
-// 64 per task (TAM, us): 256 survivors x 360 orientations 125 / 120 / 127 / 121, 1024 x 720 1138 / 1088 / 1065 / 1062,
-// 16 requests of 256 and 512 2364 / 2191 / 2174 / 2166.
+// Survivors of one band phase per TAM task: the most (32 to 64) that still give every SM about eight tasks (blocks of 4
+// orientations) of a batch of R such requests, so that the tasks spread evenly.  Measured with a least of 16 / 24 / 32 /
+// 64 (TAM, us): 256 survivors x 360 orientations with 1081 beams 117.6 / 121.0 / 115.7 / 115.4, with 541 beams 78.0 /
+// 76.0 / 74.4 / 74.9; 1024 x 720 and 16 requests of 512 x 360 take 64 in any case.
 inline int tam_chunk_for(int K, int n_orient, int R, int n_sm) {
     const long long tasks_per_survivor = (n_orient + 3) / 4;
     long long c = (long long)K * R * tasks_per_survivor / (4ll * 2 * n_sm);
     c = c / 8 * 8;
-    return (int)(c < 16 ? 16 : c > 64 ? 64 : c);
+    return (int)(c < 32 ? 32 : c > 64 ? 64 : c);
 }
 // chunks of the TAM work order: per group of survivors (each batch, or all K as one group), its survivors in
 // chunks of one phase (at most one part chunk per phase); the per-batch count bounds both
@@ -390,15 +400,16 @@ cudaError_t launch_topk(const ReqDesc *reqs, int R, int max_n_hyp, int max_K, in
 struct TamPlan {
     int total_tasks, grid, vpl;
     size_t smem;
-    int stages, lut_bytes, lut_copies;   // staged tasks per CTA; bytes of a likelihood table and how many a CTA holds
-    bool h2;   // selection counts on packed fp16 (table slot of C + 1 at most 6143: C <= 5956)
+    int stages;                // staged tasks per CTA
+    int lut_bytes, lut_tables; // bytes of a likelihood table with its copies; tables: one per stage or one for all
+    int copies;                // copies of each entry in a table
 };
 // values per lane the TAM kernel holds for max_beams valid beams (-1 if too many)
 int tam_vpl_for(int max_beams);
 // the planned launch for the batches [batch_lo[r], batch_hi[r]) of each request r: segs[R + 1] (the last is the
 // launch's task counter), grid and kernel class
-TamPlan plan_tam(const int *batch_lo, const int *batch_hi, int R, int max_beams, int max_C, int n_sm,
-                 int ctas_per_sm, int chunk, int luts, TamSeg *segs);
+TamPlan plan_tam(const int *batch_lo, const int *batch_hi, int R, int max_beams, int max_rank, int n_sm, int chunk,
+                 int luts, long long poses, TamSeg *segs);
 // TAM's work order (surv_perm, tam_chunks, chunk_cnt) of every request, after the top-K
 // per-lane stride of the TAM endpoint offsets of a values-per-lane class
 int tam_offs_stride_for(int vpl);

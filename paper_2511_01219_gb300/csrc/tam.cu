@@ -9,17 +9,17 @@
 // a cache line holds an 8 x 8 block of cells, so the endpoints of
 // neighbouring beams share lines whichever way the contour runs, and an
 // endpoint's offset from its hypothesis depends on the hypothesis only
-// through its band phase (y + P) % 8.  The likelihood l
-// (Eq. 23) falls strictly as b grows, so the descending sort of Eq. 24 is the
-// ascending order of b: the warp finds the k-th smallest b by bisection over
-// [0, C] with register-resident values, and the top-k sum of l is
+// through its band phase (y + P) % 8.  The field holds not b but its code
+// (field_code): the rank of b among the values that a clamped squared distance
+// can take, as a positive fp16 bit pattern.  Ranks order like the values, so the
+// likelihood l (Eq. 23), which falls strictly as b grows, falls with the rank:
+// the descending sort of Eq. 24 is the ascending order of ranks.  The warp finds
+// the k-th smallest rank by bisection with register-resident codes, two beams
+// per instruction, and the top-k sum of l is
 // sum_{b <= b_k} l(b) - (#{b <= b_k} - k) l(b_k), the count being the one the
-// search ends on.  The counts run on fp16 patterns 0x6400 + slot(b), two
-// beams per instruction, while slot(C + 1) <= 6143 (C <= 5956), and on 32-bit
-// slots above.  A shared-memory table holds
-// l(b) and sqrt(C) - sqrt(b) for every b in [0, C] (at slot lut_slot(b), and
-// the selection runs on slots too, see below); with those and the exact
-// integer sum of b, the warp evaluates Eq. 27-30 and, after the block's
+// search ends on.  A shared-memory table holds l(b) and sqrt(C) - sqrt(b) by
+// rank; the exact integer sum of b comes from the latter (its root is within
+// 0.002 of an integer's), and the warp evaluates Eq. 27-30 and, after the block's
 // orientations, one lane per orientation takes the exponential and Eq. 31:
 //     wp = exp(Lbar),  d_max - dbar = res * sum(sqrt(C) - sqrt(b)) / N,
 //     s_d = min(d_max - dbar, d_max - d_min) / (d_max - d_min),
@@ -51,29 +51,16 @@ namespace relo {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-// Selection values as fp16 bit patterns 0x6400 + s, s the table slot of the
-// value (lut_slot, below).  Positive fp16 numbers order like their bit
-// patterns, so this is an increasing map of s onto fp16 numbers >= 1024,
-// consecutive ones at least 1 apart; it stays finite while 0x6400 + s <=
-// 0x7bff, i.e. s <= 6143 (kHalfMaxB).
-constexpr uint32_t kHalfBias = 0x6400u;
-constexpr int kHalfMaxB = 0x7bff - 0x6400;
+// The likelihood table in shared memory.  An 8-byte entry's bank pair would be its rank mod 16, and a warp's lookups
+// then serialise on the banks that its ranks share (3.0 to 3.2 wavefronts per lookup of 32 where 2 move the bytes,
+// counted over both workloads; 2, 4 or 8 copies of the table make it worse, since lanes with the same rank no longer
+// share a read).  With kLutCopies copies, entry by entry, each lane of a half-warp reads its own copy, which lies in its
+// own bank pair, and no lookup conflicts.  506 ranks (C = 1600) take 65 KB that way, one CTA per SM; larger clamps, maps
+// with different tables in one launch and calls too small to repay the filling keep one copy.
+constexpr int kLutCopies = 16;
 
-// The table slot of value b: b + floor(b / 32), one unused slot after every 32.
-// An 8-byte entry's bank pair is its slot mod 16, and the clamped d2 of real
-// endpoints crowd onto few residues mod 16 (sums of two squares take 9 of the
-// 16; near a wall parallel to an axis they are squares, 0, 1, 4 or 9 mod 16,
-// and C itself is often a square), so value-indexed lookups serialise a warp
-// on those banks; the gap moves each block of 32 values by one more bank pair.
-// The map is strictly increasing, so the kernel holds slots instead of values:
-// the k-th smallest slot is the slot of the k-th smallest value, ties stay
-// ties, and "b <= b_k" is "slot <= slot(b_k)".  The exact sum of b is taken
-// from the values before the map.  The table of C + 2 values spans
-// lut_slot(C + 1) + 1 slots.
-__host__ __device__ constexpr uint32_t lut_slot(uint32_t b) { return b + (b >> 5); }
-
-// The smallest b in [0, C] with count_le(b) >= k, given count_le(C) = n_C >= k
-// (every valid beam is <= C); cnt receives count_le(b).  hint < 0: bisection
+// The smallest rank b in [0, C] with count_le(b) >= k, given count_le(C) = n_C >= k
+// (C the last rank: every valid beam is <= C); cnt receives count_le(b).  hint < 0: bisection
 // over [0, C].  Otherwise the search starts at hint: two counts confirm an
 // unchanged answer; else it gallops away from hint in doubling steps to a
 // bracket [lo, hi] with count_le(lo - 1) < k <= count_le(hi) and bisects it.
@@ -171,7 +158,9 @@ __global__ void __launch_bounds__(1024) k_scan_prep(const ReqDesc *__restrict__ 
 // waited for the slowest search of its task, and a table copy and offsets for
 // each of 4 to 6 CTAs per SM left the gathers a third of L1.  TAM, us, before
 // and with the stages: 256 survivors x 360 orientations x 1081 beams 140 -> 117,
-// 1024 x 720 x 1440 1127 -> 1060, 16 mixed requests 2733 -> 2140.
+// 1024 x 720 x 1440 1127 -> 1060, 16 mixed requests 2733 -> 2140; with ranks,
+// conflict-free lookups and one CTA per SM 115, 1010 and 1994 (the L1 data path
+// is then 96% busy in the 1024 x 720 launch).
 //
 // Selection.  The k-th smallest clamped d2 of a survivor rarely changes from
 // one orientation to the next (neighbouring orientations see nearly the same
@@ -183,13 +172,10 @@ __global__ void __launch_bounds__(1024) k_scan_prep(const ReqDesc *__restrict__ 
 constexpr int kTamQ = 4;
 constexpr int kTamStages = 8;   // at most
 
-// Warps per CTA, two CTAs per SM (one where their shared memory does not fit twice), by values-per-lane class: the
-// register budget they leave each other against the warps that hide the gathers.  Measured (TAM, us): up to 24 values 24
-// / 20 / 16 / 14 warps 84 / 80 / 79 / 88 (18 values, 256 survivors x 360 orientations) and 2169 / 2136 / - / 2789 (the
-// mixed batch, both lower classes); 34 values 24 / 20 / 16 / 14 / 12 warps 136 / 120 / 117 / 121 / 179; 46 values 20 / 16
-// / 14 / 12 warps 1214 / 1069 / 1060 / 1089.
-__host__ __device__ constexpr int tam_warps(int vpl, bool h2) { return h2 ? (vpl <= 24 ? 20 : vpl <= 40 ? 16 : 14) : (vpl <= 24 ? 12 : 8); }
-constexpr int kTamCtas = 2;
+// Warps of the SM's CTA by values-per-lane class: the register budget they leave each other (64 up to 40 values, 72
+// above) against the warps that hide the gathers.  Measured with two CTAs of half as many (TAM, us): 34 values 48 / 40 /
+// 32 / 28 / 24 warps 136 / 120 / 117 / 121 / 179; 46 values 40 / 32 / 28 / 24 warps 1214 / 1069 / 1060 / 1089.
+__host__ __device__ constexpr int tam_warps(int vpl) { return vpl <= 40 ? 32 : 28; }
 
 // One staged task.
 struct TamTask {
@@ -201,7 +187,8 @@ struct TamTask {
     const float2 *lut_src;     // the table the stage's copy came from (it stays when the next task shares it)
     int n;                     // survivors, -1 when there are no more tasks
     int q0, nq, n_orient;
-    int N, k, C, fine;
+    int N, k, top, C, fine;    // top: the last rank, C's
+    float root_C;              // sqrt(C), an integer
     float inv_k, res_N, span, inv_span, res2_N, d_max;   // 1 / k, res / N, span of Eq. 29, res^2 / N
     int next, left;            // the next survivor to take; warps that have left the stage
 };
@@ -234,7 +221,8 @@ __device__ __forceinline__ bool wait_full(unsigned long long *bar, uint32_t pari
 template <int VPL>
 __device__ __forceinline__ const float2 *stage_task(const ReqDesc *__restrict__ reqs, int R, const TamSeg *__restrict__ segs,
                                                     const int *s_base, int task, TamTask &t, float2 *lut,
-                                                    int lut_copies, int *offs, int tid, int nt) {
+                                                    int lut_tables, int copies, int *offs,
+                                                    int tid, int nt) {
     constexpr int kS = tam_offs_stride(VPL);
     if (task >= s_base[R]) {
         if (tid == 0) t.n = -1;
@@ -251,9 +239,9 @@ __device__ __forceinline__ const float2 *stage_task(const ReqDesc *__restrict__ 
     const int nblk = (d.n_orient + kTamQ - 1) / kTamQ;
     const int4 ck = d.tam_chunks[d.chunk_cnt[segs[lo].batch_lo] + local / nblk];   // (phase, first, end)
     const int q0 = (local % nblk) * kTamQ, nq = min(kTamQ, d.n_orient - q0);
-    const float2 *src = lut_copies > 1 || !t.lut_src ? d.lut : t.lut_src;
+    const float2 *src = lut_tables > 1 || !t.lut_src ? d.lut_rank : t.lut_src;
     if (t.lut_src != src)
-        for (int i = tid; i <= d.C + 1; i += nt) lut[lut_slot(i)] = __ldg(src + i);
+        for (int i = tid, sh = copies > 1 ? 4 : 0; i < (d.n_rank + 1) * copies; i += nt) lut[i] = __ldg(src + (i >> sh));
     {
         // the block's endpoint cells (packed x, y offsets), nq x 32 x kS contiguous, to field offsets from a cell of
         // the chunk's band phase (field_index is linear in x, and in y through the bands crossed)
@@ -285,7 +273,9 @@ __device__ __forceinline__ const float2 *stage_task(const ReqDesc *__restrict__ 
         t.n_orient = d.n_orient;
         t.N = N;
         t.k = k;
+        t.top = d.n_rank - 1;
         t.C = d.C;
+        t.root_C = sqrtf((float)d.C);
         t.fine = d.fine;
         t.inv_k = 1.0f / (float)k;
         t.res_N = d.res / (float)N;
@@ -299,119 +289,88 @@ __device__ __forceinline__ const float2 *stage_task(const ReqDesc *__restrict__ 
     return src;
 }
 
+__device__ __forceinline__ float2 lds_float2(uint32_t addr) {
+    float2 v;
+    asm("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr));
+    return v;
+}
+
 // The scores of one survivor (position s, base field pointer fh) over the orientations [ql, qh) of the staged block, by
-// one warp.
-template <int VPL, bool H2>
-__device__ __forceinline__ void score_survivor(const TamTask &tk, const float2 *lut, const int *offs, int s,
+// one warp.  lut0: the shared address that entry code 0 of this lane's copy of the table would have; stride: bytes
+// between its entries.
+template <int VPL>
+__device__ __forceinline__ void score_survivor(const TamTask &tk, uint32_t lut0, uint32_t stride, const int *offs, int s,
                                                const uint16_t *__restrict__ fh, int ql, int qh) {
     constexpr int kS = tam_offs_stride(VPL);
     const int lane = threadIdx.x & 31;
-    const int N = tk.N, k = tk.k, C = tk.C;
-    const uint32_t none = (uint32_t)C + 1u;   // table entry with zero weight
-    int hint = -1;   // the previous orientation's k-th smallest value
+    const int N = tk.N, k = tk.k, top = tk.top;
+    const uint32_t none = kFieldBias + (uint32_t)top + 1u;   // table entry with zero weight
+    const float root_C = tk.root_C;
+    int hint = -1;   // the previous orientation's k-th smallest rank
     float e_arg = 0.0f, e_sd = 0.0f;   // lane qi: orientation qi's exponent and s_d
     for (int qi = ql; qi < qh; ++qi) {
         const int *ol = offs + (qi * 32 + lane) * kS;   // this lane's offsets, slot s = beam 32 s + lane
-        int sumb = 0;
+        unsigned sumb = 0u;
         float sgs = 0.0f, sl = 0.0f;
         int bk;
         int cle;   // #{b <= bk} over the valid beams
-        if constexpr (H2) {
-            uint32_t hv[VPL / 2];   // fp16 patterns 0x6400 + b of slots 2t (low half) and 2t + 1
+        uint32_t hv[VPL / 2];   // codes of slots 2t (low half) and 2t + 1
 #pragma unroll
-            for (int u = 0; u < (VPL + 3) / 4; ++u) {
-                const int4 o4 = *reinterpret_cast<const int4 *>(ol + 4 * u);
-                const int oo[4] = {o4.x, o4.y, o4.z, o4.w};
+        for (int u = 0; u < (VPL + 3) / 4; ++u) {
+            const int4 o4 = *reinterpret_cast<const int4 *>(ol + 4 * u);
+            const int oo[4] = {o4.x, o4.y, o4.z, o4.w};
 #pragma unroll
-                for (int e = 0; e < 4; e += 2) {
-                    const int t = 2 * u + e / 2;   // pair of slots 2t, 2t + 1
-                    if (t < VPL / 2) {
-                        const int i0 = (t << 6) + lane, i1 = i0 + 32;
-                        uint32_t b0 = none, b1 = none;
-                        if (i0 < N) {
-                            b0 = (uint32_t)__ldg(fh + oo[e]);
-                            sumb += (int)b0;
-                        }
-                        if (i1 < N) {
-                            b1 = (uint32_t)__ldg(fh + oo[e + 1]);
-                            sumb += (int)b1;
-                        }
-                        // both slots at once: b + floor(b / 32) per half, plus the bias
-                        // (slot(C + 1) <= kHalfMaxB: no carry between the halves)
-                        const uint32_t v2 = b0 | (b1 << 16);
-                        hv[t] = v2 + ((v2 >> 5) & 0x07ff07ffu) + (kHalfBias | (kHalfBias << 16));
-                    }
+            for (int e = 0; e < 4; e += 2) {
+                const int t = 2 * u + e / 2;   // pair of slots 2t, 2t + 1
+                if (t < VPL / 2) {
+                    const int i0 = (t << 6) + lane, i1 = i0 + 32;
+                    uint32_t b0 = none, b1 = none;
+                    if (i0 < N) b0 = (uint32_t)__ldg(fh + oo[e]);
+                    if (i1 < N) b1 = (uint32_t)__ldg(fh + oo[e + 1]);
+                    hv[t] = b0 | (b1 << 16);
                 }
             }
-            // #{b > x} on a lane: f(b) - f(x) saturated to [0, 1] is 1 exactly when b > x (f maps
-            // b to the fp16 number of bits 0x6400 + slot(b); the exact difference is then >= 1,
-            // else <= 0, and rounding keeps both); then #{b <= x} over the warp is the 32 VPL
-            // slots less those (no-beam slots are > C)
-            auto count_le = [&](int x) -> int {
-                const unsigned short fxb = (unsigned short)(kHalfBias + lut_slot((uint32_t)x));
-                const __half2 fx = __halves2half2(__ushort_as_half(fxb), __ushort_as_half(fxb));
-                // two chains (half the add latency); the low half starts at 1024, so the
-                // total 1024 + c (c <= 64) has the fp16 bits 0x6400 + c
-                __half2 acc0 = __halves2half2(__ushort_as_half((unsigned short)kHalfBias), __float2half(0.0f));
-                __half2 acc1 = __float2half2_rn(0.0f);
+        }
+        // #{b > x} on a lane: f(b) - f(x) saturated to [0, 1] is 1 exactly when b > x (f maps rank b to the fp16 number
+        // of bits kFieldBias + b, numbers >= 1024 at least 1 apart; the exact difference is then >= 1, else <= 0, and
+        // rounding keeps both); then #{b <= x} over the warp is the 32 VPL slots less those (no-beam slots are > top)
+        auto count_le = [&](int x) -> int {
+            const unsigned short fxb = (unsigned short)(kFieldBias + (uint32_t)x);
+            const __half2 fx = __halves2half2(__ushort_as_half(fxb), __ushort_as_half(fxb));
+            // two chains (half the add latency); the low half starts at 1024, so the
+            // total 1024 + c (c <= 64) has the fp16 bits 0x6400 + c
+            __half2 acc0 = __halves2half2(__ushort_as_half((unsigned short)0x6400), __float2half(0.0f));
+            __half2 acc1 = __float2half2_rn(0.0f);
 #pragma unroll
-                for (int t = 0; t < VPL / 2; t += 2) {
-                    acc0 = __hadd2(acc0, __hsub2_sat(*reinterpret_cast<const __half2 *>(&hv[t]), fx));
-                    if (t + 1 < VPL / 2)
-                        acc1 = __hadd2(acc1, __hsub2_sat(*reinterpret_cast<const __half2 *>(&hv[t + 1]), fx));
-                }
-                const __half2 sum = __hadd2(acc0, acc1);
-                const __half2 tot = __hadd2(sum, __lowhigh2highlow(sum));
-                const int gt = __reduce_add_sync(kFull, (int)(__half_as_ushort(__low2half(tot)) & 0x3ffu));
-                return 32 * VPL - gt;
-            };
-            if (tk.fine < kFineBaseline) {
-                bk = kth_smallest(count_le, k, C, N, hint, cle);
-            } else {
-                bk = C;   // every valid beam
-                cle = N;
+            for (int t = 0; t < VPL / 2; t += 2) {
+                acc0 = __hadd2(acc0, __hsub2_sat(*reinterpret_cast<const __half2 *>(&hv[t]), fx));
+                if (t + 1 < VPL / 2)
+                    acc1 = __hadd2(acc1, __hsub2_sat(*reinterpret_cast<const __half2 *>(&hv[t + 1]), fx));
             }
-            const uint32_t bkb = kHalfBias + lut_slot((uint32_t)bk);
-#pragma unroll
-            for (int t = 0; t < VPL / 2; ++t) {
-                const uint32_t p0 = hv[t] & 0xffffu, p1 = hv[t] >> 16;
-                const float2 g0 = lut[p0 - kHalfBias], g1 = lut[p1 - kHalfBias];   // slot(C+1) (no beam) adds zero
-                sgs += g0.y + g1.y;
-                if (p0 <= bkb) sl += g0.x;
-                if (p1 <= bkb) sl += g1.x;
-            }
+            const __half2 sum = __hadd2(acc0, acc1);
+            const __half2 tot = __hadd2(sum, __lowhigh2highlow(sum));
+            const int gt = __reduce_add_sync(kFull, (int)(__half_as_ushort(__low2half(tot)) & 0x3ffu));
+            return 32 * VPL - gt;
+        };
+        if (tk.fine < kFineBaseline) {
+            bk = kth_smallest(count_le, k, top, N, hint, cle);
         } else {
-            uint32_t v[VPL];   // slots of the values
+            bk = top;   // every valid beam
+            cle = N;
+        }
+        const uint32_t bkb = kFieldBias + (uint32_t)bk;
+        // b of an entry: (sqrt(C) - g)^2 is within 0.002 of it (g is rounded to 2^-18 at most, sqrt(C) exact), so adding
+        // 1.5 2^23 leaves it as the low bits; the sum of those bit patterns, mod 2^32, is sum b + 32 VPL patterns of 0
+        // + C for every slot without a beam (g = 0 there)
 #pragma unroll
-            for (int t = 0; t < VPL; ++t) {
-                const int i = (t << 5) + lane;
-                uint32_t bv = none;
-                if (i < N) {
-                    bv = (uint32_t)__ldg(fh + ol[t]);
-                    sumb += (int)bv;
-                }
-                v[t] = lut_slot(bv);
-            }
-            auto count_le = [&](int x) -> int {
-                int c = 0;
-                const uint32_t sx = lut_slot((uint32_t)x);
-#pragma unroll
-                for (int t = 0; t < VPL; ++t) c += (v[t] <= sx) ? 1 : 0;
-                return __reduce_add_sync(kFull, c);
-            };
-            if (tk.fine < kFineBaseline) {
-                bk = kth_smallest(count_le, k, C, N, hint, cle);
-            } else {
-                bk = C;
-                cle = N;
-            }
-            const uint32_t sk = lut_slot((uint32_t)bk);
-#pragma unroll
-            for (int t = 0; t < VPL; ++t) {
-                const float2 lg = lut[v[t]];   // the slot of C+1 (no beam) adds zero
-                sgs += lg.y;
-                if (v[t] <= sk) sl += lg.x;
-            }
+        for (int t = 0; t < VPL / 2; ++t) {
+            const uint32_t p0 = hv[t] & 0xffffu, p1 = hv[t] >> 16;
+            const float2 g0 = lds_float2(lut0 + p0 * stride), g1 = lds_float2(lut0 + p1 * stride);
+            const float t0 = root_C - g0.y, t1 = root_C - g1.y;
+            sgs += g0.y + g1.y;   // the entry of no beam adds zero
+            sumb += __float_as_uint(fmaf(t0, t0, 12582912.0f)) + __float_as_uint(fmaf(t1, t1, 12582912.0f));
+            if (p0 <= bkb) sl += g0.x;
+            if (p1 <= bkb) sl += g1.x;
         }
         hint = bk;
 #pragma unroll
@@ -419,17 +378,17 @@ __device__ __forceinline__ void score_survivor(const TamTask &tk, const float2 *
             sgs += __shfl_xor_sync(kFull, sgs, o);
             sl += __shfl_xor_sync(kFull, sl, o);
         }
-        sumb = __reduce_add_sync(kFull, sumb);
+        sumb = __reduce_add_sync(kFull, sumb) - 32u * VPL * 0x4b400000u - (unsigned)(tk.C * (32 * VPL - N));
         {
             // Eq. 27-30 from the warp totals every lane holds; the top-k sum of l is every
             // b <= bk less the cle - k ties at bk beyond the k-th; lane qi keeps what its
             // orientation's score still needs: for TAM the exponent of exp(Lbar) exp(-var / 2)
             // and s_d
-            const float topsum = sl - (float)(cle - k) * lut[lut_slot(bk)].x;
+            const float topsum = sl - (float)(cle - k) * lds_float2(lut0 + bkb * stride).x;
             const float lbar = topsum * tk.inv_k;
             const float dd = tk.res_N * sgs;   // d_max - dbar
             const float dbar = tk.d_max - dd;
-            const float var = fmaxf(tk.res2_N * (float)sumb - dbar * dbar, 0.0f);
+            const float var = fmaxf(tk.res2_N * (float)(int)sumb - dbar * dbar, 0.0f);
             const float sd = fminf(dd, tk.span) * tk.inv_span;
             const int fine = tk.fine;
             float a = lbar - 0.5f * var;
@@ -456,21 +415,20 @@ __device__ __forceinline__ void score_survivor(const TamTask &tk, const float2 *
     }
 }
 
-template <int VPL, bool H2>
-__global__ void __launch_bounds__(tam_warps(VPL, H2) * 32, kTamCtas) k_tam(const ReqDesc *__restrict__ reqs, int R,
-                                                                           TamSeg *__restrict__ segs, int stages,
-                                                                           int lut_bytes, int lut_copies,
-                                                                           BatchState *bs) {
+template <int VPL>
+__global__ void __launch_bounds__(tam_warps(VPL) * 32, 1) k_tam(const ReqDesc *__restrict__ reqs, int R,
+                                                                TamSeg *__restrict__ segs, int stages, int lut_bytes,
+                                                                int lut_tables, int copies, BatchState *bs) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_base[kMaxBatchRequests + 1];
     __shared__ int s_warp[kMaxBatchRequests / 32];
     __shared__ TamTask task[kTamStages];
-    constexpr int kWarps = tam_warps(VPL, H2), kThreads = kWarps * 32;
+    constexpr int kWarps = tam_warps(VPL), kThreads = kWarps * 32;
     static_assert(kThreads >= kMaxBatchRequests, "a thread per request");
     constexpr int kOffs = kTamQ * 32 * tam_offs_stride(VPL);
     // one table for all stages when every request of the launch has the same, else one per stage
-    auto lut_of = [&](int i) { return reinterpret_cast<float2 *>(smem + (lut_copies > 1 ? i * lut_bytes : 0)); };
-    int *const offs0 = reinterpret_cast<int *>(smem + lut_copies * lut_bytes);
+    auto lut_of = [&](int i) { return reinterpret_cast<float2 *>(smem + (lut_tables > 1 ? i * lut_bytes : 0)); };
+    int *const offs0 = reinterpret_cast<int *>(smem + lut_tables * lut_bytes);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     chain_wait();
     chain_go();
@@ -512,11 +470,11 @@ __global__ void __launch_bounds__(tam_warps(VPL, H2) * 32, kTamCtas) k_tam(const
     };
     for (int i = 0; i < stages; ++i) {   // the first tasks, staged by the whole CTA
         const float2 *src = stage_task<VPL>(reqs, R, segs, s_base, (int)blockIdx.x + i * (int)gridDim.x, task[i],
-                                            lut_of(i), lut_copies, offs0 + i * kOffs, threadIdx.x, kThreads);
+                                            lut_of(i), lut_tables, copies, offs0 + i * kOffs, threadIdx.x, kThreads);
         __syncthreads();
         if (threadIdx.x == 0) {
             // a table that all stages share is filled by the first task; the others take it as theirs
-            for (int j = i; j < (lut_copies > 1 ? i + 1 : stages); ++j) task[j].lut_src = src;
+            for (int j = i; j < (lut_tables > 1 ? i + 1 : stages); ++j) task[j].lut_src = src;
             arrive(task[i]);
         }
         __syncthreads();
@@ -528,6 +486,8 @@ __global__ void __launch_bounds__(tam_warps(VPL, H2) * 32, kTamCtas) k_tam(const
             TamTask &t = task[i];
             float2 *lut = lut_of(i);
             int *offs = offs0 + i * kOffs;
+            const uint32_t stride = 8u * (uint32_t)copies;
+            const uint32_t lut0 = smem_u32(lut) + 8u * ((uint32_t)lane & (uint32_t)(copies - 1)) - kFieldBias * stride;
             if (!wait_full(&t.full, parity)) {
                 if (lane == 0) atomicExch(&bs->error, 1u);
                 return;
@@ -546,7 +506,7 @@ __global__ void __launch_bounds__(tam_warps(VPL, H2) * 32, kTamCtas) k_tam(const
                     if (j >= n * parts) break;
                     const int js = parts == 1 ? j : j / parts, ql = parts == 1 ? 0 : j - js * parts;
                     const int2 sv = __ldg(t.perm + js);
-                    score_survivor<VPL, H2>(t, lut, offs, sv.x, t.field + (unsigned)sv.y, ql, ql + part);
+                    score_survivor<VPL>(t, lut0, stride, offs, sv.x, t.field + (unsigned)sv.y, ql, ql + part);
                 }
                 __syncwarp();   // every lane's reads of the stage come before the warp counts itself out
                 int last = 0;
@@ -561,7 +521,7 @@ __global__ void __launch_bounds__(tam_warps(VPL, H2) * 32, kTamCtas) k_tam(const
                     int nt = 0;
                     if (lane == 0) nt = (int)(atomicAdd(counter, 1u) + (unsigned)stages * gridDim.x);
                     nt = __shfl_sync(kFull, nt, 0);
-                    const float2 *src = stage_task<VPL>(reqs, R, segs, s_base, nt, t, lut, lut_copies, offs, lane, 32);
+                    const float2 *src = stage_task<VPL>(reqs, R, segs, s_base, nt, t, lut, lut_tables, copies, offs, lane, 32);
                     __syncwarp();
                     if (lane == 0) {
                         t.lut_src = src;
@@ -577,17 +537,17 @@ __global__ void __launch_bounds__(tam_warps(VPL, H2) * 32, kTamCtas) k_tam(const
     }
 }
 
-template <int VPL, bool H2>
+template <int VPL>
 cudaError_t run_tam(const ReqDesc *reqs, int R, TamSeg *segs, const TamPlan &tp, BatchState *bs, cudaStream_t s) {
     // plan_tam has asked for this shape's residency, which also lets the kernel use its shared memory
-    return launch_chained(k_tam<VPL, H2>, dim3((unsigned)tp.grid), tam_warps(VPL, H2) * 32, tp.smem, s, reqs, R, segs,
-                          tp.stages, tp.lut_bytes, tp.lut_copies, bs);
+    return launch_chained(k_tam<VPL>, dim3((unsigned)tp.grid), tam_warps(VPL) * 32, tp.smem, s, reqs, R, segs,
+                          tp.stages, tp.lut_bytes, tp.lut_tables, tp.copies, bs);
 }
 
-template <int VPL, bool H2>
+template <int VPL>
 int tam_occupancy(size_t smem) {
     int occ = 0;
-    if (resident_ctas((const void *)k_tam<VPL, H2>, tam_warps(VPL, H2) * 32, smem, &occ) != cudaSuccess) {
+    if (resident_ctas((const void *)k_tam<VPL>, tam_warps(VPL) * 32, smem, &occ) != cudaSuccess) {
         cudaGetLastError();   // more than an SM has: no CTA fits
         return 0;
     }
@@ -607,9 +567,9 @@ int vpl_bucket(int max_beams) {
     return -1;
 }
 
-int occupancy_for(int vpl, bool h2, size_t smem) {
+int occupancy_for(int vpl, size_t smem) {
 #define RELO_TAM_OCC(V) \
-    if (vpl == V) return h2 ? tam_occupancy<V, true>(smem) : tam_occupancy<V, false>(smem);
+    if (vpl == V) return tam_occupancy<V>(smem);
     RELO_TAM_VPLS(RELO_TAM_OCC)
 #undef RELO_TAM_OCC
     return 0;
@@ -624,38 +584,40 @@ cudaError_t launch_scan_prep(const ReqDesc *reqs, int R, cudaStream_t s) {
 }
 
 // The launch for the batches [batch_lo[r], batch_hi[r]) of every request:
-// its kernel class (values per lane and selection precision for the longest
-// scan and the largest clamp), its stages, and a grid of every resident CTA (or
-// ctas_per_sm per SM when that is fewer); the tasks are counted by the kernel
-// from the device-built chunk tables.  chunk: survivors of a usual task; lut_copies:
-// 1 when all requests share one likelihood table.  segs: R entries and the
-// task counter.
+// its kernel class (values per lane for the longest scan), its table and
+// stages, and a grid of one CTA per SM; the tasks are counted by the kernel
+// from the device-built chunk tables.  chunk: survivors of a usual task; luts: 1
+// when all requests share one likelihood table (of max_rank ranks at most);
+// poses: survivors x orientations of the launch.  segs: R entries and the task
+// counter.
 //
 // A stage is refilled once its slowest survivor is done, so the stages together hold about twice the survivors that
-// the warps work on (never fewer than two stages); they may not cost a resident CTA.
-TamPlan plan_tam(const int *batch_lo, const int *batch_hi, int R, int max_beams, int max_C, int n_sm,
-                 int ctas_per_sm, int chunk, int luts, TamSeg *segs) {
-    TamPlan tp{0, 0, vpl_bucket(max_beams), 0, 1, 0, 1, (int)lut_slot(max_C + 1) <= kHalfMaxB};
+// the warps work on, never fewer than two stages if they fit.  The copied table wants two stages beside it and a
+// launch that gives a warp several poses.
+TamPlan plan_tam(const int *batch_lo, const int *batch_hi, int R, int max_beams, int max_rank, int n_sm, int chunk,
+                 int luts, long long poses, TamSeg *segs) {
+    TamPlan tp{0, 0, vpl_bucket(max_beams), 0, 1, 0, 1, 1};
     if (tp.vpl < 0) return tp;
-    tp.lut_bytes = (int)(((size_t)(lut_slot(max_C + 1) + 1) * sizeof(float2) + 15) & ~(size_t)15);
+    const size_t table = (size_t)(max_rank + 1) * sizeof(float2);
     const size_t offs = (size_t)kTamQ * 32 * tam_offs_stride(tp.vpl) * sizeof(int);
-    auto bytes = [&](int stages) { return (size_t)tp.lut_bytes * (luts > 1 ? stages : 1) + stages * offs; };
-    const int want = std::min(kTamStages, std::max(2, (9 * tam_warps(tp.vpl, tp.h2) + 4 * chunk - 1) / (4 * chunk)));
-    int occ = 0;
-    for (int st = want; st >= 1; --st) {   // the most stages among those with the most CTAs
-        const int o = std::min(kTamCtas, occupancy_for(tp.vpl, tp.h2, bytes(st)));
-        if (o > occ) {
-            occ = o;
+    const int want = std::min(kTamStages, std::max(3, (9 * tam_warps(tp.vpl) + 4 * chunk - 1) / (4 * chunk)));
+    const bool many = luts == 1 && poses >= 4ll * 32 * n_sm;
+    for (int copies = many ? kLutCopies : 1; copies >= 1 && !tp.smem; copies /= kLutCopies) {
+        const size_t lut = (table * copies + 15) & ~(size_t)15;
+        for (int st = want; st >= (copies > 1 ? 2 : 1) && !tp.smem; --st) {
+            const size_t bytes = lut * (luts > 1 ? st : 1) + st * offs;
+            if (bytes > 220 * 1024 || occupancy_for(tp.vpl, bytes) < 1) continue;
             tp.stages = st;
-            tp.smem = bytes(st);
+            tp.smem = bytes;
+            tp.copies = copies;
+            tp.lut_bytes = (int)lut;
         }
-        if (occ == kTamCtas) break;
     }
-    if (occ < 1) {
+    if (!tp.smem) {
         tp.vpl = -1;
         return tp;
     }
-    tp.lut_copies = luts > 1 ? tp.stages : 1;
+    tp.lut_tables = luts > 1 ? tp.stages : 1;
     bool any = false;
     for (int r = 0; r < R; ++r) {
         segs[r] = TamSeg{batch_lo[r], batch_hi[r]};
@@ -663,7 +625,7 @@ TamPlan plan_tam(const int *batch_lo, const int *batch_hi, int R, int max_beams,
     }
     segs[R] = TamSeg{0, 0};
     tp.total_tasks = any ? 1 : 0;
-    tp.grid = n_sm * (ctas_per_sm > 0 && ctas_per_sm < occ ? ctas_per_sm : occ);
+    tp.grid = n_sm;
     return tp;
 }
 
@@ -673,7 +635,7 @@ cudaError_t launch_tam(const ReqDesc *reqs, int R, TamSeg *segs, const TamPlan &
     if (tp.total_tasks <= 0) return cudaSuccess;
 #define RELO_TAM_RUN(V)                                                                 \
     if (tp.vpl == V)                                                                    \
-        return tp.h2 ? run_tam<V, true>(reqs, R, segs, tp, bs, s) : run_tam<V, false>(reqs, R, segs, tp, bs, s);
+        return run_tam<V>(reqs, R, segs, tp, bs, s);
     RELO_TAM_VPLS(RELO_TAM_RUN)
 #undef RELO_TAM_RUN
     return cudaErrorInvalidValue;
