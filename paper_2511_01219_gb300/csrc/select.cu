@@ -3,12 +3,14 @@
 // k_topk: the K hypotheses with the smallest SMAD (or CAER; Sec. III intro:
 // the coarse metric orders all positions, the ordered set is cut into
 // batches).  Keys are numerator << 21 | index, so they are unique and
-// ascending key order is (numerator, index) order.  One CTA histograms the 11 bits below the keys' highest
-// set bit, finds the digit holding the K-th smallest key, and orders the keys
-// up to that digit (by rank counting when they are few: keys are unique),
-// keeping the first K;
-// when too many keys share that digit it falls back to an MSB-first radix
-// select over 8-bit digits.
+// ascending key order is (numerator, index) order.  One CTA histograms the keys' digits (octave and the bits below its
+// leading one), finds the digit holding the K-th smallest key, moves the keys up to that digit to their digit's range and
+// counts each key's rank within it (keys are unique), keeping the first K; when a digit holds many keys it sorts them
+// instead, and when too many share the K-th key's digit it falls back to an MSB-first radix select over 8-bit digits.
+// The launch is a chain of short phases in one CTA per request, so latency bounds it, not bandwidth (20000 keys are
+// 160 KB).  With digits of equal width the best keys shared one (5000 keys, K = 256: the radix select; 20000, K = 1024: a
+// sorting network of 66 barriers, half of the launch).  Stage, us, before and now: 20.5 -> 12.2 and 41 -> 22.5; 16
+// requests of up to 8000 keys, K = 512, 67 -> 23 (there the endpoint tables of the launch's other CTAs counted most).
 //
 // k_select_batch: after TAM has scored one batch, the per-hypothesis
 // orientation argmax of Eq. 22 (already reduced by TAM into one 64-bit key per
@@ -40,7 +42,10 @@ namespace relo {
 namespace {
 
 constexpr int kTopkThreads = 1024;
-constexpr int kStageMax = 20480;   // keys staged in shared memory (160 KiB)
+// Keys a thread holds in registers from the one load to the last pass: up to kHold * kTopkThreads keys (20480) cost one
+// read, all its loads in flight; more are read from memory in every pass, kLoads in flight.
+constexpr int kHold = 20;
+constexpr int kLoads = 8;
 
 __device__ void bitonic_sort(unsigned long long *v, int n_pow2) {
     for (int k = 2; k <= n_pow2; k <<= 1) {
@@ -84,54 +89,97 @@ __device__ void order_out(unsigned long long *v, int n, int K, int32_t *survivor
     for (int i = threadIdx.x; i < K; i += blockDim.x) survivors[i] = (int32_t)(v[i] & ((1ull << kHypBits) - 1));
 }
 
-constexpr int kTopkBins = 2048;   // first pass: the 11 bits below the keys' highest set bit
+// First pass: a key's digit is its octave (the position of its highest set bit) and as many bits below that as 2048 digits
+// for all octaves present allow.  The best SMADs of thousands of hypotheses lie far below the largest, so digits of equal
+// width would put them all in one.
+constexpr int kTopkBins = 2048;
+
+struct KeyDigits {
+    int lowest, bits;   // the lowest octave present; bits below the highest set bit
+    // ascending with the key
+    __device__ __forceinline__ int operator()(unsigned long long k) const {
+        const int e = 63 - __clzll((long long)(k | 1ull));
+        const unsigned long long m = e >= bits ? k >> (e - bits) : k << (bits - e);
+        return ((e - lowest) << bits) | (int)((unsigned)m & ((1u << bits) - 1u));
+    }
+};
+// Keys of one digit up to which ranks are counted within the digit: the longest digit is then one short loop per key,
+// where the sorting network takes 55 to 66 barriers for 1024 to 2048 keys (20 us; digits of 128 to 512 keys in a request
+// of 20000, K = 1024: stage 38 us sorted, 20 us counted).
+constexpr int kDigitRankMax = 512;
 
 // The first K keys of request d in ascending order into its survivor list,
 // by one CTA (sm: the launch's dynamic shared memory).
-__device__ void topk_request(const ReqDesc &d, unsigned long long *sm, int Kp_cap, int stage_cap) {
-    const unsigned long long *keys_g = d.keys;
+__device__ __forceinline__ void topk_request(const ReqDesc &d, unsigned long long *sm, int Kp_cap) {
+    const unsigned long long *__restrict__ keys = d.keys;
     const int n = d.n_hyp, K = d.K;
     unsigned long long *sortbuf = sm;                                          // [2 * Kp_cap]
     unsigned int *hist = reinterpret_cast<unsigned int *>(sm + 2 * Kp_cap);    // [kTopkBins]
-    unsigned long long *keys_s = sm + 2 * Kp_cap + kTopkBins / 2;              // [stage_cap]
-    __shared__ unsigned long long s_or;
-    __shared__ int s_digit, s_below, s_cnt;
+    __shared__ int s_low, s_high;
+    __shared__ int s_digit, s_below, s_cnt, s_sel;
     __shared__ unsigned int s_warp[32];
-    const bool staged = n <= stage_cap;
-    const unsigned long long *keys = staged ? keys_s : keys_g;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int n_round = (n + blockDim.x - 1) / blockDim.x * blockDim.x;   // whole warps in every round
-
-    if (threadIdx.x == 0) { s_or = 0; s_cnt = 0; }
-    for (int i = threadIdx.x; i < kTopkBins; i += blockDim.x) hist[i] = 0;
-    __syncthreads();
-    unsigned long long orv = 0;
-    constexpr int kLoads = 8;   // keys a thread has in flight
-    for (int i0 = threadIdx.x; i0 < n; i0 += kLoads * blockDim.x) {
-        unsigned long long k[kLoads];
+    const bool held = n <= kHold * kTopkThreads;
+    unsigned long long mine[kHold];
+    // f(key, in) for the thread's keys; whole warps in every round, in false past the last key
+    auto each_key = [&](auto f) {
+        if (held) {
 #pragma unroll
-        for (int u = 0; u < kLoads; ++u) {
-            const int i = i0 + u * blockDim.x;
-            k[u] = i < n ? keys_g[i] : 0ull;
+            for (int u = 0; u < kHold; ++u) {
+                if (u * kTopkThreads >= n) break;
+                f(mine[u], u * kTopkThreads + (int)threadIdx.x < n);
+            }
+            return;
         }
+        for (int i0 = 0; i0 < n; i0 += kLoads * kTopkThreads) {
+            unsigned long long k[kLoads];
 #pragma unroll
-        for (int u = 0; u < kLoads; ++u) {
-            const int i = i0 + u * blockDim.x;
-            if (staged && i < n) keys_s[i] = k[u];
-            orv |= k[u];
+            for (int u = 0; u < kLoads; ++u) {
+                const int i = i0 + u * kTopkThreads + (int)threadIdx.x;
+                k[u] = i < n ? keys[i] : 0ull;
+            }
+#pragma unroll
+            for (int u = 0; u < kLoads; ++u) f(k[u], i0 + u * kTopkThreads + (int)threadIdx.x < n);
+        }
+    };
+
+    if (threadIdx.x == 0) { s_low = 63; s_high = 0; s_cnt = 0; }
+    if (held) {
+#pragma unroll
+        for (int u = 0; u < kHold; ++u) {
+            const int i = u * kTopkThreads + (int)threadIdx.x;
+            mine[u] = i < n ? keys[i] : 0ull;
         }
     }
-    for (int o = 16; o > 0; o >>= 1) orv |= __shfl_xor_sync(0xffffffffu, orv, o);
-    if (lane == 0) atomicOr(&s_or, orv);
+    for (int i = threadIdx.x; i < kTopkBins; i += blockDim.x) hist[i] = 0;
     __syncthreads();
-    const int top = s_or ? 63 - __clzll((long long)s_or) : 0;
+    int low = 63, top = 0;
+    each_key([&](unsigned long long k, bool in) {
+        const int e = 63 - __clzll((long long)(k | 1ull));
+        if (in) {
+            low = min(low, e);
+            top = max(top, e);
+        }
+    });
+    low = __reduce_min_sync(0xffffffffu, low);
+    top = __reduce_max_sync(0xffffffffu, top);
+    if (lane == 0) {
+        atomicMin(&s_low, low);
+        atomicMax(&s_high, top);
+    }
+    __syncthreads();
+    low = s_low;
+    top = max(s_high, low);
+    const KeyDigits digit{low, 31 - __clz(kTopkBins / (top - low + 1))};
 
-    // One pass over 11-bit digits finds the digit b* of the K-th smallest key;
-    // the keys with digit < b* are all in, those with digit b* are sorted with
+    // One pass over the digits finds the digit b* of the K-th smallest key;
+    // the keys with digit < b* are all in, those with digit b* are ordered with
     // them and the first K kept.
-    const int sh = top >= 10 ? top - 10 : 0;   // every key is < 2^(top + 1), so key >> sh < 2^11
-    for (int i = threadIdx.x; i < n; i += blockDim.x) atomicAdd(&hist[keys[i] >> sh], 1u);
+    each_key([&](unsigned long long k, bool in) {
+        if (in) atomicAdd(&hist[digit(k)], 1u);
+    });
     __syncthreads();
+    bool long_digit;
     {
         const unsigned a = hist[2 * threadIdx.x], b = hist[2 * threadIdx.x + 1];   // 1024 threads x 2 bins
         unsigned incl = a + b;
@@ -156,28 +204,38 @@ __device__ void topk_request(const ReqDesc &d, unsigned long long *sm, int Kp_ca
         if (excl < (unsigned)K && excl + a + b >= (unsigned)K) {
             if (excl + a >= (unsigned)K) {
                 s_digit = 2 * threadIdx.x;
-                s_below = (int)excl;
+                s_sel = (int)(excl + a);
             } else {
                 s_digit = 2 * threadIdx.x + 1;
-                s_below = (int)(excl + a);
+                s_sel = (int)(excl + a + b);
             }
         }
+        hist[2 * threadIdx.x] = excl;   // where each digit's keys begin
+        hist[2 * threadIdx.x + 1] = excl + a;
         __syncthreads();
+        const int first = 2 * threadIdx.x;
+        long_digit = __syncthreads_or((a > kDigitRankMax && first <= s_digit) || (b > kDigitRankMax && first < s_digit));
     }
-    const unsigned long long dstar = (unsigned long long)s_digit;
-    const int n_sel = s_below + (int)hist[s_digit];   // keys with digit <= b*
+    const int dstar = s_digit;
+    const int n_sel = s_sel;   // keys with digit <= b*
     if (n_sel <= 2 * Kp_cap) {
-        for (int i = threadIdx.x; i < n_round; i += blockDim.x) {   // one slot reservation per warp
-            const unsigned long long k = i < n ? keys[i] : ~0ull;
-            const bool take = i < n && (k >> sh) <= dstar;
-            const unsigned bal = __ballot_sync(0xffffffffu, take);
-            int base = 0;
-            if (lane == 0 && bal) base = atomicAdd(&s_cnt, __popc(bal));
-            base = __shfl_sync(0xffffffffu, base, 0);
-            if (take) sortbuf[base + __popc(bal & ((1u << lane) - 1u))] = k;
+        each_key([&](unsigned long long k, bool in) {
+            const int g = digit(k);
+            if (in && g <= dstar) sortbuf[atomicAdd(&hist[g], 1u)] = k;
+        });
+        __syncthreads();   // hist[g] is now where digit g ends
+        if (long_digit) {
+            order_out(sortbuf, n_sel, K, d.survivors);
+            return;
         }
-        __syncthreads();
-        order_out(sortbuf, n_sel, K, d.survivors);
+        for (int i = threadIdx.x; i < n_sel; i += blockDim.x) {
+            const unsigned long long me = sortbuf[i];
+            const int g = digit(me);
+            const int lo = g ? (int)hist[g - 1] : 0, hi = (int)hist[g];
+            int rank = lo;
+            for (int k = lo; k < hi; ++k) rank += sortbuf[k] < me ? 1 : 0;
+            if (rank < K) d.survivors[rank] = (int32_t)(me & ((1ull << kHypBits) - 1));
+        }
         return;
     }
 
@@ -188,10 +246,9 @@ __device__ void topk_request(const ReqDesc &d, unsigned long long *sm, int Kp_ca
         __syncthreads();
         for (int i = threadIdx.x; i < 256; i += blockDim.x) hist[i] = 0;
         __syncthreads();
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            const unsigned long long k = keys[i];
-            if ((k & mask) == prefix) atomicAdd(&hist[(k >> shift) & 255u], 1u);
-        }
+        each_key([&](unsigned long long k, bool in) {
+            if (in && (k & mask) == prefix) atomicAdd(&hist[(k >> shift) & 255u], 1u);
+        });
         __syncthreads();
         if (threadIdx.x < 32) {
             unsigned int local = 0;
@@ -222,15 +279,14 @@ __device__ void topk_request(const ReqDesc &d, unsigned long long *sm, int Kp_ca
         remaining -= s_below;
     }
     // prefix is now the K-th smallest key; one slot reservation per warp
-    for (int i = threadIdx.x; i < n_round; i += blockDim.x) {
-        const unsigned long long k = i < n ? keys[i] : ~0ull;
-        const bool take = i < n && k <= prefix;
+    each_key([&](unsigned long long k, bool in) {
+        const bool take = in && k <= prefix;
         const unsigned bal = __ballot_sync(0xffffffffu, take);
         int base = 0;
         if (lane == 0 && bal) base = atomicAdd(&s_cnt, __popc(bal));
         base = __shfl_sync(0xffffffffu, base, 0);
         if (take) sortbuf[base + __popc(bal & ((1u << lane) - 1u))] = k;
-    }
+    });
     __syncthreads();
     order_out(sortbuf, K, K, d.survivors);
 }
@@ -238,25 +294,26 @@ __device__ void topk_request(const ReqDesc &d, unsigned long long *sm, int Kp_ca
 // One CTA per request ranks it and then builds its TAM work order from the
 // survivors; the CTAs after the first R compute the requests' TAM endpoint
 // offsets and, for ICP, the beams' sensor-frame points meanwhile (they need the scan preparation, not the ranking).
-__global__ void __launch_bounds__(kTopkThreads) k_topk(const ReqDesc *__restrict__ reqs, int Kp_cap, int stage_cap,
-                                                       int R, int max_n_orient, int icp_chunks) {
+__global__ void __launch_bounds__(kTopkThreads) k_topk(const ReqDesc *__restrict__ reqs, int Kp_cap, int R,
+                                                       int max_n_orient, int off_block, int icp_chunks) {
     extern __shared__ __align__(16) unsigned long long sm[];
     chain_wait();
     chain_go();
     if ((int)blockIdx.x >= R) {
-        for (int t = (int)blockIdx.x - R; t < R * max_n_orient; t += (int)gridDim.x - R) {
-            const ReqDesc &o = reqs[t / max_n_orient];
-            const int q = t % max_n_orient;
-            if (q < o.n_orient && !o.state->done && o.tam_offs) tam_offsets_one(o, q);
+        const int blocks = (max_n_orient + off_block - 1) / off_block;
+        for (int t = (int)blockIdx.x - R; t < R * blocks; t += (int)gridDim.x - R) {
+            const ReqDesc &o = reqs[t / blocks];
+            const int q = t % blocks * off_block;
+            if (q < o.n_orient && !o.state->done && o.tam_offs) tam_offsets_block(o, q, min(off_block, o.n_orient - q));
         }
         for (int t = (int)gridDim.x - 1 - (int)blockIdx.x; t < R * icp_chunks; t += (int)gridDim.x - R)
             if (reqs[t / icp_chunks].icp_iters > 0) icp_points_chunk(reqs[t / icp_chunks], t % icp_chunks);
         return;
     }
     const ReqDesc &d = reqs[blockIdx.x];
-    topk_request(d, sm, Kp_cap, stage_cap);
+    topk_request(d, sm, Kp_cap);
     __syncthreads();   // every survivor is written
-    tam_chunks_one(d);
+    tam_chunks_one(d, reinterpret_cast<int2 *>(sm));   // room for 2 Kp_cap >= K cells
 }
 
 // The request's pose, score and counters into its relo_result (one thread).
@@ -412,16 +469,15 @@ cudaError_t launch_topk(const ReqDesc *reqs, int R, int max_n_hyp, int max_K, in
                         cudaStream_t s) {
     int Kp = 1;
     while (Kp < max_K) Kp <<= 1;
-    const size_t fixed = (size_t)2 * Kp * 8 + (size_t)kTopkBins * 4;
-    const size_t smem_max = 227 * 1024;
-    const int stage_cap = (max_n_hyp <= kStageMax && fixed + (size_t)max_n_hyp * 8 <= smem_max) ? max_n_hyp : 0;
-    const size_t smem = fixed + (size_t)stage_cap * 8;
+    const size_t smem = (size_t)2 * Kp * 8 + (size_t)kTopkBins * 4;
     const cudaError_t e = allow_smem((const void *)k_topk, smem);
     if (e != cudaSuccess) return e;
-    // one CTA per SM for the offsets (the ranking CTAs' shared memory leaves room for no second one)
-    const int n_off = std::max(1, std::min(R * std::max(max_n_orient, 1), n_sm));
-    return launch_chained(k_topk, dim3((unsigned)(R + n_off)), kTopkThreads, smem, s, reqs, Kp, stage_cap, R,
-                          std::max(max_n_orient, 1), (icp_beams + 31) / 32);
+    // one CTA per SM for the offsets
+    const int n_orient = std::max(max_n_orient, 1), n_off = std::max(1, std::min(R * n_orient, n_sm));
+    // orientations per task: as many as leave every CTA a task, at most the loads a thread keeps in flight
+    const int off_block = std::max(1, std::min(R * n_orient / n_off, kOffBlock));
+    return launch_chained(k_topk, dim3((unsigned)(R + n_off)), kTopkThreads, smem, s, reqs, Kp, R, n_orient, off_block,
+                          (icp_beams + 31) / 32);
 }
 
 cudaError_t launch_select_batch(const ReqDesc *reqs, int R, int batch_lo, int batch_hi, bool last, bool icp,

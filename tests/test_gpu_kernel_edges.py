@@ -5,7 +5,7 @@ import pytest
 
 import oracle
 import workloads
-from test_gpu_parity import full_case, relo, small_case   # noqa: F401  (relo: the module fixture)
+from test_gpu_parity import full_case, relo, run, small_case, stages   # noqa: F401  (relo: the module fixture)
 
 pytestmark = pytest.mark.gpu
 RES = 0.05
@@ -255,3 +255,24 @@ def test_smad_single_orientation_rows(relo, ns, gap):
         z, a = wl.ranges.copy(), wl.angles
         w = workloads.Workload("row", wl.grid, wl.res, wl.hyps, z[keep], a[keep], wl.max_range, wl.n_orient, 8, ns, (0, 0, 0))
         full_case(relo, w, 12, batch=5, local_topk=2)[0].close()
+
+
+@pytest.mark.parametrize("copies,K", [(1, 30), (40, 700), (128, 30), (140, 700), (140, 1023), (600, 700), (200, 5), (700, 700),
+                                      (700, 5)])
+def test_topk_digits(relo, copies, K):
+    """Hypotheses repeated so that many keys share a leading digit (ranks counted in short digits, long digits sorted,
+    more keys of the last digit than are sorted; keys held in registers and not): survivors equal the oracle's ranking of the same numerators."""
+    wl = small_case()
+    hyps = np.repeat(wl.hyps, copies, axis=0)
+    ctx, _, got = run(relo, wl.grid, wl.res, hyps, wl.ranges, wl.angles, wl.max_range, n_orient=wl.n_orient, topk=K,
+                      batch=256, local_topk=2, early_stop=0)
+    nb = -(-K // min(256, K))
+    st = stages(relo, ctx, len(hyps), K, wl.n_orient, nb, 2)
+    assert got.status == 0 and np.array_equal(st["surv"], oracle.rank(st["num"], K))
+    ctx.close()
+
+
+@pytest.mark.parametrize("n_orient", [305, 610, 1220])
+def test_offsets_of_several_orientations_per_task(relo, n_orient):
+    """Endpoint tables by blocks of 2, 4 and 8 orientations with a remainder: scores against the oracle (full_case)."""
+    full_case(relo, small_case(n_beams=70, ns=1220, n_orient=n_orient), 3, batch=3, local_topk=2)[0].close()
