@@ -276,3 +276,27 @@ def test_topk_digits(relo, copies, K):
 def test_offsets_of_several_orientations_per_task(relo, n_orient):
     """Endpoint tables by blocks of 2, 4 and 8 orientations with a remainder: scores against the oracle (full_case)."""
     full_case(relo, small_case(n_beams=70, ns=1220, n_orient=n_orient), 3, batch=3, local_topk=2)[0].close()
+
+
+@pytest.mark.parametrize("K,batch", [(30, 1), (700, 200), (1024, 16), (1300, 300), (2100, 1024)])
+def test_select_batches_ranked_together(relo, K, batch):
+    """Local top-k lists of many small batches, of a short last one, and of more positions than are ranked at once: the
+    order of each batch's best scores (ties to the earlier survivor), and the best of all batches."""
+    wl = small_case()
+    hyps = np.repeat(wl.hyps, 70, axis=0)
+    L = min(20, batch)
+    ctx, _, got = run(relo, wl.grid, wl.res, hyps, wl.ranges, wl.angles, wl.max_range, n_orient=wl.n_orient, topk=K,
+                      batch=batch, local_topk=L, early_stop=0)
+    nb = -(-K // batch)
+    st = stages(relo, ctx, len(hyps), K, wl.n_orient, nb, L)
+    best = st["T"].max(axis=1)
+    for b in range(nb):
+        mine = best[b * batch:(b + 1) * batch]
+        want = np.full(L, -1)
+        order = np.argsort(-mine, kind="stable")[:L] + b * batch
+        want[:len(order)] = order
+        assert np.array_equal(st["local"][b], want)
+    top = int(np.argmax(best))
+    assert got.status == 0 and got.n_batches == nb and got.n_tam_evals == K * wl.n_orient
+    assert got.hyp == st["surv"][top] and got.tam == best[top]
+    ctx.close()
