@@ -413,7 +413,6 @@ TamPlan plan_tam(const int *batch_lo, const int *batch_hi, int R, int max_beams,
 // TAM's work order (surv_perm, tam_chunks, chunk_cnt) of every request, after the top-K
 // per-lane stride of the TAM endpoint offsets of a values-per-lane class
 int tam_offs_stride_for(int vpl);
-// every request's TAM endpoint offsets for all band phases and orientations (after the scan preparation)
 cudaError_t launch_tam(const ReqDesc *reqs, int R, TamSeg *segs, const TamPlan &tp, BatchState *bs, cudaStream_t s);
 // selection of batch indexes batch_lo .. batch_hi - 1 in order; with last, also every request's result.
 // With icp, only the local top-k (launch_icp and launch_icp_best take the rest).

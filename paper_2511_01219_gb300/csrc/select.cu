@@ -104,8 +104,8 @@ struct KeyDigits {
     }
 };
 // Keys of one digit up to which ranks are counted within the digit: the longest digit is then one short loop per key,
-// where the sorting network takes 55 to 66 barriers for 1024 to 2048 keys (20 us; digits of 128 to 512 keys in a request
-// of 20000, K = 1024: stage 38 us sorted, 20 us counted).
+// where the sorting network takes 55 to 66 barriers for 1024 to 2048 keys (42000 cycles
+// for the 1024 of 20000).
 constexpr int kDigitRankMax = 512;
 
 // The first K keys of request d in ascending order into its survivor list,
