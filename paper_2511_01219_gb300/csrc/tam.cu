@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(1024) k_scan_prep(const ReqDesc *__restrict__ 
 // each of 4 to 6 CTAs per SM left the gathers a third of L1.  TAM, us, before
 // and with the stages: 256 survivors x 360 orientations x 1081 beams 140 -> 117,
 // 1024 x 720 x 1440 1127 -> 1060, 16 mixed requests 2733 -> 2140; with ranks,
-// conflict-free lookups and one CTA per SM 115, 1010 and 1994 (the L1 data path
+// conflict-free lookups and one CTA per SM 112, 975 and 1973 (the L1 data path
 // is then 96% busy in the 1024 x 720 launch).
 //
 // Selection.  The k-th smallest clamped d2 of a survivor rarely changes from
@@ -172,10 +172,12 @@ __global__ void __launch_bounds__(1024) k_scan_prep(const ReqDesc *__restrict__ 
 constexpr int kTamQ = 4;
 constexpr int kTamStages = 8;   // at most
 
-// Warps of the SM's CTA by values-per-lane class: the register budget they leave each other (64 up to 40 values, 72
-// above) against the warps that hide the gathers.  Measured with two CTAs of half as many (TAM, us): 34 values 48 / 40 /
-// 32 / 28 / 24 warps 136 / 120 / 117 / 121 / 179; 46 values 40 / 32 / 28 / 24 warps 1214 / 1069 / 1060 / 1089.
-__host__ __device__ constexpr int tam_warps(int vpl) { return vpl <= 40 ? 32 : 28; }
+// Warps of the SM's CTA by values-per-lane class: the register budget they leave each other (64 for up to 24 values, then
+// 72, 80 and 96; fewer spill) against the warps that hide the gathers.  Measured (TAM, us): 18 values 32 / 30 / 28 warps
+// 101 / 102 / 103; 30 values 32 / 28 / 24 177 / 175 / 176; 34 values 32 / 28 / 24 / 20 202 / 198 / 197 / 204; 38 values
+// 220 / 213 / 213 / 213; 46 values 32 / 28 / 24 / 22 / 20 / 16 (1024 x 720) 1152 / 1009 / 975 / 989 / 975 / 1070; 64
+// values 28 / 24 / 20 / 16 395 / 360 / 327 / 384.  An even share of the four schedulers counts: 24 and 20, not 22.
+__host__ __device__ constexpr int tam_warps(int vpl) { return vpl <= 24 ? 32 : vpl <= 30 ? 28 : vpl <= 40 ? 24 : 20; }
 
 // One staged task.
 struct TamTask {
