@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(1024) k_scan_prep(const ReqDesc *__restrict__ 
 // and with the stages: 256 survivors x 360 orientations x 1081 beams 140 -> 117,
 // 1024 x 720 x 1440 1127 -> 1060, 16 mixed requests 2733 -> 2140; with ranks,
 // conflict-free lookups and one CTA per SM 112, 975 and 1973 (the L1 data path
-// is then 96% busy in the 1024 x 720 launch).
+// is then 95% busy in the 1024 x 720 launch).
 //
 // Selection.  The k-th smallest clamped d2 of a survivor rarely changes from
 // one orientation to the next (neighbouring orientations see nearly the same
