@@ -364,15 +364,15 @@ __global__ void __launch_bounds__(kFarThreads) k_edt_far(EdtTiles t, EdtOut o, i
             if (threadIdx.x == 0) s_n = 0;
             __syncthreads();
             const int items = R * groups;
+            int n = 0;   // groups on the list: the barrier's own count, since the next round's appends change s_n at once
             for (int i0 = 0; i0 < items; i0 += kFarThreads) {
                 const int it = i0 + (int)threadIdx.x, u = it / groups, x0 = 4 * (it - u * groups), y = y0 + u0 + u;
+                bool any = false;
                 if (it < items && y >= 0 && y < t.H) {
-                    bool any = false;
                     for (int i = 0; i < 4; ++i) any = any || (x0 + i < t.W && o.d2[(size_t)y * t.W + x0 + i] == kFarMark);
                     if (any) s_list[atomicAdd(&s_n, 1)] = u << 16 | x0;
                 }
-                __syncthreads();
-                const int n = s_n;
+                n += __syncthreads_count(any);
                 if (n > kFarList - kFarThreads || i0 + kFarThreads >= items) {   // the list is full, or complete
                     for (int k = threadIdx.x; k < n; k += kFarThreads) {
                         const int lu = s_list[k] >> 16, lx = s_list[k] & 0xffff, ly = y0 + u0 + lu;
@@ -411,6 +411,7 @@ __global__ void __launch_bounds__(kFarThreads) k_edt_far(EdtTiles t, EdtOut o, i
                     }
                     __syncthreads();
                     if (threadIdx.x == 0) s_n = 0;
+                    n = 0;
                     __syncthreads();
                 }
             }

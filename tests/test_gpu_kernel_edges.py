@@ -300,3 +300,26 @@ def test_select_batches_ranked_together(relo, K, batch):
     assert got.status == 0 and got.n_batches == nb and got.n_tam_evals == K * wl.n_orient
     assert got.hyp == st["surv"][top] and got.tam == best[top]
     ctx.close()
+
+
+@pytest.mark.parametrize("shape,at", [
+    ((30, 1300), (0, 0)),      # rows of 8 whose far cells fill the list of the 32-bit pass once and more
+    ((41, 2100), (20, 1050)),  # on both sides of the occupied cell
+    ((20, 8300), (3, 4)),      # wider than 8192: 4 rows at a time, several lists
+])
+def test_edt_lists_of_far_cells(relo, shape, at):
+    """Bands with more groups of far cells than one list of the 32-bit pass holds, several times over: the oracle's
+    distances and field in every update."""
+    import torch
+    g = np.zeros(shape, np.int8)
+    g[at] = 100
+    want = oracle.edt(g)
+    ctx = relo.Relo(max_range=5.0)
+    gt = torch.from_numpy(g).cuda()
+    mid = ctx.load_map_dev(gt, RES)
+    for _ in range(8):
+        d2, field, _ = (t.cpu().numpy() for t in ctx.map_tables(mid, shape))
+        assert np.array_equal(d2, want)
+        assert np.array_equal(field, np.minimum(want, 1600))
+        ctx.update_map_dev(mid, gt)
+    ctx.close()
