@@ -284,7 +284,8 @@ __global__ void __launch_bounds__(kCols / 4 * kSplit) k_edt_band(EdtTiles t, Edt
         }
     }
     bool far = false;
-    const bool whole = x0 + 4 <= t.W && (t.W & 3) == 0;
+    // 16-byte stores where every row of d2 is aligned for them: the allocation-free entry point's output is the caller's
+    const bool whole = x0 + 4 <= t.W && (t.W & 3) == 0 && (reinterpret_cast<uintptr_t>(o.d2) & 15) == 0;
 #pragma unroll
     for (int u = 0; u < 2 * kPairs; ++u) {
         const int y = y0 + 2 * p0 + u;

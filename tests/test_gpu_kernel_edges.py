@@ -323,3 +323,23 @@ def test_edt_lists_of_far_cells(relo, shape, at):
         assert np.array_equal(field, np.minimum(want, 1600))
         ctx.update_map_dev(mid, gt)
     ctx.close()
+
+
+@pytest.mark.parametrize("shape", [(1, 4), (9, 256), (70, 300), (33, 1024)])   # rows of a multiple of 4 cells
+def test_edt_noalloc_output_at_any_int(relo, shape):
+    """An output that starts at any int32 of a buffer (a part of the caller's own pool), with a guard on both sides."""
+    import torch
+    H, W = shape
+    g = np.zeros(shape, np.int8)
+    g[np.random.default_rng(4).random(shape) < 0.01] = 100
+    g[0, 0] = 100
+    want = oracle.edt(g)
+    gt = torch.from_numpy(g).cuda()
+    for first in (4, 5, 6, 7):   # 0 to 3 ints past a 16-byte boundary
+        pool = torch.full((H * W + 12,), 7, dtype=torch.int32, device="cuda")
+        assert pool.data_ptr() % 16 == 0
+        assert relo.lib().relo_edt_noalloc(gt.data_ptr(), W, H, pool.data_ptr() + 4 * first,
+                                           torch.cuda.current_stream().cuda_stream) == 0
+        got = pool.cpu().numpy()
+        assert np.array_equal(got[first:first + H * W].reshape(shape), want)
+        assert (got[:first] == 7).all() and (got[first + H * W:] == 7).all()
