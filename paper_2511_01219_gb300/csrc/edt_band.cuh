@@ -341,6 +341,7 @@ __global__ void __launch_bounds__(kCols / 4 * kSplit) k_edt_band(EdtTiles t, Edt
 constexpr int kFarThreads = 256;
 constexpr int kFarNone = 30000;               // no occupied cell in the column: its square is above any distance
 constexpr int kFarList = 8 * kFarThreads;
+constexpr size_t kFarStatic = sizeof(int) * kFarList + 64;   // k_edt_far's static shared memory at most
 
 __host__ __device__ inline int far_rows(int W) { return W <= 8192 ? 8 : 4; }
 __host__ __device__ inline int far_width(int W) { return (W + 3) & ~3; }
@@ -436,7 +437,7 @@ inline cudaError_t launch_edt_bands(const EdtTiles &t, const EdtOut &o, int n_sm
     else
         k_edt_band<256, 2><<<dim3(strips(256), bands), 128, code, s>>>(t, o);
     const size_t smem = (size_t)far_rows(t.W) * far_width(t.W) * sizeof(uint16_t);
-    if (smem > 48 * 1024) {
+    if (smem > 48 * 1024 - kFarStatic) {   // without leave, a kernel has 48 KB for both
         const cudaError_t e = cudaFuncSetAttribute(k_edt_far, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }

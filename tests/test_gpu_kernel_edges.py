@@ -1,5 +1,9 @@
 """Kernels at the sizes where their tiling changes: remainders of tiles and
 stages, the smallest and the largest of a range, both sides of a dispatch."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -343,3 +347,27 @@ def test_edt_noalloc_output_at_any_int(relo, shape):
         got = pool.cpu().numpy()
         assert np.array_equal(got[first:first + H * W].reshape(shape), want)
         assert (got[:first] == 7).all() and (got[first + H * W:] == 7).all()
+
+
+def load_widths(widths):
+    """Maps of these widths in this order: tables equal to the oracle's."""
+    import paper_2511_01219_gb300 as relo
+    for W in widths:
+        g = np.zeros((21, W), np.int8)
+        g[np.random.default_rng(W).random(g.shape) < 0.005] = 100
+        g[:, W // 2 - 200:W // 2 + 200] = 0   # far cells in the middle
+        want = oracle.edt(g)
+        ctx = relo.Relo(max_range=5.0)
+        mid = ctx.load_map(g, RES)
+        d2, field, _ = (t.cpu().numpy() for t in ctx.map_tables(mid, g.shape))
+        ctx.close()
+        assert np.array_equal(d2, want) and np.array_equal(field, np.minimum(want, 1600)), W
+
+
+def test_map_widths_around_the_shared_memory_limits(relo):
+    """Widths on both sides of the sizes at which the 32-bit pass asks for more shared memory than a kernel gets unasked,
+    and takes 4 rows at a time; smallest first, in a process where no wider map has asked for more before."""
+    here = os.path.dirname(os.path.abspath(__file__))
+    code = "import test_gpu_kernel_edges as t; t.load_widths([2535, 2560, 2800, 3072, 3073, 8192, 8193])"
+    subprocess.check_call([sys.executable, "-c", code], cwd=here,
+                          env={**os.environ, "PYTHONPATH": os.pathsep.join([here, os.path.dirname(here)])}, timeout=300)
