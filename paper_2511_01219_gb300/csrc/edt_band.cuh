@@ -22,6 +22,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "relo_internal.h"
+
 namespace {
 
 constexpr int kSegTiles = 8;          // tile rows per column segment
@@ -438,7 +440,7 @@ inline cudaError_t launch_edt_bands(const EdtTiles &t, const EdtOut &o, int n_sm
         k_edt_band<256, 2><<<dim3(strips(256), bands), 128, code, s>>>(t, o);
     const size_t smem = (size_t)far_rows(t.W) * far_width(t.W) * sizeof(uint16_t);
     if (smem > 48 * 1024 - kFarStatic) {   // without leave, a kernel has 48 KB for both
-        const cudaError_t e = cudaFuncSetAttribute(k_edt_far, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = relo::allow_smem((const void *)k_edt_far, smem);
         if (e != cudaSuccess) return e;
     }
     k_edt_far<<<bands < 2 * n_sm ? bands : 2 * n_sm, kFarThreads, smem, s>>>(t, o, bands);
