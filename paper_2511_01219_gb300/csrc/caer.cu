@@ -138,15 +138,15 @@ __global__ void __launch_bounds__(kCaerWarps * 32) k_caer(const ReqDesc *__restr
             int held = 0;
             for (int v = 0; v < d.n_iv; ++v) {
                 const int2 iv = d.iv[v];
-                // the beam on the interval's first direction (the beams are in cyclic order, b_0 anywhere): the beam
+                // the beam on the interval's first direction (b_cyc and Rall are in cyclic order, b_0 anywhere): the beam
                 // whose direction lies (iv.x - b_0) mod N_s past the first's, found by bisection
-                const int b0 = __ldg(d.b);
+                const int b0 = __ldg(d.b_cyc);
                 int want = iv.x - b0;
                 if (want < 0) want += ns;
                 int bl = 0, bh = n - 1;
                 while (bl < bh) {
                     const int mid = (bl + bh) >> 1;
-                    int at = __ldg(d.b + mid) - b0;
+                    int at = __ldg(d.b_cyc + mid) - b0;
                     if (at < 0) at += ns;
                     if (at < want) bl = mid + 1;
                     else bh = mid;

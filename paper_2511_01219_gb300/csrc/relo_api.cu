@@ -34,6 +34,8 @@ struct SensorPlan {
     std::vector<int32_t> b;
     std::vector<int2> D, iv;
     int32_t *b_dev = nullptr;
+    // beams listed out of cyclic order only: [n] their directions in cyclic order from b_0, [n] every beam's place there
+    int32_t *cyc_dev = nullptr;
     int2 *D_dev = nullptr, *iv_dev = nullptr;
     size_t bytes = 0;
     unsigned long long last_use = 0;
@@ -410,6 +412,7 @@ int build_pairing(relo_ctx *ctx, MapSlot &m) {
 
 void free_plan(relo_ctx *ctx, SensorPlan *P) {
     dev_free(ctx, P->b_dev, sizeof(int32_t) * P->b.size());
+    dev_free(ctx, P->cyc_dev, 2 * sizeof(int32_t) * P->b.size());
     dev_free(ctx, P->D_dev, sizeof(int2) * P->D.size());
     dev_free(ctx, P->iv_dev, sizeof(int2) * P->iv.size());
     delete P;
@@ -477,6 +480,20 @@ int plan_for(relo_ctx *ctx, const float *angles_raw, int n_raw, SensorPlan **out
             }
         }
     }
+    // the beams' cyclic order from b_0; cyc stays empty when they are listed in it
+    const int32_t b0 = b[0];
+    auto turn = [&](int32_t bi) { return bi >= b0 ? bi - b0 : bi - b0 + (int32_t)ns; };
+    std::vector<int32_t> cyc;
+    if (!std::is_sorted(b.begin(), b.end(), [&](int32_t x, int32_t y) { return turn(x) < turn(y); })) {
+        std::vector<int32_t> at((size_t)n);
+        for (int i = 0; i < n; ++i) at[i] = i;
+        std::sort(at.begin(), at.end(), [&](int32_t x, int32_t y) { return turn(b[x]) < turn(b[y]); });
+        cyc.resize(2 * (size_t)n);
+        for (int k = 0; k < n; ++k) {
+            cyc[k] = b[at[k]];
+            cyc[(size_t)n + at[k]] = k;
+        }
+    }
     // directions D_j = llround((cos, sin)(2 pi j / N_s) * 2^30)
     std::vector<int2> D((size_t)ns);
     for (long long j = 0; j < ns; ++j) {
@@ -505,12 +522,16 @@ int plan_for(relo_ctx *ctx, const float *angles_raw, int n_raw, SensorPlan **out
     P->n_orient_param = ctx->p.n_orient;
     int rc;
     if ((rc = dev_alloc(ctx, (void **)&P->b_dev, sizeof(int32_t) * n, "plan beams")) ||
+        (!cyc.empty() && (rc = dev_alloc(ctx, (void **)&P->cyc_dev, sizeof(int32_t) * cyc.size(), "plan beams"))) ||
         (rc = dev_alloc(ctx, (void **)&P->D_dev, sizeof(int2) * ns, "plan directions")) ||
         (rc = dev_alloc(ctx, (void **)&P->iv_dev, sizeof(int2) * iv.size(), "plan intervals"))) {
         free_plan(ctx, P);
         return rc;
     }
     CK(cudaMemcpyAsync(P->b_dev, b.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, ctx->stream), "plan upload");
+    if (!cyc.empty())
+        CK(cudaMemcpyAsync(P->cyc_dev, cyc.data(), sizeof(int32_t) * cyc.size(), cudaMemcpyHostToDevice, ctx->stream),
+           "plan upload");
     CK(cudaMemcpyAsync(P->D_dev, D.data(), sizeof(int2) * ns, cudaMemcpyHostToDevice, ctx->stream), "plan upload");
     CK(cudaMemcpyAsync(P->iv_dev, iv.data(), sizeof(int2) * iv.size(), cudaMemcpyHostToDevice, ctx->stream),
        "plan upload");
@@ -1128,6 +1149,8 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R, HostScans
         d.n_hyp = m.n_hyp;
         d.D = P.D_dev;
         d.b = P.b_dev;
+        d.b_cyc = P.cyc_dev ? P.cyc_dev : P.b_dev;
+        d.place = P.cyc_dev ? P.cyc_dev + P.n : nullptr;
         d.iv = P.iv_dev;
         d.ns = P.ns;
         d.ns_pad = (P.ns + 31) & ~31;

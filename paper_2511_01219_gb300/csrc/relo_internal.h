@@ -243,6 +243,8 @@ struct ReqDesc {
     // sensor plan
     const int2 *D;               // [ns] Q30 directions
     const int32_t *b;            // [n_beams] panoramic index per beam
+    const int32_t *b_cyc;        // [n_beams] the same in cyclic order from the first beam's
+    const int32_t *place;        // [n_beams] every beam's place in that order; nullptr: the beams are listed in it
     const int2 *iv;              // [n_iv] (u, len) FoV intervals
     int ns, ns_pad, n_iv, n_beams, n_orient, n_enum, n_m;
     int lim;                     // floor(rmax_q16^2 / 2^32)
@@ -258,7 +260,7 @@ struct ReqDesc {
     long long n_smad_evals;
     // buffers
     int2 *vbR;                   // [n_beams]
-    int32_t *Rall;               // [n_beams] every beam's Q16 range in beam order, 0 for an invalid beam (CAER)
+    int32_t *Rall;               // [n_beams] every beam's Q16 range in the beams' cyclic order, 0 for an invalid beam (CAER)
     ScanInfo *scan;
     unsigned long long *keys;    // [n_hyp]
     long long *smad_num;         // [n_hyp]

@@ -371,3 +371,18 @@ def test_map_widths_around_the_shared_memory_limits(relo):
     code = "import test_gpu_kernel_edges as t; t.load_widths([2535, 2560, 2800, 3072, 3073, 8192, 8193])"
     subprocess.check_call([sys.executable, "-c", code], cwd=here,
                           env={**os.environ, "PYTHONPATH": os.pathsep.join([here, os.path.dirname(here)])}, timeout=300)
+
+
+@pytest.mark.parametrize("order", ["sensors", "swapped", "late_start"])
+@pytest.mark.parametrize("coarse", [0, 1])
+def test_beams_out_of_cyclic_order(relo, coarse, order):
+    """Scans whose beams are not listed in cyclic order but pass the grid's checks: three sensors one after the other, two
+    neighbours swapped, and both with a first beam in the middle of an interval.  SMAD's and CAER's numerators, shifts and
+    survivors equal the oracle's, which takes every beam by its own direction."""
+    wl = small_case(n_beams=40, ns=40, n_orient=20)
+    idx = {"sensors": [*range(10), *range(20, 30), *range(10, 20)],
+           "swapped": [0, 1, 2, 4, 3, *range(5, 30)],
+           "late_start": [*range(5, 12), *range(14, 30), 3, 4, 1, 2, 0]}[order]
+    wl.ranges, wl.angles = wl.ranges[idx].copy(), wl.angles[idx].copy()
+    wl.ranges[::7] = 100.0   # invalid beams
+    full_case(relo, wl, 12, batch=5, local_topk=2, coarse=coarse)[0].close()
