@@ -1932,7 +1932,7 @@ int relo_relocalize_batch(relo_ctx *ctx, const relo_request *reqs, int32_t n, re
        "result download");
     CK(cudaStreamSynchronize(ctx->stream), "relocalize");
     for (int i = 0; i < n; ++i)
-        if (out[i].status != RELO_OK) return fail(ctx, out[i].status, "a scan has no valid beam");
+        if (out[i].status != RELO_OK) return fail(ctx, out[i].status, result_error(out[i].status));
     return RELO_OK;
 }
 

@@ -5,7 +5,14 @@
 #include <stdint.h>
 #include <string.h>
 
+#include "../../include/relo.h"
+
 namespace relo {
+
+// what a result that is not RELO_OK reports (finalize_request, select.cu)
+inline const char *result_error(int status) {
+    return status == RELO_E_CUDA ? "the TAM kernel gave up waiting for a staged task" : "a scan has no valid beam";
+}
 
 constexpr int kTile = 8;               // the occupancy bitmap is stored in 8x8-cell tiles
 // metric codes of relo_params::coarse_metric / fine_metric
