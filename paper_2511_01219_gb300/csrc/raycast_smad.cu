@@ -346,9 +346,14 @@ __device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long v)
     return v;
 }
 
-// shared memory of one SMAD warp: in-chunk prefixes [ns_pad + 32] and chunk prefixes [ns_pad / 32 + 1]
+// shared memory of one SMAD warp: in-chunk prefixes [ns_pad + 32] of type P and chunk prefixes [ns_pad / 32 + 1]
+template <typename P>
+__host__ __device__ __forceinline__ size_t smad_inner_bytes(int ns_pad) {
+    return ((size_t)(ns_pad + 32) * sizeof(P) + 7) & ~(size_t)7;
+}
+template <typename P>
 __host__ __device__ __forceinline__ size_t smad_warp_bytes(int ns_pad) {
-    return ((((size_t)(ns_pad + 32) * 4 + 7) & ~(size_t)7) + (size_t)(ns_pad / 32 + 1) * 8 + 15) & ~(size_t)15;
+    return (smad_inner_bytes<P>(ns_pad) + (size_t)(ns_pad / 32 + 1) * 8 + 15) & ~(size_t)15;
 }
 
 // Casting.  The batch's rays form one list of work items (request r owns
@@ -461,6 +466,8 @@ __device__ __forceinline__ long long lane_sum(const uint32_t *__restrict__ row, 
 // on average x 540 to 2880 ranges: 304 us with one range per lane, 189 with
 // four (2, 4 or 5 blocks in flight instead of 6: 227, 210, 202); 20000 x 1440
 // row sums 62 and 37 us (115 MB: 17 us at the copy rate).
+// P: the type of a chunk's prefixes, 32 bits while 32 ranges fit them (kSmadNarrowLim), else 64 (one range per lane).
+template <typename P>
 __global__ void __launch_bounds__(256) k_smad(const ReqDesc *__restrict__ reqs, int R, int total_hyp,
                                               BatchState *bs, int warp_bytes) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -508,10 +515,10 @@ __global__ void __launch_bounds__(256) k_smad(const ReqDesc *__restrict__ reqs, 
             }
             continue;
         }
-        uint32_t *inner = reinterpret_cast<uint32_t *>(mine);
-        long long *chunkP = reinterpret_cast<long long *>(mine + (((size_t)(ns_pad + 32) * 4 + 7) & ~(size_t)7));
+        P *inner = reinterpret_cast<P *>(mine);
+        long long *chunkP = reinterpret_cast<long long *>(mine + smad_inner_bytes<P>(ns_pad));
         long long carry = 0;
-        if ((ns & 3) == 0) {
+        if (sizeof(P) == 4 && (ns & 3) == 0) {
             const uint4 *__restrict__ row4 = reinterpret_cast<const uint4 *>(row);
             const int n4 = ns >> 2, nblk = (ns_pad + 127) >> 7;
             for (int b0 = 0; b0 < nblk; b0 += kSmadVecs) {
@@ -557,10 +564,10 @@ __global__ void __launch_bounds__(256) k_smad(const ReqDesc *__restrict__ reqs, 
 #pragma unroll
             for (int u = 0; u < kSmadLoads; ++u) {
                 if (c0 + u >= nch) break;
-                uint32_t sc = r[u];
+                P sc = r[u];
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
-                    const uint32_t t = __shfl_up_sync(kFull, sc, o);
+                    const P t = __shfl_up_sync(kFull, sc, o);
                     if (lane >= o) sc += t;
                 }
                 inner[((c0 + u) << 5) + lane] = sc - r[u];
@@ -568,7 +575,7 @@ __global__ void __launch_bounds__(256) k_smad(const ReqDesc *__restrict__ reqs, 
                 carry += __shfl_sync(kFull, sc, 31);
             }
         }
-        inner[ns_pad + lane] = 0u;   // P(t) for t in [ns_pad, ns_pad + 32) adds nothing
+        inner[ns_pad + lane] = 0;   // P(t) for t in [ns_pad, ns_pad + 32) adds nothing
         if (lane == 0) chunkP[nch] = carry;
         __syncwarp();
         const long long sum_real = d.scan->sum_real;
@@ -621,6 +628,7 @@ __device__ __forceinline__ int list_request(const int *s_base, int R, int g) {  
     return lo;
 }
 
+template <typename P>   // as in k_smad
 __global__ void __launch_bounds__(256) k_win_build(const ReqDesc *__restrict__ reqs, int R, int total, int nm_pad_max) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_base[kMaxBatchRequests + 1];
@@ -639,17 +647,17 @@ __global__ void __launch_bounds__(256) k_win_build(const ReqDesc *__restrict__ r
         const ReqDesc &d = reqs[r];
         const int h = g - s_base[r];
         const int ns = d.ns, ns_pad = d.ns_pad, nch = ns_pad >> 5, n_m = d.n_m;
-        uint32_t *inner = reinterpret_cast<uint32_t *>(rest);
-        long long *chunkP = reinterpret_cast<long long *>(rest + (((size_t)(ns_pad + 32) * 4 + 7) & ~(size_t)7));
-        if (threadIdx.x < 32) inner[ns_pad + lane] = 0u;
+        P *inner = reinterpret_cast<P *>(rest);
+        long long *chunkP = reinterpret_cast<long long *>(rest + smad_inner_bytes<P>(ns_pad));
+        if (threadIdx.x < 32) inner[ns_pad + lane] = 0;
         const uint32_t *__restrict__ row = d.scan_table + (size_t)h * ns;
         for (int c = warp; c < nch; c += nwarps) {
             const int jj = (c << 5) + lane;
             const uint32_t rv = jj < ns ? __ldg(row + jj) : 0u;
-            uint32_t sc = rv;
+            P sc = rv;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t t = __shfl_up_sync(kFull, sc, o);
+                const P t = __shfl_up_sync(kFull, sc, o);
                 if (lane >= o) sc += t;
             }
             inner[jj] = sc - rv;
@@ -834,10 +842,14 @@ cudaError_t launch_cast(const ReqDesc *reqs, int R, int total_chunks, int cast_h
     return launch_chained(kern, dim3((unsigned)grid), kCastThreads, 0, s, reqs, R, total_chunks, bs);
 }
 
-cudaError_t launch_smad(const ReqDesc *reqs, int R, int total_hyp, int max_ns_pad, BatchState *bs, int n_sm,
+cudaError_t launch_smad(const ReqDesc *reqs, int R, int total_hyp, int max_ns_pad, bool wide, BatchState *bs, int n_sm,
                         cudaStream_t s) {
     if (R < 1 || R > kMaxBatchRequests) return cudaErrorInvalidValue;
-    const size_t wb = max_ns_pad > 0 ? smad_warp_bytes(max_ns_pad) : 0;   // no request takes prefixes: no scratch
+    void (*const kern)(const ReqDesc *, int, int, BatchState *, int) = wide ? k_smad<unsigned long long> : k_smad<uint32_t>;
+    // no request takes prefixes: no scratch
+    const size_t wb = max_ns_pad <= 0 ? 0
+                      : wide          ? smad_warp_bytes<unsigned long long>(max_ns_pad)
+                                      : smad_warp_bytes<uint32_t>(max_ns_pad);
     // warps per CTA: the most resident warps per SM that shared memory allows
     // (a long row's scratch fills an SM before its thread limit; smaller CTAs
     // waste less of it), the larger CTA on ties
@@ -845,7 +857,7 @@ cudaError_t launch_smad(const ReqDesc *reqs, int R, int total_hyp, int max_ns_pa
     for (int w = 8; w >= 1; --w) {
         if ((size_t)w * wb > (size_t)200 * 1024) continue;
         int o = 0;
-        const cudaError_t e = resident_ctas((const void *)k_smad, w * 32, (size_t)w * wb, &o);
+        const cudaError_t e = resident_ctas((const void *)kern, w * 32, (size_t)w * wb, &o);
         if (e != cudaSuccess) return e;
         if (o * w > occ * wpc) {
             wpc = w;
@@ -858,24 +870,26 @@ cudaError_t launch_smad(const ReqDesc *reqs, int R, int total_hyp, int max_ns_pa
     const long long need = ((long long)total_hyp + wpc - 1) / wpc;
     if (grid > need) grid = need;
     if (grid < 1) grid = 1;
-    return launch_chained(k_smad, dim3((unsigned)grid), wpc * 32, smem, s, reqs, R, total_hyp, bs, (int)wb);
+    return launch_chained(kern, dim3((unsigned)grid), wpc * 32, smem, s, reqs, R, total_hyp, bs, (int)wb);
 }
 
-cudaError_t launch_win_build(const ReqDesc *reqs, int R, int total, int max_ns_pad, int max_nm, cudaStream_t s) {
+cudaError_t launch_win_build(const ReqDesc *reqs, int R, int total, int max_ns_pad, int max_nm, bool wide,
+                             cudaStream_t s) {
     if (R < 1 || R > kMaxBatchRequests) return cudaErrorInvalidValue;
     if (total <= 0) return cudaSuccess;
+    void (*const kern)(const ReqDesc *, int, int, int) = wide ? k_win_build<unsigned long long> : k_win_build<uint32_t>;
     int nm_pad = 1;
     while (nm_pad < max_nm) nm_pad <<= 1;
-    const size_t smem = (size_t)nm_pad * 8 + (((size_t)(max_ns_pad + 32) * 4 + 7) & ~(size_t)7) +
-                        (size_t)(max_ns_pad / 32 + 1) * 8;
+    const size_t smem = (size_t)nm_pad * 8 + (size_t)(max_ns_pad / 32 + 1) * 8 +
+                        (wide ? smad_inner_bytes<unsigned long long>(max_ns_pad) : smad_inner_bytes<uint32_t>(max_ns_pad));
     int occ = 0, dev = 0, n_sm = 0;
-    cudaError_t e = resident_ctas((const void *)k_win_build, 256, smem, &occ);
+    cudaError_t e = resident_ctas((const void *)kern, 256, smem, &occ);
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     if (occ < 1) return cudaErrorInvalidConfiguration;
     const int grid = total < n_sm * occ ? total : n_sm * occ;
-    return launch_chained(k_win_build, dim3((unsigned)grid), 256, smem, s, reqs, R, total, nm_pad);
+    return launch_chained(kern, dim3((unsigned)grid), 256, smem, s, reqs, R, total, nm_pad);
 }
 
 cudaError_t launch_win_read(const ReqDesc *reqs, int R, int total, cudaStream_t s) {

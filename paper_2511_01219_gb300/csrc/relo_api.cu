@@ -1088,6 +1088,7 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R, HostScans
     std::vector<size_t> off((size_t)R);
     size_t total = 0;
     int total_hyp = 0, max_ns_pad = 32, smad_ns_pad = 0, max_n_hyp = 1, max_K = 1, max_beams = 1, max_C = 0, max_reps = 0, max_batches = 0;
+    bool smad_wide = false;
     long long total_chunks = 0;
     for (int r = 0; r < R; ++r) {
         const Prepared &q = pr[r];
@@ -1107,6 +1108,7 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R, HostScans
         total_hyp += nh;
         max_ns_pad = std::max(max_ns_pad, (q.P->ns + 31) & ~31);
         if (q.P->n_m > 1) smad_ns_pad = std::max(smad_ns_pad, (q.P->ns + 31) & ~31);
+        smad_wide = smad_wide || q.lim >= kSmadNarrowLim;
         max_n_hyp = std::max(max_n_hyp, nh);
         max_K = std::max(max_K, K);
         max_beams = std::max(max_beams, n);
@@ -1308,11 +1310,11 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R, HostScans
                             return launch_caer(rq, R, total_smad, max_ns_pad, sl.bs, ctx->n_sm, st);
                         return p.coarse_metric == RELO_COARSE_SMAD_DIRECT
                                    ? launch_smad_direct(rq, R, total_smad, max_ns_pad, sl.bs, ctx->n_sm, st)
-                                   : launch_smad(rq, R, total_smad, smad_ns_pad, sl.bs, ctx->n_sm, st);
+                                   : launch_smad(rq, R, total_smad, smad_ns_pad, smad_wide, sl.bs, ctx->n_sm, st);
                     }),
            "SMAD");
     if (total_build > 0) {
-        CK(timed_on(ctx, st, 6, 1, [&] { return launch_win_build(rq, R, total_build, max_ns_pad, max_nm, st); }),
+        CK(timed_on(ctx, st, 6, 1, [&] { return launch_win_build(rq, R, total_build, max_ns_pad, max_nm, smad_wide, st); }),
            "SMAD window tables");
         for (auto &x : wnew.list) CK(cudaEventRecord(x.second->built, st), "window table");
     }

@@ -387,9 +387,11 @@ cudaError_t launch_scan_prep(const ReqDesc *reqs, int R, cudaStream_t s);
 cudaError_t launch_cast(const ReqDesc *reqs, int R, int total_chunks, int cast_hyps, BatchState *bs, int n_sm, int ctas_per_sm,
                         cudaStream_t s);
 // SMAD of every hypothesis of the batch from the requests' scan tables; max_ns_pad: the longest padded row of the
-// requests with more than one orientation, 0 when there is none
-cudaError_t launch_smad(const ReqDesc *reqs, int R, int total_hyp, int max_ns_pad, BatchState *bs, int n_sm,
+// requests with more than one orientation, 0 when there is none; wide: a request has lim >= kSmadNarrowLim
+cudaError_t launch_smad(const ReqDesc *reqs, int R, int total_hyp, int max_ns_pad, bool wide, BatchState *bs, int n_sm,
                         cudaStream_t s);
+// ranges below this squared limit are below 2048 cells (2^27 in Q16), so 32 of them sum to less than 2^32
+constexpr int kSmadNarrowLim = 2048 * 2048;
 // CAER of every hypothesis of the batch (caer.cu)
 cudaError_t launch_caer(const ReqDesc *reqs, int R, int total_hyp, int max_ns_pad, BatchState *bs, int n_sm,
                         cudaStream_t s);
@@ -399,7 +401,8 @@ cudaError_t launch_smad_direct(const ReqDesc *reqs, int R, int total_hyp, int ma
 // no coarse ranking: numerator 0 and m = 0 for every hypothesis of the batch (Table II's arm without SMAD ordering)
 cudaError_t launch_rank_by_index(const ReqDesc *reqs, int R, int total_hyp, int n_sm, cudaStream_t s);
 // SMAD of the window-build requests' hypotheses, storing their sorted window keys
-cudaError_t launch_win_build(const ReqDesc *reqs, int R, int total, int max_ns_pad, int max_nm, cudaStream_t s);
+cudaError_t launch_win_build(const ReqDesc *reqs, int R, int total, int max_ns_pad, int max_nm, bool wide,
+                             cudaStream_t s);
 // SMAD of the window-read requests' hypotheses by search in their window keys
 cudaError_t launch_win_read(const ReqDesc *reqs, int R, int total, cudaStream_t s);
 // the top-K of every request with its TAM work order, and beside it (extra blocks) every request's TAM endpoint offsets

@@ -386,3 +386,44 @@ def test_beams_out_of_cyclic_order(relo, coarse, order):
     wl.ranges, wl.angles = wl.ranges[idx].copy(), wl.angles[idx].copy()
     wl.ranges[::7] = 100.0   # invalid beams
     full_case(relo, wl, 12, batch=5, local_topk=2, coarse=coarse)[0].close()
+
+
+@pytest.mark.parametrize("n_beams,ns,n_orient", [(28, 32, 32), (50, 64, 16), (65, 97, 97), (300, 361, 361), (32, 32, 8),
+                                                 (2048, 8192, 64)])
+def test_smad_ranges_whose_chunks_pass_32_bits(relo, n_beams, ns, n_orient):
+    """Ranges of some 2300 cells: 32 of them sum to more than 2^32 in Q16.  Numerators and shifts equal the oracle's by
+    prefixes, by the window tables that a cached call builds, and when it reads them; a short-range request beside them."""
+    import torch
+    n = 4200
+    g = np.zeros((n, n), np.int8)
+    g[0] = g[-1] = 100
+    g[:, 0] = g[:, -1] = 100
+    hyps = np.array([[2100, 2100], [2060, 2130], [2155, 2045]], np.int32)
+    ang = workloads.beam_angles(n_beams, ns)
+    z = np.random.default_rng(ns).uniform(95.0, 145.0, n_beams).astype(np.float32)
+    prm = oracle.Params(n_orient=n_orient, topk=2)
+    pl = oracle.plan(z, ang, 150.0, RES, prm)
+    row, _, _ = oracle.synth_scan(g, 2100, 2100, pl)
+    assert int(row[:32].astype(np.int64).sum()) > 1 << 32
+    want, shift = oracle.coarse(g, hyps, pl, prm)
+    near = workloads.make_room(3, n=40, n_boxes=4)
+    near_hyps = np.argwhere(near == 0)[:3, ::-1].astype(np.int32)
+    near_z = np.where(z > 120.0, 1.0, 0.5).astype(np.float32)
+    near_want, _ = oracle.coarse(near, near_hyps, oracle.plan(near_z, ang, 4.0, RES, prm), prm)
+
+    def numerators(ctx):
+        k = len(hyps)
+        return (ctx.stage(relo.STAGE_SMAD_NUM, torch.empty(k, dtype=torch.int64, device="cuda")).cpu().numpy(),
+                ctx.stage(relo.STAGE_SMAD_M, torch.empty(k, dtype=torch.int32, device="cuda")).cpu().numpy())
+    for cache, calls in ((0, 1), (1 << 30, 3)):
+        ctx = relo.Relo(n_orient=n_orient, topk=2, early_stop=0, max_range=150.0, scan_cache_bytes=cache)
+        far_map, near_map = ctx.load_map(g, RES), ctx.load_map(near, RES)
+        ctx.set_hypotheses(far_map, workloads.cell_centres(hyps, RES))
+        ctx.set_hypotheses(near_map, workloads.cell_centres(near_hyps, RES))
+        for _ in range(calls):
+            ctx.relocalize(far_map, z, ang, 150.0)
+            num, m = numerators(ctx)
+            assert np.array_equal(num, want) and np.array_equal(m, shift)
+        ctx.relocalize_batch([(near_map, near_z, ang, 4.0), (far_map, z, ang, 150.0)])
+        assert np.array_equal(numerators(ctx)[0], near_want)   # the first request's stages
+        ctx.close()
