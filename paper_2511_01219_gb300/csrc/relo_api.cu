@@ -1119,6 +1119,7 @@ int run_batch(relo_ctx *ctx, BatchSlot &sl, const Prepared *pr, int R, HostScans
     // hypotheses per cast work item: group while every resident warp (5 CTAs of 8 warps per SM) keeps 16 or more items
     int cast_hyps = 1;
     while (cast_hyps < kCastHypsMax && total_chunks >= 16ll * 2 * cast_hyps * 40 * ctx->n_sm) cast_hyps *= 2;
+    if (total > sl.arena_cap && ctx->last_bs == sl.bs) ctx->has_last = false;   // ensure frees the last batch's scratch
     int rc = ensure(ctx, &sl.arena, &sl.arena_cap, total, "request scratch");
     if (rc) return rc;
     for (int r = 0; r < R; ++r) {
@@ -1385,6 +1386,7 @@ int slot_init(relo_ctx *ctx, BatchSlot &sl, cudaStream_t stream) {
 
 void slot_free(relo_ctx *ctx, BatchSlot &sl) {
     if (sl.stream) cudaStreamSynchronize(sl.stream);
+    if (ctx->last_bs == sl.bs) ctx->has_last = false;   // the last batch's stages go with its slot
     dev_free(ctx, sl.reqs_dev, slot_desc_bytes());
     dev_free(ctx, sl.bs, sizeof(BatchState));
     dev_free(ctx, sl.results_dev, sizeof(relo_result) * kMaxBatchRequests);

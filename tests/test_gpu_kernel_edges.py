@@ -427,3 +427,43 @@ def test_smad_ranges_whose_chunks_pass_32_bits(relo, n_beams, ns, n_orient):
         ctx.relocalize_batch([(near_map, near_z, ang, 4.0), (far_map, z, ang, 150.0)])
         assert np.array_equal(numerators(ctx)[0], near_want)   # the first request's stages
         ctx.close()
+
+
+def test_stages_end_with_the_scratch_they_lie_in(relo):
+    """The stages of a served batch once the server has stopped, and those of a call whose scratch a later call, too large
+    for the budget, has given up: an error, not a read of freed memory."""
+    import torch
+    wl = small_case()
+
+    def stage_error(ctx):
+        with pytest.raises(relo.ReloError) as e:
+            ctx.scan_info()
+        assert e.value.code == relo.E_NOT_FOUND
+        with pytest.raises(relo.ReloError) as e:
+            ctx.stage(relo.STAGE_SURVIVORS, torch.empty(64, dtype=torch.int32, device="cuda"))
+        assert e.value.code == relo.E_NOT_FOUND
+    ctx = relo.Relo(n_orient=40, topk=8)
+    mid = ctx.load_map(wl.grid, RES)
+    ctx.set_hypotheses(mid, workloads.cell_centres(wl.hyps, RES))
+    ctx.serve_start(4, 2)
+    t = ctx.submit(mid, wl.ranges, wl.angles, wl.max_range)
+    while ctx.poll(t) is None:
+        pass
+    ctx.serve_stop()
+    stage_error(ctx)
+    ctx.relocalize(mid, wl.ranges, wl.angles, wl.max_range)
+    assert ctx.scan_info()[0] == 120   # a call's own stages are there again
+    ctx.close()
+    many = np.repeat(wl.hyps, 1000, axis=0)
+    ctx = relo.Relo(n_orient=40, topk=8, max_range=wl.max_range, hbm_budget=8 << 20)   # less than the rows below alone
+    small = ctx.load_map(wl.grid, RES)
+    ctx.set_hypotheses(small, workloads.cell_centres(wl.hyps, RES))
+    large = ctx.load_map(wl.grid, RES)
+    ctx.set_hypotheses(large, workloads.cell_centres(many, RES))
+    ctx.relocalize(small, wl.ranges, wl.angles, wl.max_range)
+    assert ctx.scan_info()[0] == 120
+    with pytest.raises(relo.ReloError) as e:
+        ctx.relocalize(large, wl.ranges, wl.angles, wl.max_range)   # 30000 rows of 120 ranges: 14 MB
+    assert e.value.code == relo.E_OVER_BUDGET
+    stage_error(ctx)
+    ctx.close()
