@@ -39,6 +39,7 @@ struct SensorPlan {
     int2 *D_dev = nullptr, *iv_dev = nullptr;
     size_t bytes = 0;
     unsigned long long last_use = 0;
+    unsigned long long call = 0;   // the last call that took it (relo_ctx::plan_call)
 };
 
 // Resident synthesized scans of one map and hypothesis set for one beam grid
@@ -159,6 +160,7 @@ struct relo_ctx {
     std::vector<MapSlot> maps;
     std::vector<SensorPlan *> plans;
     unsigned long long plan_clock = 0;
+    unsigned long long plan_call = 0;   // counts the calls that take plans: a call's plans are not evicted by its own later ones
     std::string err;
     long long held = 0;
     // batches run by the calling thread use `main` (on the context stream)
@@ -420,7 +422,8 @@ void free_plan(relo_ctx *ctx, SensorPlan *P) {
 
 // The plan for these angles, from the cache or newly built (least recently
 // used plans are evicted beyond kMaxPlans; a plan in use by queued work is
-// never evicted because eviction first waits for the stream).
+// never evicted because eviction first waits for the stream, and one that the
+// present call has taken stays: a batch of more scans than that holds them all).
 int plan_for(relo_ctx *ctx, const float *angles_raw, int n_raw, SensorPlan **out) {
     const int skip = ctx->p.n_skip_beam;
     const int n = (n_raw + skip - 1) / skip;   // Eq. 11: beams 0, skip, 2 skip, ...
@@ -429,6 +432,7 @@ int plan_for(relo_ctx *ctx, const float *angles_raw, int n_raw, SensorPlan **out
     for (SensorPlan *P : ctx->plans) {
         if (P->n_skip == skip && P->n_orient_param == ctx->p.n_orient && P->angles == a) {
             P->last_use = ++ctx->plan_clock;
+            P->call = ctx->plan_call;
             *out = P;
             return RELO_OK;
         }
@@ -537,13 +541,15 @@ int plan_for(relo_ctx *ctx, const float *angles_raw, int n_raw, SensorPlan **out
        "plan upload");
     // the host vectors of this call must outlive the asynchronous copies
     CK(cudaStreamSynchronize(ctx->stream), "plan upload");
-    if ((int)ctx->plans.size() >= kMaxPlans) {
+    while ((int)ctx->plans.size() >= kMaxPlans) {
         auto it = std::min_element(ctx->plans.begin(), ctx->plans.end(),
                                    [](SensorPlan *x, SensorPlan *y) { return x->last_use < y->last_use; });
+        if ((*it)->call == ctx->plan_call) break;
         free_plan(ctx, *it);
         ctx->plans.erase(it);
     }
     P->last_use = ++ctx->plan_clock;
+    P->call = ctx->plan_call;
     ctx->plans.push_back(P);
     *out = P;
     return RELO_OK;
@@ -1585,6 +1591,7 @@ void serve_loop(relo_ctx *ctx) {
         }
         if (cand.empty()) continue;
         // admission: prepare in FIFO order while the HBM budget allows
+        ++ctx->plan_call;
         std::vector<Ticket *> batch;
         std::vector<Prepared> pr;
         std::vector<Ticket *> back;
@@ -1880,6 +1887,7 @@ int relo_relocalize_dev(relo_ctx *ctx, int32_t map_id, const float *ranges_dev, 
                         int32_t n_beams, float max_range, relo_result *result_dev) {
     if (!ctx) return RELO_E_INVALID_ARG;
     Prepared pr;
+    ++ctx->plan_call;
     int rc = prepare(ctx, map_id, ranges_dev, angles, n_beams, max_range, result_dev, &pr);
     if (rc) return rc;
     return run_batch(ctx, ctx->main, &pr, 1);
@@ -1896,6 +1904,7 @@ int relo_relocalize_batch_dev(relo_ctx *ctx, const relo_request *reqs, int32_t n
     if (!ctx || !reqs || !results_dev || n < 1 || n > kMaxBatchRequests)
         return fail(ctx, RELO_E_INVALID_ARG, "1 to 256 requests per batch");
     std::vector<Prepared> pr((size_t)n);
+    ++ctx->plan_call;
     for (int i = 0; i < n; ++i) {
         int rc = prepare(ctx, reqs[i].map_id, reqs[i].ranges, reqs[i].angles, reqs[i].n_beams, reqs[i].max_range,
                          results_dev + i, &pr[i], reqs[i].topk);
@@ -1920,6 +1929,7 @@ int relo_relocalize_batch(relo_ctx *ctx, const relo_request *reqs, int32_t n, re
     std::vector<float> all;   // several scans go up together
     if (n > 1) all.reserve(total);
     std::vector<Prepared> pr((size_t)n);
+    ++ctx->plan_call;
     size_t pos = 0;
     for (int i = 0; i < n && !rc; ++i) {
         rc = prepare(ctx, reqs[i].map_id, sl.ranges_dev + pos, reqs[i].angles, reqs[i].n_beams, reqs[i].max_range,
@@ -1982,6 +1992,7 @@ int relo_synth_scans_dev(relo_ctx *ctx, int32_t map_id, const int32_t *cells_dev
     if (!ctx || !cells_dev || !angles || !ranges_dev || n < 0) return fail(ctx, RELO_E_INVALID_ARG, "bad arguments");
     MapSlot *m = get_map(ctx, map_id);
     if (!m) return fail(ctx, RELO_E_NOT_FOUND, "unknown map id");
+    ++ctx->plan_call;
     SensorPlan *P = nullptr;
     int rc = plan_for(ctx, angles, n_beams, &P);
     if (rc) return rc;

@@ -467,3 +467,18 @@ def test_stages_end_with_the_scratch_they_lie_in(relo):
     assert e.value.code == relo.E_OVER_BUDGET
     stage_error(ctx)
     ctx.close()
+
+
+@pytest.mark.parametrize("scans", [33, 70])
+def test_batch_of_more_scans_than_plans_are_kept(relo, scans):
+    """A batch whose requests all have a beam grid of their own, more than the context keeps between calls: every result as
+    alone, in the batch and in a second one."""
+    wl = small_case(n_beams=110)
+    ctx = relo.Relo(n_orient=40, topk=8, batch=4, local_topk=2)
+    mid = ctx.load_map(wl.grid, RES)
+    ctx.set_hypotheses(mid, workloads.cell_centres(wl.hyps, RES))
+    reqs = [(mid, wl.ranges[:40 + i], wl.angles[:40 + i], wl.max_range) for i in range(scans)]
+    alone = [ctx.relocalize(*q).as_dict() for q in reqs]
+    for _ in range(2):
+        assert [r.as_dict() for r in ctx.relocalize_batch(reqs)] == alone
+    ctx.close()
