@@ -251,7 +251,9 @@ int relo_relocalize_batch_dev(relo_ctx *ctx, const relo_request *reqs, int32_t n
 
 /* Intermediate outputs of the last relocalization (the first request of the
  * last batch), copied to caller device memory (bytes = capacity of dst_dev;
- * the call fails if it is too small):
+ * the call fails if it is too small, and with RELO_E_NOT_FOUND when none has
+ * run or its scratch is gone: after relo_serve_stop for a served batch, or
+ * after a later call that needed more scratch than the budget leaves):
  *   RELO_STAGE_SMAD_NUM   int64 [N_h]   SMAD numerators (Eq. 20)
  *   RELO_STAGE_SMAD_M     int32 [N_h]   minimising orientation shift m
  *   RELO_STAGE_SURVIVORS  int32 [K]     hypothesis indices in SMAD order

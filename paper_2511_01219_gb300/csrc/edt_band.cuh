@@ -339,7 +339,8 @@ __global__ void __launch_bounds__(kCols / 4 * kSplit) k_edt_band(EdtTiles t, Edt
 // bits each; 8 rows, or 4 and 4 on the widest maps) and lists the groups of 4 columns of a row with a cell to do, which
 // its threads then share evenly.  A group goes outward in blocks of 4 columns as above, in 32 bits, until the next block
 // is farther than its worst cell.  (One thread per cell of a row, 512 at a time over whole rows, spent 615 us on the
-// 4096 x 4096 warehouse, whose far cells lie in one strip along its edge; this takes 150 us there, most of it beside SMAD and the top-K.)
+// 4096 x 4096 warehouse, whose far cells lie in one strip along its edge; this takes 114 us there by itself,
+// most of it beside SMAD and the top-K.)
 constexpr int kFarThreads = 256;
 constexpr int kFarNone = 30000;               // no occupied cell in the column: its square is above any distance
 constexpr int kFarList = 8 * kFarThreads;

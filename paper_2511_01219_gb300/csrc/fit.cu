@@ -2,7 +2,9 @@
 // driver once: how many CTAs of a shape an SM holds, and that the kernel may
 // use that much dynamic shared memory.  The answers depend on the device, the
 // kernel and the shape alone, so they are kept for the process (at most
-// kMaxFits of them), under a mutex: any context, stream or thread may ask.  A
+// kMaxFits of them), under a mutex: any context, stream or thread may ask (a
+// limit set once held in a second driver context of the device and after
+// cudaDeviceReset and cuDevicePrimaryCtxReset: the runtime keeps it).  A
 // batch asked the driver some 20 times, 10 to 15 us of host time that a small
 // call waits for.
 #include <cuda_runtime.h>

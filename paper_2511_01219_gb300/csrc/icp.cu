@@ -19,8 +19,9 @@
 // icp_iters iterations, when fewer than 2 pairs remain, or when the motion is
 // below 1e-9 rad and 1e-9 m.  All pose arithmetic is FP64.
 //
-// What bounds it is the FP64 rate (two lanes per clock and SM) and the chain of
-// dependent steps, so a pose is spread over as many SMs as there are to spare:
+// What bounds it is the chain of dependent steps, FP64 at two lanes per clock
+// and SM and barriers (20 poses over 160 CTAs: issue slots 4% and FP64 pipes 16%
+// busy), so a pose is spread over as many SMs as there are to spare:
 // the CTAs of a cluster share its beams, their sums meet in the first CTA's
 // shared memory, one warp there solves for the motion and writes the pose to
 // all.  With one CTA per pose whose every thread solved the motion and made its

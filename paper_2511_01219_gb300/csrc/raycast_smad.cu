@@ -466,7 +466,8 @@ __device__ __forceinline__ long long lane_sum(const uint32_t *__restrict__ row, 
 // on average x 540 to 2880 ranges: 304 us with one range per lane, 189 with
 // four (2, 4 or 5 blocks in flight instead of 6: 227, 210, 202); 20000 x 1440
 // row sums 62 and 37 us (115 MB: 17 us at the copy rate).
-// P: the type of a chunk's prefixes, 32 bits while 32 ranges fit them (kSmadNarrowLim), else 64 (one range per lane).
+// P: the type of a chunk's prefixes, 32 bits while 32 ranges fit them (kSmadNarrowLim), else 64 (one range per lane): 5000
+// hypotheses x 1440 ranges, 360 orientations, 19 us with a limit of 2040 cells, 34.5 with 2060 (973 by direct window sums).
 template <typename P>
 __global__ void __launch_bounds__(256) k_smad(const ReqDesc *__restrict__ reqs, int R, int total_hyp,
                                               BatchState *bs, int warp_bytes) {

@@ -408,9 +408,10 @@ cudaError_t launch_win_read(const ReqDesc *reqs, int R, int total, cudaStream_t 
 // the top-K of every request with its TAM work order, and beside it (extra blocks) every request's TAM endpoint offsets
 cudaError_t launch_topk(const ReqDesc *reqs, int R, int max_n_hyp, int max_K, int max_n_orient, int icp_beams,
                         int n_sm, cudaStream_t s);   // icp_beams: the most beams of a request with ICP, 0 without
-// plans the TAM launch of one batch index: fills segs[R] and returns the task count and grid size
+// the TAM launch of one batch index
 struct TamPlan {
-    int total_tasks, grid, vpl;
+    int total_tasks;           // 0: none of the requests has survivors in it, else 1 (the kernel counts the tasks)
+    int grid, vpl;
     size_t smem;
     int stages;                // staged tasks per CTA
     int lut_bytes, lut_tables; // bytes of a likelihood table with its copies; tables: one per stage or one for all
@@ -422,7 +423,6 @@ int tam_vpl_for(int max_beams);
 // launch's task counter), grid and kernel class
 TamPlan plan_tam(const int *batch_lo, const int *batch_hi, int R, int max_beams, int max_rank, int n_sm, int chunk,
                  int luts, long long poses, TamSeg *segs);
-// TAM's work order (surv_perm, tam_chunks, chunk_cnt) of every request, after the top-K
 // per-lane stride of the TAM endpoint offsets of a values-per-lane class
 int tam_offs_stride_for(int vpl);
 cudaError_t launch_tam(const ReqDesc *reqs, int R, TamSeg *segs, const TamPlan &tp, BatchState *bs, cudaStream_t s);

@@ -19,9 +19,12 @@
 //
 // What bounds it: latency, a chain of a launch, a few dependent L2 reads and
 // two or more passes of a cluster barrier per sub-batch (late in a run; while
-// the tree is small the passes follow its growth).  Taking the points one by
+// the tree is small the passes follow its growth): issue slots are 24% busy, the
+// warps wait at barriers and for shared memory.  Taking the points one by
 // one in a single warp, with three launches per sub-batch, took 72 us per
-// sub-batch on the 1024 x 1024 office (161 ms per call).
+// sub-batch on the 1024 x 1024 office (161 ms per call).  Whole calls at rho =
+// 0.6 m from six seeds, 464 to 2407 sub-batches: 34 to 219 ms then, 6.8 to 43.5
+// now (74 to 91 and 14 to 18 us per sub-batch, more as the tree grows).
 //
 // A voxel of side rho is represented by its lowest-index node; a round's gain
 // is the number of voxels it claimed, and sampling stops once a round gains at

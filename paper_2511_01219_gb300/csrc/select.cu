@@ -43,7 +43,10 @@ namespace {
 
 constexpr int kTopkThreads = 1024;
 // Keys a thread holds in registers from the one load to the last pass: up to kHold * kTopkThreads keys (20480) cost one
-// read, all its loads in flight; more are read from memory in every pass, kLoads in flight.
+// read, all its loads in flight; more are read from memory in every pass, kLoads in flight.  The two ways are near each
+// other: top-K stage, us, K = 256 / 1024: 20000 keys 20.2 / 21.8, 20480 20.7 / 22.1, 20481 22.4 / 23.7, 24000 22.7 / 24.5,
+// 40000 30.4 / 31.6 (event times step by 2 us); with 10 keys a thread, so that all of these are read again, 20.2 / 22.5,
+// 20.6 / 22.4, 20.6 / 22.6, 21.0 / 23.0 and 28.5 / 30.6.
 constexpr int kHold = 20;
 constexpr int kLoads = 8;
 

@@ -55,8 +55,11 @@ constexpr unsigned kFull = 0xffffffffu;
 // then serialise on the banks that its ranks share (3.0 to 3.2 wavefronts per lookup of 32 where 2 move the bytes,
 // counted over both workloads; 2, 4 or 8 copies of the table make it worse, since lanes with the same rank no longer
 // share a read).  With kLutCopies copies, entry by entry, each lane of a half-warp reads its own copy, which lies in its
-// own bank pair, and no lookup conflicts.  506 ranks (C = 1600) take 65 KB that way, one CTA per SM; larger clamps, maps
-// with different tables in one launch and calls too small to repay the filling keep one copy.
+// own bank pair, and no lookup conflicts.  505 ranks and the entry of no beam (C = 1600) take 65 KB that way, one CTA per
+// SM; tables whose copies do not fit, maps with different tables in one launch and calls too small to repay the filling
+// keep one.  TAM, us, with 16 copies and with one, 1024 survivors x 720 orientations x 1440 beams: C = 100 812 / 797, 400
+// 843 / 846, 1600 868 / 876, 2500 878 / 885, 3600 919 / 891, 4096 919 / 894 (their copies leave room for fewer stages),
+// 6400 and 8100 (one copy in any case) 901 and 903; 256 x 360 x 1081: C = 400 104 / 105, 1600 109 / 111, 4096 118 / 113.
 constexpr int kLutCopies = 16;
 
 // The smallest rank b in [0, C] with count_le(b) >= k, given count_le(C) = n_C >= k
